@@ -28,8 +28,10 @@
  *  - Errors: every call returns a cl_status and never aborts.  A CUDA error
  *    gives CL_ERR_CUDA; its text is kept (per thread) for cl_last_error().
  *    A lattice is not thread-safe: one host thread per lattice at a time.
- *  - Precision (cl_precision): CL_FP64 keeps links and all arithmetic in
- *    FP64.  CL_FP32_STORAGE stores and multiplies links in FP32 and keeps in
+ *  - Precision (cl_precision): CL_FP64 keeps links in FP64; its matrix
+ *    products run in 60-bit fixed point with FP32 low-order terms (errors at
+ *    or below FP64's for links near SU(3); wherever a number leaves the
+ *    fixed-point range, in FP64), the rest in FP64.  CL_FP32_STORAGE stores and multiplies links in FP32 and keeps in
  *    FP64 the matrix exponentials of the Langevin and cooling updates, the
  *    det U = 1 re-projection and every global reduction.  CL_DF64 stores
  *    links as double-float pairs (hi + lo floats, ~48 significant bits) and

@@ -111,6 +111,14 @@ cl_status ensure_stage(cl_lattice* l) {
   return CL_OK;
 }
 
+// F^ = -i theta kappa F: -i (a + ib) kappa = kappa b - i kappa a.
+double clover_scale_re(const cl_lattice* l) { return KAPPA_Q * l->p.theta_im; }
+double clover_scale_im(const cl_lattice* l) { return -KAPPA_Q * l->p.theta_re; }
+// C holds the drift contributions times 2^-e in the FP64 form's fixed point.
+int contribution_exponent(const cl_lattice* l) {
+  return l->prec == 0 ? drift_exponent(l->p.beta, clover_scale_re(l), clover_scale_im(l)) : 0;
+}
+
 bool theta_nonzero(const cl_lattice* l) { return l->p.theta_re != 0.0 || l->p.theta_im != 0.0; }
 
 // The link-inverse pass: FP64 and DF64 only (the FP32-storage kernels form
@@ -119,45 +127,46 @@ bool needs_inverse_pass(const cl_lattice* l) { return l->prec != 1; }
 
 // Link inverses, plaquettes and D = P - P^{-1}, then (theta != 0) the clover
 // field scaled by (sre + i sim), then the per-plaquette drift contributions.
-cudaError_t do_force(cl_lattice* l, bool th, double sre, double sim) {
+// ce: the contributions' exponent (contribution_exponent).
+cudaError_t do_force(cl_lattice* l, bool th, double sre, double sim, int ce) {
   cudaError_t e = cudaSuccess;
   if (needs_inverse_pass(l))
-    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Ui, l->st); });
+    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); });
   if (e == cudaSuccess)
-    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Ui, l->Pq, l->Dq, l->st); });
+    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); });
   if (e == cudaSuccess && th)
     e = timed(l, CL_PHASE_CLOVER, [&] {
-      return launch_clover_rot(l->prec, l->g, l->U, l->Ui, l->Dq, l->F, sre, sim, l->st);
+      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->F, ldexp(sre, -ce), ldexp(sim, -ce), l->st);
     });
   if (e == cudaSuccess)
     e = timed(l, CL_PHASE_FORCE, [&] {
-      return launch_plaq_force(l->prec, th, l->g, l->U, l->Ui, l->Pq, l->Dq, l->F, l->Gq, l->C, l->p.beta,
-                               l->st);
+      return launch_plaq_force(l->prec, th, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->F, l->Gq, l->C, l->p.beta,
+                               ce, l->st);
     }, (th && l->prec != 1) ? 2 : 1);  // FP64 and DF64 split the theta force in two kernels
   return e;
 }
 
 cl_status do_steps(cl_lattice* l, double eps, int n) {
   const bool th = theta_nonzero(l);
-  // F^ = -i theta kappa F: -i (a + ib) kappa = kappa b - i kappa a
-  const double sre = KAPPA_Q * l->p.theta_im, sim = -KAPPA_Q * l->p.theta_re;
+  const double sre = clover_scale_re(l), sim = clover_scale_im(l);
+  const int ce = contribution_exponent(l);
   for (int i = 0; i < n; ++i) {
-    CK(do_force(l, th, sre, sim));
+    CK(do_force(l, th, sre, sim, ce));
     const bool adaptive = l->k_ref > 0.0;
     if (adaptive) {
       // drift into the plaquette buffer (dead once the force has run) with
       // max |K|, then the step size on the device, then the update from the
       // stored drift
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 2, l->g, l->U, l->C, l->Pq, eps, l->p.seed, l->sd, false, l->st);
+        return launch_update_gather(l->prec, 2, l->g, l->U, l->C, l->Pq, eps, l->p.seed, l->sd, false, ce, l->st);
       }));
       CK(timed(l, CL_PHASE_UPDATE, [&] { return launch_step_eps(l->sd, eps, l->k_ref, l->st); }));
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 3, l->g, l->U, l->Pq, l->Un, eps, l->p.seed, l->sd, true, l->st);
+        return launch_update_gather(l->prec, 3, l->g, l->U, l->Pq, l->Un, eps, l->p.seed, l->sd, true, ce, l->st);
       }));
     } else {
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 0, l->g, l->U, l->C, l->Un, eps, l->p.seed, l->sd, false, l->st);
+        return launch_update_gather(l->prec, 0, l->g, l->U, l->C, l->Un, eps, l->p.seed, l->sd, false, ce, l->st);
       }));
     }
     // one-thread bookkeeping kernel: counted as a launch, not timed (so the update
@@ -251,9 +260,9 @@ cl_status do_cool(cl_lattice* l, const cl_cool_params* cp) {
 
 cl_status do_obs(cl_lattice* l, ObsOut* dst, double* q_site) {
   if (needs_inverse_pass(l))
-    CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Ui, l->st); }));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Ui, l->Pq, l->Dq, l->st); }));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_clover_rot(l->prec, l->g, l->U, l->Ui, l->Dq, l->F, 1.0, 0.0, l->st); }));
+    CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] { return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->F, obs_clover_scale(l->prec), 0.0, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->F, 1, l->partials, q_site, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
     return launch_obs_final(l->g, l->partials, l->p.beta, l->p.theta_re, l->p.theta_im, dst, l->st);
@@ -639,8 +648,9 @@ cl_status cl_drift(cl_lattice* l, double* host_aos) {
   cl_status s = ensure_stage(l);
   if (s != CL_OK) return s;
   const bool th = theta_nonzero(l);
-  CK(do_force(l, th, KAPPA_Q * l->p.theta_im, -KAPPA_Q * l->p.theta_re));
-  CK(launch_update_gather(l->prec, 1, l->g, l->U, l->C, l->Un, 0.0, l->p.seed, l->sd, false, l->st));
+  const int ce = contribution_exponent(l);
+  CK(do_force(l, th, clover_scale_re(l), clover_scale_im(l), ce));
+  CK(launch_update_gather(l->prec, 1, l->g, l->U, l->C, l->Un, 0.0, l->p.seed, l->sd, false, ce, l->st));
   CK(launch_soa_to_aos(l->prec, l->g, l->Un, l->stage, 4, l->st));
   l->launches += 2;
   CK(cudaMemcpyAsync(host_aos, l->stage, sizeof(double) * 18 * 4 * (size_t)l->g.V,
@@ -979,8 +989,9 @@ ChainDesc describe(const cl_lattice* l, double eps, const cl_cool_params& cp, bo
   c.cs = l->cs;
   c.sd = l->sd;
   c.beta = l->p.beta;
-  c.sre = KAPPA_Q * l->p.theta_im;  // F^ = -i theta kappa F, as in do_steps
-  c.sim = -KAPPA_Q * l->p.theta_re;
+  c.cexp = contribution_exponent(l);  // as in do_steps
+  c.sre = ldexp(clover_scale_re(l), -c.cexp);
+  c.sim = ldexp(clover_scale_im(l), -c.cexp);
   c.eps = eps;
   c.sqrt_eps = sqrt(eps);
   c.k_ref = l->k_ref;

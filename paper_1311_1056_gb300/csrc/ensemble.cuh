@@ -7,6 +7,7 @@
 // k_update_f32.cu, which instantiate it for their link type.
 #pragma once
 #include "k_update.cuh"
+#include "k_update_fx.cuh"
 #include "launch.h"
 
 namespace clgc {
@@ -22,61 +23,78 @@ __device__ __forceinline__ Geo geo_of(const ChainDesc& c) {
   return g;
 }
 
+// Blocks per SM the link-algebra kernels are built for: the FP64 form's as its
+// single-chain kernels (FX_MAXNREG, k_update_f64.cu).
+#define ENS_MIN_BLOCKS(T) (std::is_same<T, double>::value ? 3 : 1)
+
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_inverse(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_link_inverse_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Ui, it.vb);
+  if constexpr (std::is_same<T, double>::value)
+    fx_links_body(geo_of(c), (const V2*)c.U, (int4*)c.Un, (int4*)c.Ui, it.vb);
+  else
+    k_link_inverse_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Ui, it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_plaq(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const ChainDesc* __restrict__ cd,
                                                              const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_plaq_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (V2*)c.Pq, (V2*)c.Dq, it.vb);
+  if constexpr (std::is_same<T, double>::value)
+    fx_plaq_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, it.vb);
+  else
+    k_plaq_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (V2*)c.Pq, (V2*)c.Dq, it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_clover(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(const ChainDesc* __restrict__ cd,
                                                                const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
+  if constexpr (std::is_same<T, double>::value)
+    fx_clover_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.F,
+                   c.sre, c.sim, it.vb);
+  else
+    k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_force_wilson(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_wilson(const ChainDesc* __restrict__ cd,
                                                                      const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_plaq_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.C,
+  if constexpr (std::is_same<T, double>::value)
+    fx_force_wilson_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C,
+                         ldexp(c.beta / 6.0, -c.cexp), it.vb);
+  else
+    k_plaq_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.C,
                               (T)(c.beta / 6.0), it.vb);
 }
 
+// FP64: the theta force's two kernels
 template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_force_a(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_a(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
-  typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_plaq_force_a_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (const V2*)c.F, (V2*)c.Gq,
-                         (V2*)c.C, (T)(c.beta / 6.0), it.vb);
+  fx_force_a_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (const int4*)c.F, (int4*)c.Gq,
+                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_force_b(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_b(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
-  typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_plaq_force_b_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Pq, (const V2*)c.Dq,
-                         (const V2*)c.F, (const V2*)c.Gq, (V2*)c.C, (T)(c.beta / 6.0), it.vb);
+  fx_force_b_body(geo_of(c), (const double2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
+                  (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), it.vb);
 }
 
 template <typename T>
@@ -100,6 +118,7 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_update(const ChainDesc* 
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   UpdArgs a;
+  a.cexp = c.cexp;
   a.beta = 0.0;
   a.eps = c.eps;
   a.sqrt_eps = c.sqrt_eps;

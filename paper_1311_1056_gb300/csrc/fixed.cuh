@@ -1,0 +1,363 @@
+// fixed.cuh -- 60-bit fixed-point 3x3 complex algebra on the integer and FP32
+// pipes, the arithmetic of the FP64 form's matrix products.
+//
+// Why: GB300 issues 2 FP64 multiply-adds per SM and clock.  Links, plaquettes
+// and everything the CL step derives from them are numbers of order one, which
+// is what fixed point is for.  A number is
+//   x = (h 2^30 + l) 2^-60,   h an int, l a float (an integer, |l| <= 2^29),
+// and a product splits by size:
+//   x y = h h' 2^-60 + (h l' + l h') 2^-90 + l l' 2^-120.
+// The first term is exact in 64 bits (IMAD.WIDE) and sums without rounding;
+// the second is below 2^-30 of the first, so float (one packed FFMA2 for its
+// two products) carries it to ~2^-56; the third is below 2^-62 and dropped.
+// A 3x3 product takes ~1,390 cycles of a scheduler and warp against ~7,500 in
+// FP64 (and 1,870 with both limbs integers), and its error is smaller: rms
+// 2.4e-17 against 3.6e-17 for random SU(3) factors, 4.8e-17 against 7.2e-17
+// after four products (FP64 rounds each of its six partial sums).
+//
+// Ranges.  |x| < FX_BOUND = 1.4375 holds for every operand and stored number:
+// a sum of six products and one summand then stays below 16 - FX_BOUND, and
+// as sums wrap at 16 a result that is out of bounds cannot look as if it were
+// in.  Every result is checked (fx_chk).  A matrix that does not fit (a
+// runaway field, NaN) is stored as plain doubles instead, marked in its first
+// word (fx_is_raw); a thread that meets one, or whose own results do not fit,
+// redoes its work in FP64 (the general path).
+#pragma once
+#include "su3.cuh"
+
+namespace clgc {
+
+// a b + c and a b.  Written in C++ the sums of products are reassociated and
+// cost twice the instructions.
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+typedef unsigned long long fx_pair;  // two packed floats
+__device__ __forceinline__ fx_pair fx_pack(float a, float b) {
+  fx_pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ fx_pair fx_fma2(fx_pair a, fx_pair b, fx_pair c) {
+  fx_pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Range check: the largest of the results' high words, offset to be unsigned.
+// WIDE: |x| < 1.4375; NARROW: |x| < 0.359375, for results that are added to
+// others before their next use.
+enum { FX_WIDE = 0, FX_NARROW = 1 };
+struct fx_chk {
+  unsigned m0, m1;
+  __device__ __forceinline__ fx_chk() : m0(0), m1(0) {}
+  template <int B>
+  __device__ __forceinline__ void see(int hi) {  // hi: units of 2^-28
+    if (B == FX_WIDE)
+      m0 = max(m0, (unsigned)hi + 0x17000000u);
+    else
+      m1 = max(m1, (unsigned)hi + 0x05C00000u);
+  }
+  __device__ __forceinline__ void fail() { m0 = 0xffffffffu; }
+  __device__ __forceinline__ bool bad() const { return m0 >= 0x2E000000u || m1 >= 0x0B800000u; }
+};
+
+__device__ __forceinline__ fx operator-(fx a) { return fx{-a.l, -a.h}; }
+__device__ __forceinline__ fx operator+(fx a, fx b) { return fx{a.l + b.l, a.h + b.h}; }
+__device__ __forceinline__ fx operator-(fx a, fx b) { return fx{a.l - b.l, a.h - b.h}; }
+__device__ __forceinline__ fx fx_twice(fx a) { return fx{2.0f * a.l, 2 * a.h}; }
+
+// The 60-bit integer of a number, and back.
+__device__ __forceinline__ long long fx_bits(fx a) { return mad_wide(a.h, 1 << 30, (long long)__float2int_rn(a.l)); }
+// r carries an offset of 2^29, which makes the truncating split a balanced one.
+__device__ __forceinline__ fx fx_split(long long r) {
+  return fx{(float)(((int)r & ((1 << 30) - 1)) - (1 << 29)), (int)(r >> 30)};
+}
+__device__ __forceinline__ fx fx_of_bits(long long v) { return fx_split(v + (1 << 29)); }
+
+// Operands: left factors carry (h, l) as floats, right factors (l, h).
+struct fx_left {
+  int h;
+  fx_pair p;
+};
+struct fx_right {
+  int h;
+  fx_pair p;
+};
+__device__ __forceinline__ fx_left fx_lhs(fx a) { return fx_left{a.h, fx_pack((float)a.h, a.l)}; }
+__device__ __forceinline__ fx_left fx_lhs_neg(fx a) { return fx_left{-a.h, fx_pack(-(float)a.h, -a.l)}; }
+__device__ __forceinline__ fx_right fx_rhs(fx a) { return fx_right{a.h, fx_pack(a.l, (float)a.h)}; }
+struct fx_cleft {
+  fx_left re, im, nim;  // nim = -im
+};
+struct fx_cright {
+  fx_right re, im;
+};
+__device__ __forceinline__ fx_cleft fx_lhs(cx<fx> a) { return fx_cleft{fx_lhs(a.re), fx_lhs(a.im), fx_lhs_neg(a.im)}; }
+__device__ __forceinline__ fx_cleft fx_lhs_neg(cx<fx> a) { return fx_cleft{fx_lhs_neg(a.re), fx_lhs_neg(a.im), fx_lhs(a.im)}; }
+__device__ __forceinline__ fx_cright fx_rhs(cx<fx> a) { return fx_cright{fx_rhs(a.re), fx_rhs(a.im)}; }
+
+// Accumulator of a sum of products: a in units of 2^-60, c (two partial sums) of 2^-90.
+struct fx_acc {
+  long long a;
+  fx_pair c;
+};
+__device__ __forceinline__ fx_acc fx_zero() { return fx_acc{0, 0ull}; }
+// S: the summand times 2^-S
+template <int S = 0>
+__device__ __forceinline__ fx_acc fx_from(fx c) {
+  return fx_acc{mad_wide(c.h, 1 << (30 - S), 0), fx_pack(c.l * (float)(1 << (30 - S)), 0.0f)};
+}
+__device__ __forceinline__ void fx_mac(fx_acc& s, const fx_left& x, const fx_right& y) {
+  s.a = mad_wide(x.h, y.h, s.a);
+  s.c = fx_fma2(x.p, y.p, s.c);
+}
+__device__ __forceinline__ void fx_cmac(fx_acc& re, fx_acc& im, const fx_cleft& a, const fx_cright& b) {
+  fx_mac(re, a.re, b.re);
+  fx_mac(im, a.re, b.im);
+  fx_mac(re, a.nim, b.im);
+  fx_mac(im, a.im, b.re);
+}
+// The sum as a 60-bit integer with an offset of 2^29: the small terms are
+// rounded to 2^-57 (in range for any operands within bounds) and folded in.
+__device__ __forceinline__ long long fx_sum(const fx_acc& s) {
+  float c0, c1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(s.c));
+  return mad_wide(__float2int_rn((c0 + c1) * 0x1p-33f) + (1 << 26), 8, s.a);
+}
+// The result times 2^-S, within bound B.
+template <int B, int S = 0>
+__device__ __forceinline__ fx fx_get(const fx_acc& s, fx_chk& ck) {
+  long long r = fx_sum(s);
+  if (S) r = (r >> S) + ((1 << 29) - (1 << (29 - S)));
+  ck.see<B>((int)(r >> 32));
+  return fx_split(r);
+}
+
+// The products run row by row in a rolled loop, the rows of the operands
+// passing through the same registers (rotated by one row each time, so that no
+// register is indexed): unrolled, the theta force is 120 KB of code and its
+// warps wait on instruction fetch (12.5 against 8.6 ms per 32^4 step with
+// integer limbs).
+__device__ __forceinline__ void fx_rotate(mat<fx>& a, const cx<fx>* last) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) a.e[k] = a.e[k + 3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) a.e[6 + k] = last[k];
+}
+struct fx_rmat {
+  fx_cright e[9];
+};
+__device__ __forceinline__ void fx_rhs(fx_rmat& r, const mat<fx>& b) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) r.e[k] = fx_rhs(b.e[k]);
+}
+// a <- 2^-S a b
+template <int B, int S = 0>
+__device__ __forceinline__ void fx_mul_left(mat<fx>& a, const mat<fx>& b, fx_chk& ck) {
+  fx_rmat y;
+  fx_rhs(y, b);
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {
+    fx_cleft x[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[k] = fx_lhs(a.e[k]);
+    cx<fx> r[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      fx_acc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(re, im, x[k], y.e[3 * k + j]);
+      r[j] = cx<fx>{fx_get<B, S>(re, ck), fx_get<B, S>(im, ck)};
+    }
+    fx_rotate(a, r);
+  }
+}
+// c <- 2^-S c + a b (SIGN > 0) or 2^-S c - a b.  Here and in fx_adj the rows
+// (columns) of a have gone round once at the end: a is what it was, without a
+// second copy.
+template <int B, int SIGN, int S = 0>
+__device__ __forceinline__ void fx_mul_acc(mat<fx>& c, mat<fx>& a, const mat<fx>& b, fx_chk& ck) {
+  fx_rmat y;
+  fx_rhs(y, b);
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {
+    cx<fx> r[3];
+    fx_cleft x[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[k] = SIGN < 0 ? fx_lhs_neg(a.e[k]) : fx_lhs(a.e[k]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      fx_acc re = fx_from<S>(c.e[j].re), im = fx_from<S>(c.e[j].im);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(re, im, x[k], y.e[3 * k + j]);
+      r[j] = cx<fx>{fx_get<B>(re, ck), fx_get<B>(im, ck)};
+    }
+    fx_rotate(c, r);
+    const cx<fx> z[3] = {a.e[0], a.e[1], a.e[2]};
+    fx_rotate(a, z);
+  }
+}
+// r = s a, s real
+template <int B>
+__device__ __forceinline__ void fx_scaled(mat<fx>& r, const mat<fx>& a, fx s, fx_chk& ck) {
+  const fx_left x = fx_lhs(s);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    fx_acc re = fx_zero(), im = fx_zero();
+    fx_mac(re, x, fx_rhs(a.e[k].re));
+    fx_mac(im, x, fx_rhs(a.e[k].im));
+    r.e[k] = cx<fx>{fx_get<B>(re, ck), fx_get<B>(im, ck)};
+  }
+}
+// c += [a, b]
+template <int B>
+__device__ __forceinline__ void fx_commutator_acc(mat<fx>& c, mat<fx>& a, mat<fx>& b, fx_chk& ck) {
+  fx_mul_acc<B, +1>(c, a, b, ck);
+  fx_mul_acc<B, -1>(c, b, a, ck);
+}
+// c = [a, b] + s a, s real
+template <int B>
+__device__ __forceinline__ void fx_commutator(mat<fx>& c, mat<fx>& a, mat<fx>& b, fx s, fx_chk& ck) {
+  fx_scaled<B>(c, a, s, ck);
+  fx_commutator_acc<B>(c, a, b, ck);
+}
+
+// Adjugate (the inverse of a matrix of determinant one): row i of r from
+// columns i + 1 and i + 2 of a, which rotate through the same registers.
+__device__ __forceinline__ void fx_adj(mat<fx>& r, mat<fx>& a, fx_chk& ck) {
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {
+    cx<fx> row[3];
+    fx_cright u[3], v[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      u[j] = fx_rhs(a.e[3 * j + 1]);
+      v[j] = fx_rhs(a.e[3 * j + 2]);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+      fx_acc re = fx_zero(), im = fx_zero();
+      fx_cmac(re, im, fx_lhs(a.e[3 * j1 + 1]), v[j2]);
+      fx_cmac(re, im, fx_lhs_neg(a.e[3 * j1 + 2]), u[j2]);
+      row[j] = cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
+    }
+    fx_rotate(r, row);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const cx<fx> z = a.e[3 * j];
+      a.e[3 * j] = a.e[3 * j + 1];
+      a.e[3 * j + 1] = a.e[3 * j + 2];
+      a.e[3 * j + 2] = z;
+    }
+  }
+}
+
+__device__ __forceinline__ void fx_add(mat<fx>& c, const mat<fx>& a) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) c.e[k] = cx<fx>{c.e[k].re + a.e[k].re, c.e[k].im + a.e[k].im};
+}
+// c <- 2 c + SIGN a
+template <int SIGN>
+__device__ __forceinline__ void fx_twice_add(mat<fx>& c, const mat<fx>& a) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const cx<fx> t = {fx_twice(c.e[k].re), fx_twice(c.e[k].im)};
+    c.e[k] = SIGN > 0 ? cx<fx>{t.re + a.e[k].re, t.im + a.e[k].im} : cx<fx>{t.re - a.e[k].re, t.im - a.e[k].im};
+  }
+}
+
+// ---------------------------------------------------------- conversions
+// Double to fixed point, rounded to nearest (ties away).  Only |x| < 2 has an
+// image; `mag` collects the magnitudes' high words for the caller's check.
+__device__ __forceinline__ long long fx_bits_of_double(double x, unsigned& mag) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  mag = max(mag, (unsigned)hi & 0x7fffffffu);
+  const int e = (hi >> 20) & 0x7ff;
+  // significand with its leading one at bit 62; x 2^60 = m 2^(e - 1025)
+  const unsigned mh = (__funnelshift_l(lo, (unsigned)hi, 10) & 0x3fffffffu) | 0x40000000u;
+  const unsigned long long m = ((unsigned long long)mh << 32) | (lo << 10);
+  const int r = max(min(1024 - e, 63), 0);
+  const long long v = (long long)(((m >> r) + 1) >> 1);
+  const long long s = (long long)(hi >> 31);
+  return (v ^ s) - s;
+}
+__device__ __forceinline__ fx fx_of_double(double x, unsigned& mag) { return fx_of_bits(fx_bits_of_double(x, mag)); }
+// Whether the largest magnitude seen is below FX_BOUND (false for NaN and Inf).
+__device__ __forceinline__ bool fx_mag_ok(unsigned mag) { return mag < 0x3FF70000u; }  // 1.4375
+
+// v 2^(e - 60) as a double, rounded to nearest even.
+__device__ __forceinline__ double fx_bits_to_double(long long v, int e = 0) {
+  const unsigned long long s = (unsigned long long)(v >> 63);
+  const unsigned long long m = ((unsigned long long)v ^ s) - s;
+  const int lz = __clzll((long long)m);
+  const unsigned long long n = m << (lz & 63);
+  unsigned long long q = n >> 11;
+  const unsigned rem = (unsigned)n & 0x7ffu;
+  q += (rem + ((unsigned)q & 1u)) > 0x400u ? 1u : 0u;
+  q += (unsigned long long)(1023 + 63 - 60 - 1 + e - lz) << 52;
+  q = m ? q : 0ull;
+  return __longlong_as_double((long long)(q | (s << 63)));
+}
+__device__ __forceinline__ double fx_to_double(fx a, int e = 0) { return fx_bits_to_double(fx_bits(a), e); }
+
+// -------------------------------------------------- stored 64-bit words
+// A matrix is stored as fixed-point words (l, h) or, all 18 of them, as
+// doubles.  Which one it is shows in its first word alone: l of a stored
+// number is below 2^31 in magnitude; the first double is stored times 2^400,
+// its high word first, which read as a float is above.  Doubles outside
+// 2^-150 .. 2^500 are stored there as 2^-150 and NaN (one has lost all meaning
+// next to the entries of a matrix of determinant one, the other overflows in
+// the next product).
+__device__ __forceinline__ bool fx_is_raw(float l) { return (__float_as_uint(l) & 0x7fffffffu) >= 0x4F000000u; }
+__device__ __forceinline__ float fx_raw_mark() { return __uint_as_float(0x7ff80000u); }
+
+__device__ __forceinline__ void fx_load(mat<fx>& a, const int4* __restrict__ f, int plane, int site, int V, fx_chk& ck) {
+  load<fx>(a, f, plane, site, V);
+  if (fx_is_raw(a.e[0].re.l)) ck.fail();
+}
+
+// The general path's view of such a field; its numbers are the field's times sc.
+struct tagged {
+  int4* p;
+  double sc;
+};
+__device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int site, int V) {
+  const int4* p = f.p + (size_t)plane * 9 * V + site;
+  const bool raw = fx_is_raw(__int_as_float(p[0].x));
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int4 v = p[(size_t)k * V];
+    if (raw) {
+      a.e[k] = cx<double>{__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
+      if (k == 0) a.e[0].re = __hiloint2double(v.x, v.y) * 0x1p-400;
+    } else {
+      const cx<fx> w = unpack(v);
+      a.e[k] = cx<double>{fx_to_double(w.re), fx_to_double(w.im)};
+    }
+    a.e[k].re *= f.sc;
+    a.e[k].im *= f.sc;
+  }
+}
+__device__ __forceinline__ void store(tagged f, int plane, int site, int V, const mat<double>& a) {
+  int4* p = f.p + (size_t)plane * 9 * V + site;
+  const double isc = 1.0 / f.sc;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    double re = a.e[k].re * isc, im = a.e[k].im * isc;
+    int4 v = make_int4(__double2loint(re), __double2hiint(re), __double2loint(im), __double2hiint(im));
+    if (k == 0) {
+      if (fabs(re) < 0x1p-150) re = 0x1p-150;
+      re = fabs(re) < 0x1p500 ? re * 0x1p400 : __longlong_as_double(0x7ff8000000000000ll);
+      v.x = __double2hiint(re);
+      v.y = __double2loint(re);
+    }
+    p[(size_t)k * V] = v;
+  }
+}
+
+}  // namespace clgc

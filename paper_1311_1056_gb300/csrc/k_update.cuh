@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "expm.cuh"
+#include "fixed.cuh"
 #include "lattice.cuh"
 #include "launch.h"
 #include "philox.cuh"
@@ -49,7 +50,12 @@ struct UpdArgs {
   uint64_t seed;
   StepDev* sd;    // device-resident step state (graph-replayable)
   int adaptive;   // 1: the step size is sd->eps_n (set by the drift pass)
+  int cexp;       // FP64: C holds the contributions times 2^-cexp (drift_exponent)
 };
+
+// FP64 form (k_update_fx.cuh): the drift of link (s, MU) from the fixed-point contributions.
+__device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
+                                           const double2* C, int cexp);
 
 // Sign flip on the integer pipe (no floating-point instruction).
 __device__ __forceinline__ double flip(double x, unsigned long long m) {
@@ -61,9 +67,8 @@ __device__ __forceinline__ float flip(float x, unsigned long long m) {
 __device__ __forceinline__ df64 flip(df64 x, unsigned long long m) {
   return df64(flip(x.hi, m), flip(x.lo, m));
 }
-template <typename T>
-__device__ __forceinline__ void load_signed(mat<T>& G, const typename vec2_of<T>::type* F, int p,
-                                            int s, int V, unsigned long long m) {
+template <typename T, class FF>
+__device__ __forceinline__ void load_signed(mat<T>& G, FF F, int p, int s, int V, unsigned long long m) {
   load(G, F, p, s, V);
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -79,6 +84,10 @@ __device__ __forceinline__ void load_rw(mat<T>& a, const typename vec2_of<T>::ty
   const typename vec2_of<T>::type* p = f + (size_t)plane * 9 * V + site;
 #pragma unroll
   for (int k = 0; k < 9; ++k) a.e[k] = unpack(p[(size_t)k * V]);
+}
+
+__device__ __forceinline__ void load_rw(mat<double>& a, tagged f, int plane, int site, int V) {
+  load(a, f, plane, site, V);
 }
 
 // c += [a, b] = a b - b a
@@ -125,10 +134,10 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_link_inverse(Geo g, const ty
 // kernel reads anyway.
 template <typename T>
 __host__ __device__ constexpr bool inverse_on_the_fly() { return sizeof(T) == 4; }
-template <typename T>
-__device__ __forceinline__ void load_inv(mat<T>& ui, const typename vec2_of<T>::type* __restrict__ U,
-                                         const typename vec2_of<T>::type* __restrict__ Ui, int mu, int site, int V) {
-  if constexpr (inverse_on_the_fly<T>()) {
+struct no_inverse {};  // in place of the U^{-1} field: form it from the link
+template <typename T, class FU, class FI>
+__device__ __forceinline__ void load_inv(mat<T>& ui, FU U, FI Ui, int mu, int site, int V) {
+  if constexpr (inverse_on_the_fly<T>() || std::is_same<FI, no_inverse>::value) {
     mat<T> u;
     load(u, U, mu, site, V);
     adj(ui, u);
@@ -140,11 +149,11 @@ __device__ __forceinline__ void load_inv(mat<T>& ui, const typename vec2_of<T>::
 // ------------------------------------------------------------- plaquettes
 // P_{mu nu}(x) = U_mu(x) U_nu(x+mu) U_mu(x+nu)^{-1} U_nu(x)^{-1} and
 // D = P - P^{-1}, six planes per site.
-template <typename T>
-__device__ __forceinline__ void k_plaq_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                              const typename vec2_of<T>::type* __restrict__ Ui,
-                                              typename vec2_of<T>::type* __restrict__ Pq,
-                                              typename vec2_of<T>::type* __restrict__ Dq, int vb) {
+template <typename T, class FU, class FUi, class FPq, class FDq>
+__device__ __forceinline__ void k_plaq_body(Geo g, FU U,
+                                              FUi Ui,
+                                              FPq Pq,
+                                              FDq Dq, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -180,11 +189,11 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq(Geo g, const typename v
 //   L4 = U_nu(x-nu)^{-1} P(x-nu) U_nu(x-nu),
 //   L3 = W^{-1} P(x-mu-nu) W with W = U_mu(x-mu-nu) U_nu(x-nu),
 // so F = D(x) + the three carried D's.  Stored times a complex scale.
-template <typename T>
-__device__ __forceinline__ void k_clover_rot_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                    const typename vec2_of<T>::type* __restrict__ Ui,
-                                                    const typename vec2_of<T>::type* __restrict__ Dq,
-                                                    typename vec2_of<T>::type* __restrict__ F,
+template <typename T, class FU, class FUi, class FDq, class FF>
+__device__ __forceinline__ void k_clover_rot_body(Geo g, FU U,
+                                                    FUi Ui,
+                                                    FDq Dq,
+                                                    FF F,
                                                     double sre, double sim, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
@@ -232,14 +241,12 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_clover_rot(Geo g, const type
 // C[4p + slot]: slot 0 U_mu(x), 1 U_nu(x), 2 U_nu(x+mu), 3 U_mu(x+nu).
 // With theta the work has two stages: a handles corners c0..c2 (G0 + G1^ +
 // G2^ and the slot 0 / slot 2 partials, parked in C); b adds corner c3, forms
-// K and completes the four slots.  In FP64 (36 registers per matrix) the
-// stages run as two kernels with the partial G^ parked in Gq, so neither
-// spills; in FP32 one kernel runs both.
-template <typename T>
-__device__ __forceinline__ void k_plaq_force_wilson_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                           const typename vec2_of<T>::type* __restrict__ Ui,
-                                                           const typename vec2_of<T>::type* __restrict__ Dq,
-                                                           typename vec2_of<T>::type* C, T beta6, int vb) {
+// K and completes the four slots.
+template <typename T, class FU, class FUi, class FDq, class FC>
+__device__ __forceinline__ void k_plaq_force_wilson_body(Geo g, FU U,
+                                                           FUi Ui,
+                                                           FDq Dq,
+                                                           FC C, T beta6, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -270,15 +277,16 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq_force_wilson(Geo g, con
 }
 
 // Corners c0..c2: G^ (partial) into Gh, slot 0 and slot 2 partials into C.
-template <typename T>
+template <typename T, class FU, class FUi, class FDq, class FF, class FC>
 __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, const int x[4], int p,
-                                              const typename vec2_of<T>::type* __restrict__ U,
-                                              const typename vec2_of<T>::type* __restrict__ Ui,
-                                              const typename vec2_of<T>::type* __restrict__ Dq,
-                                              const typename vec2_of<T>::type* __restrict__ F,
-                                              typename vec2_of<T>::type* C, T beta6) {
+                                              FU U,
+                                              FUi Ui,
+                                              FDq Dq,
+                                              FF F,
+                                              FC C, T beta6) {
   const int mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
-  const unsigned long long m = (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
+  // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
+  const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c1 = hop(g, s, x, mu, 1);
   Work<T, 4> ws(1);  // slot 0 holds Gh
   mat<T>&D = ws[0], &M = ws[1], &t = ws[2], &q = ws[3];
@@ -311,16 +319,17 @@ __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, c
 }
 
 // Corner c3, K, and the four slots completed; Gh holds the stage-a sum.
-template <typename T>
+template <typename T, class FU, class FUi, class FPq, class FDq, class FF, class FC>
 __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, const int x[4], int p,
-                                              const typename vec2_of<T>::type* __restrict__ U,
-                                              const typename vec2_of<T>::type* __restrict__ Ui,
-                                              const typename vec2_of<T>::type* __restrict__ Pq,
-                                              const typename vec2_of<T>::type* __restrict__ Dq,
-                                              const typename vec2_of<T>::type* __restrict__ F,
-                                              typename vec2_of<T>::type* C, T beta6) {
+                                              FU U,
+                                              FUi Ui,
+                                              FPq Pq,
+                                              FDq Dq,
+                                              FF F,
+                                              FC C, T beta6) {
   const int mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
-  const unsigned long long m = (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
+  // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
+  const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c3 = hop(g, s, x, nu, 1);
   Work<T, 4> ws(1);  // slot 0 holds Gh
   mat<T>&D = ws[0], &M = ws[1], &t = ws[2], &q = ws[3];
@@ -379,75 +388,22 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
   store(C, 4 * p + 3, s, g.V, M);
 }
 
-// Split form (FP64): stage a, G^ parked in Gq, stage b.  Gq is not a buffer
-// of its own: the partial of plaquette (p, s) sits in plane 4p + 1 of C (Gq
-// points at plane 1 of C, so Gq plane GQ_PLANE * p is C plane 4p + 1), the
-// slot-1 contribution of that same plaquette, which only stage b writes, and
-// only after the same thread has read the partial back.  Gq and C may alias,
-// so neither carries __restrict__ and stage b reads Gq with a plain load.
+// The FP64 and DF64 forms run the stages as two kernels, the partial G^ parked
+// in Gq.  Gq is not a buffer of its own: the partial of plaquette (p, s) sits
+// in plane 4p + 1 of C (Gq points at plane 1 of C, so Gq plane GQ_PLANE * p is
+// C plane 4p + 1), the slot-1 contribution of that same plaquette, which only
+// stage b writes, and only after the same thread has read the partial back.
+// Gq and C may alias, so neither carries __restrict__ and stage b reads Gq
+// with a plain load.
 const int GQ_PLANE = 4;
-template <typename T>
-__device__ __forceinline__ void k_plaq_force_a_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      const typename vec2_of<T>::type* __restrict__ Ui,
-                                                      const typename vec2_of<T>::type* __restrict__ Dq,
-                                                      const typename vec2_of<T>::type* __restrict__ F,
-                                                      typename vec2_of<T>::type* Gq,
-                                                      typename vec2_of<T>::type* C, T beta6, int vb) {
-  const int p = vb % 6;
-  const int s = (vb / 6) * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  int x[4];
-  site_coords(g, s, x);
-  Work<T, 1> wg(0);
-  mat<T>& Gh = wg[0];
-  force_stage_a(Gh, g, s, x, p, U, Ui, Dq, F, C, beta6);
-  store(Gq, GQ_PLANE * p, s, g.V, Gh);
-}
-template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq_force_a(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      const typename vec2_of<T>::type* __restrict__ Ui,
-                                                      const typename vec2_of<T>::type* __restrict__ Dq,
-                                                      const typename vec2_of<T>::type* __restrict__ F,
-                                                      typename vec2_of<T>::type* Gq,
-                                                      typename vec2_of<T>::type* C, T beta6) {
-  k_plaq_force_a_body<T>(g, U, Ui, Dq, F, Gq, C, beta6, blockIdx.x);
-}
-template <typename T>
-__device__ __forceinline__ void k_plaq_force_b_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      const typename vec2_of<T>::type* __restrict__ Ui,
-                                                      const typename vec2_of<T>::type* __restrict__ Pq,
-                                                      const typename vec2_of<T>::type* __restrict__ Dq,
-                                                      const typename vec2_of<T>::type* __restrict__ F,
-                                                      const typename vec2_of<T>::type* Gq,
-                                                      typename vec2_of<T>::type* C, T beta6, int vb) {
-  const int p = vb % 6;
-  const int s = (vb / 6) * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  int x[4];
-  site_coords(g, s, x);
-  Work<T, 1> wg(0);
-  mat<T>& Gh = wg[0];
-  load_rw(Gh, Gq, GQ_PLANE * p, s, g.V);  // before stage b writes slot 1 of (p, s) over it
-  force_stage_b(Gh, g, s, x, p, U, Ui, Pq, Dq, F, C, beta6);
-}
-template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq_force_b(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      const typename vec2_of<T>::type* __restrict__ Ui,
-                                                      const typename vec2_of<T>::type* __restrict__ Pq,
-                                                      const typename vec2_of<T>::type* __restrict__ Dq,
-                                                      const typename vec2_of<T>::type* __restrict__ F,
-                                                      const typename vec2_of<T>::type* Gq,
-                                                      typename vec2_of<T>::type* C, T beta6) {
-  k_plaq_force_b_body<T>(g, U, Ui, Pq, Dq, F, Gq, C, beta6, blockIdx.x);
-}
-// Fused form (FP32, which needs no split to stay in registers).
-template <typename T>
-__device__ __forceinline__ void k_plaq_force_ab_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                       const typename vec2_of<T>::type* __restrict__ Ui,
-                                                       const typename vec2_of<T>::type* __restrict__ Pq,
-                                                       const typename vec2_of<T>::type* __restrict__ Dq,
-                                                       const typename vec2_of<T>::type* __restrict__ F,
-                                                       typename vec2_of<T>::type* C, T beta6, int vb) {
+// Fused form (FP32, and the FP64 form's general path).
+template <typename T, class FU, class FUi, class FPq, class FDq, class FF, class FC>
+__device__ __forceinline__ void k_plaq_force_ab_body(Geo g, FU U,
+                                                       FUi Ui,
+                                                       FPq Pq,
+                                                       FDq Dq,
+                                                       FF F,
+                                                       FC C, T beta6, int vb) {
   const int p = vb % 6;
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -528,6 +484,8 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
   mat<T>&X = ws[0], &t = ws[1];
   if (MODE == MODE_UPDATE_X) {
     load(X, C, MU, s, g.V);  // the drift stored by the MODE_DRIFTMAX pass
+  } else if constexpr (std::is_same<T, double>::value) {
+    gather_f64(X, g, s, x, MU, C, a.cexp);
   } else {
     set_zero(X);
 #pragma unroll

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(DF_FORCE_BLOCK, 3) k_plaq_force_a_df(Geo g, co
   Work<df64, 1> wg(0);
   mat<df64>& Gh = wg[0];
   force_stage_a_df(Gh, g, s, x, p, U, Ui, Dq, F, C, beta6);
-  store(Gq, GQ_PLANE * p, s, g.V, Gh);  // plane 4p + 1 of C (see k_plaq_force_a)
+  store(Gq, GQ_PLANE * p, s, g.V, Gh);  // plane 4p + 1 of C (see GQ_PLANE)
 }
 __global__ void __launch_bounds__(DF_FORCE_BLOCK, 3) k_plaq_force_b_df(Geo g, const float4* __restrict__ U,
                                                                     const float4* __restrict__ Ui,

@@ -1,0 +1,343 @@
+// k_update_fx.cuh -- the CL step of the FP64 form in 64-bit fixed point
+// (fixed.cuh): link copies and inverses, plaquettes, clover field and
+// per-plaquette drift, the same quantities and formulas as k_update.cuh.
+//
+// Fields between the kernels (int4 words, SoA as the links): Ux, the links in
+// fixed point, in the buffer that the update writes at the step's end; Ui
+// their inverses; P, D, F, C.  F and C carry the factor 2^-e that keeps the
+// drift contributions below one (drift_exponent, launch.h): F is -i theta
+// kappa 2^-e times the clover field, negated for planes 1 and 4 (the sign of
+// the pair 02|13), C is 2^-e times the contribution.
+//
+// A thread whose inputs or results leave the fixed-point range calls the
+// general path, the FP64 bodies of k_update.cuh on the same fields, for its
+// plaquette; that code is out of line and costs the others nothing.
+//
+// Scales that keep every number within the fixed-point bound: D is stored
+// halved (|D| < 2.9), the clover sum is formed as an eighth of F.
+#pragma once
+#include "fixed.cuh"
+#include "k_update.cuh"
+
+namespace clgc {
+
+// Fields of the general path.
+__device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
+__device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
+
+// ------------------------------------------------------ links and inverses
+__device__ __forceinline__ void fx_links_body(Geo g, const double2* __restrict__ U, int4* __restrict__ Ux,
+                                              int4* __restrict__ Ui, int vb) {
+  const int mu = vb % 4;
+  const int s = (vb / 4) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  mat<double> u;
+  load(u, U, mu, s, g.V);
+  mat<fx> x, xi;
+  unsigned mag = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) x.e[k] = cx<fx>{fx_of_double(u.e[k].re, mag), fx_of_double(u.e[k].im, mag)};
+  fx_chk ck;
+  fx_adj(xi, x, ck);
+  if (!fx_mag_ok(mag) || ck.bad()) {  // readers of either turn to U itself
+    x.e[0].re.l = fx_raw_mark();
+    xi.e[0].re.l = fx_raw_mark();
+  }
+  store<fx>(Ux, mu, s, g.V, x);
+  store<fx>(Ui, mu, s, g.V, xi);
+}
+
+// ------------------------------------------------------------- plaquettes
+// (a - b) / 2
+__device__ __forceinline__ fx fx_half_diff(fx a, fx b) {
+  const int d = (a.h >> 1) - (b.h >> 1), odd = (a.h & 1) - (b.h & 1);  // a.h - b.h = 2 d + odd
+  return fx{fmaf(0.5f, a.l - b.l, (float)odd * 0x1p29f), d};
+}
+static __device__ __noinline__ void general_plaq(Geo g, const double2* U, tagged Pq, tagged Dq, int vb) {
+  k_plaq_body<double>(g, U, no_inverse(), Pq, Dq, vb);
+}
+__device__ __forceinline__ void fx_plaq_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq, int vb) {
+  const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
+  const int s = (vb / 6) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  int x[4];
+  site_coords(g, s, x);
+  fx_chk ck;
+  mat<fx> P, b;
+  fx_load(P, Ux, mu, s, g.V, ck);
+  fx_load(b, Ux, nu, hop(g, s, x, mu, 1), g.V, ck);
+  fx_mul_left<FX_WIDE>(P, b, ck);
+  fx_load(b, Ui, mu, hop(g, s, x, nu, 1), g.V, ck);
+  fx_mul_left<FX_WIDE>(P, b, ck);
+  fx_load(b, Ui, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(P, b, ck);
+  fx_adj(b, P, ck);
+  store<fx>(Pq, p, s, g.V, P);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) P.e[k] = cx<fx>{fx_half_diff(P.e[k].re, b.e[k].re), fx_half_diff(P.e[k].im, b.e[k].im)};
+  store<fx>(Dq, p, s, g.V, P);
+  if (ck.bad()) general_plaq(g, U, tag(Pq), tag_D(Dq), vb);
+}
+
+// ------------------------------------------------------------ clover field
+static __device__ __noinline__ void general_clover(Geo g, const double2* U, tagged Dq, tagged F, double sre, double sim,
+                                                   int vb) {
+  k_clover_rot_body<double>(g, U, no_inverse(), Dq, F, sre, sim, vb);
+}
+// sre, sim: the scale of plane p's F, |sre|, |sim| <= 1/32
+__device__ __forceinline__ void fx_clover_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+                                               const int4* __restrict__ Ui, const int4* __restrict__ Dq, int4* F,
+                                               double sre, double sim, int vb) {
+  const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
+  const int s = (vb / 6) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  if (p == 1 || p == 4) {
+    sre = -sre;
+    sim = -sim;
+  }
+  int x[4];
+  site_coords(g, s, x);
+  const int xmm = hop(g, s, x, mu, -1), xmn = hop(g, s, x, nu, -1);
+  const int xmm_mn = hop2(g, s, x, mu, -1, nu, -1);
+  fx_chk ck;
+  mat<fx> acc, w, d;  // sums of D / 8
+  // L3 + L4 = U_nu(x-nu)^{-1} [D(x-nu) + U_mu(x-mu-nu)^{-1} D(x-mu-nu) U_mu(x-mu-nu)] U_nu(x-nu)
+  fx_load(w, Ui, mu, xmm_mn, g.V, ck);
+  fx_load(d, Dq, p, xmm_mn, g.V, ck);
+  fx_mul_left<FX_NARROW, 2>(w, d, ck);
+  fx_load(d, Ux, mu, xmm_mn, g.V, ck);
+  fx_load(acc, Dq, p, xmn, g.V, ck);
+  fx_mul_acc<FX_WIDE, +1, 2>(acc, w, d, ck);
+  fx_load(w, Ui, nu, xmn, g.V, ck);
+  fx_mul_left<FX_WIDE>(w, acc, ck);
+  fx_load(d, Ux, nu, xmn, g.V, ck);
+  fx_load(acc, Dq, p, s, g.V, ck);
+  fx_mul_acc<FX_WIDE, +1, 2>(acc, w, d, ck);
+  // L2 = U_mu(x-mu)^{-1} D(x-mu) U_mu(x-mu)
+  fx_load(w, Ui, mu, xmm, g.V, ck);
+  fx_load(d, Dq, p, xmm, g.V, ck);
+  fx_mul_left<FX_NARROW, 2>(w, d, ck);
+  fx_load(d, Ux, mu, xmm, g.V, ck);
+  fx_mul_acc<FX_WIDE, +1>(acc, w, d, ck);
+  unsigned mag = 0;
+  const cx<fx> sc = {fx_of_double(8.0 * sre, mag), fx_of_double(8.0 * sim, mag)};
+  const fx_cleft x8 = fx_lhs(sc);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    fx_acc re = fx_zero(), im = fx_zero();
+    fx_cmac(re, im, x8, fx_rhs(acc.e[k]));
+    acc.e[k] = cx<fx>{fx_get<FX_NARROW>(re, ck), fx_get<FX_NARROW>(im, ck)};
+  }
+  store<fx>(F, p, s, g.V, acc);
+  if (ck.bad() || !fx_mag_ok(mag)) general_clover(g, U, tag_D(Dq), tag(F), sre, sim, vb);
+}
+
+// ------------------------------------------------------- plaquette drift
+static __device__ __noinline__ void general_force_wilson(Geo g, const double2* U, tagged Dq, tagged C, double b6, int vb) {
+  k_plaq_force_wilson_body<double>(g, U, no_inverse(), Dq, C, b6, vb);
+}
+__device__ __forceinline__ void fx_force_wilson_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+                                                     const int4* __restrict__ Ui, const int4* __restrict__ Dq, int4* C,
+                                                     double b6, int vb) {
+  const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
+  const int s = (vb / 6) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  fx_chk ck;
+  unsigned mag = 0;
+  const fx b = fx_of_double(2.0 * b6, mag);
+  mat<fx> M, t, a;
+  fx_load(a, Dq, p, s, g.V, ck);
+  fx_scaled<FX_WIDE>(M, a, b, ck);
+  store<fx>(C, 4 * p + 1, s, g.V, M);
+  // slot 3: u^{-1} (beta/6 D) u
+  fx_load(t, Ui, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(t, M, ck);
+  fx_load(a, Ux, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(t, a, ck);
+  store<fx>(C, 4 * p + 3, s, g.V, t);
+  // slots 0 and 2: -(beta/6) D and the same carried by a
+#pragma unroll
+  for (int k = 0; k < 9; ++k) M.e[k] = cx<fx>{-M.e[k].re, -M.e[k].im};
+  store<fx>(C, 4 * p + 0, s, g.V, M);
+  fx_load(t, Ui, mu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(t, M, ck);
+  fx_load(a, Ux, mu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(t, a, ck);
+  store<fx>(C, 4 * p + 2, s, g.V, t);
+  if (ck.bad() || !fx_mag_ok(mag)) general_force_wilson(g, U, tag_D(Dq), tag(C), b6, vb);
+}
+
+// Stage a of the theta force: corners c0 .. c2.  The sum of the dual fields
+// and the partials of slots 0 and 2 go to Gq and C (planes of this plaquette
+// that only stage b of the same thread's plaquette writes).  Both stages keep
+// at most three matrices in registers at a time, parking and re-reading the
+// rest, so that three blocks of 128 threads fit an SM.
+__device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
+                                                const int4* __restrict__ Dq, const int4* __restrict__ F, int4* Gq,
+                                                int4* C, double b6, int vb) {
+  const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
+  const int s = (vb / 6) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  int x[4];
+  site_coords(g, s, x);
+  const int c1 = hop(g, s, x, mu, 1);
+  fx_chk ck;
+  unsigned mag = 0;
+  const fx nb = fx_of_double(-b6, mag);
+  mat<fx> A, B, M;
+  // corner c0: half the slot 0 partial, [D, G0] / 2 - (beta/6) D / 2
+  fx_load(A, Dq, p, s, g.V, ck);
+  fx_load(B, F, pc, s, g.V, ck);
+  fx_commutator<FX_NARROW>(M, A, B, nb, ck);
+  store<fx>(C, 4 * p + 0, s, g.V, M);
+  // corner c1: A = G1^ = a G1 a^{-1}; slot 2 partial = slot 0 partial + [D, G1^]
+  fx_load(A, Ux, mu, s, g.V, ck);
+  fx_load(B, F, pc, c1, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, B, ck);
+  fx_load(B, Ui, mu, s, g.V, ck);
+  fx_mul_left<FX_NARROW>(A, B, ck);
+  load_rw(M, C, 4 * p + 0, s, g.V);
+  fx_load(B, Dq, p, s, g.V, ck);
+  fx_commutator_acc<FX_NARROW>(M, B, A, ck);
+  store<fx>(C, 4 * p + 2, s, g.V, M);
+  fx_load(B, F, pc, s, g.V, ck);
+  fx_add(A, B);
+  store<fx>(Gq, GQ_PLANE * p, s, g.V, A);  // G0 + G1^
+  // corner c2: G2^ = (ab) G2 (ab)^{-1}, (ab)^{-1} = adj(ab)
+  fx_load(A, Ux, mu, s, g.V, ck);
+  fx_load(B, Ux, nu, c1, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, B, ck);
+  fx_adj(B, A, ck);
+  fx_load(M, F, pc, hop(g, c1, x, nu, 1), g.V, ck);
+  fx_mul_left<FX_WIDE>(A, M, ck);
+  load_rw(M, Gq, GQ_PLANE * p, s, g.V);
+  fx_mul_acc<FX_WIDE, +1>(M, A, B, ck);
+  if (ck.bad() || !fx_mag_ok(mag)) M.e[0].re.l = fx_raw_mark();  // stage b starts over
+  store<fx>(Gq, GQ_PLANE * p, s, g.V, M);
+}
+
+static __device__ __noinline__ void general_force(Geo g, const double2* U, tagged Pq, tagged Dq, tagged F, tagged C,
+                                                  double b6, int vb) {
+  k_plaq_force_ab_body<double>(g, U, no_inverse(), Pq, Dq, F, C, b6, vb);
+}
+// Stage b: corner c3, K and the four slots.
+__device__ __forceinline__ void fx_force_b_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+                                                const int4* __restrict__ Ui, const int4* Pq, const int4* Dq,
+                                                const int4* F, const int4* Gq, int4* C, double b6, int vb) {
+  const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
+  const int s = (vb / 6) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  int x[4];
+  site_coords(g, s, x);
+  const int c3 = hop(g, s, x, nu, 1);
+  fx_chk ck;
+  unsigned mag = 0;
+  const fx pb = fx_of_double(b6, mag);
+  mat<fx> A, B, M;
+  // corner c3: A = G3r = u G3 u^{-1}; slot 3 partial = [D, G3r] + (beta/6) D
+  fx_load(A, Ux, nu, s, g.V, ck);
+  fx_load(B, F, pc, c3, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, B, ck);
+  fx_load(B, Ui, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, B, ck);
+  fx_load(B, Dq, p, s, g.V, ck);
+  fx_commutator<FX_NARROW>(M, B, A, pb, ck);
+  store<fx>(C, 4 * p + 3, s, g.V, M);
+  // M = G^ += P G3r P^{-1}, with P^{-1} = P - 2 (D / 2)
+  fx_load(B, Pq, p, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(B, A, ck);
+  fx_load(A, Dq, p, s, g.V, ck);
+  fx_load(M, Pq, p, s, g.V, ck);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) A.e[k] = cx<fx>{M.e[k].re - fx_twice(A.e[k].re), M.e[k].im - fx_twice(A.e[k].im)};
+  load_rw(M, Gq, GQ_PLANE * p, s, g.V);
+  if (fx_is_raw(M.e[0].re.l)) ck.fail();
+  fx_mul_acc<FX_WIDE, +1>(M, B, A, ck);
+  // A = K = P^{-1} G^ + G^ P
+  fx_mul_left<FX_WIDE>(A, M, ck);
+  fx_load(B, Pq, p, s, g.V, ck);
+  fx_mul_acc<FX_NARROW, +1>(A, M, B, ck);
+  // slot 0: K + partial; slot 1: -K + (beta/6) D
+  load_rw(M, C, 4 * p + 0, s, g.V);
+  fx_twice_add<+1>(M, A);
+  store<fx>(C, 4 * p + 0, s, g.V, M);
+  fx_load(M, Dq, p, s, g.V, ck);
+  fx_scaled<FX_NARROW>(M, M, pb, ck);
+  fx_twice_add<-1>(M, A);
+  store<fx>(C, 4 * p + 1, s, g.V, M);
+  // slot 3: u^{-1} (-K + partial) u
+  load_rw(M, C, 4 * p + 3, s, g.V);
+  fx_twice_add<-1>(M, A);
+  fx_load(B, Ui, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(B, M, ck);
+  fx_load(M, Ux, nu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(B, M, ck);
+  store<fx>(C, 4 * p + 3, s, g.V, B);
+  // slot 2: a^{-1} (K + partial) a
+  load_rw(M, C, 4 * p + 2, s, g.V);
+  fx_twice_add<+1>(M, A);
+  fx_load(A, Ui, mu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, M, ck);
+  fx_load(M, Ux, mu, s, g.V, ck);
+  fx_mul_left<FX_WIDE>(A, M, ck);
+  store<fx>(C, 4 * p + 2, s, g.V, A);
+  // anything out of range: the whole plaquette again (its slots are its own)
+  if (ck.bad() || !fx_mag_ok(mag)) general_force(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb);
+}
+
+// --------------------------------------------------------------- gather
+// The drift matrix 2^e sum C of link (s, MU) as doubles.
+static __device__ __noinline__ void general_gather(mat<double>& X, Geo g, int s, const int* x, int MU, tagged C, double ce) {
+  mat<double> t;
+  set_zero(X);
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == MU) continue;
+    const int p = MU < nu ? plane_index(MU, nu) : plane_index(nu, MU);
+    load(t, C, 4 * p + (MU < nu ? 0 : 1), s, g.V);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X.e[k] = cadd(X.e[k], t.e[k]);
+    load(t, C, 4 * p + (MU < nu ? 3 : 2), hop(g, s, x, nu, -1), g.V);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X.e[k] = cadd(X.e[k], t.e[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) X.e[k] = cx<double>{ce * X.e[k].re, ce * X.e[k].im};
+}
+// The sums as 60-bit integers (six contributions below 1.44 fit).
+__device__ __forceinline__ bool fx_gather(long long* X, const Geo& g, int s, const int* x, int MU, const int4* __restrict__ C) {
+  fx_chk ck;
+  mat<fx> t, l;
+#pragma unroll
+  for (int k = 0; k < 18; ++k) X[k] = 0;
+#pragma unroll
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == MU) continue;
+    const int p = MU < nu ? plane_index(MU, nu) : plane_index(nu, MU);
+    fx_load(t, C, 4 * p + (MU < nu ? 0 : 1), s, g.V, ck);
+    fx_load(l, C, 4 * p + (MU < nu ? 3 : 2), hop(g, s, x, nu, -1), g.V, ck);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      X[2 * k] += fx_bits(t.e[k].re) + fx_bits(l.e[k].re);
+      X[2 * k + 1] += fx_bits(t.e[k].im) + fx_bits(l.e[k].im);
+    }
+  }
+  return !ck.bad();
+}
+__device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
+                                           const double2* C, int cexp) {
+  const int4* c = reinterpret_cast<const int4*>(C);
+  long long v[18];
+  if (fx_gather(v, g, s, x, MU, c)) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      X.e[k] = cx<double>{fx_bits_to_double(v[2 * k], cexp), fx_bits_to_double(v[2 * k + 1], cexp)};
+  } else {
+    mat<double> Xg;  // a local of its own: its address goes out of line
+    general_gather(Xg, g, s, x, MU, tag(c), ldexp(1.0, cexp));
+    X = Xg;
+  }
+}
+
+}  // namespace clgc

@@ -5,6 +5,7 @@
 
 #include "cvt.cuh"
 #include "expm.cuh"
+#include "fixed.cuh"
 #include "launch.h"
 #include "lattice.cuh"
 #include "philox.cuh"
@@ -873,15 +874,21 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
       cx<double> q = {0.0, 0.0};
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
-        load(F1, F, p, s, g.V);
-        load(F2, F, 5 - p, s, g.V);
+        if constexpr (std::is_same<T, double>::value) {
+          load(F1, tagged{(int4*)F, 1.0}, p, s, g.V);
+          load(F2, tagged{(int4*)F, 1.0}, 5 - p, s, g.V);
+        } else {
+          load(F1, F, p, s, g.V);
+          load(F2, F, 5 - p, s, g.V);
+        }
         cx<T> t = trace_mul(F1, F2);
         double sg = (p == 1) ? -1.0 : 1.0;
         q.re += sg * (double)t.re;
         q.im += sg * (double)t.im;
       }
-      q.re *= KAPPA_Q;
-      q.im *= KAPPA_Q;
+      // F carries obs_clover_scale, 1/32 in the FP64 form
+      q.re *= std::is_same<T, double>::value ? 1024.0 * KAPPA_Q : KAPPA_Q;
+      q.im *= std::is_same<T, double>::value ? 1024.0 * KAPPA_Q : KAPPA_Q;
       v[5] += q.re;
       v[6] += q.im;
       if (q_site) {

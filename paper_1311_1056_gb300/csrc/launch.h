@@ -65,7 +65,8 @@ struct ChainDesc {
   double* arec;             // the single-pass apply's tile records
   CoolState* cs;
   StepDev* sd;
-  double beta, sre, sim;    // coupling; clover scale -i theta kappa = sre + i sim
+  double beta, sre, sim;    // coupling; clover scale -i theta kappa = sre + i sim (FP64: times 2^-cexp)
+  int cexp;                 // drift_exponent (FP64)
   double eps, sqrt_eps, k_ref;
   uint64_t seed;
   CoolArgs ca;
@@ -109,6 +110,14 @@ cudaError_t launch_aos_to_soa(int prec, const GeoH& g, const double* aos, void* 
                               cudaStream_t st);
 cudaError_t launch_soa_to_aos(int prec, const GeoH& g, const void* U, double* aos, int nplanes,
                               cudaStream_t st);
+// The FP64 form runs the step's link algebra in 64-bit fixed point
+// (k_update_fx.cuh): Ux receives the links in fixed point (the update's target
+// buffer, free until then), the clover scale and the contributions C carry the
+// factor 2^-cexp, cexp = drift_exponent(beta, scale_re, scale_im).  The other
+// forms ignore Ux and take cexp = 0.
+int drift_exponent(double beta, double sre, double sim);
+// Scale of the clover field that launch_obs expects (fixed point: entries below one).
+inline double obs_clover_scale(int prec) { return prec == 0 ? 0.03125 : 1.0; }
 // The CL step (k_update.cuh): link inverses Ui; plaquettes P and D = P - P^{-1}
 // (six planes); the clover field F^ = scale * F_{mu nu}(x) built from the D's;
 // the per-plaquette drift contributions C (24 planes: 4 links x 6 planes);
@@ -119,21 +128,22 @@ cudaError_t launch_soa_to_aos(int prec, const GeoH& g, const void* U, double* ao
 cudaError_t prepare_df64_kernels();
 cudaError_t launch_noise_sample(int prec, int site0, int n, uint64_t seed, uint32_t step, int mu, double* out,
                                 cudaStream_t st);
-cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ui, cudaStream_t st);
-cudaError_t launch_plaq(int prec, const GeoH& g, const void* U, const void* Ui, void* Pq, void* Dq,
+cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ux, void* Ui, cudaStream_t st);
+cudaError_t launch_plaq(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
                         cudaStream_t st);
-cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void* Ui, const void* Dq,
+cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, const void* Dq,
                               void* F, double scale_re, double scale_im, cudaStream_t st);
 // (theta != 0 runs two kernels, parking partial sums of the transported dual
 // fields in Gq, six planes.)
-cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ui,
+cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
-                              double beta, cudaStream_t st);
+                              double beta, int cexp, cudaStream_t st);
 // mode 0: update from the gathered drift (eps, or the device step size when
 // sd_adaptive); 1: write the drift X_S to out; 2: write X_S to out and fold
 // max |K|^2 into sd->kmax2_bits; 3: update reading X_S from C (a mode-2 output).
 cudaError_t launch_update_gather(int prec, int mode, const GeoH& g, const void* U, const void* C, void* out,
-                                 double eps, uint64_t seed, StepDev* sd, bool sd_adaptive, cudaStream_t st);
+                                 double eps, uint64_t seed, StepDev* sd, bool sd_adaptive, int cexp,
+                                 cudaStream_t st);
 // step += 1 on the device (the Philox step counter read by the update).
 // After an update: step += 1 and t += the step size taken (eps, or the
 // device step size when adaptive).

@@ -59,7 +59,14 @@ struct Work<df64, N> {
   __device__ __forceinline__ mat<df64>& operator[](int i) { return base[i * blockDim.x]; }
 };
 
+// Fixed point (fixed.cuh): x = (h 2^30 + l) 2^-60.
+struct fx {
+  float l;
+  int h;
+};
+
 template <typename T> struct vec2_of;
+template <> struct vec2_of<fx> { typedef int4 type; };
 template <> struct vec2_of<double> { typedef double2 type; };
 template <> struct vec2_of<float> { typedef float2 type; };
 template <> struct vec2_of<df64> { typedef float4 type; };  // (re.hi, re.lo, im.hi, im.lo)
@@ -68,6 +75,8 @@ template <> struct vec2_of<df64> { typedef float4 type; };  // (re.hi, re.lo, im
 __device__ __forceinline__ cx<double> unpack(double2 v) { return cx<double>{v.x, v.y}; }
 __device__ __forceinline__ cx<float> unpack(float2 v) { return cx<float>{v.x, v.y}; }
 __device__ __forceinline__ cx<df64> unpack(float4 v) { return cx<df64>{df64(v.x, v.y), df64(v.z, v.w)}; }
+__device__ __forceinline__ cx<fx> unpack(int4 v) { return cx<fx>{fx{__int_as_float(v.x), v.y}, fx{__int_as_float(v.z), v.w}}; }
+__device__ __forceinline__ int4 pack(cx<fx> c) { return make_int4(__float_as_int(c.re.l), c.re.h, __float_as_int(c.im.l), c.im.h); }
 __device__ __forceinline__ double2 pack(cx<double> c) { return make_double2(c.re, c.im); }
 __device__ __forceinline__ float2 pack(cx<float> c) { return make_float2(c.re, c.im); }
 __device__ __forceinline__ float4 pack(cx<df64> c) { return df_pack(c.re, c.im); }
