@@ -217,10 +217,16 @@ cl_status do_cool(cl_lattice* l, const cl_cool_params* cp) {
   CoolArgs a = cool_args(cp);
   const int n_iter = cp->forced_sweeps >= 0 ? cp->forced_sweeps : cp->n_max;
   const bool single_pass = (cp->mode == CL_D0 || cp->mode == CL_D1) && l->prec != 2;
+  // FP64: the sweeps work on the fixed-point links in Un (launch.h)
+  void* X = l->prec == 0 ? l->Un : l->U;
+  auto unload = [&] {
+    if (l->prec != 0) return cudaSuccess;
+    return timed(l, CL_PHASE_COOL_APPLY, [&] { return launch_cool_unload(l->g, l->U, l->Un, l->cs, l->st); });
+  };
   if (single_pass) {
     // sweep 0: the rule's first inputs from a plain gradient pass
     CK(timed(l, CL_PHASE_COOL_GRAD, [&] {
-      return launch_cool_grad(l->prec, l->g, l->U, l->f, l->partials, nullptr, l->st);
+      return launch_cool_grad(l->prec, l->g, l->U, X, l->f, l->partials, nullptr, l->st);
     }));
     CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt(l->g, l->partials, a, l->cs, 1, l->st); }));
     if (n_iter == 0) return CL_OK;
@@ -228,33 +234,35 @@ cl_status do_cool(cl_lattice* l, const cl_cool_params* cp) {
       return launch_cool_omega(l->prec, l->g, l->f, l->Om, l->Omi, cp->eps, l->cs, l->st);
     }));
     CK(timed(l, CL_PHASE_COOL_APPLY, [&] {
-      return launch_cool_apply_tiles(l->prec, l->g, l->U, l->Om, l->Omi, l->crec, l->cs, l->st);
+      return launch_cool_apply_tiles(l->prec, l->g, X, l->Om, l->Omi, l->crec, l->cs, l->st);
     }));
     for (int k = 1; k <= n_iter; ++k) {
       CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt_tiles(l->g, l->crec, a, l->cs, l->st); }));
       if (k == n_iter) break;
       CK(timed(l, CL_PHASE_COOL_GRAD_OMEGA, [&] {
-        return launch_cool_grad_omega(l->prec, l->g, l->U, l->Om, l->Omi, cp->eps, l->cs, l->st);
+        return launch_cool_grad_omega(l->prec, l->g, X, l->Om, l->Omi, cp->eps, l->cs, l->st);
       }));
       CK(timed(l, CL_PHASE_COOL_APPLY, [&] {
-        return launch_cool_apply_tiles(l->prec, l->g, l->U, l->Om, l->Omi, l->crec, l->cs, l->st);
+        return launch_cool_apply_tiles(l->prec, l->g, X, l->Om, l->Omi, l->crec, l->cs, l->st);
       }));
     }
+    CK(unload());
     return CL_OK;
   }
   for (int k = 0; k <= n_iter; ++k) {
     // the first gradient of a call always runs: the done flag still holds
     // the previous call's decision until the rule resets it (first = 1)
     CK(timed(l, CL_PHASE_COOL_GRAD, [&] {
-      return launch_cool_grad(l->prec, l->g, l->U, l->f, l->partials, k == 0 ? nullptr : l->cs, l->st);
+      return launch_cool_grad(l->prec, l->g, l->U, X, l->f, l->partials, k == 0 ? nullptr : l->cs, l->st);
     }));
     CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt(l->g, l->partials, a, l->cs, k == 0, l->st); }));
     if (k == n_iter) break;
     CK(timed(l, CL_PHASE_COOL_OMEGA, [&] {
       return launch_cool_omega(l->prec, l->g, l->f, l->Om, l->Omi, cp->eps, l->cs, l->st);
     }));
-    CK(timed(l, CL_PHASE_COOL_APPLY, [&] { return launch_cool_apply(l->prec, l->g, l->U, l->Om, l->Omi, l->cs, l->st); }));
+    CK(timed(l, CL_PHASE_COOL_APPLY, [&] { return launch_cool_apply(l->prec, l->g, X, l->Om, l->Omi, l->cs, l->st); }));
   }
+  if (n_iter > 0) CK(unload());
   return CL_OK;
 }
 
@@ -316,7 +324,14 @@ cudaError_t init_state(cl_lattice* l) {
   l->launches++;
   if (e == cudaSuccess && params->gauge_sigma > 0.0) {
     e = launch_gauge_omega(l->prec, l->g, l->Om, l->Omi, params->seed, params->gauge_sigma, l->st);
-    if (e == cudaSuccess) e = launch_cool_apply(l->prec, l->g, l->U, l->Om, l->Omi, nullptr, l->st);
+    if (l->prec == 0) {  // on the fixed-point words (launch.h)
+      if (e == cudaSuccess) e = launch_cool_load(l->g, l->U, l->Un, l->st);
+      if (e == cudaSuccess) e = launch_cool_apply(l->prec, l->g, l->Un, l->Om, l->Omi, nullptr, l->st);
+      if (e == cudaSuccess) e = launch_cool_unload(l->g, l->U, l->Un, nullptr, l->st);
+      l->launches += 2;
+    } else if (e == cudaSuccess) {
+      e = launch_cool_apply(l->prec, l->g, l->U, l->Om, l->Omi, nullptr, l->st);
+    }
     l->launches += 2;
   }
   return e;
@@ -661,7 +676,7 @@ cl_status cl_drift(cl_lattice* l, double* host_aos) {
 
 cl_status cl_cool_gradient(cl_lattice* l, double* host_f) {
   if (!l || !host_f) return fail(CL_ERR_INVALID, "NULL argument");
-  CK(launch_cool_grad(l->prec, l->g, l->U, l->f, l->partials, nullptr, l->st));
+  CK(launch_cool_grad(l->prec, l->g, l->U, l->Un, l->f, l->partials, nullptr, l->st));
   l->launches++;
   const size_t n = 8 * (size_t)l->g.V;
   CK(cudaMemcpyAsync(host_f, l->f, sizeof(double) * n, cudaMemcpyDeviceToHost, l->st));
@@ -931,6 +946,7 @@ FusedPlan plan_fused(const cl_batch* b) {
   add(ENS_COOL_OMEGA, four, tiles);
   add(ENS_COOL_APPLY, four, x4);
   add(ENS_COOL_GRAD_OMEGA, sp, red);
+  add(ENS_COOL_UNLOAD, [&](int i) { return b->with_cooling && b->lats[i]->prec == 0; }, x4);
   P.fam[ENS_COOL_APPLY_UN].off = P.items.size();
   for (int i = 0; i < n; ++i)
     if (sp(i)) {
@@ -1058,6 +1074,7 @@ cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainD
       CK(fam(ENS_COOL_APPLY, ENS_COOL_APPLY, 0));
       CK(fam(ENS_COOL_APPLY_UN, ENS_COOL_APPLY_UN, 0));
     }
+    if (P.n_iter > 0) CK(fam(ENS_COOL_UNLOAD, ENS_COOL_UNLOAD, 0));
   }
   *launches = nl;
   return CL_OK;

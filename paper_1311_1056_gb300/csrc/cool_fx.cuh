@@ -1,0 +1,423 @@
+// cool_fx.cuh -- the cooling sweeps of the FP64 form in fixed point
+// (fixed.cuh): gradient, Omega and apply, the formulas of kernels.cu.
+//
+// A cooling call keeps the links as fixed-point words Ux in the lattice's
+// second link buffer: its first gradient reads the FP64 links and writes them,
+// every sweep reads and writes Ux, and one pass at the end (fx_unload) writes
+// the FP64 links back if any sweep ran.  (Converting 64-bit words both ways in
+// every sweep would cost two fifths of it.)  Omega and Omega^{-1} are packed
+// Hermitian fields of 9 words per site.  A link, Omega or f that leaves the
+// fixed-point range is stored as doubles (fixed.cuh) and the threads that meet
+// it work in FP64.
+#pragma once
+#include "expm.cuh"
+#include "fixed.cuh"
+#include "lattice.cuh"
+#include "launch.h"
+
+namespace clgc {
+
+// ---------------------------------------------------------- packed fields
+struct fx_herm {
+  fx d[3];
+  cx<fx> o[3];  // 01, 02, 12
+};
+__device__ __forceinline__ fx fx_word(int2 w) { return fx{__int_as_float(w.x), w.y}; }
+__device__ __forceinline__ void fx_load_herm(fx_herm& h, const int2* __restrict__ P, int s, int V, fx_chk& ck) {
+  fx w[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) w[k] = fx_word(__ldg(P + (size_t)k * V + s));
+  if (fx_is_raw(w[0].l)) ck.fail();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    h.d[k] = w[k];
+    h.o[k] = cx<fx>{w[3 + 2 * k], w[4 + 2 * k]};
+  }
+}
+__device__ __forceinline__ void fx_store_herm(int2* P, int s, int V, const fx_herm& h) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    P[(size_t)k * V + s] = make_int2(__float_as_int(h.d[k].l), h.d[k].h);
+    P[(size_t)(3 + 2 * k) * V + s] = make_int2(__float_as_int(h.o[k].re.l), h.o[k].re.h);
+    P[(size_t)(4 + 2 * k) * V + s] = make_int2(__float_as_int(h.o[k].im.l), h.o[k].im.h);
+  }
+}
+// The general path's packed fields: doubles in, doubles out.
+struct tagged_herm {
+  int2* p;
+};
+__device__ __forceinline__ void store_herm(tagged_herm f, int s, int V, const herm& h) {
+  const double w[9] = {h.d0, h.d1, h.d2, h.o01.re, h.o01.im, h.o02.re, h.o02.im, h.o12.re, h.o12.im};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) f.p[(size_t)k * V + s] = k == 0 ? fx_raw_first(w[0]) : make_int2(__double2loint(w[k]), __double2hiint(w[k]));
+}
+__device__ __forceinline__ void load_herm_mat(mat<double>& m, tagged_herm f, int s, int V) {
+  double w[9];
+  const bool raw = fx_is_raw(__int_as_float(f.p[s].x));
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int2 v = f.p[(size_t)k * V + s];
+    w[k] = !raw ? fx_to_double(fx_word(v)) : k == 0 ? fx_raw_first(v) : __hiloint2double(v.y, v.x);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) m.e[4 * k] = cx<double>{w[k], 0.0};
+  m.e[1] = cx<double>{w[3], w[4]};
+  m.e[3] = cx<double>{w[3], -w[4]};
+  m.e[2] = cx<double>{w[5], w[6]};
+  m.e[6] = cx<double>{w[5], -w[6]};
+  m.e[5] = cx<double>{w[7], w[8]};
+  m.e[7] = cx<double>{w[7], -w[8]};
+}
+
+// -------------------------------------------------------------- gradient
+// G_x = sum_mu (U U^+ - U^+_{x-mu} U_{x-mu}) as 60-bit integers (d, o01, o02,
+// o12), and the three diagonal sums of its first part (Tr U U^+ of the links
+// at x).  The sums must stay below 8 (they are about 4 near SU(3)): their
+// squares are followed in float too, and ok is false beyond 7.5.
+struct fx_gradient {
+  long long d[3], o[6], un[3];
+  bool ok;
+};
+// rows (or conjugated columns) r0, r1, r2 of one link: += sign r_i conj(r_j)
+__device__ __forceinline__ void fx_outer(fx_acc* D, fx_acc* O, float* n, cx<fx> r0, cx<fx> r1, cx<fx> r2, bool neg) {
+  const cx<fx> r[3] = {r0, r1, r2};
+  fx_cright R[3];
+  fx_cleft X[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    R[i] = fx_rhs(r[i]);
+    X[i] = neg ? fx_lhs_neg(r[i]) : fx_lhs(r[i]);
+    fx_mac(D[i], X[i].re, R[i].re);
+    fx_mac(D[i], X[i].im, R[i].im);
+    const float a = (float)r[i].re.h, b = (float)r[i].im.h;
+    n[i] = fmaf(a, a, fmaf(b, b, n[i]));
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {  // (0,1), (0,2), (1,2)
+    const int i = q < 2 ? 0 : 1, j = q == 0 ? 1 : 2;
+    // x conj(y): re x.re y.re + x.im y.im, im x.im y.re - x.re y.im
+    fx_mac(O[2 * q], X[i].re, R[j].re);
+    fx_mac(O[2 * q], X[i].im, R[j].im);
+    fx_mac(O[2 * q + 1], X[i].im, R[j].re);
+    const fx_left nre = {-X[i].re.h, fx_neg(X[i].re.p)};
+    fx_mac(O[2 * q + 1], nre, R[j].im);
+  }
+}
+// load(u, mu, site): link (mu, site) as fixed point
+template <class Load>
+__device__ __forceinline__ void fx_grad_site(fx_gradient& G, const Geo& g, int s, const int x[4], Load load) {
+  fx_acc D[3], O[6];
+  float nf[3], nb[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    D[i] = fx_zero();
+    nf[i] = nb[i] = 0.0f;
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) O[i] = fx_zero();
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    mat<fx> u;
+    load(u, mu, s);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) fx_outer(D, O, nf, u.e[k], u.e[3 + k], u.e[6 + k], false);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) G.un[i] = fx_sum<true>(D[i]) - (1 << 29);
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    mat<fx> u;
+    load(u, mu, hop(g, s, x, mu, -1));
+    // - (U^+ U)_ij = - conj(U_ki) U_kj: x conj(y) with x = conj(U_ki), y = conj(U_kj)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const cx<fx> a = u.e[3 * k], b = u.e[3 * k + 1], c = u.e[3 * k + 2];
+      fx_outer(D, O, nb, cx<fx>{a.re, -a.im}, cx<fx>{b.re, -b.im}, cx<fx>{c.re, -c.im}, true);
+    }
+  }
+  G.ok = true;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    G.d[i] = fx_sum<true>(D[i]) - (1 << 29);
+    G.ok = G.ok && nf[i] < 7.5f * 0x1p60f && nb[i] < 7.5f * 0x1p60f;
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) G.o[i] = fx_sum<true>(O[i]) - (1 << 29);
+}
+
+// ----------------------------------------------------------- exponential
+// exp(H) and exp(-H) of a traceless Hermitian H, as expm_hermitian_pair:
+// H^2, the two invariants, Horner's rule on the three Cayley-Hamilton
+// coefficients of both, all in fixed point.  False (nothing useful in om, omi)
+// when a number leaves the range: |H| above ~1/3.
+struct fx_const {
+  int h, l;
+};
+// 1 / n! in units of 2^-60, rounded, as high and (balanced) low limb
+__host__ __device__ constexpr long long fx_inv_factorial(int n) {
+  long long f = 1;
+  for (int k = 2; k <= n; ++k) f *= k;
+  return n > 19 ? 0 : ((1ll << 60) + f / 2) / f;
+}
+__host__ __device__ constexpr fx_const fx_split_const(long long v) {
+  const long long h = (v + (1ll << 29)) >> 30;
+  return fx_const{(int)h, (int)(v - (h << 30))};
+}
+#define FX_F(n) fx_split_const(fx_inv_factorial(n))
+__constant__ fx_const c_fx_invfact[20] = {FX_F(0),  FX_F(1),  FX_F(2),  FX_F(3),  FX_F(4),  FX_F(5),  FX_F(6),
+                                          FX_F(7),  FX_F(8),  FX_F(9),  FX_F(10), FX_F(11), FX_F(12), FX_F(13),
+                                          FX_F(14), FX_F(15), FX_F(16), FX_F(17), FX_F(18), FX_F(19)};
+#undef FX_F
+__device__ __forceinline__ fx_acc fx_from_invfact(int n) {
+  const fx_const c = c_fx_invfact[n];
+  return fx_acc{mad_wide(c.h, 1 << 30, (long long)c.l), 0ull};
+}
+
+__device__ __forceinline__ bool fx_expm_hermitian_pair(fx_herm& om, fx_herm& omi, const fx_herm& H, float tol) {
+  fx_chk ck;
+  fx_herm Q;  // H^2
+  {
+    fx_cleft L[3];
+    fx_cright R[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      L[q] = fx_lhs(H.o[q]);
+      R[q] = fx_rhs(H.o[q]);
+    }
+    // |o01|^2, |o02|^2, |o12|^2 into the two diagonals each belongs to
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      fx_acc a = fx_zero();
+      fx_mac(a, fx_lhs(H.d[i]), fx_rhs(H.d[i]));
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const int qi = q < 2 ? 0 : 1, qj = q == 0 ? 1 : 2;
+        if (qi != i && qj != i) continue;
+        fx_mac(a, L[q].re, R[q].re);
+        fx_mac(a, L[q].im, R[q].im);
+      }
+      Q.d[i] = fx_get<FX_WIDE>(a, ck);
+    }
+    // (H^2)_01 = (d0 + d1) o01 + o02 conj(o12), _02 = (d0 + d2) o02 + o01 o12,
+    // _12 = (d1 + d2) o12 + conj(o01) o02; d_i + d_j = -d_k
+    fx_acc re, im;
+    fx_left nd = fx_lhs(-H.d[2]);
+    re = im = fx_zero();
+    fx_mac(re, nd, R[0].re);
+    fx_mac(im, nd, R[0].im);
+    fx_mac(re, L[1].re, R[2].re);
+    fx_mac(re, L[1].im, R[2].im);
+    fx_mac(im, L[1].im, R[2].re);
+    fx_mac(im, fx_lhs_neg(H.o[1].re), R[2].im);
+    Q.o[0] = cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
+    nd = fx_lhs(-H.d[1]);
+    re = im = fx_zero();
+    fx_mac(re, nd, R[1].re);
+    fx_mac(im, nd, R[1].im);
+    fx_cmac(re, im, L[0], R[2]);
+    Q.o[1] = cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
+    nd = fx_lhs(-H.d[0]);
+    re = im = fx_zero();
+    fx_mac(re, nd, R[2].re);
+    fx_mac(im, nd, R[2].im);
+    fx_mac(re, L[0].re, R[1].re);
+    fx_mac(re, L[0].im, R[1].im);
+    fx_mac(im, L[0].re, R[1].im);
+    fx_mac(im, L[0].nim, R[1].re);
+    Q.o[2] = cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
+  }
+  // c1 = Tr H^2 / 2, c0 = det H = Tr H^3 / 3 = (sum_i Q_ii d_i + 2 Re sum Q_ij conj(o_ij)) / 3
+  const fx c1 = fx_of_bits((fx_bits(Q.d[0]) + fx_bits(Q.d[1]) + fx_bits(Q.d[2])) >> 1);
+  fx_acc t = fx_zero(), t2 = fx_zero();
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    fx_mac(t, fx_lhs(Q.d[i]), fx_rhs(H.d[i]));
+    fx_mac(t2, fx_lhs(Q.o[i].re), fx_rhs(H.o[i].re));
+    fx_mac(t2, fx_lhs(Q.o[i].im), fx_rhs(H.o[i].im));
+  }
+  const fx t3 = fx_of_bits(fx_sum(t) + 2 * (fx_sum(t2) - (1 << 29)) - (1 << 29));
+  fx_acc z = fx_zero();
+  const fx_const third = fx_split_const(((1ll << 60) + 1) / 3);
+  fx_mac(z, fx_lhs(fx{(float)third.l, third.h}), fx_rhs(t3));
+  const fx c0 = fx_get<FX_WIDE>(z, ck);
+  const float r = sqrtf(2.0f * fmaxf(fmaf(c1.l, 0x1p-60f, (float)c1.h * 0x1p-30f), 0.0f));
+  if (ck.bad() || !(r < 0.34f)) return false;
+  const int N = taylor_terms(r, tol);
+  const fx_right b1 = fx_rhs(c1), b0 = fx_rhs(c0), nb0 = fx_rhs(-c0);
+  // exp(H) = a + b H + c H^2, exp(-H) = ap - bp H + cp H^2
+  const fx_const f = c_fx_invfact[N];
+  fx a = {(float)f.l, f.h}, b = {0.0f, 0}, c = {0.0f, 0}, ap = a, bp = b, cp = c;
+#pragma unroll 1
+  for (int k = N - 1; k >= 0; --k) {
+    fx_acc s = fx_from_invfact(k), u = fx_from(a), sp = s, up = fx_from(ap);
+    const fx_left x = fx_lhs(c), xp = fx_lhs(cp);
+    fx_mac(s, x, b0);
+    fx_mac(u, x, b1);
+    fx_mac(sp, xp, nb0);
+    fx_mac(up, xp, b1);
+    c = b;
+    b = fx_get<FX_WIDE>(u, ck);
+    a = fx_get<FX_WIDE>(s, ck);
+    cp = bp;
+    bp = fx_get<FX_WIDE>(up, ck);
+    ap = fx_get<FX_WIDE>(sp, ck);
+  }
+  const fx_left lb = fx_lhs(b), lc = fx_lhs(c), lbp = fx_lhs(-bp), lcp = fx_lhs(cp);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int q = (k - 3) >> 1;
+    const fx hk = k < 3 ? H.d[k] : (k & 1) ? H.o[q].re : H.o[q].im, qk = k < 3 ? Q.d[k] : (k & 1) ? Q.o[q].re : Q.o[q].im;
+    const fx_right hr = fx_rhs(hk), qr = fx_rhs(qk);
+    fx_acc s = k < 3 ? fx_from(a) : fx_zero(), sp = k < 3 ? fx_from(ap) : fx_zero();
+    fx_mac(s, lb, hr);
+    fx_mac(s, lc, qr);
+    fx_mac(sp, lbp, hr);
+    fx_mac(sp, lcp, qr);
+    const fx w = fx_get<FX_WIDE>(s, ck), wp = fx_get<FX_WIDE>(sp, ck);
+    if (k < 3) {
+      om.d[k] = w;
+      omi.d[k] = wp;
+    } else if (k & 1) {
+      om.o[q].re = w;
+      omi.o[q].re = wp;
+    } else {
+      om.o[q].im = w;
+      omi.o[q].im = wp;
+    }
+  }
+  return !ck.bad();
+}
+
+// H = 4 c (G - Tr G / 3), c = -eps alpha_ad (f_a lambda_a = 4 (G - Tr G / 3)).
+__device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradient& G, double c) {
+  fx_chk ck;
+  unsigned mag = 0;
+  const fx_left c4 = fx_lhs(fx_of_double(4.0 * c, mag));
+  const long long third = (G.d[0] + G.d[1] + G.d[2]) / 3;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const long long v = k < 3 ? G.d[k] - third : G.o[k - 3];
+    ck.see<FX_WIDE>((int)(v >> 32));
+    fx_acc a = fx_zero();
+    fx_mac(a, c4, fx_rhs(fx_of_bits(v)));
+    const fx w = fx_get<FX_WIDE>(a, ck);
+    const int q = (k - 3) >> 1;
+    if (k < 3)
+      H.d[k] = w;
+    else if (k & 1)
+      H.o[q].re = w;
+    else
+      H.o[q].im = w;
+  }
+  return !ck.bad() && fx_mag_ok(mag);
+}
+// The same from f: H = c f_a lambda_a.
+__device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const double* f, double c) {
+  fx_chk ck;
+  unsigned mag = 0;
+  const fx_left cl = fx_lhs(fx_of_double(c, mag)), cn = fx_lhs(fx_of_double(-c, mag)),
+                c3 = fx_lhs(fx_of_double(c * 0.57735026918962576451, mag)),
+                m3 = fx_lhs(fx_of_double(-2.0 * (c * 0.57735026918962576451), mag));
+  fx_right F[8];
+#pragma unroll
+  for (int a = 0; a < 8; ++a) F[a] = fx_rhs(fx_of_double(f[a], mag));
+  auto one = [&](const fx_left& x, const fx_right& y) {
+    fx_acc s = fx_zero();
+    fx_mac(s, x, y);
+    return fx_get<FX_WIDE>(s, ck);
+  };
+  auto two = [&](const fx_left& x, const fx_right& y, const fx_left& x2, const fx_right& y2) {
+    fx_acc s = fx_zero();
+    fx_mac(s, x, y);
+    fx_mac(s, x2, y2);
+    return fx_get<FX_WIDE>(s, ck);
+  };
+  H.d[0] = two(cl, F[2], c3, F[7]);
+  H.d[1] = two(cn, F[2], c3, F[7]);
+  H.d[2] = one(m3, F[7]);
+  H.o[0] = cx<fx>{one(cl, F[0]), one(cn, F[1])};
+  H.o[1] = cx<fx>{one(cl, F[3]), one(cn, F[4])};
+  H.o[2] = cx<fx>{one(cl, F[5]), one(cn, F[6])};
+  return !ck.bad() && fx_mag_ok(mag);
+}
+
+// ----------------------------------------------------------------- apply
+// u <- Omega u Omega'^{-1}, row by row (each row of Omega u goes straight into
+// the second product); with WITH_NORM also Tr u u^+ - 3 as a 60-bit integer.
+struct fx_apply_ops {  // Omega as left factors
+  fx_left d[3];
+  fx_cleft o[3];
+};
+__device__ __forceinline__ void fx_lhs(fx_apply_ops& L, const fx_herm& h) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    L.d[q] = fx_lhs(h.d[q]);
+    L.o[q] = fx_lhs(h.o[q]);
+  }
+}
+__device__ __forceinline__ fx_cleft fx_conj(const fx_cleft& a) { return fx_cleft{a.re, a.nim, a.im}; }
+template <bool WITH_NORM>
+__device__ __forceinline__ void fx_apply_link(mat<fx>& u, const fx_apply_ops& L, const fx_herm& oi, fx_chk& ck, long long& dev) {
+  fx_rmat y;
+  fx_rhs(y, u);
+  fx_right rd[3], ro[3][3];  // Omega'^{-1} as right factors: re, im, -im
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    rd[q] = fx_rhs(oi.d[q]);
+    ro[q][0] = fx_rhs(oi.o[q].re);
+    ro[q][1] = fx_rhs(oi.o[q].im);
+    ro[q][2] = fx_rhs(-oi.o[q].im);
+  }
+  fx_acc n = fx_zero();
+  float nf = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    fx_cleft t[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      fx_acc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (k == i) {
+          fx_mac(re, L.d[i], y.e[3 * k + j].re);
+          fx_mac(im, L.d[i], y.e[3 * k + j].im);
+        } else {
+          const int q = i + k - 1;  // 01 -> 0, 02 -> 1, 12 -> 2
+          fx_cmac(re, im, k > i ? L.o[q] : fx_conj(L.o[q]), y.e[3 * k + j]);
+        }
+      }
+      t[j] = fx_lhs(cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)});
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      fx_acc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (k == j) {
+          fx_mac(re, t[k].re, rd[j]);
+          fx_mac(im, t[k].im, rd[j]);
+        } else {  // element (k, j): o_kj for k < j, conj(o_jk) for k > j
+          const int q = j + k - 1, c = k < j ? 1 : 2;
+          fx_mac(re, t[k].re, ro[q][0]);
+          fx_mac(re, t[k].nim, ro[q][c]);
+          fx_mac(im, t[k].re, ro[q][c]);
+          fx_mac(im, t[k].im, ro[q][0]);
+        }
+      }
+      const cx<fx> r = {fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
+      u.e[3 * i + j] = r;
+      if (WITH_NORM) {
+        fx_mac(n, fx_lhs(r.re), fx_rhs(r.re));
+        fx_mac(n, fx_lhs(r.im), fx_rhs(r.im));
+        const float a = (float)r.re.h, b = (float)r.im.h;
+        nf = fmaf(a, a, fmaf(b, b, nf));
+      }
+    }
+  }
+  if (WITH_NORM) {
+    dev += fx_sum(n) - ((3ll << 60) + (1 << 29));
+    if (!(nf < 4.9f * 0x1p60f)) ck.fail();  // the sum of four deviations must fit
+  }
+}
+
+}  // namespace clgc

@@ -46,6 +46,8 @@ __device__ __forceinline__ fx_pair fx_fma2(fx_pair a, fx_pair b, fx_pair c) {
   return r;
 }
 
+__device__ __forceinline__ fx_pair fx_neg(fx_pair a) { return a ^ 0x8000000080000000ull; }
+
 // Range check: the largest of the results' high words, offset to be unsigned.
 // WIDE: |x| < 1.4375; NARROW: |x| < 0.359375, for results that are added to
 // others before their next use.
@@ -122,10 +124,13 @@ __device__ __forceinline__ void fx_cmac(fx_acc& re, fx_acc& im, const fx_cleft& 
 }
 // The sum as a 60-bit integer with an offset of 2^29: the small terms are
 // rounded to 2^-57 (in range for any operands within bounds) and folded in.
+// LONG: sums of up to 48 products (rounded to 2^-56).
+template <bool LONG = false>
 __device__ __forceinline__ long long fx_sum(const fx_acc& s) {
   float c0, c1;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(s.c));
-  return mad_wide(__float2int_rn((c0 + c1) * 0x1p-33f) + (1 << 26), 8, s.a);
+  return LONG ? mad_wide(__float2int_rn((c0 + c1) * 0x1p-34f) + (1 << 25), 16, s.a)
+              : mad_wide(__float2int_rn((c0 + c1) * 0x1p-33f) + (1 << 26), 8, s.a);
 }
 // The result times 2^-S, within bound B.
 template <int B, int S = 0>
@@ -321,6 +326,23 @@ __device__ __forceinline__ void fx_load(mat<fx>& a, const int4* __restrict__ f, 
   if (fx_is_raw(a.e[0].re.l)) ck.fail();
 }
 
+// Plain (coherent) load, for words this kernel also writes; |v| < 1 for a 60-bit integer.
+__device__ __forceinline__ void fx_load_plain(mat<fx>& a, const int4* f, int plane, int site, int V) {
+  const int4* p = f + (size_t)plane * 9 * V + site;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a.e[k] = unpack(p[(size_t)k * V]);
+}
+__device__ __forceinline__ bool fx_below_one(long long v) { return (unsigned)((int)(v >> 32) + (1 << 28)) < (1u << 29); }
+
+// The first double of a raw matrix, to and from its stored words.
+__device__ __forceinline__ int2 fx_raw_first(double x) {
+  const double ax = fabs(x);
+  if (ax < 0x1p-150) x = 0x1p-150;
+  x = ax < 0x1p500 ? x * 0x1p400 : __longlong_as_double(0x7ff8000000000000ll);
+  return make_int2(__double2hiint(x), __double2loint(x));
+}
+__device__ __forceinline__ double fx_raw_first(int2 v) { return __hiloint2double(v.x, v.y) * 0x1p-400; }
+
 // The general path's view of such a field; its numbers are the field's times sc.
 struct tagged {
   int4* p;
@@ -334,7 +356,7 @@ __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int si
     const int4 v = p[(size_t)k * V];
     if (raw) {
       a.e[k] = cx<double>{__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
-      if (k == 0) a.e[0].re = __hiloint2double(v.x, v.y) * 0x1p-400;
+      if (k == 0) a.e[0].re = fx_raw_first(make_int2(v.x, v.y));
     } else {
       const cx<fx> w = unpack(v);
       a.e[k] = cx<double>{fx_to_double(w.re), fx_to_double(w.im)};
@@ -348,15 +370,9 @@ __device__ __forceinline__ void store(tagged f, int plane, int site, int V, cons
   const double isc = 1.0 / f.sc;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    double re = a.e[k].re * isc, im = a.e[k].im * isc;
-    int4 v = make_int4(__double2loint(re), __double2hiint(re), __double2loint(im), __double2hiint(im));
-    if (k == 0) {
-      if (fabs(re) < 0x1p-150) re = 0x1p-150;
-      re = fabs(re) < 0x1p500 ? re * 0x1p400 : __longlong_as_double(0x7ff8000000000000ll);
-      v.x = __double2hiint(re);
-      v.y = __double2loint(re);
-    }
-    p[(size_t)k * V] = v;
+    const double re = a.e[k].re * isc, im = a.e[k].im * isc;
+    const int2 w = k == 0 ? fx_raw_first(re) : make_int2(__double2loint(re), __double2hiint(re));
+    p[(size_t)k * V] = make_int4(w.x, w.y, __double2loint(im), __double2hiint(im));
   }
 }
 

@@ -3,6 +3,7 @@
 // (instantiated by k_update_f64.cu / k_update_f32.cu).
 #include <type_traits>
 
+#include "cool_fx.cuh"
 #include "cvt.cuh"
 #include "expm.cuh"
 #include "fixed.cuh"
@@ -137,7 +138,6 @@ __global__ void k_hot(Geo g, typename vec2_of<T>::type* U, uint64_t seed) {
 }
 
 // Read-only load of one real of a packed field.
-__device__ __forceinline__ double ldg_real(const double* p) { return __ldg(p); }
 __device__ __forceinline__ float ldg_real(const float* p) { return __ldg(p); }
 __device__ __forceinline__ df64 ldg_real(const df64* p) {
   const float2 v = __ldg(reinterpret_cast<const float2*>(p));
@@ -223,8 +223,13 @@ __global__ void k_gauge_omega(Geo g, T* Om, T* Omi, uint64_t seed, double sigma)
   normals_f64<4>(r, seed, 0u, (uint32_t)s, 0u, STREAM_GAUGE);
   herm h = herm_from_algebra(r, -sigma), om, omi;
   expm_hermitian_pair(om, omi, h, taylor_tol<T>());
-  store_herm(Om, s, g.V, om);
-  store_herm(Omi, s, g.V, omi);
+  if constexpr (std::is_same<T, double>::value) {
+    store_herm(tagged_herm{(int2*)Om}, s, g.V, om);
+    store_herm(tagged_herm{(int2*)Omi}, s, g.V, omi);
+  } else {
+    store_herm(Om, s, g.V, om);
+    store_herm(Omi, s, g.V, omi);
+  }
 }
 
 // The CL noise of links (site0 + i, mu) as form T draws it (a diagnostic).
@@ -397,9 +402,8 @@ __device__ __forceinline__ void cool_grad_df(const Geo& g, const float4* __restr
 // f_ax = 2 Tr[lambda_a G_x], G_x = sum_mu (U_{x,mu} U_{x,mu}^+ - U_{x-mu,mu}^+ U_{x-mu,mu})
 // (Sec. 2, eq. "eq:24") at site s, in the link type; returns the sum over
 // the four links at x of Tr U U^+.
-template <typename T>
-__device__ __forceinline__ T cool_grad_site(const Geo& g, const typename vec2_of<T>::type* __restrict__ U, int s,
-                                            const int x[4], T fa[8]) {
+template <typename T, class FU>
+__device__ __forceinline__ T cool_grad_site(const Geo& g, FU U, int s, const int x[4], T fa[8]) {
   T g00 = T(0), g11 = T(0), g22 = T(0);
   cx<T> g01 = {T(0), T(0)}, g02 = {T(0), T(0)}, g12 = {T(0), T(0)};
 #pragma unroll
@@ -449,39 +453,183 @@ __device__ __forceinline__ T cool_grad_site(const Geo& g, const typename vec2_of
   return un;
 }
 
+// FP64 form: the links as a cooling call sees them.  FIRST (its first
+// gradient): the FP64 links, whose fixed-point words go to Ux on the way;
+// later: Ux.
+template <bool FIRST>
+__device__ __forceinline__ bool cool_fx_gradient(fx_gradient& G, const Geo& g, const double2* __restrict__ U, int4* Ux,
+                                                 int s, const int x[4]) {
+  fx_chk ck;
+  if constexpr (FIRST) {
+    fx_grad_site(G, g, s, x, [&](mat<fx>& u, int mu, int site) {
+      mat<double> d;
+      load(d, U, mu, site, g.V);
+      unsigned mag = 0;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_double(d.e[k].re, mag), fx_of_double(d.e[k].im, mag)};
+      const bool fits = fx_mag_ok(mag);
+      if (!fits) ck.fail();
+      if (site == s) {
+        if (fits)
+          store<fx>(Ux, mu, s, g.V, u);
+        else
+          store(tagged{Ux, 1.0}, mu, s, g.V, d);
+      }
+    });
+  } else {
+    fx_grad_site(G, g, s, x, [&](mat<fx>& u, int mu, int site) { fx_load(u, Ux, mu, site, g.V, ck); });
+  }
+  // |G| below 1, as everything formed from it expects
+#pragma unroll
+  for (int k = 0; k < 3; ++k) G.ok = G.ok && fx_below_one(G.d[k]) && fx_below_one(G.o[2 * k]) && fx_below_one(G.o[2 * k + 1]);
+  return G.ok && !ck.bad();
+}
+// The general path: f in fa, the norm of the site's links returned.
+static __device__ __noinline__ double general_cool_grad(const Geo g, const double2* U, int4* Ux, int s, double* fa) {
+  int x[4];
+  site_coords(g, s, x);
+  double f[8];
+  const double un = U ? cool_grad_site<double>(g, U, s, x, f) : cool_grad_site<double>(g, tagged{Ux, 1.0}, s, x, f);
+#pragma unroll
+  for (int a = 0; a < 8; ++a) fa[a] = f[a];
+  return un;
+}
+// f, and the rule's sums of one site into v: sum |f|, sum f^2, (1/3) sum Tr U U^+, nonfinite.
+template <bool FIRST>
+__device__ __forceinline__ void cool_grad_f64(const Geo& g, const double2* __restrict__ U, int4* Ux, double* f, int s,
+                                              double* v) {
+  int x[4];
+  site_coords(g, s, x);
+  fx_gradient G;
+  double fa[8], un, abs_sum, sq_sum;
+  if (cool_fx_gradient<FIRST>(G, g, U, Ux, s, x)) {
+    long long o = 0;
+    fx_acc sq = fx_zero();  // sum (f / 4)^2
+    fx_chk ck;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      o += G.o[k] < 0 ? -G.o[k] : G.o[k];
+      const fx w = fx_of_bits(G.o[k]);
+      fx_mac(sq, fx_lhs(w), fx_rhs(w));
+      const int a = k < 2 ? k : k + 1;
+      const double d = fx_bits_to_double(G.o[k], 2);
+      fa[a] = (k & 1) ? -d : d;
+    }
+    const long long d01 = G.d[0] - G.d[1], d2 = G.d[0] + G.d[1] - 2 * G.d[2];
+    fa[2] = fx_bits_to_double(d01, 1);
+    fa[7] = fx_bits_to_double(d2, 1) * 0.57735026918962576451;
+    abs_sum = fx_bits_to_double(o, 2) + (fabs(fa[2]) + fabs(fa[7]));
+    // (f_2 / 4)^2 + (f_7 / 4)^2 with f_2 / 4 = d01 / 2, f_7 / 4 = d2 / (2 sqrt 3)
+    const fx w2 = fx_of_bits(d01 >> 1);
+    unsigned mag = 0;
+    const fx c7 = fx_of_double(0.28867513459481288225, mag);
+    fx_acc z = fx_zero();
+    fx_mac(z, fx_lhs(c7), fx_rhs(fx_of_bits(d2 >> 2)));
+    const fx w7 = fx_twice(fx_twice(fx_get<FX_WIDE>(z, ck)));
+    fx_mac(sq, fx_lhs(w2), fx_rhs(w2));
+    fx_mac(sq, fx_lhs(w7), fx_rhs(w7));
+    sq_sum = fx_bits_to_double(fx_sum(sq) - (1 << 29), 4);
+    un = 12.0 + fx_bits_to_double(G.un[0] + G.un[1] + G.un[2] - (12ll << 60));
+  } else {
+    un = general_cool_grad(g, FIRST ? U : nullptr, Ux, s, fa);
+    abs_sum = sq_sum = 0.0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      abs_sum += fabs(fa[a]);
+      sq_sum = fma(fa[a], fa[a], sq_sum);
+    }
+    v[3] += isfinite(un) && isfinite(abs_sum) ? 0.0 : 1.0;
+  }
+#pragma unroll
+  for (int a = 0; a < 8; ++a) f[(size_t)a * g.V + s] = fa[a];
+  v[0] += abs_sum;
+  v[1] += sq_sum;
+  v[2] += un * (1.0 / 3.0);
+}
+
 // The gradient f into [a][V] (FP64) with, per block, sum |f|, sum f^2,
 // sum (1/3) Tr U U^+ of the links at x and the nonfinite count.
 // Block vb of nvb (the grid-stride loop over sites and the record index).
-template <typename T>
-__device__ __forceinline__ void cool_grad_body(const Geo& g, const typename vec2_of<T>::type* __restrict__ U,
+// FIRST: a call's first gradient (cs NULL), which always runs.
+template <typename T, bool FIRST>
+__device__ __forceinline__ void cool_grad_body(const Geo& g, const typename vec2_of<T>::type* __restrict__ U, void* Ux,
                                                double* __restrict__ f, double* partials, const CoolState* cs,
                                                int vb, int nvb) {
-  if (cs && cs->done) return;
+  if (!FIRST && cs->done) return;
   double v[NQ_COOL] = {0.0, 0.0, 0.0, 0.0};
   for (int s = vb * blockDim.x + threadIdx.x; s < g.V; s += nvb * blockDim.x) {
-    int x[4];
-    site_coords(g, s, x);
-    T fa[8];
-    const T un = cool_grad_site<T>(g, U, s, x, fa);
-    bool ok = isfinite(un);
+    if constexpr (std::is_same<T, double>::value) {
+      cool_grad_f64<FIRST>(g, U, (int4*)Ux, f, s, v);
+    } else {
+      int x[4];
+      site_coords(g, s, x);
+      T fa[8];
+      const T un = cool_grad_site<T>(g, U, s, x, fa);
+      bool ok = isfinite(un);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const double d = cvt<double>(fa[a]);
-      f[(size_t)a * g.V + s] = d;
-      v[0] += fabs(d);
-      v[1] = fma(d, d, v[1]);
-      ok = ok && isfinite(fa[a]);
+      for (int a = 0; a < 8; ++a) {
+        const double d = cvt<double>(fa[a]);
+        f[(size_t)a * g.V + s] = d;
+        v[0] += fabs(d);
+        v[1] = fma(d, d, v[1]);
+        ok = ok && isfinite(fa[a]);
+      }
+      v[2] += cvt<double>(un) * (1.0 / 3.0);
+      v[3] += ok ? 0.0 : 1.0;
     }
-    v[2] += cvt<double>(un) * (1.0 / 3.0);
-    v[3] += ok ? 0.0 : 1.0;
   }
   block_reduce_store<NQ_COOL, -1>(v, partials + (size_t)vb * NQ_COOL);
 }
-template <typename T>
+template <typename T, bool FIRST>
 __global__ void __launch_bounds__(RED_THREADS) k_cool_grad(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                          double* __restrict__ f, double* partials,
+                                                          void* Ux, double* __restrict__ f, double* partials,
                                                           const CoolState* cs) {
-  cool_grad_body<T>(g, U, f, partials, cs, blockIdx.x, gridDim.x);
+  cool_grad_body<T, FIRST>(g, U, Ux, f, partials, cs, blockIdx.x, gridDim.x);
+}
+
+// FP64 form: one link of Ux to or from the FP64 links.  The way back only when
+// the call applied a sweep (cs; NULL: always), so that a call without one
+// leaves the links bit for bit as they were.
+__device__ __forceinline__ void cool_unload_body(const Geo& g, double2* U, const int4* Ux, const CoolState* cs, int vb) {
+  if (cs && cs->sweeps == 0) return;
+  const int mu = vb % 4;
+  const int s = (vb / 4) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  mat<double> u;
+  load(u, tagged{const_cast<int4*>(Ux), 1.0}, mu, s, g.V);
+  store(U, mu, s, g.V, u);
+}
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_cool_unload(Geo g, double2* U, const int4* Ux, const CoolState* cs) {
+  cool_unload_body(g, U, Ux, cs, blockIdx.x);
+}
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_cool_load(Geo g, const double2* __restrict__ U, int4* Ux) {
+  const int mu = blockIdx.x % 4;
+  const int s = (blockIdx.x / 4) * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  mat<double> d;
+  load(d, U, mu, s, g.V);
+  mat<fx> u;
+  unsigned mag = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_double(d.e[k].re, mag), fx_of_double(d.e[k].im, mag)};
+  if (fx_mag_ok(mag))
+    store<fx>(Ux, mu, s, g.V, u);
+  else
+    store(tagged{Ux, 1.0}, mu, s, g.V, d);
+}
+
+// Omega_x and its inverse from f in FP64: the FP64 form's general path.
+static __device__ __noinline__ void general_cool_omega(const double* fa, double c, int2* Om, int2* Omi, int s, int V) {
+  const herm h = herm_from_algebra(fa, c);
+  herm om, omi;
+  expm_hermitian_pair(om, omi, h);
+  store_herm(tagged_herm{Om}, s, V, om);
+  store_herm(tagged_herm{Omi}, s, V, omi);
+}
+static __device__ __noinline__ void general_cool_grad_omega(const Geo g, int4* Ux, double c, int2* Om, int2* Omi, int s) {
+  double fa[8];
+  general_cool_grad(g, nullptr, Ux, s, fa);
+  general_cool_omega(fa, c, Om, Omi, s, g.V);
 }
 
 // Single-pass sweep of the D_0 / D_1 rules, part 1: the strength alpha_ad of
@@ -489,8 +637,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_cool_grad(Geo g, const typename
 // (k_cool_apply_tiles) summed, so the rule has decided before this kernel runs
 // and the gradient never leaves the thread: f_ax at x, then Omega_x =
 // exp(-eps alpha_ad f_ax lambda_a) and its inverse (FP64), stored packed.
+// FP64 form: U is Ux.
 template <typename T>
-__device__ __forceinline__ void cool_grad_omega_body(const Geo& g, const typename vec2_of<T>::type* __restrict__ U,
+__device__ __forceinline__ void cool_grad_omega_body(const Geo& g, const typename vec2_of<T>::type* U,
                                                      T* __restrict__ Om, T* __restrict__ Omi, double eps,
                                                      const CoolState* cs, int vb, int nvb) {
   if (cs->done) return;
@@ -498,20 +647,31 @@ __device__ __forceinline__ void cool_grad_omega_body(const Geo& g, const typenam
   for (int s = vb * blockDim.x + threadIdx.x; s < g.V; s += nvb * blockDim.x) {
     int x[4];
     site_coords(g, s, x);
-    T fa[8];
-    cool_grad_site<T>(g, U, s, x, fa);
-    double fd[8];
+    if constexpr (std::is_same<T, double>::value) {
+      fx_gradient G;
+      fx_herm H, om, omi;
+      if (cool_fx_gradient<false>(G, g, nullptr, (int4*)U, s, x) && fx_herm_of_gradient(H, G, c) &&
+          fx_expm_hermitian_pair(om, omi, H, TAYLOR_TOL_FP64)) {
+        fx_store_herm((int2*)Om, s, g.V, om);
+        fx_store_herm((int2*)Omi, s, g.V, omi);
+      } else {
+        general_cool_grad_omega(g, (int4*)U, c, (int2*)Om, (int2*)Omi, s);
+      }
+    } else {
+      T fa[8];
+      cool_grad_site<T>(g, U, s, x, fa);
+      double fd[8];
 #pragma unroll
-    for (int a = 0; a < 8; ++a) fd[a] = cvt<double>(fa[a]);
-    herm h = herm_from_algebra(fd, c), om, omi;
-    expm_hermitian_pair(om, omi, h, taylor_tol<T>());
-    store_herm(Om, s, g.V, om);
-    store_herm(Omi, s, g.V, omi);
+      for (int a = 0; a < 8; ++a) fd[a] = cvt<double>(fa[a]);
+      herm h = herm_from_algebra(fd, c), om, omi;
+      expm_hermitian_pair(om, omi, h, taylor_tol<T>());
+      store_herm(Om, s, g.V, om);
+      store_herm(Omi, s, g.V, omi);
+    }
   }
 }
 template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_cool_grad_omega(Geo g,
-                                                                const typename vec2_of<T>::type* __restrict__ U,
+__global__ void __launch_bounds__(RED_THREADS) k_cool_grad_omega(Geo g, const typename vec2_of<T>::type* U,
                                                                 T* __restrict__ Om, T* __restrict__ Omi, double eps,
                                                                 const CoolState* cs) {
   cool_grad_omega_body<T>(g, U, Om, Omi, eps, cs, blockIdx.x, gridDim.x);
@@ -618,10 +778,24 @@ __device__ __forceinline__ void cool_omega_body(const Geo& g, const double* __re
     double fa[8];
 #pragma unroll
     for (int a = 0; a < 8; ++a) fa[a] = __ldg(f + (size_t)a * g.V + s);
-    herm h = herm_from_algebra(fa, -eps * cs->alpha_ad), om, omi;
-    expm_hermitian_pair(om, omi, h, taylor_tol<T>());
-    store_herm(Om, s, g.V, om);
-    store_herm(Omi, s, g.V, omi);
+    if constexpr (std::is_same<T, double>::value) {
+      const double c = -eps * cs->alpha_ad;
+      fx_herm H, om, omi;
+      if (fx_herm_of_f(H, fa, c) && fx_expm_hermitian_pair(om, omi, H, TAYLOR_TOL_FP64)) {
+        fx_store_herm((int2*)Om, s, g.V, om);
+        fx_store_herm((int2*)Omi, s, g.V, omi);
+      } else {
+        double fg[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) fg[a] = fa[a];
+        general_cool_omega(fg, c, (int2*)Om, (int2*)Omi, s, g.V);
+      }
+    } else {
+      herm h = herm_from_algebra(fa, -eps * cs->alpha_ad), om, omi;
+      expm_hermitian_pair(om, omi, h, taylor_tol<T>());
+      store_herm(Om, s, g.V, om);
+      store_herm(Omi, s, g.V, omi);
+    }
   }
 }
 template <typename T>
@@ -630,8 +804,20 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_cool_omega(Geo g, const doub
   cool_omega_body<T>(g, f, Om, Omi, eps, cs, blockIdx.x);
 }
 
+// FP64 form's general path of one link; returns Tr U U^+.
+static __device__ __noinline__ double general_cool_apply(const Geo g, int4* Ux, int2* Om, int2* Omi, int mu, int s, int sp) {
+  mat<double> o, oi, u, t;
+  load_herm_mat(o, tagged_herm{Om}, s, g.V);
+  load_herm_mat(oi, tagged_herm{Omi}, sp, g.V);
+  load(u, tagged{Ux, 1.0}, mu, s, g.V);
+  mul_herm_left(t, o, u);
+  mul_herm_right(u, t, oi);
+  store(tagged{Ux, 1.0}, mu, s, g.V, u);
+  return norm2(u);
+}
+
 // U_{x,mu} <- Omega_x U_{x,mu} Omega_{x+mu}^{-1}, all links at once (in place:
-// every link is read and written by the same thread).
+// every link is read and written by the same thread).  FP64 form: U is Ux.
 template <typename T>
 __device__ __forceinline__ void cool_apply_body(const Geo& g, typename vec2_of<T>::type* U, const T* __restrict__ Om,
                                                 const T* __restrict__ Omi, const CoolState* cs, int vb) {
@@ -641,13 +827,33 @@ __device__ __forceinline__ void cool_apply_body(const Geo& g, typename vec2_of<T
   if (s >= g.V) return;
   int x[4];
   site_coords(g, s, x);
-  mat<T> o, oi, u, t;
-  load_herm_mat(o, Om, s, g.V);
-  load_herm_mat(oi, Omi, hop(g, s, x, mu, 1), g.V);
-  load(u, U, mu, s, g.V);
-  mul_herm_left(t, o, u);
-  mul_herm_right(u, t, oi);
-  store(U, mu, s, g.V, u);
+  if constexpr (std::is_same<T, double>::value) {
+    const int sp = hop(g, s, x, mu, 1);
+    int4* Ux = (int4*)U;
+    fx_chk ck;
+    fx_herm o, oi;
+    mat<fx> u;
+    fx_load_herm(o, (const int2*)Om, s, g.V, ck);
+    fx_load_herm(oi, (const int2*)Omi, sp, g.V, ck);
+    fx_load_plain(u, Ux, mu, s, g.V);
+    if (fx_is_raw(u.e[0].re.l)) ck.fail();
+    fx_apply_ops L;
+    fx_lhs(L, o);
+    long long dev = 0;
+    fx_apply_link<false>(u, L, oi, ck, dev);
+    if (!ck.bad())
+      store<fx>(Ux, mu, s, g.V, u);
+    else
+      general_cool_apply(g, Ux, (int2*)Om, (int2*)Omi, mu, s, sp);
+  } else {
+    mat<T> o, oi, u, t;
+    load_herm_mat(o, Om, s, g.V);
+    load_herm_mat(oi, Omi, hop(g, s, x, mu, 1), g.V);
+    load(u, U, mu, s, g.V);
+    mul_herm_left(t, o, u);
+    mul_herm_right(u, t, oi);
+    store(U, mu, s, g.V, u);
+  }
 }
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_cool_apply(Geo g, typename vec2_of<T>::type* U, const T* __restrict__ Om,
@@ -667,8 +873,11 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_cool_apply(Geo g, typename v
 // sum independent of the launch shape: a fused batch, which runs the tiles of
 // many chains in one launch, gives each chain the records of its lone run.
 // Resident blocks of COOL_TILE threads the tile kernels are built for: 72
-// registers a thread with FP32 links, 128 with FP64 ones (a few bytes of spills).
-#define COOL_TILE_MIN_BLOCKS(T) (sizeof(T) == 4 ? 7 : 4)
+// registers a thread with FP32 links, 168 with fixed-point ones (100 bytes of
+// spills; four blocks at 128 registers spill 300).  The FP64 form's apply is
+// bound by the integer and FP32 pipes: 0.35 ms per 32^4 sweep against 1.42 ms
+// in FP64 arithmetic, gradient + Omega 0.28 against 0.91 ms.
+#define COOL_TILE_MIN_BLOCKS(T) (sizeof(T) == 4 ? 7 : 3)
 __device__ __forceinline__ int layer_sites(const Geo& g) { return g.V / g.L[3]; }
 __device__ __forceinline__ int tiles_per_layer(const Geo& g) { return (layer_sites(g) + COOL_TILE - 1) / COOL_TILE; }
 
@@ -683,18 +892,50 @@ __device__ __forceinline__ void cool_apply_tile(const Geo& g, typename vec2_of<T
   if (s < s1) {
     int x[4];
     site_coords(g, s, x);
-    mat<T> o;
-    load_herm_mat(o, Om, s, g.V);
     T un = T(0);
+    if constexpr (std::is_same<T, double>::value) {
+      int4* Ux = (int4*)U;
+      fx_chk ck0;
+      fx_apply_ops L;
+      {
+        fx_herm o;
+        fx_load_herm(o, (const int2*)Om, s, g.V, ck0);
+        fx_lhs(L, o);
+      }
+      long long dev = 0;  // Tr U U^+ - 3 of the links in range, 2^-60
+      double wild = 0.0;  // of the others
+#pragma unroll 1
+      for (int mu = 0; mu < 4; ++mu) {
+        const int sp = hop(g, s, x, mu, 1);
+        fx_chk ck = ck0;
+        fx_herm oi;
+        mat<fx> u;
+        fx_load_herm(oi, (const int2*)Omi, sp, g.V, ck);
+        fx_load_plain(u, Ux, mu, s, g.V);
+        if (fx_is_raw(u.e[0].re.l)) ck.fail();
+        long long d = 0;
+        fx_apply_link<true>(u, L, oi, ck, d);
+        if (!ck.bad()) {
+          store<fx>(Ux, mu, s, g.V, u);
+          dev += d;
+        } else {
+          wild += general_cool_apply(g, Ux, (int2*)Om, (int2*)Omi, mu, s, sp) - 3.0;
+        }
+      }
+      un = 12.0 + (fx_bits_to_double(dev) + wild);
+    } else {
+      mat<T> o;
+      load_herm_mat(o, Om, s, g.V);
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      mat<T> oi, u, t;
-      load_herm_mat(oi, Omi, hop(g, s, x, mu, 1), g.V);
-      load(u, U, mu, s, g.V);
-      mul_herm_left(t, o, u);
-      mul_herm_right(u, t, oi);
-      store(U, mu, s, g.V, u);
-      un += norm2(u);
+      for (int mu = 0; mu < 4; ++mu) {
+        mat<T> oi, u, t;
+        load_herm_mat(oi, Omi, hop(g, s, x, mu, 1), g.V);
+        load(u, U, mu, s, g.V);
+        mul_herm_left(t, o, u);
+        mul_herm_right(u, t, oi);
+        store(U, mu, s, g.V, u);
+        un += norm2(u);
+      }
     }
     v.x = cvt<double>(un) * (1.0 / 3.0);
     v.y = isfinite(un) ? 0.0 : 1.0;
@@ -1014,15 +1255,28 @@ __device__ __forceinline__ int ens_reduce_blocks(int V) {
   return b < RED_MAX_BLOCKS ? b : RED_MAX_BLOCKS;
 }
 
-// first = 1: the call's first gradient, which always runs (as k_cool_grad with no state)
+// The links a sweep works on: the step's new links, or (FP64) their
+// fixed-point words in the old links' buffer.
 template <typename T>
+__device__ __forceinline__ typename vec2_of<T>::type* ens_links(const ChainDesc& c) {
+  return (typename vec2_of<T>::type*)(std::is_same<T, double>::value ? c.U : c.Un);
+}
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_cool_unload(const ChainDesc* __restrict__ cd,
+                                                                   const WorkItem* __restrict__ w) {
+  const WorkItem it = w[blockIdx.x];
+  const ChainDesc& c = cd[it.chain];
+  cool_unload_body(ens_geo(c), (double2*)c.Un, (const int4*)c.U, c.cs, it.vb);
+}
+
+// FIRST: the call's first gradient, which always runs (as k_cool_grad with no state)
+template <typename T, bool FIRST>
 __global__ void __launch_bounds__(RED_THREADS) k_ens_cool_grad(const ChainDesc* __restrict__ cd,
-                                                              const WorkItem* __restrict__ w, int first) {
+                                                              const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  cool_grad_body<T>(ens_geo(c), (const V2*)c.Un, (double*)c.f, c.partials, first ? nullptr : c.cs, it.vb,
-                    ens_reduce_blocks(c.V));
+  cool_grad_body<T, FIRST>(ens_geo(c), (const V2*)c.Un, c.U, (double*)c.f, c.partials, c.cs, it.vb,
+                           ens_reduce_blocks(c.V));
 }
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_cool_omega(const ChainDesc* __restrict__ cd,
@@ -1037,7 +1291,7 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_cool_apply(const ChainDe
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  cool_apply_body<T>(ens_geo(c), (V2*)c.Un, (const T*)c.Om, (const T*)c.Omi, c.cs, it.vb);
+  cool_apply_body<T>(ens_geo(c), ens_links<T>(c), (const T*)c.Om, (const T*)c.Omi, c.cs, it.vb);
 }
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_ens_cool_grad_omega(const ChainDesc* __restrict__ cd,
@@ -1045,7 +1299,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_ens_cool_grad_omega(const Chain
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  cool_grad_omega_body<T>(ens_geo(c), (const V2*)c.Un, (T*)c.Om, (T*)c.Omi, c.ca.eps, c.cs, it.vb,
+  cool_grad_omega_body<T>(ens_geo(c), ens_links<T>(c), (T*)c.Om, (T*)c.Omi, c.ca.eps, c.cs, it.vb,
                           ens_reduce_blocks(c.V));
 }
 template <typename T>
@@ -1057,7 +1311,7 @@ __global__ void __launch_bounds__(COOL_TILE, COOL_TILE_MIN_BLOCKS(T)) k_ens_cool
   const Geo g = ens_geo(c);
   if (c.cs->done) return;
   const int tpl = tiles_per_layer(g);
-  cool_apply_tile<T>(g, (V2*)c.Un, (const T*)c.Om, (const T*)c.Omi, (double2*)c.arec, it.vb / tpl, it.vb % tpl);
+  cool_apply_tile<T>(g, ens_links<T>(c), (const T*)c.Om, (const T*)c.Omi, (double2*)c.arec, it.vb / tpl, it.vb % tpl);
 }
 // the rule, one block of 256 threads per listed chain
 __global__ void k_ens_cool_adapt(const ChainDesc* __restrict__ cd, const int* __restrict__ chains, int first) {
@@ -1076,11 +1330,20 @@ template <typename T>
 cudaError_t launch_ens_cool_family(int fam, const ChainDesc* cd, const WorkItem* w, int nw, int arg, cudaStream_t st) {
   const unsigned n = (unsigned)nw;
   switch (fam) {
-    case ENS_COOL_GRAD: k_ens_cool_grad<T><<<n, RED_THREADS, 0, st>>>(cd, w, arg); break;
+    case ENS_COOL_GRAD:
+      if (arg)
+        k_ens_cool_grad<T, true><<<n, RED_THREADS, 0, st>>>(cd, w);
+      else
+        k_ens_cool_grad<T, false><<<n, RED_THREADS, 0, st>>>(cd, w);
+      break;
     case ENS_COOL_OMEGA: k_ens_cool_omega<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_COOL_APPLY: k_ens_cool_apply<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_COOL_GRAD_OMEGA: k_ens_cool_grad_omega<T><<<n, RED_THREADS, 0, st>>>(cd, w); break;
     case ENS_COOL_APPLY_UN: k_ens_cool_apply_tiles<T><<<n, COOL_TILE, 0, st>>>(cd, w); break;
+    case ENS_COOL_UNLOAD:
+      if (!std::is_same<T, double>::value) return cudaErrorInvalidValue;
+      k_ens_cool_unload<<<n, ENS_BLOCK, 0, st>>>(cd, w);
+      break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -1194,7 +1457,7 @@ cudaError_t launch_noise_sample(int prec, int site0, int n, uint64_t seed, uint3
   });
 }
 
-cudaError_t launch_cool_grad(int prec, const GeoH& h, const void* U, void* f, double* partials,
+cudaError_t launch_cool_grad(int prec, const GeoH& h, const void* U, void* Ux, void* f, double* partials,
                              const CoolState* cs, cudaStream_t st) {
   Geo g = to_geo(h);
   return by_prec(prec, [&](auto t) {
@@ -1202,8 +1465,13 @@ cudaError_t launch_cool_grad(int prec, const GeoH& h, const void* U, void* f, do
     if constexpr (std::is_same<T, df64>::value)
       k_cool_grad_df<<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const float4*)U, (float2*)f, partials, cs);
     else
-      k_cool_grad<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const typename vec2_of<T>::type*)U, (double*)f,
-                                                                partials, cs);
+    {
+      auto* u = (const typename vec2_of<T>::type*)U;
+      if (cs)
+        k_cool_grad<T, false><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, u, Ux, (double*)f, partials, cs);
+      else
+        k_cool_grad<T, true><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, u, Ux, (double*)f, partials, cs);
+    }
   });
 }
 
@@ -1252,6 +1520,19 @@ cudaError_t launch_cool_grad_omega(int prec, const GeoH& h, const void* U, void*
                                                                          (float*)Omi, eps, cs);
   else
     return cudaErrorInvalidValue;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cool_load(const GeoH& h, const void* U, void* Ux, cudaStream_t st) {
+  Geo g = to_geo(h);
+  const int bs = block_of(h, TUNE_APPLY);
+  k_cool_load<<<(unsigned)(((g.V + bs - 1) / bs) * 4), bs, 0, st>>>(g, (const double2*)U, (int4*)Ux);
+  return cudaGetLastError();
+}
+cudaError_t launch_cool_unload(const GeoH& h, void* U, const void* Ux, const CoolState* cs, cudaStream_t st) {
+  Geo g = to_geo(h);
+  const int bs = block_of(h, TUNE_APPLY);
+  k_cool_unload<<<(unsigned)(((g.V + bs - 1) / bs) * 4), bs, 0, st>>>(g, (double2*)U, (const int4*)Ux, cs);
   return cudaGetLastError();
 }
 

@@ -92,7 +92,8 @@ enum {
   ENS_COOL_APPLY = 10,  // apply, 4 directions
   ENS_COOL_GRAD_OMEGA = 11, // single-pass sweeps (D_0 / D_1): gradient + Omega
   ENS_COOL_APPLY_UN = 12,   // single-pass sweeps: apply per tile + norm sums (one item per tile)
-  ENS_NFAM = 13
+  ENS_COOL_UNLOAD = 13,     // FP64: fixed-point links back to doubles, 4 directions
+  ENS_NFAM = 14
 };
 const int ENS_BLOCK = 128;
 
@@ -152,8 +153,15 @@ cudaError_t launch_step_bump(StepDev* sd, double eps, bool adaptive, cudaStream_
 cudaError_t launch_step_eps(StepDev* sd, double eps, double k_ref, cudaStream_t st);
 // Cooling: gradient f (8 FP64 values per site, [a][V]) + partial sums; the
 // rule; Omega; apply.
-cudaError_t launch_cool_grad(int prec, const GeoH& g, const void* U, void* f, double* partials,
+// FP64 form: the sweeps run on the links' fixed-point words Ux (the second link
+// buffer), which the call's first gradient (cs NULL) writes from U; the Omega,
+// apply and later gradient launches take Ux as U, and launch_cool_unload at the
+// end writes U back if a sweep ran (cs NULL: always).  launch_cool_load writes
+// Ux without a gradient.
+cudaError_t launch_cool_grad(int prec, const GeoH& g, const void* U, void* Ux, void* f, double* partials,
                              const CoolState* cs, cudaStream_t st);
+cudaError_t launch_cool_load(const GeoH& g, const void* U, void* Ux, cudaStream_t st);
+cudaError_t launch_cool_unload(const GeoH& g, void* U, const void* Ux, const CoolState* cs, cudaStream_t st);
 cudaError_t launch_cool_adapt(const GeoH& g, const double* partials, CoolArgs a, CoolState* cs,
                               int first, cudaStream_t st);
 cudaError_t launch_cool_omega(int prec, const GeoH& g, const void* f, void* Om, void* Omi,

@@ -78,3 +78,48 @@ def test_non_finite_links_are_reported(cl):
             with pytest.raises(cl.CLError) as e:
                 lat.observables()
             assert e.value.status == cl.CL_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("L", [(4, 4, 4, 4), (3, 5, 2, 4), (1, 4, 4, 2), (7, 3, 2, 5)])
+@pytest.mark.parametrize("spread", [0, 0.05, 0.2, 0.4, "mixed"])
+@pytest.mark.parametrize("mode", ["D0", "D1", "D2_MEANABS", "D2_RMS"])
+def test_cooling_inside_and_outside_the_range(cl, L, spread, mode):
+    """Two sweeps of a step small enough that no field blows up: a sweep multiplies each link by two
+    matrices near 1, a few tens of roundings of the link's size; 1e-12 of max |U| is a hundred times that.
+    (D_2 divides by <|f|>, at rounding level for SU(3) links: there the guard stops it on both sides.)"""
+    U = field(L, spread, 21)
+    kw = dict(eps=1e-3, alpha=1.0, forced_sweeps=2, d_guard=1e-9)
+    ref, rep = O.cool(L, U, O.cool_params(mode=getattr(O, mode), **kw))
+    with cl.Lattice(L) as lat:
+        lat.set_links(U)
+        got = lat.cool(cl.make_cool(mode=getattr(cl, "CL_" + mode), **kw))
+        Ug = lat.links()
+        f = lat.cool_gradient()
+    assert got["sweeps"] == rep["sweeps"]
+    assert np.abs(Ug - ref).max() <= 1e-12 * np.abs(ref).max()
+    fr = O.cool_gradient(L, ref)
+    assert np.abs(f - fr).max() <= 1e-11 * np.abs(ref).max() ** 2
+    for k in ("un_before", "un_after"):
+        assert abs(got[k] - rep[k]) <= 1e-12 * rep[k], k
+
+
+def test_cooling_with_a_large_exponent(cl):
+    """eps alpha |f| of order one: Omega leaves the fixed-point range and is formed in FP64."""
+    L = (4, 2, 3, 4)
+    U = field(L, 0.2, 9)
+    kw = dict(eps=0.1, alpha=1.0, forced_sweeps=1)
+    ref, _ = O.cool(L, U, O.cool_params(mode=O.D0, **kw))
+    with cl.Lattice(L) as lat:
+        lat.set_links(U)
+        lat.cool(cl.make_cool(mode=cl.CL_D0, **kw))
+        assert np.abs(lat.links() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def test_a_cooling_call_without_a_sweep_keeps_the_links(cl):
+    L = (4, 4, 2, 3)
+    U = field(L, 0.2, 2)
+    with cl.Lattice(L) as lat:
+        lat.set_links(U)
+        rep = lat.cool(cl.make_cool(0.01, mode=cl.CL_D1, n_min=0, n_max=5, d_floor=1e9))
+        assert rep["sweeps"] == 0
+        assert np.array_equal(lat.links(), U)
