@@ -10,7 +10,7 @@
 // fixed-point range is stored as doubles (fixed.cuh) and the threads that meet
 // it work in FP64.
 #pragma once
-#include "expm.cuh"
+#include "expm_fx.cuh"
 #include "fixed.cuh"
 #include "lattice.cuh"
 #include "launch.h"
@@ -40,6 +40,15 @@ __device__ __forceinline__ void fx_store_herm(int2* P, int s, int V, const fx_he
     P[(size_t)k * V + s] = make_int2(__float_as_int(h.d[k].l), h.d[k].h);
     P[(size_t)(3 + 2 * k) * V + s] = make_int2(__float_as_int(h.o[k].re.l), h.o[k].re.h);
     P[(size_t)(4 + 2 * k) * V + s] = make_int2(__float_as_int(h.o[k].im.l), h.o[k].im.h);
+  }
+}
+// FP32-storage form: the packed field of floats.
+__device__ __forceinline__ void fx_store_herm(float* P, int s, int V, const fx_herm& h) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    P[(size_t)k * V + s] = fx_to_float(h.d[k]);
+    P[(size_t)(3 + 2 * k) * V + s] = fx_to_float(h.o[k].re);
+    P[(size_t)(4 + 2 * k) * V + s] = fx_to_float(h.o[k].im);
   }
 }
 // The general path's packed fields: doubles in, doubles out.
@@ -150,29 +159,6 @@ __device__ __forceinline__ void fx_grad_site(fx_gradient& G, const Geo& g, int s
 // H^2, the two invariants, Horner's rule on the three Cayley-Hamilton
 // coefficients of both, all in fixed point.  False (nothing useful in om, omi)
 // when a number leaves the range: |H| above ~1/3.
-struct fx_const {
-  int h, l;
-};
-// 1 / n! in units of 2^-60, rounded, as high and (balanced) low limb
-__host__ __device__ constexpr long long fx_inv_factorial(int n) {
-  long long f = 1;
-  for (int k = 2; k <= n; ++k) f *= k;
-  return n > 19 ? 0 : ((1ll << 60) + f / 2) / f;
-}
-__host__ __device__ constexpr fx_const fx_split_const(long long v) {
-  const long long h = (v + (1ll << 29)) >> 30;
-  return fx_const{(int)h, (int)(v - (h << 30))};
-}
-#define FX_F(n) fx_split_const(fx_inv_factorial(n))
-__constant__ fx_const c_fx_invfact[20] = {FX_F(0),  FX_F(1),  FX_F(2),  FX_F(3),  FX_F(4),  FX_F(5),  FX_F(6),
-                                          FX_F(7),  FX_F(8),  FX_F(9),  FX_F(10), FX_F(11), FX_F(12), FX_F(13),
-                                          FX_F(14), FX_F(15), FX_F(16), FX_F(17), FX_F(18), FX_F(19)};
-#undef FX_F
-__device__ __forceinline__ fx_acc fx_from_invfact(int n) {
-  const fx_const c = c_fx_invfact[n];
-  return fx_acc{mad_wide(c.h, 1 << 30, (long long)c.l), 0ull};
-}
-
 __device__ __forceinline__ bool fx_expm_hermitian_pair(fx_herm& om, fx_herm& omi, const fx_herm& H, float tol) {
   fx_chk ck;
   fx_herm Q;  // H^2
@@ -237,8 +223,7 @@ __device__ __forceinline__ bool fx_expm_hermitian_pair(fx_herm& om, fx_herm& omi
   }
   const fx t3 = fx_of_bits(fx_sum(t) + 2 * (fx_sum(t2) - (1 << 29)) - (1 << 29));
   fx_acc z = fx_zero();
-  const fx_const third = fx_split_const(((1ll << 60) + 1) / 3);
-  fx_mac(z, fx_lhs(fx{(float)third.l, third.h}), fx_rhs(t3));
+  fx_mac(z, fx_lhs(fx_third()), fx_rhs(t3));
   const fx c0 = fx_get<FX_WIDE>(z, ck);
   const float r = sqrtf(2.0f * fmaxf(fmaf(c1.l, 0x1p-60f, (float)c1.h * 0x1p-30f), 0.0f));
   if (ck.bad() || !(r < 0.34f)) return false;
@@ -312,7 +297,13 @@ __device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradien
   return !ck.bad() && fx_mag_ok(mag);
 }
 // The same from f: H = c f_a lambda_a.
-__device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const double* f, double c) {
+__device__ __forceinline__ fx fx_of_real(double x, unsigned& mag) { return fx_of_double(x, mag); }
+__device__ __forceinline__ fx fx_of_real(float x, unsigned& mag) {
+  if (!(fabsf(x) < 1.4375f)) mag = 0xffffffffu;
+  return fx_of_float(x);
+}
+template <typename T>
+__device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const T* f, double c) {
   fx_chk ck;
   unsigned mag = 0;
   const fx_left cl = fx_lhs(fx_of_double(c, mag)), cn = fx_lhs(fx_of_double(-c, mag)),
@@ -320,7 +311,7 @@ __device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const double* f, double
                 m3 = fx_lhs(fx_of_double(-2.0 * (c * 0.57735026918962576451), mag));
   fx_right F[8];
 #pragma unroll
-  for (int a = 0; a < 8; ++a) F[a] = fx_rhs(fx_of_double(f[a], mag));
+  for (int a = 0; a < 8; ++a) F[a] = fx_rhs(fx_of_real(f[a], mag));
   auto one = [&](const fx_left& x, const fx_right& y) {
     fx_acc s = fx_zero();
     fx_mac(s, x, y);

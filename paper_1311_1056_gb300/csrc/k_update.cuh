@@ -34,7 +34,7 @@
 #pragma once
 #include <type_traits>
 
-#include "expm.cuh"
+#include "expm_fx.cuh"
 #include "fixed.cuh"
 #include "lattice.cuh"
 #include "launch.h"
@@ -53,7 +53,12 @@ struct UpdArgs {
   int cexp;       // FP64: C holds the contributions times 2^-cexp (drift_exponent)
 };
 
-// FP64 form (k_update_fx.cuh): the drift of link (s, MU) from the fixed-point contributions.
+// FP64 form (k_update_fx.cuh): the update of link (s, MU), from the fixed-point
+// contributions C (X NULL) or from the drift in X; and its drift alone.
+__device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const double2* C, const double2* X,
+                                           double2* out, const UpdArgs& a, int s, const int* x, int MU);
+__device__ __forceinline__ double drift_f64(const Geo& g, const double2* C, double2* out, int cexp, int s, const int* x,
+                                            int MU, bool write);
 __device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
                                            const double2* C, int cexp);
 
@@ -463,6 +468,46 @@ __device__ __forceinline__ void exponent(mat<R>& A, const R* g, R eps, R sqrt_ep
   add_noise(A, g, sqrt_eps * (R)1.41421356237309504880);  // eta = sqrt(2) * normal
 }
 
+// 2 |X - Tr X / 3|_F^2 in FP64.
+__device__ __forceinline__ double general_k2(mat<double>& X) {
+  const double tr_re = (X.e[0].re + X.e[4].re + X.e[8].re) * (1.0 / 3.0);
+  const double tr_im = (X.e[0].im + X.e[4].im + X.e[8].im) * (1.0 / 3.0);
+  X.e[0].re -= tr_re; X.e[4].re -= tr_re; X.e[8].re -= tr_re;
+  X.e[0].im -= tr_im; X.e[4].im -= tr_im; X.e[8].im -= tr_im;
+  return 2.0 * norm2(X);
+}
+
+// U' = exp(A) U det^{-1/3} with everything in FP64: the FP64 and FP32-storage
+// forms beyond the fixed-point range (expm_fx.cuh).
+static __device__ __noinline__ void general_update_f64(mat<double>& Un, mat<double>& A, const mat<double>& U,
+                                                       uint64_t seed, uint32_t step, int s, int mu, double eps,
+                                                       double sqrt_eps) {
+  double eta[8];
+  normals_f64<4>(eta, seed, step, (uint32_t)s, (uint32_t)mu, STREAM_CL);
+  exponent<double>(A, eta, eps, sqrt_eps);
+  mat<double> E;
+  expm_traceless(E, A);
+  mul(Un, E, U);
+  const cx<double> z = det_inv_cuberoot(det(Un));
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], z);
+}
+static __device__ __noinline__ void general_update_f32(mat<float>& Un, const mat<float>& Af, const mat<float>& U,
+                                                       float rA) {
+  mat<double> A, E;
+  convert(A, Af);
+  expm_traceless(E, A, rA, taylor_tol<float>());
+  mat<float> Et;
+  convert(Et, E);
+  mul(Un, Et, U);
+  mat<double> Und;
+  convert(Und, Un);
+  const cx<double> z = det_inv_cuberoot(det(Und));
+  const cx<float> zt = {cvt<float>(z.re), cvt<float>(z.im)};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], zt);
+}
+
 // ------------------------------------------------ gather + exponential update
 // X of link (x, mu) = sum of its six plaquette contributions: for nu != mu,
 // mu < nu: slot 0 of (x, p) and slot 3 of (x - nu, p); mu > nu: slot 1 of
@@ -482,7 +527,12 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
   site_coords(g, s, x);
   Work<T, 2> ws(0);
   mat<T>&X = ws[0], &t = ws[1];
-  if (MODE == MODE_UPDATE_X) {
+  if constexpr (std::is_same<T, double>::value && (MODE == MODE_UPDATE || MODE == MODE_UPDATE_X)) {
+    update_f64(g, U, MODE == MODE_UPDATE ? C : nullptr, MODE == MODE_UPDATE ? nullptr : C, out, a, s, x, MU);
+    return;
+  } else if constexpr (std::is_same<T, double>::value && MODE == MODE_DRIFTMAX) {
+    // the gather is part of drift_f64
+  } else if (MODE == MODE_UPDATE_X) {
     load(X, C, MU, s, g.V);  // the drift stored by the MODE_DRIFTMAX pass
   } else if constexpr (std::is_same<T, double>::value) {
     gather_f64(X, g, s, x, MU, C, a.cexp);
@@ -506,15 +556,17 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
     return;
   }
   if (MODE == MODE_DRIFTMAX) {
-    if (s_raw < g.V) store(out, MU, s, g.V, X);
     // |K|^2 = sum_a |Tr(lambda_a X)|^2 = 2 |X - Tr X / 3|_F^2 (Tr l_a l_b = 2 delta_ab)
-    mat<double> Xd;
-    convert(Xd, X);
-    const double tr_re = (Xd.e[0].re + Xd.e[4].re + Xd.e[8].re) * (1.0 / 3.0);
-    const double tr_im = (Xd.e[0].im + Xd.e[4].im + Xd.e[8].im) * (1.0 / 3.0);
-    Xd.e[0].re -= tr_re; Xd.e[4].re -= tr_re; Xd.e[8].re -= tr_re;
-    Xd.e[0].im -= tr_im; Xd.e[4].im -= tr_im; Xd.e[8].im -= tr_im;
-    unsigned long long k2 = (unsigned long long)__double_as_longlong(2.0 * norm2(Xd));
+    double kk;
+    if constexpr (std::is_same<T, double>::value) {
+      kk = drift_f64(g, C, out, a.cexp, s, x, MU, s_raw < g.V);
+    } else {
+      if (s_raw < g.V) store(out, MU, s, g.V, X);
+      mat<double> Xd;
+      convert(Xd, X);
+      kk = general_k2(Xd);
+    }
+    unsigned long long k2 = (unsigned long long)__double_as_longlong(kk);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const unsigned long long v = __shfl_xor_sync(0xffffffffu, k2, o);
@@ -523,9 +575,9 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
     if ((threadIdx.x & 31) == 0) atomicMax(&a.sd->kmax2_bits, k2);
     return;
   }
-  // exponent A = 2 eps (X - Tr X/3) + i sqrt(eps) eta_a lambda_a; exp in FP64.
-  // The FP64 form builds A in FP64; the FP32-storage form builds it in FP32
-  // (X and the noise carry FP32 information only) and widens it for the exp.
+  // exponent A = 2 eps (X - Tr X/3) + i sqrt(eps) eta_a lambda_a.  The
+  // FP32-storage form builds it in FP32 (X and the noise carry FP32
+  // information only) and widens it for the exponential.
   const uint32_t step = a.sd->step;
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
@@ -549,35 +601,51 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
     store(out, MU, s, g.V, Un);
     return;
   }
-  mat<double> A;
-  float rA = -1.f;
-  if (sizeof(T) == 8) {
-    double eta[8];
-    normals_f64<4>(eta, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
-    convert(A, X);
-    exponent<double>(A, eta, eps, sqrt_eps);
-  } else {
+  if constexpr (std::is_same<T, float>::value) {
+    // the exponent in FP32, the exponential in fixed point; beyond its range in FP64
     float ef[8];
     normals_f32<4>(ef, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
-    mat<float> Af;
-    convert(Af, X);
-    exponent<float>(Af, ef, (float)eps, (float)sqrt_eps);
-    rA = sqrtf(norm2(Af));
-    convert(A, Af);
-  }
-  mat<double> E;
-  expm_traceless(E, A, rA, taylor_tol<T>());
-  mat<T> Et, Ul, Un;
-  convert(Et, E);
-  load(Ul, U, MU, s, g.V);
-  mul(Un, Et, Ul);
-  mat<double> Und;
-  convert(Und, Un);
-  cx<double> z = det_inv_cuberoot(det(Und));
-  cx<T> zt = {cvt<T>(z.re), cvt<T>(z.im)};
+    exponent<float>(X, ef, (float)eps, (float)sqrt_eps);
+    const float rA = sqrtf(norm2(X));
+    mat<float> Et, Ul, Un;
+    load(Ul, U, MU, s, g.V);
+    bool done = false;
+    if (rA < 1.4f) {  // every entry below the bound
+      mat<fx> A;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], zt);
-  store(out, MU, s, g.V, Un);
+      for (int k = 0; k < 9; ++k) A.e[k] = cx<fx>{fx_of_float(X.e[k].re), fx_of_float(X.e[k].im)};
+      if (fx_expm_traceless(A, rA, taylor_tol<float>())) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) Et.e[k] = cx<float>{fx_to_float(A.e[k].re), fx_to_float(A.e[k].im)};
+        mul(Un, Et, Ul);
+        float mx = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          mx = fmaxf(mx, fmaxf(fabsf(Un.e[k].re), fabsf(Un.e[k].im)));
+          A.e[k] = cx<fx>{fx_of_float(Un.e[k].re), fx_of_float(Un.e[k].im)};
+        }
+        fx_chk ck;
+        const cx<fx> d = fx_det_minus_one(A, ck);
+        const cx<float> e = {fx_to_float(d.re), fx_to_float(d.im)};
+        if (mx < 1.43f && !ck.bad() && fmaf(e.re, e.re, e.im * e.im) < 1e-11f) {
+          // det^{-1/3} = 1 - e/3 + 2 e^2/9 (the next term is below 5e-18), rounded to float
+          const float q = 2.0f / 9.0f;
+          const cx<float> z = {1.0f + fmaf(q * e.re, e.re, fmaf(-q * e.im, e.im, e.re * (-1.0f / 3.0f))),
+                               fmaf(2.0f * q * e.re, e.im, e.im * (-1.0f / 3.0f))};
+#pragma unroll
+          for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], z);
+          done = true;
+        }
+      }
+    }
+    if (!done) {
+      mat<float> Xg = X, Ug = Ul, Ung;
+      general_update_f32(Ung, Xg, Ug, rA);
+      Un = Ung;
+    }
+    store(out, MU, s, g.V, Un);
+    return;
+  }
 }
 template <typename T, int MODE>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_update_gather(Geo g, const typename vec2_of<T>::type* __restrict__ U,

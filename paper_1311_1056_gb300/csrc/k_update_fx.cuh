@@ -18,6 +18,7 @@
 #pragma once
 #include "fixed.cuh"
 #include "k_update.cuh"
+#include "noise_fx.cuh"
 
 namespace clgc {
 
@@ -305,15 +306,17 @@ static __device__ __noinline__ void general_gather(mat<double>& X, Geo g, int s,
 #pragma unroll
   for (int k = 0; k < 9; ++k) X.e[k] = cx<double>{ce * X.e[k].re, ce * X.e[k].im};
 }
-// The sums as 60-bit integers (six contributions below 1.44 fit).
+// The sums as 60-bit integers.  Six contributions below 1.44 could just pass
+// the 64-bit range at 8: the first four must stay below 5.
 __device__ __forceinline__ bool fx_gather(long long* X, const Geo& g, int s, const int* x, int MU, const int4* __restrict__ C) {
   fx_chk ck;
+  unsigned m = 0;
   mat<fx> t, l;
 #pragma unroll
   for (int k = 0; k < 18; ++k) X[k] = 0;
 #pragma unroll
-  for (int nu = 0; nu < 4; ++nu) {
-    if (nu == MU) continue;
+  for (int j = 0; j < 3; ++j) {
+    const int nu = j + (j >= MU ? 1 : 0);
     const int p = MU < nu ? plane_index(MU, nu) : plane_index(nu, MU);
     fx_load(t, C, 4 * p + (MU < nu ? 0 : 1), s, g.V, ck);
     fx_load(l, C, 4 * p + (MU < nu ? 3 : 2), hop(g, s, x, nu, -1), g.V, ck);
@@ -321,9 +324,11 @@ __device__ __forceinline__ bool fx_gather(long long* X, const Geo& g, int s, con
     for (int k = 0; k < 9; ++k) {
       X[2 * k] += fx_bits(t.e[k].re) + fx_bits(l.e[k].re);
       X[2 * k + 1] += fx_bits(t.e[k].im) + fx_bits(l.e[k].im);
+      if (j == 1)
+        m = max(m, max((unsigned)(int)(X[2 * k] >> 32) + (5u << 28), (unsigned)(int)(X[2 * k + 1] >> 32) + (5u << 28)));
     }
   }
-  return !ck.bad();
+  return !ck.bad() && m < (10u << 28);
 }
 __device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
                                            const double2* C, int cexp) {
@@ -338,6 +343,159 @@ __device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, 
     general_gather(Xg, g, s, x, MU, tag(c), ldexp(1.0, cexp));
     X = Xg;
   }
+}
+
+// --------------------------------------------------------------- update
+// (X - Tr X / 3) / 4 of the 60-bit integers X; false out of range.
+__device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long* X) {
+  fx_chk ck;
+  const long long tr = (X[0] + X[8] + X[16]) / 3, ti = (X[1] + X[9] + X[17]) / 3;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const long long re = (X[2 * k] - (k % 4 == 0 ? tr : 0)) >> 2, im = (X[2 * k + 1] - (k % 4 == 0 ? ti : 0)) >> 2;
+    ck.see<FX_WIDE>((int)(re >> 32));
+    ck.see<FX_WIDE>((int)(im >> 32));
+    Q.e[k] = cx<fx>{fx_of_bits(re), fx_of_bits(im)};
+  }
+  return !ck.bad();
+}
+// A = 2 eps (X - Tr X / 3) + i sqrt(eps) sqrt(2) g_a lambda_a from the traceless
+// quarter of X 2^-cexp and g / 8.  The noise constant 8 sqrt(2 eps) passes the fixed-point
+// bound at eps = 0.016; from there on A is formed as a quarter.
+__device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, const fx* gs, double eps, double sqrt_eps,
+                                            int cexp) {
+  fx_chk ck;
+  unsigned mag = 0;
+  const bool quarter = !(sqrt_eps < 0.12);
+  const double ks = sqrt_eps * (quarter ? 2.0 * 1.41421356237309504880 : 8.0 * 1.41421356237309504880);
+  const double kd = ldexp(quarter ? 2.0 * eps : 8.0 * eps, cexp);  // times X / 4
+  const fx kf = fx_of_double(ks, mag);
+  const fx_left d = fx_lhs(fx_of_double(kd, mag)), n = fx_lhs(kf), m = fx_lhs_neg(kf),
+                n3 = fx_lhs(fx_times(n, fx_rhs(fx_constant(NFX_RSQRT3_H, NFX_RSQRT3_L))));
+  if (!fx_mag_ok(mag)) return false;
+  fx_right R[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) R[j] = fx_rhs(gs[j]);
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+#pragma unroll
+    for (int im = 0; im < 2; ++im) {
+      fx_acc s = fx_zero();
+      fx_mac(s, d, fx_rhs(im ? A.e[k].im : A.e[k].re));
+      // i H: H01 = g0 - i g1, H02 = g3 - i g4, H12 = g5 - i g6, Hermitian;
+      // H00 = g2 + g7 / sqrt 3, H11 = -g2 + g7 / sqrt 3, H22 = -2 g7 / sqrt 3
+      const int i = k / 3, j = k % 3;
+      if (i == j) {
+        if (im) {
+          if (i < 2) fx_mac(s, i == 0 ? n : m, R[2]);
+          fx_mac(s, n3, i < 2 ? R[7] : fx_rhs(fx_twice(-gs[7])));
+        }
+      } else {
+        const int q = i + j == 1 ? 0 : i + j == 2 ? 3 : 5;
+        if (im)
+          fx_mac(s, n, R[q]);
+        else
+          fx_mac(s, i < j ? n : m, R[q + 1]);
+      }
+      const long long r = fx_sum(s) - (1 << 29);
+      if (quarter)
+        ck.see<FX_NARROW>((int)(r >> 32));
+      else
+        ck.see<FX_WIDE>((int)(r >> 32));
+      const fx w = fx_of_bits(quarter ? r << 2 : r);
+      if (im)
+        A.e[k].im = w;
+      else
+        A.e[k].re = w;
+    }
+  return !ck.bad();
+}
+
+// The adaptive step's drift pass: the operand of the update (the traceless
+// quarter of X 2^-cexp, or X itself as doubles) into out; returns |K|^2 =
+// 2 |X - Tr X / 3|_F^2.
+__device__ __forceinline__ double drift_f64(const Geo& g, const double2* C, double2* out, int cexp, int s, const int* x,
+                                            int MU, bool write) {
+  const int4* c = reinterpret_cast<const int4*>(C);
+  int4* o = reinterpret_cast<int4*>(out);
+  long long v[18];
+  mat<fx> Q;
+  if (fx_gather(v, g, s, x, MU, c) && fx_traceless_quarter(Q, v)) {
+    fx_acc n = fx_zero();
+    float nf = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      fx_mac(n, fx_lhs(Q.e[k].re), fx_rhs(Q.e[k].re));
+      fx_mac(n, fx_lhs(Q.e[k].im), fx_rhs(Q.e[k].im));
+      nf = fmaf((float)Q.e[k].re.h, (float)Q.e[k].re.h, fmaf((float)Q.e[k].im.h, (float)Q.e[k].im.h, nf));
+    }
+    if (nf < 7.5f * 0x1p60f) {
+      if (write) store<fx>(o, MU, s, g.V, Q);
+      return fx_bits_to_double(fx_sum(n) - (1 << 29), 2 * cexp + 5);
+    }
+  }
+  mat<double> Xd;
+  gather_f64(Xd, g, s, x, MU, C, cexp);
+  if (write) store(tagged{o, ldexp(1.0, cexp + 2)}, MU, s, g.V, Xd);
+  return general_k2(Xd);
+}
+
+// The whole update in fixed point: exp(A) U with U the fixed-point word that
+// the links pass left in `out`, times det^{-1/3} = 1 - e/3 for |e = det - 1| <
+// 2^-31 (the drift of the determinant over a step is 1e-15; the next term is
+// below 2^-62).  What does not fit goes through general_update_f64.
+__device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const double2* C, const double2* X,
+                                           double2* out, const UpdArgs& a, int s, const int* x, int MU) {
+  const uint32_t step = a.sd->step;
+  const double eps = a.adaptive ? a.sd->eps_n : a.eps;
+  const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
+  const tagged Xt = {reinterpret_cast<int4*>(const_cast<double2*>(X)), ldexp(1.0, a.cexp + 2)};
+  mat<fx> A;
+  bool ok;
+  if (C) {
+    long long v[18];
+    ok = fx_gather(v, g, s, x, MU, reinterpret_cast<const int4*>(C)) && fx_traceless_quarter(A, v);
+  } else {
+    fx_chk ck;
+    fx_load(A, Xt.p, MU, s, g.V, ck);
+    ok = !ck.bad();
+  }
+  if (ok) {
+    {
+      fx gs[8];
+      normals_fx<4>(gs, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
+      ok = fx_exponent(A, gs, eps, sqrt_eps, a.cexp);
+    }
+    ok = ok && fx_expm_traceless(A, fx_norm(A), TAYLOR_TOL_FP64);
+    if (ok) {
+      fx_chk ck;
+      mat<fx> u;
+      fx_load_plain(u, reinterpret_cast<const int4*>(out), MU, s, g.V);
+      if (fx_is_raw(u.e[0].re.l)) ck.fail();
+      fx_mul_left<FX_WIDE>(A, u, ck);
+      const cx<fx> e = fx_det_minus_one(A, ck);
+      if (!ck.bad() && e.re.h == 0 && e.im.h == 0) {
+        const float er = e.re.l * (-1.0f / 3.0f), ei = e.im.l * (-1.0f / 3.0f);  // units of 2^-60
+        double2* p = out + (size_t)MU * 9 * g.V + s;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          const float ur = (float)A.e[k].re.h * 0x1p-30f, ui = (float)A.e[k].im.h * 0x1p-30f;
+          const fx re = {A.e[k].re.l + fmaf(er, ur, -ei * ui), A.e[k].re.h};
+          const fx im = {A.e[k].im.l + fmaf(er, ui, ei * ur), A.e[k].im.h};
+          p[(size_t)k * g.V] = make_double2(fx_to_double(re), fx_to_double(im));
+        }
+        return;
+      }
+    }
+  }
+  mat<double> Xg, u, r;
+  if (C)
+    gather_f64(Xg, g, s, x, MU, C, a.cexp);
+  else
+    load(Xg, Xt, MU, s, g.V);
+  load(u, U, MU, s, g.V);
+  general_update_f64(r, Xg, u, a.seed, step, s, MU, eps, sqrt_eps);
+  store(out, MU, s, g.V, r);
 }
 
 }  // namespace clgc

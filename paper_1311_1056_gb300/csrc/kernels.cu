@@ -9,6 +9,7 @@
 #include "fixed.cuh"
 #include "launch.h"
 #include "lattice.cuh"
+#include "noise_fx.cuh"
 #include "philox.cuh"
 #include "su3.cuh"
 
@@ -239,7 +240,10 @@ __global__ void k_noise_sample(int site0, int n, uint64_t seed, uint32_t step, u
   if (i >= n) return;
   const uint32_t s = (uint32_t)(site0 + i);
   if constexpr (std::is_same<T, double>::value) {
-    normals_f64<4>(out + 8 * (size_t)i, seed, step, s, mu, STREAM_CL);
+    fx e[8];
+    normals_fx<4>(e, seed, step, s, mu, STREAM_CL);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) out[8 * (size_t)i + j] = fx_to_double(e[j], 3);
   } else if constexpr (std::is_same<T, float>::value) {
     float e[8];
     normals_f32<4>(e, seed, step, s, mu, STREAM_CL);
@@ -632,6 +636,29 @@ static __device__ __noinline__ void general_cool_grad_omega(const Geo g, int4* U
   general_cool_omega(fa, c, Om, Omi, s, g.V);
 }
 
+// FP32-storage form: Omega_x and its inverse from f (FP32 or, read back from
+// the rule's pass, FP64), the exponential in fixed point and rounded to float.
+static __device__ __noinline__ void general_omega_f32(const double* fa, double c, float* Om, float* Omi, int s, int V) {
+  const herm h = herm_from_algebra(fa, c);
+  herm om, omi;
+  expm_hermitian_pair(om, omi, h, TAYLOR_TOL_FP32_STORAGE);
+  store_herm(Om, s, V, om);
+  store_herm(Omi, s, V, omi);
+}
+template <typename R>
+__device__ __forceinline__ void omega_f32(const R* fa, double c, float* Om, float* Omi, int s, int V) {
+  fx_herm H, om, omi;
+  if (fx_herm_of_f(H, fa, c) && fx_expm_hermitian_pair(om, omi, H, TAYLOR_TOL_FP32_STORAGE)) {
+    fx_store_herm(Om, s, V, om);
+    fx_store_herm(Omi, s, V, omi);
+  } else {
+    double fd[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) fd[a] = cvt<double>(fa[a]);
+    general_omega_f32(fd, c, Om, Omi, s, V);
+  }
+}
+
 // Single-pass sweep of the D_0 / D_1 rules, part 1: the strength alpha_ad of
 // these rules needs only the unitarity norm, which the previous sweep's apply
 // (k_cool_apply_tiles) summed, so the rule has decided before this kernel runs
@@ -660,13 +687,7 @@ __device__ __forceinline__ void cool_grad_omega_body(const Geo& g, const typenam
     } else {
       T fa[8];
       cool_grad_site<T>(g, U, s, x, fa);
-      double fd[8];
-#pragma unroll
-      for (int a = 0; a < 8; ++a) fd[a] = cvt<double>(fa[a]);
-      herm h = herm_from_algebra(fd, c), om, omi;
-      expm_hermitian_pair(om, omi, h, taylor_tol<T>());
-      store_herm(Om, s, g.V, om);
-      store_herm(Omi, s, g.V, omi);
+      omega_f32(fa, c, Om, Omi, s, g.V);
     }
   }
 }
@@ -791,10 +812,7 @@ __device__ __forceinline__ void cool_omega_body(const Geo& g, const double* __re
         general_cool_omega(fg, c, (int2*)Om, (int2*)Omi, s, g.V);
       }
     } else {
-      herm h = herm_from_algebra(fa, -eps * cs->alpha_ad), om, omi;
-      expm_hermitian_pair(om, omi, h, taylor_tol<T>());
-      store_herm(Om, s, g.V, om);
-      store_herm(Omi, s, g.V, omi);
+      omega_f32(fa, -eps * cs->alpha_ad, Om, Omi, s, g.V);
     }
   }
 }

@@ -123,3 +123,53 @@ def test_a_cooling_call_without_a_sweep_keeps_the_links(cl):
         rep = lat.cool(cl.make_cool(0.01, mode=cl.CL_D1, n_min=0, n_max=5, d_floor=1e9))
         assert rep["sweeps"] == 0
         assert np.array_equal(lat.links(), U)
+
+
+@pytest.mark.parametrize("spread", [0, 0.1, 0.4, "mixed"])
+@pytest.mark.parametrize("eps", [1e-6, 1e-3, 0.0143, 0.0145, 0.05, 0.4])
+@pytest.mark.parametrize("k_ref", [0.0, 3.0])
+def test_update_over_step_sizes(cl, spread, eps, k_ref):
+    """One CL step.  The step sizes put the exponent's norm below, next to and beyond the halvings of its
+    series and the fixed-point range, and lie on both sides of the noise constant's (eps = 0.0144).  The update
+    is three products of matrices of size max |U| exp(|A|); 1e-12 of the result is several hundred roundings.
+    (The drift itself is off by up to 1e-11 of its size for links far from SU(3), times eps.)"""
+    L = (4, 3, 2, 5)
+    U = field(L, spread, 31)
+    if k_ref:
+        ref, _, _ = O.cl_step_adaptive(L, U, 6.0, 1.0, eps, k_ref, 99, 4)
+    else:
+        ref = O.cl_step(L, U, 6.0, 1.0, eps, 99, 4)
+    if not np.isfinite(ref).all():
+        pytest.skip("the reference step itself overflows")
+    with cl.Lattice(L, beta=6.0, theta=1.0, seed=99) as lat:
+        lat.set_links(U)
+        cl.cl_set_step(lat.h, 4)
+        lat.set_adaptive_step(k_ref)
+        lat.step(eps)
+        Ug = lat.links()
+    assert np.abs(Ug - ref).max() <= 1e-12 * np.abs(ref).max() + 1e-11 * eps * np.abs(ref).max() ** 2
+
+
+@pytest.mark.parametrize("eps", [1e-4, 0.02, 0.4])
+def test_fp32_storage_update_over_step_sizes(cl, eps):
+    """The FP32-storage exponential is rounded to float once; the product and the determinant's root are
+    ~20 dependent roundings of 6e-8 on links of order one: 5e-6 of the result."""
+    L = (4, 3, 2, 5)
+    U = field(L, 0, 31).astype(np.complex64).astype(np.complex128)
+    ref = O.cl_step(L, U, 6.0, 1.0, eps, 99, 0)
+    with cl.Lattice(L, beta=6.0, theta=1.0, seed=99, prec=cl.CL_FP32_STORAGE) as lat:
+        lat.set_links(U)
+        lat.step(eps)
+        assert np.abs(lat.links() - ref).max() <= 5e-6 * np.abs(ref).max()
+
+
+def test_reprojection_of_links_off_determinant_one(cl):
+    """det U away from 1 (beyond the fixed-point series): the principal cube root, as everywhere."""
+    L = (2, 4, 3, 2)
+    U = field(L, 0, 8) * (1.0 + 1e-6)
+    U[3, 1] *= 1.01 * np.exp(0.2j)
+    ref = O.cl_step(L, U, 0.0, 0.0, 1e-3, 5, 0)
+    with cl.Lattice(L, beta=0.0, theta=0.0, seed=5) as lat:
+        lat.set_links(U)
+        lat.step(1e-3)
+        assert np.abs(lat.links() - ref).max() <= 1e-12
