@@ -271,7 +271,7 @@ cl_status do_obs(cl_lattice* l, ObsOut* dst, double* q_site) {
     CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->F, obs_clover_scale(l->prec), 0.0, l->st); }));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->F, 1, l->partials, q_site, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->Un, l->Pq, l->Dq, l->F, l->partials, q_site, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
     return launch_obs_final(l->g, l->partials, l->p.beta, l->p.theta_re, l->p.theta_im, dst, l->st);
   }));

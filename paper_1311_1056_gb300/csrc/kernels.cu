@@ -753,6 +753,7 @@ __device__ __forceinline__ void cool_rule(const Geo& g, const double* tot, const
 }
 __device__ __forceinline__ void cool_adapt_body(const Geo& g, const double* partials, int nb, const CoolArgs& a,
                                                 CoolState* cs, int first) {
+  if (!first && cs->done) return;
   __shared__ double tot[NQ_COOL];
   reduce_partials<NQ_COOL, -1>(partials, nb, tot);
   __syncthreads();
@@ -995,6 +996,7 @@ __global__ void __launch_bounds__(COOL_TILE, COOL_TILE_MIN_BLOCKS(T))
 enum { COOL_RULE_THREADS = 1024 };
 __device__ __forceinline__ void cool_adapt_tiles_body(const Geo& g, const double2* __restrict__ rec, int nrec,
                                                       const CoolArgs& a, CoolState* cs) {
+  if (cs->done) return;
   __shared__ double2 sm[COOL_RULE_THREADS / 32];
   double2 v = make_double2(0.0, 0.0);
 #pragma unroll 4
@@ -1083,12 +1085,218 @@ __global__ void __launch_bounds__(DF_APPLY_BLOCK, 4) k_cool_apply_df(Geo g, floa
 }
 
 // ----------------------------------------------------------- observables
-// Per site: the six plaquettes P_{mu nu}(x) = U_mu(x) U_nu(x+mu) U_mu(x+nu)^{-1} U_nu(x)^{-1}
-// (Tr P / 3 and Tr P + Tr P^{-1} for S_W), (1/3) Tr U U^+ of the four links,
-// max |det U - 1| (FP64), nonfinite count and, with the clover field,
-// q_L(x) = kappa [Tr F01 F23 - Tr F02 F13 + Tr F03 F12].
+// Per site: Tr P / 3 and Tr P + Tr P^{-1} of the six plaquettes (from the
+// plaquette pass's P and D = P - P^{-1}), (1/3) Tr U U^+ of the four links,
+// max |det U - 1|^2, nonfinite count and q_L(x) = kappa [Tr F01 F23 - Tr F02 F13
+// + Tr F03 F12] of the clover field.  Sums of a site run in fixed point and
+// are widened to FP64 once (GB300's FP64 rate again: 430 us at 16^4 with the
+// plaquettes, determinants and traces formed in FP64).
+
+// One link's Tr U U^+ - 3 (60-bit integer) and |det U - 1|^2; false out of range.
+__device__ __forceinline__ bool obs_link(const mat<fx>& u, long long& dev, double& det2) {
+  fx_chk ck;
+  fx_acc n = fx_zero();
+  float nf = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    fx_mac(n, fx_lhs(u.e[k].re), fx_rhs(u.e[k].re));
+    fx_mac(n, fx_lhs(u.e[k].im), fx_rhs(u.e[k].im));
+    nf = fmaf((float)u.e[k].re.h, (float)u.e[k].re.h, fmaf((float)u.e[k].im.h, (float)u.e[k].im.h, nf));
+  }
+  const cx<fx> e = fx_det_minus_one(u, ck);
+  if (ck.bad() || !(nf < 4.9f * 0x1p60f)) return false;
+  dev += fx_sum(n) - ((3ll << 60) + (1 << 29));
+  const double re = fx_to_double(e.re), im = fx_to_double(e.im);
+  det2 = fmax(det2, fma(re, re, im * im));
+  return true;
+}
+// The same of a link beyond the range (or not finite), in FP64; returns Tr U U^+.
+template <typename T>
+static __device__ __noinline__ double general_obs_link(const typename vec2_of<T>::type* U, int mu, int s, int V, double* det2,
+                                                       double* bad) {
+  mat<T> u;
+  load(u, U, mu, s, V);
+  if (!finite_mat(u)) *bad = 1.0;
+  mat<double> ud;
+  convert(ud, u);
+  const cx<double> d = det(ud);
+  const double h = hypot(d.re - 1.0, d.im);
+  *det2 = fmax(*det2, h * h);
+  return (double)norm2(u);
+}
+// Tr of a stored matrix times 1/4 as a 60-bit integer (FP32 storage: of its float trace).
+__device__ __forceinline__ bool obs_trace(long long& re, long long& im, const float2* f, int p, int s, int V) {
+  float tr = 0.0f, ti = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 9; k += 4) {
+    const float2 w = __ldg(f + ((size_t)p * 9 + k) * V + s);
+    tr += w.x;
+    ti += w.y;
+  }
+  if (!(fabsf(tr) < 7.0f && fabsf(ti) < 7.0f)) return false;
+  re = fx_bits(fx_of_float(0.25f * tr));
+  im = fx_bits(fx_of_float(0.25f * ti));
+  return true;
+}
+__device__ __forceinline__ bool obs_trace(long long& re, long long& im, const double2* f, int p, int s, int V) {
+  const int4* P = reinterpret_cast<const int4*>(f);
+  bool ok = true;
+  re = im = 0;
+#pragma unroll
+  for (int k = 0; k < 9; k += 4) {
+    const cx<fx> w = unpack(__ldg(P + ((size_t)p * 9 + k) * V + s));
+    if (k == 0 && fx_is_raw(w.re.l)) ok = false;
+    re += fx_bits(w.re) >> 2;
+    im += fx_bits(w.im) >> 2;
+  }
+  return ok;
+}
+template <typename T>
+static __device__ __noinline__ void general_obs_trace(const typename vec2_of<T>::type* f, int p, int s, int V, double sc,
+                                                      double* out) {
+  mat<T> m;
+  if constexpr (std::is_same<T, double>::value)
+    load(m, tagged{(int4*)f, sc}, p, s, V);
+  else
+    load(m, f, p, s, V);
+  const cx<T> t = trace(m);
+  out[0] = (double)t.re;
+  out[1] = (double)t.im;
+}
+// Tr F_p F_{5-p} in FP64.
+template <typename T>
+static __device__ __noinline__ void general_obs_ff(const typename vec2_of<T>::type* F, int p, int s, int V, double* out) {
+  mat<T> F1, F2;
+  if constexpr (std::is_same<T, double>::value) {
+    load(F1, tagged{(int4*)F, 1.0}, p, s, V);
+    load(F2, tagged{(int4*)F, 1.0}, 5 - p, s, V);
+  } else {
+    load(F1, F, p, s, V);
+    load(F2, F, 5 - p, s, V);
+  }
+  const cx<T> t = trace_mul(F1, F2);
+  out[0] = (double)t.re;
+  out[1] = (double)t.im;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_of<T>::type* __restrict__ U,
+                                                    const int4* __restrict__ Ux,
+                                                    const typename vec2_of<T>::type* __restrict__ Pq,
+                                                    const typename vec2_of<T>::type* __restrict__ Dq,
+                                                    const typename vec2_of<T>::type* __restrict__ F,
+                                                    double* partials, double* q_site) {
+  constexpr bool FX = std::is_same<T, double>::value;
+  double v[NQ_OBS];
+#pragma unroll
+  for (int q = 0; q < NQ_OBS; ++q) v[q] = 0.0;
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
+    // links
+    long long dev = 0;
+    double wild = 0.0, det2 = 0.0, bad = 0.0;
+#pragma unroll 1
+    for (int mu = 0; mu < 4; ++mu) {
+      mat<fx> u;
+      bool in;
+      if constexpr (FX) {
+        load<fx>(u, Ux, mu, s, g.V);
+        in = !fx_is_raw(u.e[0].re.l);
+      } else {
+        mat<T> w;
+        load(w, U, mu, s, g.V);
+        in = true;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          in = in && fabsf((float)w.e[k].re) < 1.4375f && fabsf((float)w.e[k].im) < 1.4375f;
+          u.e[k] = cx<fx>{fx_of_float((float)w.e[k].re), fx_of_float((float)w.e[k].im)};
+        }
+      }
+      if (!in || !obs_link(u, dev, det2)) wild += general_obs_link<T>(U, mu, s, g.V, &det2, &bad) - 3.0;
+    }
+    v[4] += (12.0 + (fx_bits_to_double(dev) + wild)) * (1.0 / 3.0);
+    v[7] = fmax(v[7], det2);
+    v[8] += bad;
+    // plaquettes: Tr P and Tr P^{-1} = Tr P - Tr D (the fixed-point D is halved)
+    long long pr = 0, pi = 0, dr = 0, di = 0;  // units of 2^-58
+    double wp[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int p = 0; p < 6; ++p) {
+      long long a, b, c, d;
+      if (obs_trace(a, b, Pq, p, s, g.V) && obs_trace(c, d, Dq, p, s, g.V)) {
+        pr += a;
+        pi += b;
+        dr += c;
+        di += d;
+      } else {
+        double t[2];
+        general_obs_trace<T>(Pq, p, s, g.V, 1.0, t);
+        wp[0] += t[0];
+        wp[1] += t[1];
+        general_obs_trace<T>(Dq, p, s, g.V, 2.0, t);
+        wp[2] += t[0];
+        wp[3] += t[1];
+      }
+    }
+    const double tr = fx_bits_to_double(pr, 2) + wp[0], ti = fx_bits_to_double(pi, 2) + wp[1];
+    v[0] += tr * (1.0 / 3.0);
+    v[1] += ti * (1.0 / 3.0);
+    v[2] += 2.0 * tr - (fx_bits_to_double(dr, FX ? 3 : 2) + wp[2]);
+    v[3] += 2.0 * ti - (fx_bits_to_double(di, FX ? 3 : 2) + wp[3]);
+    // topological charge density; F carries obs_clover_scale
+    cx<double> q = {0.0, 0.0};
+    if constexpr (FX) {
+      fx_acc re = fx_zero(), im = fx_zero();
+      fx_chk ck;
+#pragma unroll 1
+      for (int p = 0; p < 3; ++p) {  // the planes 1 and 4 are both stored negated
+        mat<fx> F1, F2;
+        fx_load(F1, (const int4*)F, p, s, g.V, ck);
+        fx_load(F2, (const int4*)F, 5 - p, s, g.V, ck);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            fx_cmac(re, im, p == 1 ? fx_lhs_neg(F1.e[3 * i + k]) : fx_lhs(F1.e[3 * i + k]), fx_rhs(F2.e[3 * k + i]));
+      }
+      if (!ck.bad()) {  // |F| < 0.36: 54 products stay below 7
+        q.re = fx_bits_to_double(fx_sum<true>(re) - (1 << 29));
+        q.im = fx_bits_to_double(fx_sum<true>(im) - (1 << 29));
+      } else {
+        for (int p = 0; p < 3; ++p) {
+          double t[2];
+          general_obs_ff<T>(F, p, s, g.V, t);
+          q.re += p == 1 ? -t[0] : t[0];
+          q.im += p == 1 ? -t[1] : t[1];
+        }
+      }
+      q.re *= 1024.0 * KAPPA_Q;
+      q.im *= 1024.0 * KAPPA_Q;
+    } else {
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        mat<T> F1, F2;
+        load(F1, F, p, s, g.V);
+        load(F2, F, 5 - p, s, g.V);
+        const cx<T> t = trace_mul(F1, F2);
+        q.re += p == 1 ? -cvt<double>(t.re) : cvt<double>(t.re);
+        q.im += p == 1 ? -cvt<double>(t.im) : cvt<double>(t.im);
+      }
+      q.re *= KAPPA_Q;
+      q.im *= KAPPA_Q;
+    }
+    v[5] += q.re;
+    v[6] += q.im;
+    if (q_site) {
+      q_site[2 * (size_t)s] = q.re;
+      q_site[2 * (size_t)s + 1] = q.im;
+    }
+  }
+  block_reduce_store<NQ_OBS, 7>(v, partials + (size_t)blockIdx.x * NQ_OBS);
+}
+
+// DF64 form: the plaquettes formed here.
+template <typename T>
+__global__ void __launch_bounds__(RED_THREADS) k_obs_direct(Geo g, const typename vec2_of<T>::type* __restrict__ U,
                                                     const typename vec2_of<T>::type* __restrict__ F,
                                                     int with_q, double* partials, double* q_site) {
   double v[NQ_OBS];
@@ -1107,7 +1315,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
       mat<double> ud;
       convert(ud, u);
       cx<double> d = det(ud);
-      v[7] = fmax(v[7], hypot(d.re - 1.0, d.im));
+      const double h = hypot(d.re - 1.0, d.im);
+      v[7] = fmax(v[7], h * h);
     }
 #pragma unroll
     for (int p = 0; p < 6; ++p) {
@@ -1133,21 +1342,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
       cx<double> q = {0.0, 0.0};
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
-        if constexpr (std::is_same<T, double>::value) {
-          load(F1, tagged{(int4*)F, 1.0}, p, s, g.V);
-          load(F2, tagged{(int4*)F, 1.0}, 5 - p, s, g.V);
-        } else {
-          load(F1, F, p, s, g.V);
-          load(F2, F, 5 - p, s, g.V);
-        }
+        load(F1, F, p, s, g.V);
+        load(F2, F, 5 - p, s, g.V);
         cx<T> t = trace_mul(F1, F2);
         double sg = (p == 1) ? -1.0 : 1.0;
         q.re += sg * (double)t.re;
         q.im += sg * (double)t.im;
       }
-      // F carries obs_clover_scale, 1/32 in the FP64 form
-      q.re *= std::is_same<T, double>::value ? 1024.0 * KAPPA_Q : KAPPA_Q;
-      q.im *= std::is_same<T, double>::value ? 1024.0 * KAPPA_Q : KAPPA_Q;
+      q.re *= KAPPA_Q;
+      q.im *= KAPPA_Q;
       v[5] += q.re;
       v[6] += q.im;
       if (q_site) {
@@ -1177,7 +1380,7 @@ __global__ void k_obs_final(Geo g, const double* partials, int nb, double beta, 
   // S = S_W - i theta Q
   out->s_re = out->sw_re + th_re * tot[6] + th_im * tot[5];
   out->s_im = out->sw_im - th_re * tot[5] + th_im * tot[6];
-  out->max_det_dev = tot[7];
+  out->max_det_dev = sqrt(tot[7]);
   out->nonfinite = tot[8];
 }
 
@@ -1580,14 +1783,17 @@ cudaError_t launch_cool_adapt_tiles(const GeoH& h, const double* rec, CoolArgs a
   return cudaGetLastError();
 }
 
-cudaError_t launch_obs(int prec, const GeoH& h, const void* U, const void* F, int with_q,
-                       double* partials, double* q_site, cudaStream_t st) {
+cudaError_t launch_obs(int prec, const GeoH& h, const void* U, const void* Ux, const void* Pq, const void* Dq,
+                       const void* F, double* partials, double* q_site, cudaStream_t st) {
   Geo g = to_geo(h);
   return by_prec(prec, [&](auto t) {
     using T = decltype(t);
-    k_obs<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const typename vec2_of<T>::type*)U,
-                                                        (const typename vec2_of<T>::type*)F, with_q, partials,
-                                                        q_site);
+    typedef typename vec2_of<T>::type V2;
+    if constexpr (std::is_same<T, df64>::value)
+      k_obs_direct<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const V2*)U, (const V2*)F, 1, partials, q_site);
+    else
+      k_obs<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const V2*)U, (const int4*)Ux, (const V2*)Pq,
+                                                          (const V2*)Dq, (const V2*)F, partials, q_site);
   });
 }
 

@@ -181,10 +181,11 @@ cudaError_t launch_cool_grad_omega(int prec, const GeoH& g, const void* U, void*
 cudaError_t launch_cool_apply_tiles(int prec, const GeoH& g, void* U, const void* Om, const void* Omi,
                                     double* rec, const CoolState* cs, cudaStream_t st);
 cudaError_t launch_cool_adapt_tiles(const GeoH& g, const double* rec, CoolArgs a, CoolState* cs, cudaStream_t st);
-// Observables: per-site pass (F must hold the unscaled clover field when
-// with_q) then the final fixed-order reduction into *out.
-cudaError_t launch_obs(int prec, const GeoH& g, const void* U, const void* F, int with_q,
-                       double* partials, double* q_site, cudaStream_t st);
+// Observables: per-site pass over the links, the plaquette pass's fields and
+// the clover field F (scale obs_clover_scale), then the final fixed-order
+// reduction into *out.
+cudaError_t launch_obs(int prec, const GeoH& g, const void* U, const void* Ux, const void* Pq, const void* Dq,
+                       const void* F, double* partials, double* q_site, cudaStream_t st);
 cudaError_t launch_obs_final(const GeoH& g, const double* partials, double beta, double th_re,
                              double th_im, ObsOut* out, cudaStream_t st);
 // Fused batch: one launch of family fam (ENS_*) over nw work items (device
