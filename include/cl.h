@@ -175,7 +175,9 @@ cl_status cl_trajectory(cl_lattice* lat, double eps, int n_steps, const cl_cool_
  * CL_TUNE_FORCE (per-plaquette drift), CL_TUNE_UPDATE (noise + exponential
  * update), CL_TUNE_OMEGA (cooling transformation), CL_TUNE_APPLY (cooling
  * apply).  The reductions keep a fixed shape so that their summation order,
- * and hence every result, is the same under any tuning.
+ * and hence every result, is the same under any tuning.  The cooling kernels
+ * choose their own shape by lattice size: the last two families are accepted,
+ * timed and stored, and change no launch.
  * cl_set_blocks: blocks[CL_NTUNE], each 0 (default, 128) or a multiple of 32
  *   in [32, 256]; takes effect for later launches (graphs already captured
  *   keep the shape they were captured with).
@@ -473,7 +475,7 @@ enum {
   CL_PHASE_CLOVER = 0,     /* link inverses, plaquettes, clover field */
   CL_PHASE_UPDATE = 1,     /* drift gather + noise + exponential update */
   CL_PHASE_COOL_GRAD = 2,  /* cooling gradient f_ax + partial sums */
-  CL_PHASE_COOL_RULE = 3,  /* adaptive rule (one block) */
+  CL_PHASE_COOL_RULE = 3,  /* adaptive rule: runs inside the gradient and apply kernels, no launch of its own */
   CL_PHASE_COOL_OMEGA = 4, /* Omega_x, Omega_x^{-1} */
   CL_PHASE_COOL_APPLY = 5, /* U <- Omega U Omega^{-1} */
   CL_PHASE_OBS = 6,        /* observables */

@@ -179,8 +179,9 @@ cl_status do_steps(cl_lattice* l, double eps, int n) {
   return CL_OK;
 }
 
-CoolArgs cool_args(const cl_cool_params* cp) {
+CoolArgs cool_args(const cl_cool_params* cp, int V) {
   CoolArgs a;
+  a.inv_links = 1.0 / (4.0 * (double)V);
   a.eps = cp->eps;
   a.alpha = cp->alpha;
   a.tol_rel = cp->tol_rel;
@@ -191,6 +192,10 @@ CoolArgs cool_args(const cl_cool_params* cp) {
   a.n_max = cp->n_max;
   a.forced_sweeps = cp->forced_sweeps;
   return a;
+}
+
+CoolBufs cool_bufs(cl_lattice* l, const CoolArgs& a, CoolState* cs) {
+  return CoolBufs{l->U, l->prec == 1 ? l->U : l->Un, l->f, l->Om, l->Omi, l->crec, l->sd, cs, a};
 }
 
 cl_status check_cool(const cl_cool_params* cp) {
@@ -205,64 +210,31 @@ cl_status check_cool(const cl_cool_params* cp) {
 // Enqueue the whole cooling loop; the device rule decides how many sweeps
 // actually run (later launches return at once once it says done).
 //
-// D_0 and D_1 (FP64, FP32 storage) run single-pass sweeps: their strength
-// needs only the unitarity norm, so after the first sweep each apply also
-// sums the norm of the links it writes (one record per tile), the rule
-// decides the next sweep from those records, and one kernel forms the
-// gradient and Omega together (f stays in registers): rule, gradient +
-// Omega, apply per sweep instead of gradient, rule, Omega, apply.  D_2 needs
-// sum |f_ax| before Omega, so it keeps the four-kernel sweep, as does the
-// DF64 form.
+// The rule runs in the last block of the kernel whose sums it needs.  D_0 and
+// D_1 need only the unitarity norm, so after the first sweep each apply also
+// sums the norm of the links it writes and one kernel forms the gradient and
+// Omega together (gradient + Omega, apply per sweep).  D_2 needs sum |f_ax|
+// before Omega: gradient, Omega, apply per sweep and a last gradient.
 cl_status do_cool(cl_lattice* l, const cl_cool_params* cp) {
-  CoolArgs a = cool_args(cp);
+  CoolArgs a = cool_args(cp, l->g.V);
   const int n_iter = cp->forced_sweeps >= 0 ? cp->forced_sweeps : cp->n_max;
-  const bool single_pass = (cp->mode == CL_D0 || cp->mode == CL_D1) && l->prec != 2;
-  // FP64: the sweeps work on the fixed-point links in Un (launch.h)
-  void* X = l->prec == 0 ? l->Un : l->U;
-  auto unload = [&] {
-    if (l->prec != 0) return cudaSuccess;
-    return timed(l, CL_PHASE_COOL_APPLY, [&] { return launch_cool_unload(l->g, l->U, l->Un, l->cs, l->st); });
-  };
-  if (single_pass) {
-    // sweep 0: the rule's first inputs from a plain gradient pass
-    CK(timed(l, CL_PHASE_COOL_GRAD, [&] {
-      return launch_cool_grad(l->prec, l->g, l->U, X, l->f, l->partials, nullptr, l->st);
-    }));
-    CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt(l->g, l->partials, a, l->cs, 1, l->st); }));
-    if (n_iter == 0) return CL_OK;
-    CK(timed(l, CL_PHASE_COOL_OMEGA, [&] {
-      return launch_cool_omega(l->prec, l->g, l->f, l->Om, l->Omi, cp->eps, l->cs, l->st);
-    }));
+  const bool single_pass = cp->mode == CL_D0 || cp->mode == CL_D1;
+  const CoolBufs B = cool_bufs(l, a, l->cs);
+  CK(timed(l, CL_PHASE_COOL_GRAD, [&] { return launch_cool_grad(l->prec, l->g, B, true, true, l->st); }));
+  if (n_iter == 0) return CL_OK;
+  for (int k = 0; k < n_iter; ++k) {
+    if (single_pass && k > 0)
+      CK(timed(l, CL_PHASE_COOL_GRAD_OMEGA, [&] { return launch_cool_grad_omega(l->prec, l->g, B, l->st); }));
+    else
+      CK(timed(l, CL_PHASE_COOL_OMEGA, [&] { return launch_cool_omega(l->prec, l->g, B, l->st); }));
     CK(timed(l, CL_PHASE_COOL_APPLY, [&] {
-      return launch_cool_apply_tiles(l->prec, l->g, X, l->Om, l->Omi, l->crec, l->cs, l->st);
+      return launch_cool_apply(l->prec, l->g, B, single_pass, k == n_iter - 1, l->st);
     }));
-    for (int k = 1; k <= n_iter; ++k) {
-      CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt_tiles(l->g, l->crec, a, l->cs, l->st); }));
-      if (k == n_iter) break;
-      CK(timed(l, CL_PHASE_COOL_GRAD_OMEGA, [&] {
-        return launch_cool_grad_omega(l->prec, l->g, X, l->Om, l->Omi, cp->eps, l->cs, l->st);
+    if (!single_pass)
+      CK(timed(l, CL_PHASE_COOL_GRAD, [&] {
+        return launch_cool_grad(l->prec, l->g, B, false, true, l->st);
       }));
-      CK(timed(l, CL_PHASE_COOL_APPLY, [&] {
-        return launch_cool_apply_tiles(l->prec, l->g, X, l->Om, l->Omi, l->crec, l->cs, l->st);
-      }));
-    }
-    CK(unload());
-    return CL_OK;
   }
-  for (int k = 0; k <= n_iter; ++k) {
-    // the first gradient of a call always runs: the done flag still holds
-    // the previous call's decision until the rule resets it (first = 1)
-    CK(timed(l, CL_PHASE_COOL_GRAD, [&] {
-      return launch_cool_grad(l->prec, l->g, l->U, X, l->f, l->partials, k == 0 ? nullptr : l->cs, l->st);
-    }));
-    CK(timed(l, CL_PHASE_COOL_RULE, [&] { return launch_cool_adapt(l->g, l->partials, a, l->cs, k == 0, l->st); }));
-    if (k == n_iter) break;
-    CK(timed(l, CL_PHASE_COOL_OMEGA, [&] {
-      return launch_cool_omega(l->prec, l->g, l->f, l->Om, l->Omi, cp->eps, l->cs, l->st);
-    }));
-    CK(timed(l, CL_PHASE_COOL_APPLY, [&] { return launch_cool_apply(l->prec, l->g, X, l->Om, l->Omi, l->cs, l->st); }));
-  }
-  if (n_iter > 0) CK(unload());
   return CL_OK;
 }
 
@@ -324,14 +296,11 @@ cudaError_t init_state(cl_lattice* l) {
   l->launches++;
   if (e == cudaSuccess && params->gauge_sigma > 0.0) {
     e = launch_gauge_omega(l->prec, l->g, l->Om, l->Omi, params->seed, params->gauge_sigma, l->st);
-    if (l->prec == 0) {  // on the fixed-point words (launch.h)
-      if (e == cudaSuccess) e = launch_cool_load(l->g, l->U, l->Un, l->st);
-      if (e == cudaSuccess) e = launch_cool_apply(l->prec, l->g, l->Un, l->Om, l->Omi, nullptr, l->st);
-      if (e == cudaSuccess) e = launch_cool_unload(l->g, l->U, l->Un, nullptr, l->st);
-      l->launches += 2;
-    } else if (e == cudaSuccess) {
-      e = launch_cool_apply(l->prec, l->g, l->U, l->Om, l->Omi, nullptr, l->st);
+    if (e == cudaSuccess && l->prec != 1) {  // the apply works on the fixed-point words (launch.h)
+      e = launch_cool_load(l->prec, l->g, l->U, l->Un, l->st);
+      l->launches++;
     }
+    if (e == cudaSuccess) e = launch_cool_apply(l->prec, l->g, cool_bufs(l, CoolArgs(), nullptr), false, true, l->st);
     l->launches += 2;
   }
   return e;
@@ -676,18 +645,11 @@ cl_status cl_drift(cl_lattice* l, double* host_aos) {
 
 cl_status cl_cool_gradient(cl_lattice* l, double* host_f) {
   if (!l || !host_f) return fail(CL_ERR_INVALID, "NULL argument");
-  CK(launch_cool_grad(l->prec, l->g, l->U, l->Un, l->f, l->partials, nullptr, l->st));
+  CK(launch_cool_grad(l->prec, l->g, cool_bufs(l, CoolArgs(), l->cs), true, false, l->st));
   l->launches++;
   const size_t n = 8 * (size_t)l->g.V;
   CK(cudaMemcpyAsync(host_f, l->f, sizeof(double) * n, cudaMemcpyDeviceToHost, l->st));
   CK(cudaStreamSynchronize(l->st));
-  if (l->prec == 2) {  // DF64 keeps f as (hi, lo) float pairs: widen in place
-    for (size_t i = 0; i < n; ++i) {
-      float hl[2];
-      std::memcpy(hl, host_f + i, sizeof(hl));
-      host_f[i] = (double)hl[0] + (double)hl[1];
-    }
-  }
   return CL_OK;
 }
 
@@ -900,15 +862,13 @@ struct FusedPlan {
     int n;
   };
   List fam[ENS_NFAM + 3];  // + the gradient of the first sweep (all chains), the first Omega (all), spare
-  List all_chains, adaptive_chains, adaptive_flags, sp_chains, four_chains;
+  List all_chains, adaptive_chains, adaptive_flags;
   int n_iter;
   bool any_adaptive;
 };
 enum { ENS_FIRST_GRAD = ENS_NFAM, ENS_FIRST_OMEGA = ENS_NFAM + 1 };
 
-bool single_pass_chain(const cl_lattice* l, const cl_cool_params& cp) {
-  return (cp.mode == CL_D0 || cp.mode == CL_D1) && l->prec != 2;
-}
+bool single_pass_chain(const cl_cool_params& cp) { return cp.mode == CL_D0 || cp.mode == CL_D1; }
 
 FusedPlan plan_fused(const cl_batch* b) {
   FusedPlan P;
@@ -924,14 +884,13 @@ FusedPlan plan_fused(const cl_batch* b) {
   };
   auto th = [&](int i) { return theta_nonzero(b->lats[i]); };
   auto ad = [&](int i) { return b->lats[i]->k_ref > 0.0; };
-  auto sp = [&](int i) { return b->with_cooling && single_pass_chain(b->lats[i], b->cps[i]); };
+  auto sp = [&](int i) { return b->with_cooling && single_pass_chain(b->cps[i]); };
   auto cool = [&](int i) { return b->with_cooling != 0; };
-  auto four = [&](int i) { return b->with_cooling && !single_pass_chain(b->lats[i], b->cps[i]); };
+  auto four = [&](int i) { return b->with_cooling && !single_pass_chain(b->cps[i]); };
   auto all = [&](int) { return true; };
   auto tiles = [](int V) { return (V + ENS_BLOCK - 1) / ENS_BLOCK; };
   auto x4 = [&](int V) { return 4 * tiles(V); };
   auto x6 = [&](int V) { return 6 * tiles(V); };
-  auto red = [](int V) { return reduce_blocks(V); };
   add(ENS_INVERSE, [&](int i) { return needs_inverse_pass(b->lats[i]); }, x4);
   add(ENS_PLAQ, all, x6);
   add(ENS_CLOVER, th, x6);
@@ -940,20 +899,14 @@ FusedPlan plan_fused(const cl_batch* b) {
   add(ENS_UPDATE, [&](int i) { return !ad(i); }, x4);
   add(ENS_DRIFTMAX, ad, x4);
   add(ENS_UPDATE_X, ad, x4);
-  add(ENS_FIRST_GRAD, cool, red);
-  add(ENS_FIRST_OMEGA, cool, tiles);
-  add(ENS_COOL_GRAD, four, red);
-  add(ENS_COOL_OMEGA, four, tiles);
-  add(ENS_COOL_APPLY, four, x4);
-  add(ENS_COOL_GRAD_OMEGA, sp, red);
-  add(ENS_COOL_UNLOAD, [&](int i) { return b->with_cooling && b->lats[i]->prec == 0; }, x4);
-  P.fam[ENS_COOL_APPLY_UN].off = P.items.size();
-  for (int i = 0; i < n; ++i)
-    if (sp(i)) {
-      const int nt = cool_tiles(b->lats[i]->g);
-      for (int t = 0; t < nt; ++t) P.items.push_back(WorkItem{i, t});
-    }
-  P.fam[ENS_COOL_APPLY_UN].n = (int)(P.items.size() - P.fam[ENS_COOL_APPLY_UN].off);
+  auto cb = [&](int fam) { return [=](int V) { return ens_cool_blocks(b->lats[0]->prec, fam, V); }; };
+  add(ENS_FIRST_GRAD, cool, cb(ENS_COOL_GRAD));
+  add(ENS_FIRST_OMEGA, cool, cb(ENS_COOL_OMEGA));
+  add(ENS_COOL_GRAD, four, cb(ENS_COOL_GRAD));
+  add(ENS_COOL_OMEGA, four, cb(ENS_COOL_OMEGA));
+  add(ENS_COOL_APPLY, four, cb(ENS_COOL_APPLY));
+  add(ENS_COOL_GRAD_OMEGA, sp, cb(ENS_COOL_GRAD_OMEGA));
+  add(ENS_COOL_APPLY_UN, sp, cb(ENS_COOL_APPLY_UN));
   P.all_chains.off = P.ints.size();
   for (int i = 0; i < n; ++i) P.ints.push_back(i);
   P.all_chains.n = n;
@@ -964,14 +917,6 @@ FusedPlan plan_fused(const cl_batch* b) {
   P.adaptive_flags.off = P.ints.size();
   for (int i = 0; i < n; ++i) P.ints.push_back(ad(i) ? 1 : 0);
   P.adaptive_flags.n = n;
-  P.sp_chains.off = P.ints.size();
-  for (int i = 0; i < n; ++i)
-    if (sp(i)) P.ints.push_back(i);
-  P.sp_chains.n = (int)(P.ints.size() - P.sp_chains.off);
-  P.four_chains.off = P.ints.size();
-  for (int i = 0; i < n; ++i)
-    if (four(i)) P.ints.push_back(i);
-  P.four_chains.n = (int)(P.ints.size() - P.four_chains.off);
   P.any_adaptive = P.adaptive_chains.n > 0;
   P.n_iter = 0;
   if (b->with_cooling)
@@ -1012,7 +957,7 @@ ChainDesc describe(const cl_lattice* l, double eps, const cl_cool_params& cp, bo
   c.sqrt_eps = sqrt(eps);
   c.k_ref = l->k_ref;
   c.seed = l->p.seed;
-  c.ca = cool_args(&cp);
+  c.ca = cool_args(&cp, l->g.V);
   return c;
 }
 
@@ -1046,35 +991,18 @@ cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainD
   CK(launch_ens_step_bump(cd, ints + P.all_chains.off, ints + P.adaptive_flags.off, P.all_chains.n, st));
   ++nl;
   if (b->with_cooling) {
-    const int* all = ints + P.all_chains.off;
-    const int n = P.all_chains.n;
     CK(fam(ENS_COOL_GRAD, ENS_FIRST_GRAD, 1));
-    CK(launch_ens_cool_adapt(cd, all, n, 1, st));
-    ++nl;
-    if (P.n_iter > 0) {
-      CK(fam(ENS_COOL_OMEGA, ENS_FIRST_OMEGA, 0));
-      CK(fam(ENS_COOL_APPLY, ENS_COOL_APPLY, 0));
-      CK(fam(ENS_COOL_APPLY_UN, ENS_COOL_APPLY_UN, 0));
-    }
-    for (int k = 1; k <= P.n_iter; ++k) {
+    for (int k = 0; k < P.n_iter; ++k) {
+      if (k == 0) {
+        CK(fam(ENS_COOL_OMEGA, ENS_FIRST_OMEGA, 0));
+      } else {
+        CK(fam(ENS_COOL_OMEGA, ENS_COOL_OMEGA, 0));
+        CK(fam(ENS_COOL_GRAD_OMEGA, ENS_COOL_GRAD_OMEGA, 0));
+      }
+      CK(fam(ENS_COOL_APPLY, ENS_COOL_APPLY, k));
+      CK(fam(ENS_COOL_APPLY_UN, ENS_COOL_APPLY_UN, k));
       CK(fam(ENS_COOL_GRAD, ENS_COOL_GRAD, 0));
-      // the rule: four-kernel chains from the gradient's records, single-pass
-      // chains from their apply's tile records
-      if (P.four_chains.n) {
-        CK(launch_ens_cool_adapt(cd, ints + P.four_chains.off, P.four_chains.n, 0, st));
-        ++nl;
-      }
-      if (P.sp_chains.n) {
-        CK(launch_ens_cool_adapt_tiles(cd, ints + P.sp_chains.off, P.sp_chains.n, st));
-        ++nl;
-      }
-      if (k == P.n_iter) break;
-      CK(fam(ENS_COOL_OMEGA, ENS_COOL_OMEGA, 0));
-      CK(fam(ENS_COOL_GRAD_OMEGA, ENS_COOL_GRAD_OMEGA, 0));
-      CK(fam(ENS_COOL_APPLY, ENS_COOL_APPLY, 0));
-      CK(fam(ENS_COOL_APPLY_UN, ENS_COOL_APPLY_UN, 0));
     }
-    if (P.n_iter > 0) CK(fam(ENS_COOL_UNLOAD, ENS_COOL_UNLOAD, 0));
   }
   *launches = nl;
   return CL_OK;

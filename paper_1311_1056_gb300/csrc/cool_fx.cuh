@@ -2,13 +2,12 @@
 // (fixed.cuh): gradient, Omega and apply, the formulas of kernels.cu.
 //
 // A cooling call keeps the links as fixed-point words Ux in the lattice's
-// second link buffer: its first gradient reads the FP64 links and writes them,
-// every sweep reads and writes Ux, and one pass at the end (fx_unload) writes
-// the FP64 links back if any sweep ran.  (Converting 64-bit words both ways in
-// every sweep would cost two fifths of it.)  Omega and Omega^{-1} are packed
-// Hermitian fields of 9 words per site.  A link, Omega or f that leaves the
-// fixed-point range is stored as doubles (fixed.cuh) and the threads that meet
-// it work in FP64.
+// second link buffer: its first gradient reads the links and writes them, every
+// sweep reads and writes Ux, and the last apply writes the links back.
+// (Converting 64-bit words both ways in every sweep would cost two fifths of
+// it.)  Omega and Omega^{-1} are packed Hermitian fields of 9 words per site.  A
+// link, Omega or f that leaves the fixed-point range is stored as doubles
+// (fixed.cuh) and the threads that meet it work in FP64.
 #pragma once
 #include "expm_fx.cuh"
 #include "fixed.cuh"
@@ -79,15 +78,12 @@ __device__ __forceinline__ void load_herm_mat(mat<double>& m, tagged_herm f, int
 }
 
 // -------------------------------------------------------------- gradient
-// G_x = sum_mu (U U^+ - U^+_{x-mu} U_{x-mu}) as 60-bit integers (d, o01, o02,
-// o12), and the three diagonal sums of its first part (Tr U U^+ of the links
-// at x).  The sums must stay below 8 (they are about 4 near SU(3)): their
-// squares are followed in float too, and ok is false beyond 7.5.
+// G_x = sum_mu (U U^+ - U^+_{x-mu} U_{x-mu}) as 60-bit integers: diagonal, and
+// re / im of 01, 02, 12.
 struct fx_gradient {
-  long long d[3], o[6], un[3];
-  bool ok;
+  long long d[3], o[6];
 };
-// rows (or conjugated columns) r0, r1, r2 of one link: += sign r_i conj(r_j)
+// rows (or conjugated columns) r0, r1, r2 of one link: += sign r_i conj(r_j); n: their squares in float
 __device__ __forceinline__ void fx_outer(fx_acc* D, fx_acc* O, float* n, cx<fx> r0, cx<fx> r1, cx<fx> r2, bool neg) {
   const cx<fx> r[3] = {r0, r1, r2};
   fx_cright R[3];
@@ -112,56 +108,21 @@ __device__ __forceinline__ void fx_outer(fx_acc* D, fx_acc* O, float* n, cx<fx> 
     fx_mac(O[2 * q + 1], nre, R[j].im);
   }
 }
-// load(u, mu, site): link (mu, site) as fixed point
-template <class Load>
-__device__ __forceinline__ void fx_grad_site(fx_gradient& G, const Geo& g, int s, const int x[4], Load load) {
-  fx_acc D[3], O[6];
-  float nf[3], nb[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    D[i] = fx_zero();
-    nf[i] = nb[i] = 0.0f;
-  }
-#pragma unroll
-  for (int i = 0; i < 6; ++i) O[i] = fx_zero();
-#pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
-    mat<fx> u;
-    load(u, mu, s);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) fx_outer(D, O, nf, u.e[k], u.e[3 + k], u.e[6 + k], false);
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) G.un[i] = fx_sum<true>(D[i]) - (1 << 29);
-#pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
-    mat<fx> u;
-    load(u, mu, hop(g, s, x, mu, -1));
-    // - (U^+ U)_ij = - conj(U_ki) U_kj: x conj(y) with x = conj(U_ki), y = conj(U_kj)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const cx<fx> a = u.e[3 * k], b = u.e[3 * k + 1], c = u.e[3 * k + 2];
-      fx_outer(D, O, nb, cx<fx>{a.re, -a.im}, cx<fx>{b.re, -b.im}, cx<fx>{c.re, -c.im}, true);
-    }
-  }
-  G.ok = true;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    G.d[i] = fx_sum<true>(D[i]) - (1 << 29);
-    G.ok = G.ok && nf[i] < 7.5f * 0x1p60f && nb[i] < 7.5f * 0x1p60f;
-  }
-#pragma unroll
-  for (int i = 0; i < 6; ++i) G.o[i] = fx_sum<true>(O[i]) - (1 << 29);
-}
-
 // ----------------------------------------------------------- exponential
-// exp(H) and exp(-H) of a traceless Hermitian H, as expm_hermitian_pair:
-// H^2, the two invariants, Horner's rule on the three Cayley-Hamilton
-// coefficients of both, all in fixed point.  False (nothing useful in om, omi)
-// when a number leaves the range: |H| above ~1/3.
-__device__ __forceinline__ bool fx_expm_hermitian_pair(fx_herm& om, fx_herm& omi, const fx_herm& H, float tol) {
+// exp(H), or exp(-H), of a traceless Hermitian H, as expm_hermitian_pair: H^2,
+// the two invariants, Horner's rule on the Cayley-Hamilton coefficients, in
+// fixed point.  (One sign: two threads share a site's pair.)  False when a
+// number leaves the range: |H|_F above 0.34.  Both signs agree on that: they see
+// the same numbers up to the test of |H|, and below it no coefficient and no
+// entry of the result can exceed exp(0.34) < 1.4375.
+struct fx_exp_series {  // what both signs share
+  fx_herm Q;            // H^2
+  fx c0, c1;            // det H, Tr H^2 / 2
+  int N;                // terms
+};
+__device__ __forceinline__ bool fx_exp_setup(fx_exp_series& S, const fx_herm& H, float tol) {
   fx_chk ck;
-  fx_herm Q;  // H^2
+  fx_herm& Q = S.Q;
   {
     fx_cleft L[3];
     fx_cright R[3];
@@ -227,50 +188,45 @@ __device__ __forceinline__ bool fx_expm_hermitian_pair(fx_herm& om, fx_herm& omi
   const fx c0 = fx_get<FX_WIDE>(z, ck);
   const float r = sqrtf(2.0f * fmaxf(fmaf(c1.l, 0x1p-60f, (float)c1.h * 0x1p-30f), 0.0f));
   if (ck.bad() || !(r < 0.34f)) return false;
-  const int N = taylor_terms(r, tol);
-  const fx_right b1 = fx_rhs(c1), b0 = fx_rhs(c0), nb0 = fx_rhs(-c0);
-  // exp(H) = a + b H + c H^2, exp(-H) = ap - bp H + cp H^2
+  S.c0 = c0;
+  S.c1 = c1;
+  S.N = taylor_terms(r, tol);
+  return true;
+}
+// exp(H), inverse: exp(-H).  det(-H) = -det H: exp(-H) = a - b H + c H^2 with c0 negated.
+__device__ __forceinline__ void fx_exp_sum(fx_herm& om, const fx_exp_series& S, const fx_herm& H, bool inverse) {
+  fx_chk ck;  // nothing to check: see above
+  const fx_herm& Q = S.Q;
+  const int N = S.N;
+  const fx_right b1 = fx_rhs(S.c1), b0 = fx_rhs(inverse ? -S.c0 : S.c0);
   const fx_const f = c_fx_invfact[N];
-  fx a = {(float)f.l, f.h}, b = {0.0f, 0}, c = {0.0f, 0}, ap = a, bp = b, cp = c;
+  fx a = {(float)f.l, f.h}, b = {0.0f, 0}, c = {0.0f, 0};
 #pragma unroll 1
   for (int k = N - 1; k >= 0; --k) {
-    fx_acc s = fx_from_invfact(k), u = fx_from(a), sp = s, up = fx_from(ap);
-    const fx_left x = fx_lhs(c), xp = fx_lhs(cp);
+    fx_acc s = fx_from_invfact(k), u = fx_from(a);
+    const fx_left x = fx_lhs(c);
     fx_mac(s, x, b0);
     fx_mac(u, x, b1);
-    fx_mac(sp, xp, nb0);
-    fx_mac(up, xp, b1);
     c = b;
     b = fx_get<FX_WIDE>(u, ck);
     a = fx_get<FX_WIDE>(s, ck);
-    cp = bp;
-    bp = fx_get<FX_WIDE>(up, ck);
-    ap = fx_get<FX_WIDE>(sp, ck);
   }
-  const fx_left lb = fx_lhs(b), lc = fx_lhs(c), lbp = fx_lhs(-bp), lcp = fx_lhs(cp);
+  const fx_left lb = fx_lhs(inverse ? -b : b), lc = fx_lhs(c);
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const int q = (k - 3) >> 1;
     const fx hk = k < 3 ? H.d[k] : (k & 1) ? H.o[q].re : H.o[q].im, qk = k < 3 ? Q.d[k] : (k & 1) ? Q.o[q].re : Q.o[q].im;
-    const fx_right hr = fx_rhs(hk), qr = fx_rhs(qk);
-    fx_acc s = k < 3 ? fx_from(a) : fx_zero(), sp = k < 3 ? fx_from(ap) : fx_zero();
-    fx_mac(s, lb, hr);
-    fx_mac(s, lc, qr);
-    fx_mac(sp, lbp, hr);
-    fx_mac(sp, lcp, qr);
-    const fx w = fx_get<FX_WIDE>(s, ck), wp = fx_get<FX_WIDE>(sp, ck);
-    if (k < 3) {
+    fx_acc s = k < 3 ? fx_from(a) : fx_zero();
+    fx_mac(s, lb, fx_rhs(hk));
+    fx_mac(s, lc, fx_rhs(qk));
+    const fx w = fx_get<FX_WIDE>(s, ck);
+    if (k < 3)
       om.d[k] = w;
-      omi.d[k] = wp;
-    } else if (k & 1) {
+    else if (k & 1)
       om.o[q].re = w;
-      omi.o[q].re = wp;
-    } else {
+    else
       om.o[q].im = w;
-      omi.o[q].im = wp;
-    }
   }
-  return !ck.bad();
 }
 
 // H = 4 c (G - Tr G / 3), c = -eps alpha_ad (f_a lambda_a = 4 (G - Tr G / 3)).

@@ -25,7 +25,7 @@ inline int block_of(const GeoH& h, int fam) { return h.blk[fam] > 0 ? h.blk[fam]
 // replay with fresh noise and the adaptive step size is decided on the GPU.
 struct StepDev {
   uint32_t step;                 // Philox step counter (the noise key's step word)
-  uint32_t pad;
+  uint32_t pad;                  // counter of finished blocks (last-block reductions), zero between launches
   double eps_n, sqrt_eps_n;      // step size of the current step (adaptive mode)
   double t;                      // Langevin time: sum of the step sizes taken
   double kmax;                   // K_max of the last adaptive step
@@ -42,6 +42,7 @@ struct CoolState {
 };
 
 struct CoolArgs {
+  double inv_links;  // 1 / (4 V)
   double eps, alpha, tol_rel, d_floor, d_guard;
   int mode, n_min, n_max, forced_sweeps;
 };
@@ -62,7 +63,7 @@ struct ChainDesc {
   int L[4], stride[4], V;
   void *U, *Un, *Ui, *Pq, *Dq, *F, *C, *Gq, *f, *Om, *Omi;
   double* partials;
-  double* arec;             // the single-pass apply's tile records
+  double* arec;             // the cooling kernels' block records
   CoolState* cs;
   StepDev* sd;
   double beta, sre, sim;    // coupling; clover scale -i theta kappa = sre + i sim (FP64: times 2^-cexp)
@@ -87,13 +88,12 @@ enum {
   ENS_UPDATE = 5,       // gather + update, fixed step size
   ENS_DRIFTMAX = 6,     // gather, drift into Ui, max |K|^2 (adaptive step size)
   ENS_UPDATE_X = 7,     // update from the drift in Ui (adaptive step size)
-  ENS_COOL_GRAD = 8,    // gradient + rule sums (RED_THREADS blocks, grid-stride per chain)
+  ENS_COOL_GRAD = 8,    // gradient + rule
   ENS_COOL_OMEGA = 9,   // Omega, Omega^{-1}
-  ENS_COOL_APPLY = 10,  // apply, 4 directions
+  ENS_COOL_APPLY = 10,  // apply
   ENS_COOL_GRAD_OMEGA = 11, // single-pass sweeps (D_0 / D_1): gradient + Omega
-  ENS_COOL_APPLY_UN = 12,   // single-pass sweeps: apply per tile + norm sums (one item per tile)
-  ENS_COOL_UNLOAD = 13,     // FP64: fixed-point links back to doubles, 4 directions
-  ENS_NFAM = 14
+  ENS_COOL_APPLY_UN = 12,   // single-pass sweeps: apply + rule
+  ENS_NFAM = 13
 };
 const int ENS_BLOCK = 128;
 
@@ -151,36 +151,34 @@ cudaError_t launch_update_gather(int prec, int mode, const GeoH& g, const void* 
 cudaError_t launch_step_bump(StepDev* sd, double eps, bool adaptive, cudaStream_t st);
 // Adaptive step size from the drift pass: eps_n = eps min(1, k_ref / K_max).
 cudaError_t launch_step_eps(StepDev* sd, double eps, double k_ref, cudaStream_t st);
-// Cooling: gradient f (8 FP64 values per site, [a][V]) + partial sums; the
-// rule; Omega; apply.
-// FP64 form: the sweeps run on the links' fixed-point words Ux (the second link
-// buffer), which the call's first gradient (cs NULL) writes from U; the Omega,
-// apply and later gradient launches take Ux as U, and launch_cool_unload at the
-// end writes U back if a sweep ran (cs NULL: always).  launch_cool_load writes
-// Ux without a gradient.
-cudaError_t launch_cool_grad(int prec, const GeoH& g, const void* U, void* Ux, void* f, double* partials,
-                             const CoolState* cs, cudaStream_t st);
-cudaError_t launch_cool_load(const GeoH& g, const void* U, void* Ux, cudaStream_t st);
-cudaError_t launch_cool_unload(const GeoH& g, void* U, const void* Ux, const CoolState* cs, cudaStream_t st);
-cudaError_t launch_cool_adapt(const GeoH& g, const double* partials, CoolArgs a, CoolState* cs,
-                              int first, cudaStream_t st);
-cudaError_t launch_cool_omega(int prec, const GeoH& g, const void* f, void* Om, void* Omi,
-                              double eps, const CoolState* cs, cudaStream_t st);
-cudaError_t launch_cool_apply(int prec, const GeoH& g, void* U, const void* Om, const void* Omi,
-                              const CoolState* cs, cudaStream_t st);
-// Single-pass sweep of the D_0 / D_1 rules (FP64 and FP32 storage only):
-// Omega and Omega^{-1} straight from the gradient with the strength the rule
-// already set; the apply over tiles of COOL_TILE sites inside one x3 layer,
-// one record per tile of the rule's inputs for the next sweep ((1/3) Tr U U^+
-// and nonfinite count, 2 doubles; cool_tiles(g) records); the rule from
-// those records.
-enum { COOL_TILE = 128 };
-int cool_tiles(const GeoH& g);
-cudaError_t launch_cool_grad_omega(int prec, const GeoH& g, const void* U, void* Om, void* Omi, double eps,
-                                   const CoolState* cs, cudaStream_t st);
-cudaError_t launch_cool_apply_tiles(int prec, const GeoH& g, void* U, const void* Om, const void* Omi,
-                                    double* rec, const CoolState* cs, cudaStream_t st);
-cudaError_t launch_cool_adapt_tiles(const GeoH& g, const double* rec, CoolArgs a, CoolState* cs, cudaStream_t st);
+// Cooling (cool_sweep.cuh).  What a call works on: the links U; the second link
+// buffer Ux, which holds their fixed-point words during a call of the FP64 and
+// DF64 forms (FP32 storage: Ux = U); f (8 FP64 values per site, [a][V]); the
+// packed Omega, Omega^{-1}; records of 32 bytes, one per 32 sites, and 160 bytes;
+// the rule's parameters and state.
+struct CoolBufs {
+  void *U, *Ux, *f, *Om, *Omi;
+  double* rec;
+  StepDev* sd;
+  CoolState* cs;
+  CoolArgs ca;
+};
+int ens_cool_blocks(int prec, int fam, int V);  // a chain's blocks in a fused launch of family ENS_COOL_*
+// Gradient f and (rule) the adaptive rule in its last block; first: a call's
+// first one, which reads U and writes Ux.
+cudaError_t launch_cool_grad(int prec, const GeoH& g, const CoolBufs& b, bool first, bool rule, cudaStream_t st);
+// Omega and its inverse from f.
+cudaError_t launch_cool_omega(int prec, const GeoH& g, const CoolBufs& b, cudaStream_t st);
+// Single-pass sweeps of the D_0 / D_1 rules: Omega and its inverse straight
+// from the gradient with the strength the rule already set.
+cudaError_t launch_cool_grad_omega(int prec, const GeoH& g, const CoolBufs& b, cudaStream_t st);
+// Apply; rule: single-pass sweeps, the rule for the next sweep from the new
+// links' norm.  last: the call's last enqueued sweep, after which U holds the
+// links again (also when the rule has stopped the call before).  b.cs NULL:
+// no rule state, always applied.
+cudaError_t launch_cool_apply(int prec, const GeoH& g, const CoolBufs& b, bool rule, bool last, cudaStream_t st);
+// Ux from U (FP64, DF64), for an apply without a gradient before it.
+cudaError_t launch_cool_load(int prec, const GeoH& g, const void* U, void* Ux, cudaStream_t st);
 // Observables: per-site pass over the links, the plaquette pass's fields and
 // the clover field F (scale obs_clover_scale), then the final fixed-order
 // reduction into *out.
@@ -192,14 +190,11 @@ cudaError_t launch_obs_final(const GeoH& g, const double* partials, double beta,
 // arrays cd, w); FP64 and FP32 storage only.  Per-chain kernels (one thread
 // or one block per chain): the adaptive step size, the step counter, and the
 // cooling rule (first = the call's first sweep).
-// arg: ENS_COOL_GRAD's `first` flag (the call's first gradient runs whatever the rule state).
+// arg: ENS_COOL_GRAD's `first` flag (the call's first gradient runs whatever the rule state); the applies' sweep number.
 cudaError_t launch_ens(int prec, int fam, const ChainDesc* cd, const WorkItem* w, int nw, int arg, cudaStream_t st);
 cudaError_t launch_ens_step_eps(const ChainDesc* cd, const int* chains, int n, cudaStream_t st);
 cudaError_t launch_ens_step_bump(const ChainDesc* cd, const int* chains, const int* adaptive, int n,
                                  cudaStream_t st);
-cudaError_t launch_ens_cool_adapt(const ChainDesc* cd, const int* chains, int n, int first, cudaStream_t st);
-// the rule of single-pass chains from their tile records (ChainDesc::arec)
-cudaError_t launch_ens_cool_adapt_tiles(const ChainDesc* cd, const int* chains, int n, cudaStream_t st);
 // Integer-pipe float <-> double conversions (cvt.cuh) against the hardware
 // ones on n generated cases; mismatch counts added into bad[0] (float ->
 // double) and bad[1] (double -> float).
