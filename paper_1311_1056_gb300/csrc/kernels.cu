@@ -189,8 +189,12 @@ __global__ void k_noise_sample(int site0, int n, uint64_t seed, uint32_t step, u
 // page-locked memory, read or written over the host link) is one contiguous
 // run per block, and the SoA side is CONV_SITES consecutive sites per row.
 // The tile's pitch is odd in 16-byte units, so the column-wise accesses of a
-// quarter warp hit distinct banks.
+// quarter warp hit distinct banks.  16-byte accesses with a tile's loads in
+// flight at once where the buffer is aligned: both directions then run at the
+// host link's rate (24^3 x 32 links from / to page-locked memory 1.22 / 1.33 ms,
+// the copy engine's 1.23 / 1.34; out in 8-byte writes 1.82 ms).
 const int CONV_SITES = 32, CONV_MAX_ROWS = 54;  // up to 6 planes
+const int CONV_BATCH = 5;  // AoS loads in flight per thread (36 rows: the whole tile)
 __host__ __device__ constexpr int conv_pitch(int rows) { return rows + 1 + (rows & 1); }
 
 template <typename T>
@@ -199,11 +203,23 @@ __global__ void __launch_bounds__(256) k_aos_to_soa(Geo g, const double* __restr
   __shared__ double2 buf[CONV_SITES * conv_pitch(CONV_MAX_ROWS)];
   const int R = 9 * nplanes, pitch = conv_pitch(R);
   const int s0 = blockIdx.x * CONV_SITES;
-  const int ns = min(CONV_SITES, g.V - s0);
+  const int ns = min(CONV_SITES, g.V - s0), n = ns * R;
   const double* src = aos + 2 * (size_t)s0 * R;
-  for (int e = threadIdx.x; e < ns * R; e += blockDim.x) {
-    const int j = e / R, r = e - j * R;
-    buf[j * pitch + r] = make_double2(src[2 * e], src[2 * e + 1]);
+  // a caller's buffer need only be aligned to 8 bytes
+  const bool wide = (reinterpret_cast<size_t>(src) & 15) == 0;
+  for (int e0 = threadIdx.x; e0 < n; e0 += CONV_BATCH * 256) {
+    double2 v[CONV_BATCH];
+#pragma unroll
+    for (int q = 0; q < CONV_BATCH; ++q) {
+      const int e = e0 + q * 256;
+      if (e < n) v[q] = wide ? __ldcs(reinterpret_cast<const double2*>(src) + e) : make_double2(src[2 * e], src[2 * e + 1]);
+    }
+#pragma unroll
+    for (int q = 0; q < CONV_BATCH; ++q) {
+      const int e = e0 + q * 256;
+      const int j = e / R, r = e - j * R;
+      if (e < n) buf[j * pitch + r] = v[q];
+    }
   }
   __syncthreads();
   for (int e = threadIdx.x; e < R * CONV_SITES; e += blockDim.x) {
@@ -230,11 +246,16 @@ __global__ void __launch_bounds__(256) k_soa_to_aos(Geo g, const typename vec2_o
   }
   __syncthreads();
   double* dst = aos + 2 * (size_t)s0 * R;
+  const bool wide = (reinterpret_cast<size_t>(dst) & 15) == 0;
   for (int e = threadIdx.x; e < ns * R; e += blockDim.x) {
     const int j = e / R, r = e - j * R;
     const double2 v = buf[j * pitch + r];
-    dst[2 * e] = v.x;
-    dst[2 * e + 1] = v.y;
+    if (wide) {
+      __stcs(reinterpret_cast<double2*>(dst) + e, v);
+    } else {
+      dst[2 * e] = v.x;
+      dst[2 * e + 1] = v.y;
+    }
   }
 }
 
