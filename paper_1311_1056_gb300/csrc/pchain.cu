@@ -5,9 +5,10 @@
 // One CTA per chain and one thread per link; the chain lives in shared memory
 // for a whole chunk of steps, so one launch runs [CL step, cooling sweeps,
 // observables] many times with no HBM traffic but the records.  The drift of
-// link k needs the cyclic product P_k = U_k ... U_N U_1 ... U_{k-1}; it is
-// P_k = Suf_k Pre_{k-1} from an inclusive prefix and suffix product scan
-// (Hillis-Steele, log2 N rounds).  With sum_a sigma_a Tr(sigma_a M) =
+// link k needs the cyclic product P_k = U_k ... U_N U_1 ... U_{k-1}: products
+// of 1, 2, 4, ... links from k on by doubling, and P_k from those of N's binary
+// digits (floor(log2 N) + ones(N) - 1 products of a thread: 7 at N = 30, where
+// a prefix and a suffix scan take 11).  With sum_a sigma_a Tr(sigma_a M) =
 // 2 (M - Tr M / 2) the exponent of the update is
 //   A = -eps beta (P_k - Tr P_k / 2) + i sqrt(eps) sqrt(2) g_a sigma_a,
 // and exp of a traceless 2x2 matrix is cosh(s) + sinh(s)/s A with s^2 = -det A.
@@ -15,6 +16,13 @@
 // Omega_k = exp(-eps alpha_ad f_ak sigma_a) (Hermitian: cosh r + sinh r / r H),
 // U_k <- Omega_k U_k Omega_{k+1}^{-1}; the adaptive rule (alpha_ad = alpha / D,
 // sweep-count stop rule) runs on the block's fixed-order reductions.
+//
+// Arithmetic.  Chains of up to 512 links hold their links in fixed point
+// (pchain_fx.cuh) while every number of a step fits; a block-wide vote sends
+// the part of a step that does not (a runaway chain, a large step) through the
+// FP64 code, and the chain comes back at the next step that fits.  At the end of
+// a step the links are rounded to doubles, so that runs split over calls equal
+// one run.  Longer chains (64 registers a thread) stay in FP64.
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -22,6 +30,7 @@
 
 #include "../../include/cl.h"
 #include "launch.h"
+#include "pchain_fx.cuh"
 #include "philox.cuh"
 #include "runtime.h"
 #include "su3.cuh"
@@ -187,109 +196,282 @@ __device__ __forceinline__ void block_reduce4(double v[4], double* red) {
   for (int q = 0; q < 4; ++q) v[q] = t[q];
 }
 
-// As[k] = U_0 ... U_k, Bs[k] = U_k ... U_{n-1}.
-__device__ __forceinline__ void scan_products(const SM2& Us, const SM2& As, const SM2& Bs, int n) {
-  const int k = threadIdx.x;
-  const bool act = k < n;
-  if (act) {
-    const M2 u = Us.get(k);
-    As.set(k, u);
-    Bs.set(k, u);
-  }
+// The sum of v over the block, in every thread.
+__device__ __forceinline__ long long block_sum(long long v, long long* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (blockDim.x == 32) return v;
+  __syncthreads();  // red may still be read from the previous call
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int off = 1; off < n; off <<= 1) {
-    const bool da = act && k >= off, db = act && k + off < n;
-    M2 pa, pb;
-    if (da) pa = As.get(k - off);
-    if (db) pb = Bs.get(k + off);
+  v = 0;
+  for (int i = 0; i < blockDim.x >> 5; ++i) v += red[i];
+  return v;
+}
+
+// U_k U_{k+1} ... (n links, cyclic) for link k, whose matrix is u.  a and b are
+// scratch; the caller synchronises before their next use.
+template <class Arr, class M, class Mul>
+__device__ __forceinline__ M cyclic_product(const M& u, Arr a, Arr b, int k, bool act, int n, Mul mul) {
+  M w = u, p = u;
+  int off = 0;
+  if (act) a.set(k, w);
+  __syncthreads();
+  for (int m = n, len = 1;; len *= 2) {
+    if (m & 1) {
+      const int j = k + off < n ? k + off : k + off - n;
+      p = off > 0 ? mul(p, a.get(j)) : w;
+      off += len;
+    }
+    m >>= 1;
+    if (m == 0) break;
+    w = mul(w, a.get(k + len < n ? k + len : k + len - n));
+    if (act) b.set(k, w);
     __syncthreads();
-    if (da) As.set(k, m2mul(pa, As.get(k)));
-    if (db) Bs.set(k, m2mul(Bs.get(k), pb));
+    const Arr t = a;
+    a = b;
+    b = t;
+  }
+  return p;
+}
+
+// One chain's block.  Threads beyond the last link work on its copy and write
+// nothing, so that a warp stays whole.
+struct Chain {
+  int n, k;  // links, this thread's
+  bool act;
+  double* smem;
+  __device__ __forceinline__ SM2 Us() const { return SM2{smem, n}; }
+  __device__ __forceinline__ SM2 As() const { return SM2{smem + 8 * n, n}; }
+  __device__ __forceinline__ SM2 Bs() const { return SM2{smem + 16 * n, n}; }
+  __device__ __forceinline__ SF2 Uf() const { return SF2{(int2*)smem, n}; }
+  __device__ __forceinline__ SF2 Af() const { return SF2{(int2*)(smem + 8 * n), n}; }
+  __device__ __forceinline__ SF2 Bf() const { return SF2{(int2*)(smem + 16 * n), n}; }
+  __device__ __forceinline__ double* red() const { return smem + 24 * n; }
+
+  // This thread's link between doubles and fixed point, in place (the caller synchronises).
+  __device__ __forceinline__ bool fits(F2& f) const {
+    const M2 u = Us().get(k);
+    unsigned mag = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f.e[q] = cx<fx>{fx_of_double(u.e[q].re, mag), fx_of_double(u.e[q].im, mag)};
+    return fx_mag_ok(mag);
+  }
+  __device__ __forceinline__ M2 as_double() const {
+    const F2 f = Uf().get(k);
+    M2 u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u.e[q] = C{fx_to_double(f.e[q].re), fx_to_double(f.e[q].im)};
+    return u;
+  }
+  __device__ __forceinline__ void to_double() const {
+    const M2 u = as_double();
+    __syncthreads();  // (threads beyond the last link read its copy)
+    if (act) Us().set(k, u);
     __syncthreads();
   }
+
+  __device__ __forceinline__ M2 product_f64() const {
+    return cyclic_product(Us().get(k), As(), Bs(), k, act, n, [](const M2& x, const M2& y) { return m2mul(x, y); });
+  }
+  // The cyclic product times 2^-S, S = 0, 1 or 2: links away from unitarity
+  // leave the range by a little (1.8 at 30 links, 2.3 at 60 of the same start).
+  __device__ __forceinline__ bool product_fx(F2& P, int& S) const {
+    const F2 u = Uf().get(k);
+    fx_chk ck;
+    P = cyclic_product(u, Af(), Bf(), k, act, n, [&](const F2& x, const F2& y) { return f2_mul<false>(x, y, 0, ck); });
+    S = 0;
+    if (!__syncthreads_or(ck.bad())) return true;
+#pragma unroll 1
+    for (S = 1; S <= 2; ++S) {
+      F2 v;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        v.e[q] = cx<fx>{fx_of_bits(fx_bits(u.e[q].re) >> S), fx_of_bits(fx_bits(u.e[q].im) >> S)};
+      fx_chk cs;
+      P = cyclic_product(v, Af(), Bf(), k, act, n, [&](const F2& x, const F2& y) { return f2_mul<true>(x, y, S, cs); });
+      if (!__syncthreads_or(cs.bad())) return true;
+    }
+    return false;
+  }
+
+  __device__ __forceinline__ bool step_fx(const PcStepFx& c, uint64_t seed, uint32_t step) const {
+    F2 P;
+    int S;
+    if (!product_fx(P, S)) return false;
+    fx g[4];
+    normals_fx<2>(g, seed, step, (uint32_t)k, 0u, STREAM_PC_CL);
+    fx_chk ck;
+    const F2 W = pc_update_fx(P, S, Uf().get(k), g, c, ck);
+    if (__syncthreads_or(ck.bad())) return false;
+    if (act) Uf().set(k, W);
+    __syncthreads();
+    return true;
+  }
+  __device__ __forceinline__ void step_f64(C mb, double sq, uint64_t seed, uint32_t step) const {
+    const M2 P = product_f64();
+    double g[4];
+    normals_f64<2>(g, seed, step, (uint32_t)k, 0u, STREAM_PC_CL);
+    const C htr = cscale(cadd(P.e[0], P.e[3]), 0.5);
+    M2 A;
+    A.e[0] = cmul(mb, csub(P.e[0], htr));
+    A.e[3] = cmul(mb, csub(P.e[3], htr));
+    A.e[1] = cmul(mb, P.e[1]);
+    A.e[2] = cmul(mb, P.e[2]);
+    // + i sq [[g3, g1 - i g2], [g1 + i g2, -g3]]
+    A.e[0].im += sq * g[2];
+    A.e[3].im -= sq * g[2];
+    A.e[1].re += sq * g[1];
+    A.e[1].im += sq * g[0];
+    A.e[2].re -= sq * g[1];
+    A.e[2].im += sq * g[0];
+    M2 W = m2mul(exp_traceless(A), Us().get(k));
+    const C z = cinv(csqrt_p(m2det(W)));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) W.e[q] = cmul(W.e[q], z);
+    __syncthreads();
+    if (act) Us().set(k, W);
+    __syncthreads();
+  }
+
+  // f_a and Tr U U^+ / 2 of this thread's link
+  __device__ __forceinline__ double grad_f64(double f[3]) const {
+    const M2 u = Us().get(k);
+    const M2 w = Us().get(k == 0 ? n - 1 : k - 1);
+    // G = u u^+ - w^+ w (Hermitian)
+    C G00 = C{0.0, 0.0}, G01 = C{0.0, 0.0}, G10 = C{0.0, 0.0}, G11 = C{0.0, 0.0};
+    G00 = cfma(u.e[0], cconj(u.e[0]), cfma(u.e[1], cconj(u.e[1]), G00));
+    G01 = cfma(u.e[0], cconj(u.e[2]), cfma(u.e[1], cconj(u.e[3]), G01));
+    G10 = cfma(u.e[2], cconj(u.e[0]), cfma(u.e[3], cconj(u.e[1]), G10));
+    G11 = cfma(u.e[2], cconj(u.e[2]), cfma(u.e[3], cconj(u.e[3]), G11));
+    G00 = cfms(cconj(w.e[0]), w.e[0], cfms(cconj(w.e[2]), w.e[2], G00));
+    G01 = cfms(cconj(w.e[0]), w.e[1], cfms(cconj(w.e[2]), w.e[3], G01));
+    G10 = cfms(cconj(w.e[1]), w.e[0], cfms(cconj(w.e[3]), w.e[2], G10));
+    G11 = cfms(cconj(w.e[1]), w.e[1], cfms(cconj(w.e[3]), w.e[3], G11));
+    f[0] = 2.0 * (G01.re + G10.re);
+    f[1] = 2.0 * (G10.im - G01.im);
+    f[2] = 2.0 * (G00.re - G11.re);
+    return 0.5 * (u.e[0].re * u.e[0].re + u.e[0].im * u.e[0].im + u.e[1].re * u.e[1].re + u.e[1].im * u.e[1].im +
+                  u.e[2].re * u.e[2].re + u.e[2].im * u.e[2].im + u.e[3].re * u.e[3].re + u.e[3].im * u.e[3].im);
+  }
+  // The norms' sums, from the gradients: v = {sum Tr / 2, sum |f|, sum f^2}
+  __device__ __forceinline__ void norms_f64(double v[4], double tr, const double f[3]) const {
+    v[0] = act ? tr : 0.0;
+    v[1] = act ? fabs(f[0]) + fabs(f[1]) + fabs(f[2]) : 0.0;
+    v[2] = act ? f[0] * f[0] + f[1] * f[1] + f[2] * f[2] : 0.0;
+    v[3] = 0.0;
+    block_reduce4(v, red());
+  }
+  __device__ __forceinline__ void apply_f64(const double f[3], double ea) const {
+    const double h[3] = {ea * f[0], ea * f[1], ea * f[2]};
+    M2 om, omi;
+    exp_herm_pair(h, om, omi);
+    if (act) {
+      As().set(k, om);
+      Bs().set(k, omi);
+    }
+    __syncthreads();
+    const M2 r = m2mul(m2mul(As().get(k), Us().get(k)), Bs().get(k + 1 == n ? 0 : k + 1));
+    __syncthreads();
+    if (act) Us().set(k, r);
+    __syncthreads();
+  }
+  __device__ __forceinline__ bool apply_fx(const fx g[3], double ea) const {
+    unsigned mag = 0;
+    const fx s = fx_of_double(4.0 * ea, mag);
+    fx om[4], on[4];
+    fx_chk ck;
+    pc_omega_fx(om, g, s, ck);
+    if (act) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) Af().word(q, k, om[q]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) on[q] = Af().word(q, k + 1 == n ? 0 : k + 1);
+    const F2 r = pc_apply_fx(om, Uf().get(k), on, ck);
+    if (__syncthreads_or(ck.bad() || !fx_mag_ok(mag))) return false;
+    if (act) Uf().set(k, r);
+    __syncthreads();
+    return true;
+  }
+};
+
+// 1 / x to FP64 precision: the float reciprocal and two Newton steps.
+__device__ __forceinline__ double pc_recip(double x) {
+  if (!(x > 0x1p-60 && x < 0x1p60)) return 1.0 / x;
+  double r = (double)(1.0f / (float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
 }
 
 // MAXT = 512 for chains of up to 512 links (128 registers a thread, no
 // spills); 1024 for longer ones (64 registers: some spilling to L1).
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_pchain(PcArgs a) {
+  constexpr bool FX = MAXT <= 512;
   extern __shared__ double smem[];
-  const int n = a.n, c = blockIdx.x, k = threadIdx.x;
-  const bool act = k < n;
-  const SM2 Us{smem, n}, As{smem + 8 * n, n}, Bs{smem + 16 * n, n};
-  double* red = smem + 24 * n;
+  const int n = a.n, c = blockIdx.x;
+  const Chain ch = {n, min((int)threadIdx.x, n - 1), threadIdx.x < n, smem};
+  const int k = ch.k;
   double2* Ug = a.U + (size_t)c * n * 4;
-  if (act) {
+  if (ch.act) {
     M2 u;
     for (int q = 0; q < 4; ++q) {
       const double2 v = Ug[4 * k + q];
       u.e[q] = C{v.x, v.y};
     }
-    Us.set(k, u);
+    ch.Us().set(k, u);
   }
   __syncthreads();
-  const C beta = C{a.beta[2 * c], a.beta[2 * c + 1]};
+  const C mb = C{-a.eps * a.beta[2 * c], -a.eps * a.beta[2 * c + 1]};  // -eps beta
   const uint64_t seed = a.seed[c];
   const double sq = sqrt(a.eps) * 1.41421356237309504880;  // sqrt(eps) * sqrt(2)
+  const double inv_n = 1.0 / n;
+  PcStepFx cf;
+  if (FX) cf = pc_step_fx(mb.re, mb.im, sq);
+  const bool sums = a.cool && (a.ca.mode == CL_D2_MEANABS || a.ca.mode == CL_D2_RMS);
+  bool raw = true;  // the links stand as doubles (block-uniform)
   for (int s = 0; s < a.n_steps; ++s) {
-    // ---- CL step, all links at once
-    scan_products(Us, As, Bs, n);
-    // (each thread reads only its own link of Us, so it writes it in place)
-    if (act) {
-      const M2 P = k == 0 ? Bs.get(0) : m2mul(Bs.get(k), As.get(k - 1));
-      double g[4];
-      normals_f64<2>(g, seed, a.step0 + (uint32_t)s, (uint32_t)k, 0u, STREAM_PC_CL);
-      const C htr = cscale(cadd(P.e[0], P.e[3]), 0.5);
-      const C mb = C{-a.eps * beta.re, -a.eps * beta.im};  // -eps beta
-      M2 A;
-      A.e[0] = cmul(mb, csub(P.e[0], htr));
-      A.e[3] = cmul(mb, csub(P.e[3], htr));
-      A.e[1] = cmul(mb, P.e[1]);
-      A.e[2] = cmul(mb, P.e[2]);
-      // + i sq [[g3, g1 - i g2], [g1 + i g2, -g3]]
-      A.e[0].im += sq * g[2];
-      A.e[3].im -= sq * g[2];
-      A.e[1].re += sq * g[1];
-      A.e[1].im += sq * g[0];
-      A.e[2].re -= sq * g[1];
-      A.e[2].im += sq * g[0];
-      M2 W = m2mul(exp_traceless(A), Us.get(k));
-      const C z = cinv(csqrt_p(m2det(W)));
-#pragma unroll
-      for (int q = 0; q < 4; ++q) W.e[q] = cmul(W.e[q], z);
-      Us.set(k, W);
+    if (FX && raw && cf.ok) {
+      F2 f;
+      raw = __syncthreads_or(!ch.fits(f));
+      if (!raw && ch.act) ch.Uf().set(k, f);
+      __syncthreads();
     }
-    __syncthreads();
+    // ---- CL step, all links at once
+    if (FX && !raw && !ch.step_fx(cf, seed, a.step0 + (uint32_t)s)) {
+      ch.to_double();
+      raw = true;
+    }
+    if (!FX || raw) ch.step_f64(mb, sq, seed, a.step0 + (uint32_t)s);
     // ---- gauge cooling (the adaptive rule of the SU(3) path, per chain)
     int sweeps = 0;
     double un = 0.0, un_prev = 0.0;
     for (int it = 0;; ++it) {
       double v[4] = {0.0, 0.0, 0.0, 0.0}, f[3] = {0.0, 0.0, 0.0};
-      if (act) {
-        const M2 u = Us.get(k);
-        const M2 w = Us.get(k == 0 ? n - 1 : k - 1);
-        // G = u u^+ - w^+ w (Hermitian)
-        C G00 = C{0.0, 0.0}, G01 = C{0.0, 0.0}, G10 = C{0.0, 0.0}, G11 = C{0.0, 0.0};
-        G00 = cfma(u.e[0], cconj(u.e[0]), cfma(u.e[1], cconj(u.e[1]), G00));
-        G01 = cfma(u.e[0], cconj(u.e[2]), cfma(u.e[1], cconj(u.e[3]), G01));
-        G10 = cfma(u.e[2], cconj(u.e[0]), cfma(u.e[3], cconj(u.e[1]), G10));
-        G11 = cfma(u.e[2], cconj(u.e[2]), cfma(u.e[3], cconj(u.e[3]), G11));
-        G00 = cfms(cconj(w.e[0]), w.e[0], cfms(cconj(w.e[2]), w.e[2], G00));
-        G01 = cfms(cconj(w.e[0]), w.e[1], cfms(cconj(w.e[2]), w.e[3], G01));
-        G10 = cfms(cconj(w.e[1]), w.e[0], cfms(cconj(w.e[3]), w.e[2], G10));
-        G11 = cfms(cconj(w.e[1]), w.e[1], cfms(cconj(w.e[3]), w.e[3], G11));
-        f[0] = 2.0 * (G01.re + G10.re);
-        f[1] = 2.0 * (G10.im - G01.im);
-        f[2] = 2.0 * (G00.re - G11.re);
-        const double tuu = u.e[0].re * u.e[0].re + u.e[0].im * u.e[0].im + u.e[1].re * u.e[1].re +
-                           u.e[1].im * u.e[1].im + u.e[2].re * u.e[2].re + u.e[2].im * u.e[2].im +
-                           u.e[3].re * u.e[3].re + u.e[3].im * u.e[3].im;
-        v[0] = 0.5 * tuu;
-        v[1] = fabs(f[0]) + fabs(f[1]) + fabs(f[2]);
-        v[2] = f[0] * f[0] + f[1] * f[1] + f[2] * f[2];
+      fx g[3];
+      if (FX && !raw) {
+        long long t;
+        fx_chk ck;
+        pc_grad_fx(ch.Uf().get(k), ch.Uf().get(k == 0 ? n - 1 : k - 1), g, t, ck);
+        if (__syncthreads_or(ck.bad())) {
+          ch.to_double();
+          raw = true;
+        } else {
+          un = 1.0 + (double)block_sum(ch.act ? (t + 256) >> 9 : 0, (long long*)ch.red()) * (inv_n * 0x1p-52);
+          if (sums) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) f[q] = fx_to_double(g[q], 2);
+            ch.norms_f64(v, 0.0, f);
+          }
+        }
       }
-      block_reduce4(v, red);
-      un = v[0] / n;
+      if (!FX || raw) {
+        const double tr = ch.grad_f64(f);
+        ch.norms_f64(v, tr, f);
+        un = v[0] / n;
+      }
       if (!a.cool) break;
       double D = 1.0;
       if (a.ca.mode == CL_D1) D = un;
@@ -307,36 +489,61 @@ __global__ void __launch_bounds__(MAXT, 1) k_pchain(PcArgs a) {
       }
       if (D < a.ca.d_guard) stop = true;
       if (stop) break;
-      const double alpha_ad = a.ca.alpha / D;
-      if (act) {
-        const double ea = -a.ca.eps * alpha_ad;  // the cooling eps, not the Langevin one
-        const double h[3] = {ea * f[0], ea * f[1], ea * f[2]};
-        M2 om, omi;
-        exp_herm_pair(h, om, omi);
-        As.set(k, om);
-        Bs.set(k, omi);
+      const double ea = -a.ca.eps * a.ca.alpha * pc_recip(D);  // the cooling eps, not the Langevin one
+      if (FX && !raw && !ch.apply_fx(g, ea)) {
+        ch.to_double();
+        raw = true;
+        ch.grad_f64(f);
       }
-      __syncthreads();
-      if (act) Us.set(k, m2mul(m2mul(As.get(k), Us.get(k)), Bs.get(k + 1 == n ? 0 : k + 1)));
-      __syncthreads();
+      if (!FX || raw) ch.apply_f64(f, ea);
       ++sweeps;
       un_prev = un;
+    }
+    if (FX && !raw) {  // round to doubles
+      const M2 u = ch.as_double();
+      unsigned mag = 0;
+      F2 r;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r.e[q] = cx<fx>{fx_of_double(u.e[q].re, mag), fx_of_double(u.e[q].im, mag)};
+      __syncthreads();
+      if (ch.act) ch.Uf().set(k, r);
+      __syncthreads();
     }
     // ---- records
     const int done = a.done0 + s + 1;
     if (a.obs_every > 0 && done % a.obs_every == 0) {
-      scan_products(Us, As, Bs, n);
-      double v[4] = {0.0, 0.0, 0.0, 0.0};
-      if (act) {
-        const C d = m2det(Us.get(k));
-        v[3] = hypot(d.re - 1.0, d.im);
+      C tr, d;
+      bool have = false;
+      if (FX && !raw) {
+        F2 P;
+        int S;
+        have = ch.product_fx(P, S);
+        if (have) {
+          tr = C{fx_bits_to_double(fx_bits(P.e[0].re) + fx_bits(P.e[3].re), S),
+                 fx_bits_to_double(fx_bits(P.e[0].im) + fx_bits(P.e[3].im), S)};
+          const F2 u = ch.Uf().get(k);
+          fx_acc re = fx_acc{-(1ll << 60), 0ull}, im = fx_zero();
+          fx_cmac(re, im, fx_lhs(u.e[0]), fx_rhs(u.e[3]));
+          fx_cmac(re, im, fx_lhs_neg(u.e[1]), fx_rhs(u.e[2]));
+          d = C{fx_bits_to_double(fx_sum(re) - (1 << 29)), fx_bits_to_double(fx_sum(im) - (1 << 29))};
+        } else {
+          ch.to_double();
+          raw = true;
+        }
       }
-      block_reduce4(v, red);
-      if (k == 0) {
+      if (!have) {
+        const M2 P = ch.product_f64();
+        __syncthreads();
+        tr = cadd(P.e[0], P.e[3]);
+        d = m2det(ch.Us().get(k));
+        d.re -= 1.0;
+      }
+      double v[4] = {0.0, 0.0, 0.0, hypot(d.re, d.im)};
+      block_reduce4(v, ch.red());
+      if (threadIdx.x == 0) {
         double* o = a.obs + ((size_t)(done / a.obs_every - 1) * a.n_chains + c) * 5;
-        const M2 tot = As.get(n - 1);
-        o[0] = 0.5 * (tot.e[0].re + tot.e[3].re);
-        o[1] = 0.5 * (tot.e[0].im + tot.e[3].im);
+        o[0] = 0.5 * tr.re;
+        o[1] = 0.5 * tr.im;
         o[2] = un;
         o[3] = v[3];
         o[4] = (double)sweeps;
@@ -344,8 +551,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_pchain(PcArgs a) {
       __syncthreads();
     }
   }
-  if (act) {
-    const M2 u = Us.get(k);
+  if (FX && !raw) ch.to_double();
+  if (ch.act) {
+    const M2 u = ch.Us().get(k);
     for (int q = 0; q < 4; ++q) Ug[4 * k + q] = make_double2(u.e[q].re, u.e[q].im);
   }
 }
