@@ -29,17 +29,15 @@
  *    gives CL_ERR_CUDA; its text is kept (per thread) for cl_last_error().
  *    A lattice is not thread-safe: one host thread per lattice at a time.
  *  - Precision (cl_precision): CL_FP64 keeps links in FP64; its matrix
- *    products run in 60-bit fixed point with FP32 low-order terms (errors at
- *    or below FP64's for links near SU(3); wherever a number leaves the
- *    fixed-point range, in FP64), the rest in FP64.  CL_FP32_STORAGE stores and multiplies links in FP32 and keeps in
- *    FP64 the matrix exponentials of the Langevin and cooling updates, the
- *    det U = 1 re-projection and every global reduction.  CL_DF64 stores
- *    links as double-float pairs (hi + lo floats, ~48 significant bits) and
- *    does the link algebra (products, inverses, plaquettes, clover, drift,
- *    cooling transformations), the noise, the exponentials and the
- *    re-projection in double-float arithmetic on the FP32 pipe, with only
- *    the reductions' final sums in FP64; its results agree with CL_FP64 to
- *    ~1e-14 per step.
+ *    products, noise and exponentials run in 60-bit fixed point with FP32
+ *    low-order terms (errors at or below FP64's for links near SU(3); wherever
+ *    a number leaves the fixed-point range, in FP64), the rest in FP64.
+ *    CL_FP32_STORAGE stores and multiplies links in FP32; the matrix
+ *    exponentials of the Langevin and cooling updates and the det U = 1
+ *    re-projection keep FP64's precision, every global reduction is FP64.
+ *    CL_DF64 stores links as double-float pairs (hi + lo floats, ~48
+ *    significant bits) and is the FP64 form in everything else; its results
+ *    agree with CL_FP64 to ~1e-14 per step.
  *  - Noise: Philox4x32-10 keyed by (seed, step, site, mu), so results do not
  *    depend on launch shape, and a run resumed from cl_get_links /
  *    cl_get_step reproduces the uninterrupted one.
@@ -435,8 +433,8 @@ cl_status cl_cool_gradient(cl_lattice* lat, double* host_f);
  * draw them (Philox4x32-10 stream 0, Box-Muller): for each of the nsites
  * sites site0 .. site0 + nsites - 1 and direction mu, the 8 numbers of link
  * (site, mu) at step `step` (the update's eta_a = sqrt(2) times them, a =
- * 1..8, so that <eta_a eta_b> = 2 delta_ab), host doubles [site][8].  FP64 draws them in FP64,
- * DF64 in double-float, FP32 storage in float.  A diagnostic: it uses the
+ * 1..8, so that <eta_a eta_b> = 2 delta_ab), host doubles [site][8].  FP64 and DF64 draw them
+ * in fixed point to FP64's precision, FP32 storage in float.  A diagnostic: it uses the
  * current device and the legacy default stream, allocates and frees its own
  * device buffer, and synchronises.  Errors: CL_ERR_INVALID (NULL out, bad
  * precision, nsites < 0, site0 < 0, mu outside 0..3), CL_ERR_OOM, CL_ERR_CUDA. */

@@ -114,9 +114,9 @@ cl_status ensure_stage(cl_lattice* l) {
 // F^ = -i theta kappa F: -i (a + ib) kappa = kappa b - i kappa a.
 double clover_scale_re(const cl_lattice* l) { return KAPPA_Q * l->p.theta_im; }
 double clover_scale_im(const cl_lattice* l) { return -KAPPA_Q * l->p.theta_re; }
-// C holds the drift contributions times 2^-e in the FP64 form's fixed point.
+// C holds the drift contributions times 2^-e in fixed point (FP64, DF64).
 int contribution_exponent(const cl_lattice* l) {
-  return l->prec == 0 ? drift_exponent(l->p.beta, clover_scale_re(l), clover_scale_im(l)) : 0;
+  return l->prec != 1 ? drift_exponent(l->p.beta, clover_scale_re(l), clover_scale_im(l)) : 0;
 }
 
 bool theta_nonzero(const cl_lattice* l) { return l->p.theta_re != 0.0 || l->p.theta_im != 0.0; }
@@ -379,8 +379,7 @@ cl_status cl_init_lattice(const cl_params* params, void* cuda_stream, cl_lattice
     l->Omi = c + sizeof(double) * 8 * Vs + real_size(l) * 9 * Vs;
     l->crec = (double*)(c + align256(sizeof(double) * 8 * Vs + 2 * real_size(l) * 9 * Vs));
   }
-  cudaError_t e = l->prec == 2 ? prepare_df64_kernels() : cudaSuccess;
-  if (e == cudaSuccess) e = init_state(l);
+  cudaError_t e = init_state(l);
   if (e != cudaSuccess) {
     cl_free(l);
     return fail(CL_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e));

@@ -24,8 +24,8 @@ __device__ __forceinline__ Geo geo_of(const ChainDesc& c) {
 }
 
 // Blocks per SM the link-algebra kernels are built for: the FP64 form's as its
-// single-chain kernels (FX_MAXNREG, k_update_f64.cu).
-#define ENS_MIN_BLOCKS(T) (std::is_same<T, double>::value ? 3 : 1)
+// single-chain kernels (FX_MAXNREG, k_update_fx_launch.cuh).
+#define ENS_MIN_BLOCKS(T) (is_fx<T>() ? 3 : 1)
 
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_inverse(const ChainDesc* __restrict__ cd,
@@ -33,10 +33,7 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_inverse(const ChainDesc*
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  if constexpr (std::is_same<T, double>::value)
-    fx_links_body(geo_of(c), (const V2*)c.U, (int4*)c.Un, (int4*)c.Ui, it.vb);
-  else
-    k_link_inverse_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Ui, it.vb);
+  fx_links_body<T>(geo_of(c), (const V2*)c.U, (int4*)c.Un, (int4*)c.Ui, it.vb);
 }
 
 template <typename T>
@@ -45,10 +42,10 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  if constexpr (std::is_same<T, double>::value)
-    fx_plaq_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, it.vb);
+  if constexpr (is_fx<T>())
+    fx_plaq_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, it.vb);
   else
-    k_plaq_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (V2*)c.Pq, (V2*)c.Dq, it.vb);
+    k_plaq_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Pq, (V2*)c.Dq, it.vb);
 }
 
 template <typename T>
@@ -57,11 +54,11 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(con
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  if constexpr (std::is_same<T, double>::value)
-    fx_clover_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.F,
+  if constexpr (is_fx<T>())
+    fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.F,
                    c.sre, c.sim, it.vb);
   else
-    k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
+    k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }
 
 template <typename T>
@@ -70,11 +67,11 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_wils
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  if constexpr (std::is_same<T, double>::value)
-    fx_force_wilson_body(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C,
+  if constexpr (is_fx<T>())
+    fx_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C,
                          ldexp(c.beta / 6.0, -c.cexp), it.vb);
   else
-    k_plaq_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Dq, (V2*)c.C,
+    k_plaq_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.C,
                               (T)(c.beta / 6.0), it.vb);
 }
 
@@ -93,7 +90,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_b(co
                                                                 const WorkItem* __restrict__ w) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  fx_force_b_body(geo_of(c), (const double2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
+  fx_force_b_body<T>(geo_of(c), (const typename vec2_of<T>::type*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
                   (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), it.vb);
 }
 
@@ -103,7 +100,7 @@ __global__ void __maxnreg__(FORCE_AB_MAXNREG) k_ens_force_ab(const ChainDesc* __
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  k_plaq_force_ab_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Ui, (const V2*)c.Pq, (const V2*)c.Dq,
+  k_plaq_force_ab_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Pq, (const V2*)c.Dq,
                           (const V2*)c.F, (V2*)c.C, (T)(c.beta / 6.0), it.vb);
 }
 
@@ -125,9 +122,12 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_update(const ChainDesc* 
   a.seed = c.seed;
   a.sd = c.sd;
   a.adaptive = MODE == MODE_UPDATE_X ? 1 : 0;
-  const V2* in = (const V2*)(MODE == MODE_UPDATE_X ? c.Pq : c.C);
-  V2* out = (V2*)(MODE == MODE_DRIFTMAX ? c.Pq : c.Un);
-  k_update_gather_body<T, MODE>(geo_of(c), (const V2*)c.U, in, out, a, it.vb);
+  const void* in = MODE == MODE_UPDATE_X ? c.Pq : c.C;
+  void* out = MODE == MODE_DRIFTMAX ? c.Pq : c.Un;
+  if constexpr (is_fx<T>())
+    fx_update_body<T, MODE>(geo_of(c), (const V2*)c.U, (const int4*)in, out, a, it.vb);
+  else
+    k_update_gather_body<T, MODE>(geo_of(c), (const V2*)c.U, (const V2*)in, (V2*)out, a, it.vb);
 }
 
 // Launch family fam of the CL step for link type T (FP64 runs the theta
@@ -137,12 +137,14 @@ cudaError_t launch_ens_step_family(int fam, const ChainDesc* cd, const WorkItem*
   if (nw <= 0) return cudaSuccess;
   const unsigned n = (unsigned)nw;
   switch (fam) {
-    case ENS_INVERSE: k_ens_inverse<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
+    case ENS_INVERSE:
+      if constexpr (is_fx<T>()) k_ens_inverse<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
+      break;
     case ENS_PLAQ: k_ens_plaq<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_CLOVER: k_ens_clover<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_FORCE_WILSON: k_ens_force_wilson<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_FORCE_THETA:
-      if constexpr (sizeof(T) == 8) {  // FP64: the split form (only it is instantiated)
+      if constexpr (is_fx<T>()) {
         k_ens_force_a<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
         k_ens_force_b<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
       } else {

@@ -50,17 +50,8 @@ struct UpdArgs {
   uint64_t seed;
   StepDev* sd;    // device-resident step state (graph-replayable)
   int adaptive;   // 1: the step size is sd->eps_n (set by the drift pass)
-  int cexp;       // FP64: C holds the contributions times 2^-cexp (drift_exponent)
+  int cexp;       // fixed point: C holds the contributions times 2^-cexp (drift_exponent)
 };
-
-// FP64 form (k_update_fx.cuh): the update of link (s, MU), from the fixed-point
-// contributions C (X NULL) or from the drift in X; and its drift alone.
-__device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const double2* C, const double2* X,
-                                           double2* out, const UpdArgs& a, int s, const int* x, int MU);
-__device__ __forceinline__ double drift_f64(const Geo& g, const double2* C, double2* out, int cexp, int s, const int* x,
-                                            int MU, bool write);
-__device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
-                                           const double2* C, int cexp);
 
 // Sign flip on the integer pipe (no floating-point instruction).
 __device__ __forceinline__ double flip(double x, unsigned long long m) {
@@ -68,9 +59,6 @@ __device__ __forceinline__ double flip(double x, unsigned long long m) {
 }
 __device__ __forceinline__ float flip(float x, unsigned long long m) {
   return __int_as_float(__float_as_int(x) ^ (int)(m >> 32));
-}
-__device__ __forceinline__ df64 flip(df64 x, unsigned long long m) {
-  return df64(flip(x.hi, m), flip(x.lo, m));
 }
 template <typename T, class FF>
 __device__ __forceinline__ void load_signed(mat<T>& G, FF F, int p, int s, int V, unsigned long long m) {
@@ -112,51 +100,21 @@ __device__ __forceinline__ void scaled(mat<T>& r, T c, const mat<T>& a) {
 }
 
 // ---------------------------------------------------------------- inverses
-// Ui = adj(U) = U^{-1} for every link (det U = 1 by the re-projection).
-template <typename T>
-__device__ __forceinline__ void k_link_inverse_body(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      typename vec2_of<T>::type* __restrict__ Ui, int vb) {
-  const int mu = vb % 4;
-  const int s = (vb / 4) * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  mat<T> u, ui;
-  load(u, U, mu, s, g.V);
+// The inverse of link (mu, site) from the link (det U = 1 by the
+// re-projection): the adjugate, on the FP32 pipe that the FP32-storage form's
+// memory- and latency-bound kernels leave idle.
+template <typename T, class FU>
+__device__ __forceinline__ void load_inv(mat<T>& ui, FU U, int mu, int site, int V) {
+  mat<T> u;
+  load(u, U, mu, site, V);
   adj(ui, u);
-  store(Ui, mu, s, g.V, ui);
-}
-template <typename T>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_link_inverse(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                      typename vec2_of<T>::type* __restrict__ Ui) {
-  k_link_inverse_body<T>(g, U, Ui, blockIdx.x);
-}
-
-// The inverse of link (mu, site) as the plaquette, clover and force kernels
-// use it.  FP64: loaded from the U^{-1} field the link-inverse pass wrote
-// (forming it costs 126 flops on the FP64 pipe these kernels are bound by).
-// FP32 storage: formed from the link (the same adjugate, so the same bits,
-// on the FP32 pipe, which these memory- and latency-bound kernels leave
-// idle); no link-inverse pass runs and the load usually hits a line of U the
-// kernel reads anyway.
-template <typename T>
-__host__ __device__ constexpr bool inverse_on_the_fly() { return sizeof(T) == 4; }
-struct no_inverse {};  // in place of the U^{-1} field: form it from the link
-template <typename T, class FU, class FI>
-__device__ __forceinline__ void load_inv(mat<T>& ui, FU U, FI Ui, int mu, int site, int V) {
-  if constexpr (inverse_on_the_fly<T>() || std::is_same<FI, no_inverse>::value) {
-    mat<T> u;
-    load(u, U, mu, site, V);
-    adj(ui, u);
-  } else {
-    load(ui, Ui, mu, site, V);
-  }
 }
 
 // ------------------------------------------------------------- plaquettes
 // P_{mu nu}(x) = U_mu(x) U_nu(x+mu) U_mu(x+nu)^{-1} U_nu(x)^{-1} and
 // D = P - P^{-1}, six planes per site.
-template <typename T, class FU, class FUi, class FPq, class FDq>
+template <typename T, class FU, class FPq, class FDq>
 __device__ __forceinline__ void k_plaq_body(Geo g, FU U,
-                                              FUi Ui,
                                               FPq Pq,
                                               FDq Dq, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
@@ -164,13 +122,12 @@ __device__ __forceinline__ void k_plaq_body(Geo g, FU U,
   if (s >= g.V) return;
   int x[4];
   site_coords(g, s, x);
-  Work<T, 5> ws(0);
-  mat<T>&a = ws[0], &b = ws[1], &A = ws[2], &B = ws[3], &P = ws[4];
+  mat<T> a, b, A, B, P;
   load(a, U, mu, s, g.V);
   load(b, U, nu, hop(g, s, x, mu, 1), g.V);
   mul(A, a, b);
-  load_inv(a, U, Ui, mu, hop(g, s, x, nu, 1), g.V);
-  load_inv(b, U, Ui, nu, s, g.V);
+  load_inv(a, U, mu, hop(g, s, x, nu, 1), g.V);
+  load_inv(b, U, nu, s, g.V);
   mul(B, a, b);
   mul(P, A, B);
   store(Pq, p, s, g.V, P);
@@ -181,10 +138,9 @@ __device__ __forceinline__ void k_plaq_body(Geo g, FU U,
 }
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                              const typename vec2_of<T>::type* __restrict__ Ui,
                                               typename vec2_of<T>::type* __restrict__ Pq,
                                               typename vec2_of<T>::type* __restrict__ Dq) {
-  k_plaq_body<T>(g, U, Ui, Pq, Dq, blockIdx.x);
+  k_plaq_body<T>(g, U, Pq, Dq, blockIdx.x);
 }
 
 // ------------------------------------------------------------ clover field
@@ -194,9 +150,8 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq(Geo g, const typename v
 //   L4 = U_nu(x-nu)^{-1} P(x-nu) U_nu(x-nu),
 //   L3 = W^{-1} P(x-mu-nu) W with W = U_mu(x-mu-nu) U_nu(x-nu),
 // so F = D(x) + the three carried D's.  Stored times a complex scale.
-template <typename T, class FU, class FUi, class FDq, class FF>
+template <typename T, class FU, class FDq, class FF>
 __device__ __forceinline__ void k_clover_rot_body(Geo g, FU U,
-                                                    FUi Ui,
                                                     FDq Dq,
                                                     FF F,
                                                     double sre, double sim, int vb) {
@@ -207,23 +162,22 @@ __device__ __forceinline__ void k_clover_rot_body(Geo g, FU U,
   site_coords(g, s, x);
   const int xmm = hop(g, s, x, mu, -1), xmn = hop(g, s, x, nu, -1);
   const int xmm_mn = hop2(g, s, x, mu, -1, nu, -1);
-  Work<T, 4> ws(0);
-  mat<T>&acc = ws[0], &w = ws[1], &d = ws[2], &t = ws[3];
+  mat<T> acc, w, d, t;
   load(acc, Dq, p, s, g.V);
   // L2 = U_mu(x-mu)^{-1} D(x-mu) U_mu(x-mu)
-  load_inv(w, U, Ui, mu, xmm, g.V);
+  load_inv(w, U, mu, xmm, g.V);
   load(d, Dq, p, xmm, g.V);
   mul(t, w, d);
   load(w, U, mu, xmm, g.V);
   mul_acc<+1>(acc, t, w);
   // L3 + L4 = U_nu(x-nu)^{-1} [D(x-nu) + U_mu(x-mu-nu)^{-1} D(x-mu-nu) U_mu(x-mu-nu)] U_nu(x-nu)
-  load_inv(w, U, Ui, mu, xmm_mn, g.V);
+  load_inv(w, U, mu, xmm_mn, g.V);
   load(d, Dq, p, xmm_mn, g.V);
   mul(t, w, d);
   load(w, U, mu, xmm_mn, g.V);
   load(d, Dq, p, xmn, g.V);
   mul_acc<+1>(d, t, w);
-  load_inv(w, U, Ui, nu, xmn, g.V);
+  load_inv(w, U, nu, xmn, g.V);
   mul(t, w, d);
   load(w, U, nu, xmn, g.V);
   mul_acc<+1>(acc, t, w);
@@ -234,11 +188,10 @@ __device__ __forceinline__ void k_clover_rot_body(Geo g, FU U,
 }
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_clover_rot(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                    const typename vec2_of<T>::type* __restrict__ Ui,
                                                     const typename vec2_of<T>::type* __restrict__ Dq,
                                                     typename vec2_of<T>::type* __restrict__ F,
                                                     double sre, double sim) {
-  k_clover_rot_body<T>(g, U, Ui, Dq, F, sre, sim, blockIdx.x);
+  k_clover_rot_body<T>(g, U, Dq, F, sre, sim, blockIdx.x);
 }
 
 // ----------------------------------------------------- plaquette drift
@@ -247,27 +200,25 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_clover_rot(Geo g, const type
 // With theta the work has two stages: a handles corners c0..c2 (G0 + G1^ +
 // G2^ and the slot 0 / slot 2 partials, parked in C); b adds corner c3, forms
 // K and completes the four slots.
-template <typename T, class FU, class FUi, class FDq, class FC>
+template <typename T, class FU, class FDq, class FC>
 __device__ __forceinline__ void k_plaq_force_wilson_body(Geo g, FU U,
-                                                           FUi Ui,
                                                            FDq Dq,
                                                            FC C, T beta6, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
-  Work<T, 4> ws(0);
-  mat<T>&D = ws[0], &M = ws[1], &t = ws[2], &a = ws[3];
+  mat<T> D, M, t, a;
   load(D, Dq, p, s, g.V);
   scaled(M, -beta6, D);
   store(C, 4 * p + 0, s, g.V, M);
-  load_inv(a, U, Ui, mu, s, g.V);
+  load_inv(a, U, mu, s, g.V);
   mul(t, a, M);
   load(a, U, mu, s, g.V);
   mul(M, t, a);
   store(C, 4 * p + 2, s, g.V, M);
   scaled(M, beta6, D);
   store(C, 4 * p + 1, s, g.V, M);
-  load_inv(a, U, Ui, nu, s, g.V);
+  load_inv(a, U, nu, s, g.V);
   mul(t, a, M);
   load(a, U, nu, s, g.V);
   mul(M, t, a);
@@ -275,17 +226,15 @@ __device__ __forceinline__ void k_plaq_force_wilson_body(Geo g, FU U,
 }
 template <typename T>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_plaq_force_wilson(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                           const typename vec2_of<T>::type* __restrict__ Ui,
                                                            const typename vec2_of<T>::type* __restrict__ Dq,
                                                            typename vec2_of<T>::type* C, T beta6) {
-  k_plaq_force_wilson_body<T>(g, U, Ui, Dq, C, beta6, blockIdx.x);
+  k_plaq_force_wilson_body<T>(g, U, Dq, C, beta6, blockIdx.x);
 }
 
 // Corners c0..c2: G^ (partial) into Gh, slot 0 and slot 2 partials into C.
-template <typename T, class FU, class FUi, class FDq, class FF, class FC>
+template <typename T, class FU, class FDq, class FF, class FC>
 __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, const int x[4], int p,
                                               FU U,
-                                              FUi Ui,
                                               FDq Dq,
                                               FF F,
                                               FC C, T beta6) {
@@ -293,8 +242,7 @@ __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, c
   // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
   const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c1 = hop(g, s, x, mu, 1);
-  Work<T, 4> ws(1);  // slot 0 holds Gh
-  mat<T>&D = ws[0], &M = ws[1], &t = ws[2], &q = ws[3];
+  mat<T> D, M, t, q;
   load(D, Dq, p, s, g.V);
   // corner c0: slot 0 partial = [D, G0] - (beta/6) D
   load_signed(Gh, F, pc, s, g.V, m);
@@ -305,7 +253,7 @@ __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, c
   load_signed(t, F, pc, c1, g.V, m);
   load(q, U, mu, s, g.V);
   mul(D, q, t);  // a G1 (D is re-read below)
-  load_inv(q, U, Ui, mu, s, g.V);
+  load_inv(q, U, mu, s, g.V);
   mul(t, D, q);  // G1^
 #pragma unroll
   for (int k = 0; k < 9; ++k) Gh.e[k] = cadd(Gh.e[k], t.e[k]);
@@ -324,10 +272,9 @@ __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, c
 }
 
 // Corner c3, K, and the four slots completed; Gh holds the stage-a sum.
-template <typename T, class FU, class FUi, class FPq, class FDq, class FF, class FC>
+template <typename T, class FU, class FPq, class FDq, class FF, class FC>
 __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, const int x[4], int p,
                                               FU U,
-                                              FUi Ui,
                                               FPq Pq,
                                               FDq Dq,
                                               FF F,
@@ -336,13 +283,12 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
   // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
   const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c3 = hop(g, s, x, nu, 1);
-  Work<T, 4> ws(1);  // slot 0 holds Gh
-  mat<T>&D = ws[0], &M = ws[1], &t = ws[2], &q = ws[3];
+  mat<T> D, M, t, q;
   // corner c3: G3r = u G3 u^{-1}; slot 3 partial = [D, G3r] + (beta/6) D
   load_signed(q, F, pc, c3, g.V, m);
   load(M, U, nu, s, g.V);
   mul(t, M, q);
-  load_inv(M, U, Ui, nu, s, g.V);
+  load_inv(M, U, nu, s, g.V);
   mul(q, t, M);
   load(D, Dq, p, s, g.V);
   scaled(M, beta6, D);
@@ -377,7 +323,7 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
   load_rw(M, C, 4 * p + 2, s, g.V);
 #pragma unroll
   for (int k = 0; k < 9; ++k) M.e[k] = cadd(M.e[k], K.e[k]);
-  load_inv(Gh, U, Ui, mu, s, g.V);
+  load_inv(Gh, U, mu, s, g.V);
   mul(t, Gh, M);
   load(Gh, U, mu, s, g.V);
   mul(M, t, Gh);
@@ -386,7 +332,7 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
   load_rw(M, C, 4 * p + 3, s, g.V);
 #pragma unroll
   for (int k = 0; k < 9; ++k) M.e[k] = csub(M.e[k], K.e[k]);
-  load_inv(Gh, U, Ui, nu, s, g.V);
+  load_inv(Gh, U, nu, s, g.V);
   mul(t, Gh, M);
   load(Gh, U, nu, s, g.V);
   mul(M, t, Gh);
@@ -402,9 +348,8 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
 // with a plain load.
 const int GQ_PLANE = 4;
 // Fused form (FP32, and the FP64 form's general path).
-template <typename T, class FU, class FUi, class FPq, class FDq, class FF, class FC>
+template <typename T, class FU, class FPq, class FDq, class FF, class FC>
 __device__ __forceinline__ void k_plaq_force_ab_body(Geo g, FU U,
-                                                       FUi Ui,
                                                        FPq Pq,
                                                        FDq Dq,
                                                        FF F,
@@ -414,10 +359,9 @@ __device__ __forceinline__ void k_plaq_force_ab_body(Geo g, FU U,
   if (s >= g.V) return;
   int x[4];
   site_coords(g, s, x);
-  Work<T, 1> wg(0);
-  mat<T>& Gh = wg[0];
-  force_stage_a(Gh, g, s, x, p, U, Ui, Dq, F, C, beta6);
-  force_stage_b(Gh, g, s, x, p, U, Ui, Pq, Dq, F, C, beta6);
+  mat<T> Gh;
+  force_stage_a(Gh, g, s, x, p, U, Dq, F, C, beta6);
+  force_stage_b(Gh, g, s, x, p, U, Pq, Dq, F, C, beta6);
 }
 // Left to itself the compiler gives the fused FP32 force 228 registers, two
 // blocks of 128 per SM; capped at 160 it keeps three (a few hundred bytes of
@@ -428,12 +372,11 @@ __device__ __forceinline__ void k_plaq_force_ab_body(Geo g, FU U,
 const int FORCE_AB_MAXNREG = 160;
 template <typename T>
 __global__ void __maxnreg__(FORCE_AB_MAXNREG) k_plaq_force_ab(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                       const typename vec2_of<T>::type* __restrict__ Ui,
                                                        const typename vec2_of<T>::type* __restrict__ Pq,
                                                        const typename vec2_of<T>::type* __restrict__ Dq,
                                                        const typename vec2_of<T>::type* __restrict__ F,
                                                        typename vec2_of<T>::type* C, T beta6) {
-  k_plaq_force_ab_body<T>(g, U, Ui, Pq, Dq, F, C, beta6, blockIdx.x);
+  k_plaq_force_ab_body<T>(g, U, Pq, Dq, F, C, beta6, blockIdx.x);
 }
 
 // Noise matrix sum_a eta_a lambda_a (Hermitian) into the imaginary part of A,
@@ -509,6 +452,17 @@ static __device__ __noinline__ void general_update_f32(mat<float>& Un, const mat
 }
 
 // ------------------------------------------------ gather + exponential update
+// Running maximum of |K|^2 over the lattice (whole warps; lanes past the end repeat the last site).
+__device__ __forceinline__ void kmax_update(StepDev* sd, double kk) {
+  unsigned long long k2 = (unsigned long long)__double_as_longlong(kk);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, k2, o);
+    k2 = v > k2 ? v : k2;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(&sd->kmax2_bits, k2);
+}
+
 // X of link (x, mu) = sum of its six plaquette contributions: for nu != mu,
 // mu < nu: slot 0 of (x, p) and slot 3 of (x - nu, p); mu > nu: slot 1 of
 // (x, p) and slot 2 of (x - nu, p), p the plane of (mu, nu).
@@ -525,17 +479,9 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
   const int s = s_raw < g.V ? s_raw : g.V - 1;
   int x[4];
   site_coords(g, s, x);
-  Work<T, 2> ws(0);
-  mat<T>&X = ws[0], &t = ws[1];
-  if constexpr (std::is_same<T, double>::value && (MODE == MODE_UPDATE || MODE == MODE_UPDATE_X)) {
-    update_f64(g, U, MODE == MODE_UPDATE ? C : nullptr, MODE == MODE_UPDATE ? nullptr : C, out, a, s, x, MU);
-    return;
-  } else if constexpr (std::is_same<T, double>::value && MODE == MODE_DRIFTMAX) {
-    // the gather is part of drift_f64
-  } else if (MODE == MODE_UPDATE_X) {
+  mat<T> X, t;
+  if (MODE == MODE_UPDATE_X) {
     load(X, C, MU, s, g.V);  // the drift stored by the MODE_DRIFTMAX pass
-  } else if constexpr (std::is_same<T, double>::value) {
-    gather_f64(X, g, s, x, MU, C, a.cexp);
   } else {
     set_zero(X);
 #pragma unroll
@@ -557,22 +503,10 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
   }
   if (MODE == MODE_DRIFTMAX) {
     // |K|^2 = sum_a |Tr(lambda_a X)|^2 = 2 |X - Tr X / 3|_F^2 (Tr l_a l_b = 2 delta_ab)
-    double kk;
-    if constexpr (std::is_same<T, double>::value) {
-      kk = drift_f64(g, C, out, a.cexp, s, x, MU, s_raw < g.V);
-    } else {
-      if (s_raw < g.V) store(out, MU, s, g.V, X);
-      mat<double> Xd;
-      convert(Xd, X);
-      kk = general_k2(Xd);
-    }
-    unsigned long long k2 = (unsigned long long)__double_as_longlong(kk);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long v = __shfl_xor_sync(0xffffffffu, k2, o);
-      k2 = v > k2 ? v : k2;
-    }
-    if ((threadIdx.x & 31) == 0) atomicMax(&a.sd->kmax2_bits, k2);
+    if (s_raw < g.V) store(out, MU, s, g.V, X);
+    mat<double> Xd;
+    convert(Xd, X);
+    kmax_update(a.sd, general_k2(Xd));
     return;
   }
   // exponent A = 2 eps (X - Tr X/3) + i sqrt(eps) eta_a lambda_a.  The
@@ -581,71 +515,48 @@ __device__ __forceinline__ void k_update_gather_body(Geo g, const typename vec2_
   const uint32_t step = a.sd->step;
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
-  if constexpr (std::is_same<T, df64>::value) {
-    // DF64: the noise, the exponent, the exponential (its scalar recurrences
-    // too), the update and the re-projection in double-float; no FP64
-    // instruction on the common path
-    df64 eta[8];
-    normals_df64<4>(eta, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
-    exponent<df64>(X, eta, df64(eps), df64(sqrt_eps));
-    // three workspace slots: E overwrites X (entry by entry), the link U
-    // takes the slot of X^2 once E is formed
-    Work<df64, 1> wu(2);
-    mat<df64>&E = X, &Ul = t, &Un = wu[0];
-    expm_traceless_df(E, X, t);
-    load(Ul, U, MU, s, g.V);
-    mul_df_compact(Un, E, Ul);
-    const cx<df64> z = det_inv_cuberoot_df(det(Un));
-#pragma unroll 1
-    for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], z);  // rolled: Un is in the workspace; saves code
-    store(out, MU, s, g.V, Un);
-    return;
-  }
-  if constexpr (std::is_same<T, float>::value) {
-    // the exponent in FP32, the exponential in fixed point; beyond its range in FP64
-    float ef[8];
-    normals_f32<4>(ef, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
-    exponent<float>(X, ef, (float)eps, (float)sqrt_eps);
-    const float rA = sqrtf(norm2(X));
-    mat<float> Et, Ul, Un;
-    load(Ul, U, MU, s, g.V);
-    bool done = false;
-    if (rA < 1.4f) {  // every entry below the bound
-      mat<fx> A;
+  // the exponent in FP32, the exponential in fixed point; beyond its range in FP64
+  float ef[8];
+  normals_f32<4>(ef, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
+  exponent<float>(X, ef, (float)eps, (float)sqrt_eps);
+  const float rA = sqrtf(norm2(X));
+  mat<float> Et, Ul, Un;
+  load(Ul, U, MU, s, g.V);
+  bool done = false;
+  if (rA < 1.4f) {  // every entry below the bound
+    mat<fx> A;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) A.e[k] = cx<fx>{fx_of_float(X.e[k].re), fx_of_float(X.e[k].im)};
-      if (fx_expm_traceless(A, rA, taylor_tol<float>())) {
+    for (int k = 0; k < 9; ++k) A.e[k] = cx<fx>{fx_of_float(X.e[k].re), fx_of_float(X.e[k].im)};
+    if (fx_expm_traceless(A, rA, taylor_tol<float>())) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Et.e[k] = cx<float>{fx_to_float(A.e[k].re), fx_to_float(A.e[k].im)};
-        mul(Un, Et, Ul);
-        float mx = 0.0f;
+      for (int k = 0; k < 9; ++k) Et.e[k] = cx<float>{fx_to_float(A.e[k].re), fx_to_float(A.e[k].im)};
+      mul(Un, Et, Ul);
+      float mx = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-          mx = fmaxf(mx, fmaxf(fabsf(Un.e[k].re), fabsf(Un.e[k].im)));
-          A.e[k] = cx<fx>{fx_of_float(Un.e[k].re), fx_of_float(Un.e[k].im)};
-        }
-        fx_chk ck;
-        const cx<fx> d = fx_det_minus_one(A, ck);
-        const cx<float> e = {fx_to_float(d.re), fx_to_float(d.im)};
-        if (mx < 1.43f && !ck.bad() && fmaf(e.re, e.re, e.im * e.im) < 1e-11f) {
-          // det^{-1/3} = 1 - e/3 + 2 e^2/9 (the next term is below 5e-18), rounded to float
-          const float q = 2.0f / 9.0f;
-          const cx<float> z = {1.0f + fmaf(q * e.re, e.re, fmaf(-q * e.im, e.im, e.re * (-1.0f / 3.0f))),
-                               fmaf(2.0f * q * e.re, e.im, e.im * (-1.0f / 3.0f))};
+      for (int k = 0; k < 9; ++k) {
+        mx = fmaxf(mx, fmaxf(fabsf(Un.e[k].re), fabsf(Un.e[k].im)));
+        A.e[k] = cx<fx>{fx_of_float(Un.e[k].re), fx_of_float(Un.e[k].im)};
+      }
+      fx_chk ck;
+      const cx<fx> d = fx_det_minus_one(A, ck);
+      const cx<float> e = {fx_to_float(d.re), fx_to_float(d.im)};
+      if (mx < 1.43f && !ck.bad() && fmaf(e.re, e.re, e.im * e.im) < 1e-11f) {
+        // det^{-1/3} = 1 - e/3 + 2 e^2/9 (the next term is below 5e-18), rounded to float
+        const float q = 2.0f / 9.0f;
+        const cx<float> z = {1.0f + fmaf(q * e.re, e.re, fmaf(-q * e.im, e.im, e.re * (-1.0f / 3.0f))),
+                             fmaf(2.0f * q * e.re, e.im, e.im * (-1.0f / 3.0f))};
 #pragma unroll
-          for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], z);
-          done = true;
-        }
+        for (int k = 0; k < 9; ++k) Un.e[k] = cmul(Un.e[k], z);
+        done = true;
       }
     }
-    if (!done) {
-      mat<float> Xg = X, Ug = Ul, Ung;
-      general_update_f32(Ung, Xg, Ug, rA);
-      Un = Ung;
-    }
-    store(out, MU, s, g.V, Un);
-    return;
   }
+  if (!done) {
+    mat<float> Xg = X, Ug = Ul, Ung;
+    general_update_f32(Ung, Xg, Ug, rA);
+    Un = Ung;
+  }
+  store(out, MU, s, g.V, Un);
 }
 template <typename T, int MODE>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_update_gather(Geo g, const typename vec2_of<T>::type* __restrict__ U,

@@ -12,38 +12,32 @@ typedef vec2_of<float>::type V2;
 inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 1) / bs) * planes)); }
 }  // namespace
 
-cudaError_t launch_link_inverse_f32(const GeoH& h, const void* U, void* Ui, cudaStream_t st) {
-  Geo g = make_geo(h.L, h.V);
-  k_link_inverse<float><<<grid(g.V, 4, block_of(h, TUNE_CLOVER)), block_of(h, TUNE_CLOVER), 0, st>>>(g, (const V2*)U, (V2*)Ui);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_plaq_f32(const GeoH& h, const void* U, const void* Ui, void* Pq, void* Dq,
+cudaError_t launch_plaq_f32(const GeoH& h, const void* U, void* Pq, void* Dq,
                            cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  k_plaq<float><<<grid(g.V, 6, block_of(h, TUNE_CLOVER)), block_of(h, TUNE_CLOVER), 0, st>>>(g, (const V2*)U, (const V2*)Ui, (V2*)Pq, (V2*)Dq);
+  k_plaq<float><<<grid(g.V, 6, block_of(h, TUNE_CLOVER)), block_of(h, TUNE_CLOVER), 0, st>>>(g, (const V2*)U, (V2*)Pq, (V2*)Dq);
   return cudaGetLastError();
 }
 
-cudaError_t launch_clover_rot_f32(const GeoH& h, const void* U, const void* Ui, const void* Dq,
+cudaError_t launch_clover_rot_f32(const GeoH& h, const void* U, const void* Dq,
                                  void* F, double sre, double sim, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  k_clover_rot<float><<<grid(g.V, 6, block_of(h, TUNE_CLOVER)), block_of(h, TUNE_CLOVER), 0, st>>>(g, (const V2*)U, (const V2*)Ui, (const V2*)Dq,
+  k_clover_rot<float><<<grid(g.V, 6, block_of(h, TUNE_CLOVER)), block_of(h, TUNE_CLOVER), 0, st>>>(g, (const V2*)U, (const V2*)Dq,
                                                   (V2*)F, sre, sim);
   return cudaGetLastError();
 }
 
-cudaError_t launch_plaq_force_f32(bool theta, const GeoH& h, const void* U, const void* Ui,
-                                 const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
+cudaError_t launch_plaq_force_f32(bool theta, const GeoH& h, const void* U,
+                                 const void* Pq, const void* Dq, const void* F, void* C,
                                  double beta, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const float b6 = (float)(beta / 6.0);
   if (!theta) {
-    k_plaq_force_wilson<float><<<grid(g.V, 6, block_of(h, TUNE_FORCE)), block_of(h, TUNE_FORCE), 0, st>>>(g, (const V2*)U, (const V2*)Ui, (const V2*)Dq,
+    k_plaq_force_wilson<float><<<grid(g.V, 6, block_of(h, TUNE_FORCE)), block_of(h, TUNE_FORCE), 0, st>>>(g, (const V2*)U, (const V2*)Dq,
                                                          (V2*)C, b6);
     return cudaGetLastError();
   }
-  k_plaq_force_ab<float><<<grid(g.V, 6, block_of(h, TUNE_FORCE)), block_of(h, TUNE_FORCE), 0, st>>>(g, (const V2*)U, (const V2*)Ui, (const V2*)Pq,
+  k_plaq_force_ab<float><<<grid(g.V, 6, block_of(h, TUNE_FORCE)), block_of(h, TUNE_FORCE), 0, st>>>(g, (const V2*)U, (const V2*)Pq,
                                                       (const V2*)Dq, (const V2*)F, (V2*)C, b6);
   return cudaGetLastError();
 }
@@ -52,6 +46,7 @@ cudaError_t launch_update_gather_f32(int mode, const GeoH& h, const void* U, con
                                     double eps, uint64_t seed, StepDev* sd, bool adaptive, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   UpdArgs a;
+  a.cexp = 0;
   a.beta = 0.0;
   a.eps = eps;
   a.sqrt_eps = sqrt(eps);

@@ -1,5 +1,5 @@
-// k_update_fx.cuh -- the CL step of the FP64 form in 64-bit fixed point
-// (fixed.cuh): link copies and inverses, plaquettes, clover field and
+// k_update_fx.cuh -- the CL step of the FP64 and DF64 forms (link type L) in
+// 64-bit fixed point (fixed.cuh): link copies and inverses, plaquettes, clover field and
 // per-plaquette drift, the same quantities and formulas as k_update.cuh.
 //
 // Fields between the kernels (int4 words, SoA as the links): Ux, the links in
@@ -18,6 +18,7 @@
 #pragma once
 #include "fixed.cuh"
 #include "k_update.cuh"
+#include "link_fx.cuh"
 #include "noise_fx.cuh"
 
 namespace clgc {
@@ -27,20 +28,17 @@ __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
 
 // ------------------------------------------------------ links and inverses
-__device__ __forceinline__ void fx_links_body(Geo g, const double2* __restrict__ U, int4* __restrict__ Ux,
-                                              int4* __restrict__ Ui, int vb) {
+template <typename L>
+__device__ __forceinline__ void fx_links_body(Geo g, const typename vec2_of<L>::type* __restrict__ U,
+                                              int4* __restrict__ Ux, int4* __restrict__ Ui, int vb) {
   const int mu = vb % 4;
   const int s = (vb / 4) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
-  mat<double> u;
-  load(u, U, mu, s, g.V);
   mat<fx> x, xi;
-  unsigned mag = 0;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) x.e[k] = cx<fx>{fx_of_double(u.e[k].re, mag), fx_of_double(u.e[k].im, mag)};
+  const bool in = fx_load_link<L>(x, U, mu, s, g.V);
   fx_chk ck;
   fx_adj(xi, x, ck);
-  if (!fx_mag_ok(mag) || ck.bad()) {  // readers of either turn to U itself
+  if (!in || ck.bad()) {  // readers of either turn to U itself
     x.e[0].re.l = fx_raw_mark();
     xi.e[0].re.l = fx_raw_mark();
   }
@@ -54,10 +52,12 @@ __device__ __forceinline__ fx fx_half_diff(fx a, fx b) {
   const int d = (a.h >> 1) - (b.h >> 1), odd = (a.h & 1) - (b.h & 1);  // a.h - b.h = 2 d + odd
   return fx{fmaf(0.5f, a.l - b.l, (float)odd * 0x1p29f), d};
 }
-static __device__ __noinline__ void general_plaq(Geo g, const double2* U, tagged Pq, tagged Dq, int vb) {
-  k_plaq_body<double>(g, U, no_inverse(), Pq, Dq, vb);
+template <typename L>
+static __device__ __noinline__ void general_plaq(Geo g, const typename vec2_of<L>::type* U, tagged Pq, tagged Dq, int vb) {
+  k_plaq_body<double>(g, link_field<L>{U}, Pq, Dq, vb);
 }
-__device__ __forceinline__ void fx_plaq_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+template <typename L>
+__device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                              const int4* __restrict__ Ui, int4* Pq, int4* Dq, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
@@ -78,16 +78,18 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const double2* U, const int4
 #pragma unroll
   for (int k = 0; k < 9; ++k) P.e[k] = cx<fx>{fx_half_diff(P.e[k].re, b.e[k].re), fx_half_diff(P.e[k].im, b.e[k].im)};
   store<fx>(Dq, p, s, g.V, P);
-  if (ck.bad()) general_plaq(g, U, tag(Pq), tag_D(Dq), vb);
+  if (ck.bad()) general_plaq<L>(g, U, tag(Pq), tag_D(Dq), vb);
 }
 
 // ------------------------------------------------------------ clover field
-static __device__ __noinline__ void general_clover(Geo g, const double2* U, tagged Dq, tagged F, double sre, double sim,
+template <typename L>
+static __device__ __noinline__ void general_clover(Geo g, const typename vec2_of<L>::type* U, tagged Dq, tagged F, double sre, double sim,
                                                    int vb) {
-  k_clover_rot_body<double>(g, U, no_inverse(), Dq, F, sre, sim, vb);
+  k_clover_rot_body<double>(g, link_field<L>{U}, Dq, F, sre, sim, vb);
 }
 // sre, sim: the scale of plane p's F, |sre|, |sim| <= 1/32
-__device__ __forceinline__ void fx_clover_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+template <typename L>
+__device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                const int4* __restrict__ Ui, const int4* __restrict__ Dq, int4* F,
                                                double sre, double sim, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
@@ -131,14 +133,16 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const double2* U, const in
     acc.e[k] = cx<fx>{fx_get<FX_NARROW>(re, ck), fx_get<FX_NARROW>(im, ck)};
   }
   store<fx>(F, p, s, g.V, acc);
-  if (ck.bad() || !fx_mag_ok(mag)) general_clover(g, U, tag_D(Dq), tag(F), sre, sim, vb);
+  if (ck.bad() || !fx_mag_ok(mag)) general_clover<L>(g, U, tag_D(Dq), tag(F), sre, sim, vb);
 }
 
 // ------------------------------------------------------- plaquette drift
-static __device__ __noinline__ void general_force_wilson(Geo g, const double2* U, tagged Dq, tagged C, double b6, int vb) {
-  k_plaq_force_wilson_body<double>(g, U, no_inverse(), Dq, C, b6, vb);
+template <typename L>
+static __device__ __noinline__ void general_force_wilson(Geo g, const typename vec2_of<L>::type* U, tagged Dq, tagged C, double b6, int vb) {
+  k_plaq_force_wilson_body<double>(g, link_field<L>{U}, Dq, C, b6, vb);
 }
-__device__ __forceinline__ void fx_force_wilson_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+template <typename L>
+__device__ __forceinline__ void fx_force_wilson_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                      const int4* __restrict__ Ui, const int4* __restrict__ Dq, int4* C,
                                                      double b6, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
@@ -166,7 +170,7 @@ __device__ __forceinline__ void fx_force_wilson_body(Geo g, const double2* U, co
   fx_load(a, Ux, mu, s, g.V, ck);
   fx_mul_left<FX_WIDE>(t, a, ck);
   store<fx>(C, 4 * p + 2, s, g.V, t);
-  if (ck.bad() || !fx_mag_ok(mag)) general_force_wilson(g, U, tag_D(Dq), tag(C), b6, vb);
+  if (ck.bad() || !fx_mag_ok(mag)) general_force_wilson<L>(g, U, tag_D(Dq), tag(C), b6, vb);
 }
 
 // Stage a of the theta force: corners c0 .. c2.  The sum of the dual fields
@@ -218,12 +222,14 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
   store<fx>(Gq, GQ_PLANE * p, s, g.V, M);
 }
 
-static __device__ __noinline__ void general_force(Geo g, const double2* U, tagged Pq, tagged Dq, tagged F, tagged C,
+template <typename L>
+static __device__ __noinline__ void general_force(Geo g, const typename vec2_of<L>::type* U, tagged Pq, tagged Dq, tagged F, tagged C,
                                                   double b6, int vb) {
-  k_plaq_force_ab_body<double>(g, U, no_inverse(), Pq, Dq, F, C, b6, vb);
+  k_plaq_force_ab_body<double>(g, link_field<L>{U}, Pq, Dq, F, C, b6, vb);
 }
 // Stage b: corner c3, K and the four slots.
-__device__ __forceinline__ void fx_force_b_body(Geo g, const double2* U, const int4* __restrict__ Ux,
+template <typename L>
+__device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                 const int4* __restrict__ Ui, const int4* Pq, const int4* Dq,
                                                 const int4* F, const int4* Gq, int4* C, double b6, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
@@ -284,7 +290,7 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const double2* U, const i
   fx_mul_left<FX_WIDE>(A, M, ck);
   store<fx>(C, 4 * p + 2, s, g.V, A);
   // anything out of range: the whole plaquette again (its slots are its own)
-  if (ck.bad() || !fx_mag_ok(mag)) general_force(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb);
+  if (ck.bad() || !fx_mag_ok(mag)) general_force<L>(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb);
 }
 
 // --------------------------------------------------------------- gather
@@ -331,16 +337,15 @@ __device__ __forceinline__ bool fx_gather(long long* X, const Geo& g, int s, con
   return !ck.bad() && m < (10u << 28);
 }
 __device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, const int* x, int MU,
-                                           const double2* C, int cexp) {
-  const int4* c = reinterpret_cast<const int4*>(C);
+                                           const int4* C, int cexp) {
   long long v[18];
-  if (fx_gather(v, g, s, x, MU, c)) {
+  if (fx_gather(v, g, s, x, MU, C)) {
 #pragma unroll
     for (int k = 0; k < 9; ++k)
       X.e[k] = cx<double>{fx_bits_to_double(v[2 * k], cexp), fx_bits_to_double(v[2 * k + 1], cexp)};
   } else {
     mat<double> Xg;  // a local of its own: its address goes out of line
-    general_gather(Xg, g, s, x, MU, tag(c), ldexp(1.0, cexp));
+    general_gather(Xg, g, s, x, MU, tag(C), ldexp(1.0, cexp));
     X = Xg;
   }
 }
@@ -414,13 +419,11 @@ __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, co
 // The adaptive step's drift pass: the operand of the update (the traceless
 // quarter of X 2^-cexp, or X itself as doubles) into out; returns |K|^2 =
 // 2 |X - Tr X / 3|_F^2.
-__device__ __forceinline__ double drift_f64(const Geo& g, const double2* C, double2* out, int cexp, int s, const int* x,
-                                            int MU, bool write) {
-  const int4* c = reinterpret_cast<const int4*>(C);
-  int4* o = reinterpret_cast<int4*>(out);
+__device__ __forceinline__ double drift_fx(const Geo& g, const int4* C, int4* o, int cexp, int s, const int* x, int MU,
+                                           bool write) {
   long long v[18];
   mat<fx> Q;
-  if (fx_gather(v, g, s, x, MU, c) && fx_traceless_quarter(Q, v)) {
+  if (fx_gather(v, g, s, x, MU, C) && fx_traceless_quarter(Q, v)) {
     fx_acc n = fx_zero();
     float nf = 0.0f;
 #pragma unroll
@@ -444,17 +447,18 @@ __device__ __forceinline__ double drift_f64(const Geo& g, const double2* C, doub
 // the links pass left in `out`, times det^{-1/3} = 1 - e/3 for |e = det - 1| <
 // 2^-31 (the drift of the determinant over a step is 1e-15; the next term is
 // below 2^-62).  What does not fit goes through general_update_f64.
-__device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const double2* C, const double2* X,
-                                           double2* out, const UpdArgs& a, int s, const int* x, int MU) {
+template <typename L>
+__device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L>::type* U, const int4* C, const int4* X,
+                                          typename vec2_of<L>::type* out, const UpdArgs& a, int s, const int* x, int MU) {
   const uint32_t step = a.sd->step;
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
-  const tagged Xt = {reinterpret_cast<int4*>(const_cast<double2*>(X)), ldexp(1.0, a.cexp + 2)};
+  const tagged Xt = {const_cast<int4*>(X), ldexp(1.0, a.cexp + 2)};
   mat<fx> A;
   bool ok;
   if (C) {
     long long v[18];
-    ok = fx_gather(v, g, s, x, MU, reinterpret_cast<const int4*>(C)) && fx_traceless_quarter(A, v);
+    ok = fx_gather(v, g, s, x, MU, C) && fx_traceless_quarter(A, v);
   } else {
     fx_chk ck;
     fx_load(A, Xt.p, MU, s, g.V, ck);
@@ -476,13 +480,13 @@ __device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const
       const cx<fx> e = fx_det_minus_one(A, ck);
       if (!ck.bad() && e.re.h == 0 && e.im.h == 0) {
         const float er = e.re.l * (-1.0f / 3.0f), ei = e.im.l * (-1.0f / 3.0f);  // units of 2^-60
-        double2* p = out + (size_t)MU * 9 * g.V + s;
+        typename vec2_of<L>::type* p = out + (size_t)MU * 9 * g.V + s;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
           const float ur = (float)A.e[k].re.h * 0x1p-30f, ui = (float)A.e[k].im.h * 0x1p-30f;
           const fx re = {A.e[k].re.l + fmaf(er, ur, -ei * ui), A.e[k].re.h};
           const fx im = {A.e[k].im.l + fmaf(er, ui, ei * ur), A.e[k].im.h};
-          p[(size_t)k * g.V] = make_double2(fx_to_double(re), fx_to_double(im));
+          p[(size_t)k * g.V] = fx_link_word(out, cx<fx>{re, im});
         }
         return;
       }
@@ -493,9 +497,32 @@ __device__ __forceinline__ void update_f64(const Geo& g, const double2* U, const
     gather_f64(Xg, g, s, x, MU, C, a.cexp);
   else
     load(Xg, Xt, MU, s, g.V);
-  load(u, U, MU, s, g.V);
+  load_link_d<L>(u, U, MU, s, g.V);
   general_update_f64(r, Xg, u, a.seed, step, s, MU, eps, sqrt_eps);
-  store(out, MU, s, g.V, r);
+  store_link(out, MU, s, g.V, r);
+}
+
+// The modes of k_update_gather_body (k_update.cuh).  C and (DRIFTMAX's out,
+// UPDATE_X's C) the drift are fixed-point fields.
+template <typename L, int MODE>
+__device__ __forceinline__ void fx_update_body(Geo g, const typename vec2_of<L>::type* __restrict__ U,
+                                               const int4* __restrict__ C, void* __restrict__ out, UpdArgs a, int vb) {
+  typedef typename vec2_of<L>::type V2;
+  const int MU = vb % 4;
+  const int s_raw = (vb / 4) * blockDim.x + threadIdx.x;
+  if (MODE != MODE_DRIFTMAX && s_raw >= g.V) return;
+  const int s = s_raw < g.V ? s_raw : g.V - 1;
+  int x[4];
+  site_coords(g, s, x);
+  if (MODE == MODE_DRIFT) {
+    mat<double> X;
+    gather_f64(X, g, s, x, MU, C, a.cexp);
+    store_link((V2*)out, MU, s, g.V, X);
+  } else if (MODE == MODE_DRIFTMAX) {
+    kmax_update(a.sd, drift_fx(g, C, (int4*)out, a.cexp, s, x, MU, s_raw < g.V));
+  } else {
+    update_fx<L>(g, U, MODE == MODE_UPDATE ? C : nullptr, MODE == MODE_UPDATE ? nullptr : C, (V2*)out, a, s, x, MU);
+  }
 }
 
 }  // namespace clgc

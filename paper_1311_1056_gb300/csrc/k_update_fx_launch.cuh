@@ -1,0 +1,147 @@
+// k_update_fx_launch.cuh -- kernels and launches of the CL step in fixed point
+// (k_update_fx.cuh) for one link type, instantiated by k_update_f64.cu and
+// k_update_df64.cu.
+#pragma once
+#include <cmath>
+
+#include "k_update_fx.cuh"
+#include "launch.h"
+
+namespace clgc {
+
+// The step's launches for links of type L (k_update_fx_launch.cuh).
+template <typename L>
+struct StepFx {
+  static cudaError_t links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st);
+  static cudaError_t plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq, cudaStream_t st);
+  static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* F, double sre, double sim, cudaStream_t st);
+  static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6, cudaStream_t st);
+  static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, uint64_t seed, StepDev* sd, bool adaptive, int cexp, cudaStream_t st);
+};
+
+namespace {
+// 1-D grid, plane (or direction) fastest: the blocks resident at one time
+// cover every plane of a range of sites, so shared neighbours stay in cache.
+inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 1) / bs) * planes)); }
+
+// Registers of the plaquette, clover and force kernels: three blocks of 128
+// threads per SM.  Per 32^4 step at caps of 144 / 168 / 208: clover and
+// plaquettes 3.33 / 3.00 / 3.37 ms, force 7.37 / 6.49 / 6.98 ms (two blocks at
+// 208; 144 spills more, 420 bytes a thread at 168).  FP64 arithmetic took 11.95
+// and 26.0 ms.
+const int FX_MAXNREG = 168;
+template <typename L>
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui) {
+  fx_links_body<L>(g, U, Ux, Ui, blockIdx.x);
+}
+template <typename L>
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_plaq(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+                                                            const int4* __restrict__ Ui, int4* Pq, int4* Dq) {
+  fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, blockIdx.x);
+}
+template <typename L>
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+                                                              const int4* __restrict__ Ui,
+                                                              const int4* __restrict__ Dq, int4* F, double sre,
+                                                              double sim) {
+  fx_clover_body<L>(g, U, Ux, Ui, Dq, F, sre, sim, blockIdx.x);
+}
+template <typename L>
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
+                                                                    const int4* __restrict__ Ux,
+                                                                    const int4* __restrict__ Ui,
+                                                                    const int4* __restrict__ Dq, int4* C, double b6) {
+  fx_force_wilson_body<L>(g, U, Ux, Ui, Dq, C, b6, blockIdx.x);
+}
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
+                                                               const int4* __restrict__ Ui,
+                                                               const int4* __restrict__ Dq,
+                                                               const int4* __restrict__ F, int4* Gq, int4* C,
+                                                               double b6) {
+  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, blockIdx.x);
+}
+template <typename L>
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+                                                               const int4* __restrict__ Ui, const int4* Pq,
+                                                               const int4* Dq, const int4* F, const int4* Gq, int4* C,
+                                                               double b6) {
+  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, blockIdx.x);
+}
+template <typename L, int MODE>
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
+                                                              const int4* __restrict__ C, void* __restrict__ out, UpdArgs a) {
+  fx_update_body<L, MODE>(g, U, C, out, a, blockIdx.x);
+}
+}  // namespace
+
+template <typename L>
+cudaError_t StepFx<L>::links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st) {
+  Geo g = make_geo(h.L, h.V);
+  const int bs = block_of(h, TUNE_CLOVER);
+  k_fx_links<L><<<grid(g.V, 4, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (int4*)Ux, (int4*)Ui);
+  return cudaGetLastError();
+}
+
+template <typename L>
+cudaError_t StepFx<L>::plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
+                            cudaStream_t st) {
+  Geo g = make_geo(h.L, h.V);
+  const int bs = block_of(h, TUNE_CLOVER);
+  k_fx_plaq<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (int4*)Pq, (int4*)Dq);
+  return cudaGetLastError();
+}
+
+template <typename L>
+cudaError_t StepFx<L>::clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
+                                  void* F, double sre, double sim, cudaStream_t st) {
+  Geo g = make_geo(h.L, h.V);
+  const int bs = block_of(h, TUNE_CLOVER);
+  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq,
+                                               (int4*)F, sre, sim);
+  return cudaGetLastError();
+}
+
+template <typename L>
+cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui,
+                                  const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
+                                  cudaStream_t st) {
+  Geo g = make_geo(h.L, h.V);
+  const int bs = block_of(h, TUNE_FORCE);
+  const dim3 gr = grid(g.V, 6, bs);
+  if (!theta) {
+    k_fx_force_wilson<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)C, b6);
+    return cudaGetLastError();
+  }
+  k_fx_force_a<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)F, (int4*)Gq,
+                                  (int4*)C, b6);
+  k_fx_force_b<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Pq, (const int4*)Dq,
+                                  (const int4*)F, (const int4*)Gq, (int4*)C, b6);
+  return cudaGetLastError();
+}
+
+template <typename L>
+cudaError_t StepFx<L>::update(int mode, const GeoH& h, const void* U, const void* C, void* out,
+                                    double eps, uint64_t seed, StepDev* sd, bool adaptive, int cexp, cudaStream_t st) {
+  Geo g = make_geo(h.L, h.V);
+  UpdArgs a;
+  a.cexp = cexp;
+  a.beta = 0.0;
+  a.eps = eps;
+  a.sqrt_eps = sqrt(eps);
+  a.seed = seed;
+  a.sd = sd;
+  a.adaptive = adaptive ? 1 : 0;
+  const int bs = block_of(h, TUNE_UPDATE);
+  const dim3 gr = grid(g.V, 4, bs);
+  const typename vec2_of<L>::type* u = (const typename vec2_of<L>::type*)U;
+  const int4* c = (const int4*)C;
+  switch (mode) {
+    case MODE_DRIFT: k_fx_update<L, MODE_DRIFT><<<gr, bs, 0, st>>>(g, u, c, out, a); break;
+    case MODE_DRIFTMAX: k_fx_update<L, MODE_DRIFTMAX><<<gr, bs, 0, st>>>(g, u, c, out, a); break;
+    case MODE_UPDATE_X: k_fx_update<L, MODE_UPDATE_X><<<gr, bs, 0, st>>>(g, u, c, out, a); break;
+    default: k_fx_update<L, MODE_UPDATE><<<gr, bs, 0, st>>>(g, u, c, out, a); break;
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace clgc

@@ -165,19 +165,14 @@ __global__ void k_noise_sample(int site0, int n, uint64_t seed, uint32_t step, u
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t s = (uint32_t)(site0 + i);
-  if constexpr (std::is_same<T, double>::value) {
+  if constexpr (is_fx<T>()) {
     fx e[8];
     normals_fx<4>(e, seed, step, s, mu, STREAM_CL);
 #pragma unroll
     for (int j = 0; j < 8; ++j) out[8 * (size_t)i + j] = fx_to_double(e[j], 3);
-  } else if constexpr (std::is_same<T, float>::value) {
+  } else {
     float e[8];
     normals_f32<4>(e, seed, step, s, mu, STREAM_CL);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) out[8 * (size_t)i + j] = (double)e[j];
-  } else {
-    df64 e[8];
-    normals_df64<4>(e, seed, step, s, mu, STREAM_CL);
 #pragma unroll
     for (int j = 0; j < 8; ++j) out[8 * (size_t)i + j] = (double)e[j];
   }
@@ -322,15 +317,13 @@ __device__ __forceinline__ bool obs_link(const mat<fx>& u, long long& dev, doubl
 template <typename T>
 static __device__ __noinline__ double general_obs_link(const typename vec2_of<T>::type* U, int mu, int s, int V, double* det2,
                                                        double* bad) {
-  mat<T> u;
-  load(u, U, mu, s, V);
+  mat<double> u;
+  load_link_d<T>(u, U, mu, s, V);
   if (!finite_mat(u)) *bad = 1.0;
-  mat<double> ud;
-  convert(ud, u);
-  const cx<double> d = det(ud);
+  const cx<double> d = det(u);
   const double h = hypot(d.re - 1.0, d.im);
   *det2 = fmax(*det2, h * h);
-  return (double)norm2(u);
+  return norm2(u);
 }
 // Tr of a stored matrix times 1/4 as a 60-bit integer (FP32 storage: of its float trace).
 __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const float2* f, int p, int s, int V) {
@@ -346,8 +339,7 @@ __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const fl
   im = fx_bits(fx_of_float(0.25f * ti));
   return true;
 }
-__device__ __forceinline__ bool obs_trace(long long& re, long long& im, const double2* f, int p, int s, int V) {
-  const int4* P = reinterpret_cast<const int4*>(f);
+__device__ __forceinline__ bool obs_trace(long long& re, long long& im, const int4* P, int p, int s, int V) {
   bool ok = true;
   re = im = 0;
 #pragma unroll
@@ -359,42 +351,41 @@ __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const do
   }
   return ok;
 }
-template <typename T>
-static __device__ __noinline__ void general_obs_trace(const typename vec2_of<T>::type* f, int p, int s, int V, double sc,
-                                                      double* out) {
-  mat<T> m;
-  if constexpr (std::is_same<T, double>::value)
-    load(m, tagged{(int4*)f, sc}, p, s, V);
-  else
-    load(m, f, p, s, V);
-  const cx<T> t = trace(m);
+static __device__ __noinline__ void general_obs_trace(const int4* f, int p, int s, int V, double sc, double* out) {
+  mat<double> m;
+  load(m, tagged{const_cast<int4*>(f), sc}, p, s, V);
+  const cx<double> t = trace(m);
+  out[0] = t.re;
+  out[1] = t.im;
+}
+static __device__ __noinline__ void general_obs_trace(const float2* f, int p, int s, int V, double, double* out) {
+  mat<float> m;
+  load(m, f, p, s, V);
+  const cx<float> t = trace(m);
   out[0] = (double)t.re;
   out[1] = (double)t.im;
 }
 // Tr F_p F_{5-p} in FP64.
-template <typename T>
-static __device__ __noinline__ void general_obs_ff(const typename vec2_of<T>::type* F, int p, int s, int V, double* out) {
-  mat<T> F1, F2;
-  if constexpr (std::is_same<T, double>::value) {
-    load(F1, tagged{(int4*)F, 1.0}, p, s, V);
-    load(F2, tagged{(int4*)F, 1.0}, 5 - p, s, V);
-  } else {
-    load(F1, F, p, s, V);
-    load(F2, F, 5 - p, s, V);
-  }
-  const cx<T> t = trace_mul(F1, F2);
-  out[0] = (double)t.re;
-  out[1] = (double)t.im;
+static __device__ __noinline__ void general_obs_ff(const int4* F, int p, int s, int V, double* out) {
+  mat<double> F1, F2;
+  load(F1, tagged{const_cast<int4*>(F), 1.0}, p, s, V);
+  load(F2, tagged{const_cast<int4*>(F), 1.0}, 5 - p, s, V);
+  const cx<double> t = trace_mul(F1, F2);
+  out[0] = t.re;
+  out[1] = t.im;
 }
 
+// The type of the plaquette and clover fields' words.
+template <typename T>
+struct obs_word { typedef typename std::conditional<is_fx<T>(), int4, float2>::type type; };
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_of<T>::type* __restrict__ U,
                                                     const int4* __restrict__ Ux,
-                                                    const typename vec2_of<T>::type* __restrict__ Pq,
-                                                    const typename vec2_of<T>::type* __restrict__ Dq,
-                                                    const typename vec2_of<T>::type* __restrict__ F,
+                                                    const typename obs_word<T>::type* __restrict__ Pq,
+                                                    const typename obs_word<T>::type* __restrict__ Dq,
+                                                    const typename obs_word<T>::type* __restrict__ F,
                                                     double* partials, double* q_site) {
-  constexpr bool FX = std::is_same<T, double>::value;
+  constexpr bool FX = is_fx<T>();
   double v[NQ_OBS];
 #pragma unroll
   for (int q = 0; q < NQ_OBS; ++q) v[q] = 0.0;
@@ -437,10 +428,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
         di += d;
       } else {
         double t[2];
-        general_obs_trace<T>(Pq, p, s, g.V, 1.0, t);
+        general_obs_trace(Pq, p, s, g.V, 1.0, t);
         wp[0] += t[0];
         wp[1] += t[1];
-        general_obs_trace<T>(Dq, p, s, g.V, 2.0, t);
+        general_obs_trace(Dq, p, s, g.V, 2.0, t);
         wp[2] += t[0];
         wp[3] += t[1];
       }
@@ -458,8 +449,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
 #pragma unroll 1
       for (int p = 0; p < 3; ++p) {  // the planes 1 and 4 are both stored negated
         mat<fx> F1, F2;
-        fx_load(F1, (const int4*)F, p, s, g.V, ck);
-        fx_load(F2, (const int4*)F, 5 - p, s, g.V, ck);
+        fx_load(F1, F, p, s, g.V, ck);
+        fx_load(F2, F, 5 - p, s, g.V, ck);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -472,7 +463,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
       } else {
         for (int p = 0; p < 3; ++p) {
           double t[2];
-          general_obs_ff<T>(F, p, s, g.V, t);
+          general_obs_ff(F, p, s, g.V, t);
           q.re += p == 1 ? -t[0] : t[0];
           q.im += p == 1 ? -t[1] : t[1];
         }
@@ -498,75 +489,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
       q_site[2 * (size_t)s] = q.re;
       q_site[2 * (size_t)s + 1] = q.im;
     }
-  }
-  block_reduce_store<NQ_OBS, 7>(v, partials + (size_t)blockIdx.x * NQ_OBS);
-}
-
-// DF64 form: the plaquettes formed here.
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_obs_direct(Geo g, const typename vec2_of<T>::type* __restrict__ U,
-                                                    const typename vec2_of<T>::type* __restrict__ F,
-                                                    int with_q, double* partials, double* q_site) {
-  double v[NQ_OBS];
-#pragma unroll
-  for (int q = 0; q < NQ_OBS; ++q) v[q] = 0.0;
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
-    int x[4];
-    site_coords(g, s, x);
-    bool ok = true;
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      mat<T> u;
-      load(u, U, mu, s, g.V);
-      ok = ok && finite_mat(u);
-      v[4] += (double)norm2(u) * (1.0 / 3.0);
-      mat<double> ud;
-      convert(ud, u);
-      cx<double> d = det(ud);
-      const double h = hypot(d.re - 1.0, d.im);
-      v[7] = fmax(v[7], h * h);
-    }
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      const int mu = plane_mu(p), nu = plane_nu(p);
-      mat<T> a, b, A, B, Ai, Bi;
-      load(a, U, mu, s, g.V);
-      load(b, U, nu, hop(g, s, x, mu, 1), g.V);
-      mul(A, a, b);
-      load(a, U, nu, s, g.V);
-      load(b, U, mu, hop(g, s, x, nu, 1), g.V);
-      mul(B, a, b);
-      adj(Bi, B);
-      adj(Ai, A);
-      cx<T> tp = trace_mul(A, Bi);   // Tr P
-      cx<T> tpi = trace_mul(B, Ai);  // Tr P^{-1}
-      v[0] += (double)tp.re * (1.0 / 3.0);
-      v[1] += (double)tp.im * (1.0 / 3.0);
-      v[2] += (double)tp.re + (double)tpi.re;
-      v[3] += (double)tp.im + (double)tpi.im;
-    }
-    if (with_q) {
-      mat<T> F1, F2;
-      cx<double> q = {0.0, 0.0};
-#pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        load(F1, F, p, s, g.V);
-        load(F2, F, 5 - p, s, g.V);
-        cx<T> t = trace_mul(F1, F2);
-        double sg = (p == 1) ? -1.0 : 1.0;
-        q.re += sg * (double)t.re;
-        q.im += sg * (double)t.im;
-      }
-      q.re *= KAPPA_Q;
-      q.im *= KAPPA_Q;
-      v[5] += q.re;
-      v[6] += q.im;
-      if (q_site) {
-        q_site[2 * (size_t)s] = q.re;
-        q_site[2 * (size_t)s + 1] = q.im;
-      }
-    }
-    v[8] += ok ? 0.0 : 1.0;
   }
   block_reduce_store<NQ_OBS, 7>(v, partials + (size_t)blockIdx.x * NQ_OBS);
 }
@@ -910,12 +832,9 @@ cudaError_t launch_obs(int prec, const GeoH& h, const void* U, const void* Ux, c
   Geo g = to_geo(h);
   return by_prec(prec, [&](auto t) {
     using T = decltype(t);
-    typedef typename vec2_of<T>::type V2;
-    if constexpr (std::is_same<T, df64>::value)
-      k_obs_direct<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const V2*)U, (const V2*)F, 1, partials, q_site);
-    else
-      k_obs<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const V2*)U, (const int4*)Ux, (const V2*)Pq,
-                                                          (const V2*)Dq, (const V2*)F, partials, q_site);
+    typedef typename obs_word<T>::type W;
+    k_obs<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const typename vec2_of<T>::type*)U, (const int4*)Ux,
+                                                        (const W*)Pq, (const W*)Dq, (const W*)F, partials, q_site);
   });
 }
 

@@ -111,22 +111,19 @@ cudaError_t launch_aos_to_soa(int prec, const GeoH& g, const double* aos, void* 
                               cudaStream_t st);
 cudaError_t launch_soa_to_aos(int prec, const GeoH& g, const void* U, double* aos, int nplanes,
                               cudaStream_t st);
-// The FP64 form runs the step's link algebra in 64-bit fixed point
+// The FP64 and DF64 forms run the step's link algebra in 64-bit fixed point
 // (k_update_fx.cuh): Ux receives the links in fixed point (the update's target
 // buffer, free until then), the clover scale and the contributions C carry the
-// factor 2^-cexp, cexp = drift_exponent(beta, scale_re, scale_im).  The other
-// forms ignore Ux and take cexp = 0.
+// factor 2^-cexp, cexp = drift_exponent(beta, scale_re, scale_im).  FP32
+// storage ignores Ux and Ui and takes cexp = 0.
 int drift_exponent(double beta, double sre, double sim);
 // Scale of the clover field that launch_obs expects (fixed point: entries below one).
-inline double obs_clover_scale(int prec) { return prec == 0 ? 0.03125 : 1.0; }
+inline double obs_clover_scale(int prec) { return prec != 1 ? 0.03125 : 1.0; }
 // The CL step (k_update.cuh): link inverses Ui; plaquettes P and D = P - P^{-1}
 // (six planes); the clover field F^ = scale * F_{mu nu}(x) built from the D's;
 // the per-plaquette drift contributions C (24 planes: 4 links x 6 planes);
 // then per link the gather of its six contributions followed by the update
 // (mode 0) or by storing the drift matrix X_S (mode 1).
-// Lets the double-float link-algebra kernels take their shared-memory matrix
-// workspace (up to 5 x 144 B per thread); called before the first DF64 launch.
-cudaError_t prepare_df64_kernels();
 cudaError_t launch_noise_sample(int prec, int site0, int n, uint64_t seed, uint32_t step, int mu, double* out,
                                 cudaStream_t st);
 cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ux, void* Ui, cudaStream_t st);

@@ -173,3 +173,34 @@ def test_reprojection_of_links_off_determinant_one(cl):
         lat.set_links(U)
         lat.step(1e-3)
         assert np.abs(lat.links() - ref).max() <= 1e-12
+
+
+@pytest.mark.parametrize("spread", [0, 0.1, 0.4, "mixed"])
+@pytest.mark.parametrize("k_ref", [0.0, 3.0])
+def test_df64_form_inside_and_outside_the_range(cl, spread, k_ref):
+    """The same kernels on double-float links: drift, one step, observables.  Links and drift are rounded to 2^-48
+    on their way out, below the FP64 form's bounds above."""
+    L, eps = (4, 3, 2, 5), 1e-3
+    w = field(L, spread, 31).view(np.float64)
+    hi = w.astype(np.float32).astype(np.float64)
+    U = (hi + (w - hi).astype(np.float32)).view(np.complex128)  # exact double-float numbers
+    top = np.abs(U).max()
+    if k_ref:
+        ref, _, _ = O.cl_step_adaptive(L, U, 6.0, 1.0, eps, k_ref, 99, 0)
+    else:
+        ref = O.cl_step(L, U, 6.0, 1.0, eps, 99, 0)
+    Xr, obs_r = O.drift(L, U, 6.0, 1.0), O.observables(L, U, 6.0, 1.0)
+    with cl.Lattice(L, beta=6.0, theta=1.0, seed=99, prec=cl.CL_DF64) as lat:
+        lat.set_links(U)
+        assert np.array_equal(lat.links(), U)
+        X, obs = lat.drift(), lat.observables()
+        lat.set_adaptive_step(k_ref)
+        lat.step(eps)
+        Ug = lat.links()
+    assert np.abs(X - Xr).max() <= 1e-11 * np.abs(Xr).max()
+    scale = max(abs(obs_r["sw_re"]), 6.0 * 6 * I.volume(L))
+    for k in ("plaq_re", "plaq_im", "un"):
+        assert abs(obs[k] - obs_r[k]) <= 1e-12 * max(1.0, abs(obs_r[k])), k
+    for k in ("q_re", "q_im", "sw_re", "sw_im"):
+        assert abs(obs[k] - obs_r[k]) <= 1e-12 * scale, k
+    assert np.abs(Ug - ref).max() <= 1e-12 * np.abs(ref).max() + 1e-11 * eps * top ** 2
