@@ -124,6 +124,8 @@ bool theta_nonzero(const cl_lattice* l) { return l->p.theta_re != 0.0 || l->p.th
 // The link-inverse pass: FP64 and DF64 only (the FP32-storage kernels form
 // each inverse from its link where they use it).
 bool needs_inverse_pass(const cl_lattice* l) { return l->prec != 1; }
+// FP64 and DF64 form the clover field in two kernels.
+int clover_kernels(const cl_lattice* l) { return l->prec != 1 ? 2 : 1; }
 
 // Link inverses, plaquettes and D = P - P^{-1}, then (theta != 0) the clover
 // field scaled by (sre + i sim), then the per-plaquette drift contributions.
@@ -136,13 +138,14 @@ cudaError_t do_force(cl_lattice* l, bool th, double sre, double sim, int ce) {
     e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); });
   if (e == cudaSuccess && th)
     e = timed(l, CL_PHASE_CLOVER, [&] {
-      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->F, ldexp(sre, -ce), ldexp(sim, -ce), l->st);
-    });
+      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, ldexp(sre, -ce), ldexp(sim, -ce),
+                               l->st);
+    }, clover_kernels(l));
   if (e == cudaSuccess)
     e = timed(l, CL_PHASE_FORCE, [&] {
       return launch_plaq_force(l->prec, th, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->F, l->Gq, l->C, l->p.beta,
                                ce, l->st);
-    }, (th && l->prec != 1) ? 2 : 1);  // FP64 and DF64 split the theta force in two kernels
+    }, (th && l->prec != 1) ? 3 : 1);  // FP64 and DF64 split the theta force in three kernels
   return e;
 }
 
@@ -242,7 +245,9 @@ cl_status do_obs(cl_lattice* l, ObsOut* dst, double* q_site) {
   if (needs_inverse_pass(l))
     CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); }));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->F, obs_clover_scale(l->prec), 0.0, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] {
+    return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, obs_clover_scale(l->prec), 0.0, l->st);
+  }, clover_kernels(l)));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->Un, l->Pq, l->Dq, l->F, l->partials, q_site, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
     return launch_obs_final(l->g, l->partials, l->p.beta, l->p.theta_re, l->p.theta_im, dst, l->st);
@@ -972,7 +977,7 @@ cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainD
   int64_t nl = 0;
   auto fam = [&](int f, int list, int arg) -> cudaError_t {
     if (P.fam[list].n == 0) return cudaSuccess;
-    nl += (f == ENS_FORCE_THETA && prec == 0) ? 2 : 1;
+    nl += prec != 0 ? 1 : f == ENS_FORCE_THETA ? 3 : f == ENS_CLOVER ? 2 : 1;
     return launch_ens(prec, f, cd, w + P.fam[list].off, P.fam[list].n, arg, st);
   };
   CK(fam(ENS_INVERSE, ENS_INVERSE, 0));

@@ -48,6 +48,22 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const
     k_plaq_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Pq, (V2*)c.Dq, it.vb);
 }
 
+// FP64: the clover field's first kernel and the theta force's
+template <typename T>
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover_half(const ChainDesc* __restrict__ cd,
+                                                                    const WorkItem* __restrict__ w) {
+  const WorkItem it = w[blockIdx.x];
+  const ChainDesc& c = cd[it.chain];
+  fx_clover_half_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C, it.vb);
+}
+template <typename T>
+__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_t(const ChainDesc* __restrict__ cd,
+                                                                const WorkItem* __restrict__ w) {
+  const WorkItem it = w[blockIdx.x];
+  const ChainDesc& c = cd[it.chain];
+  fx_force_t_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.F, (int4*)c.C, it.vb);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(const ChainDesc* __restrict__ cd,
                                                                const WorkItem* __restrict__ w) {
@@ -55,8 +71,8 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(con
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
-    fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.F,
-                   c.sre, c.sim, it.vb);
+    fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq,
+                      (const int4*)c.C, (int4*)c.F, c.sre, c.sim, it.vb);
   else
     k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }
@@ -75,7 +91,6 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_wils
                               (T)(c.beta / 6.0), it.vb);
 }
 
-// FP64: the theta force's two kernels
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_a(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
@@ -130,8 +145,8 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_update(const ChainDesc* 
     k_update_gather_body<T, MODE>(geo_of(c), (const V2*)c.U, (const V2*)in, (V2*)out, a, it.vb);
 }
 
-// Launch family fam of the CL step for link type T (FP64 runs the theta
-// force as its two kernels).
+// Launch family fam of the CL step for link type T (FP64 runs the clover
+// field and the theta force as two and three kernels).
 template <typename T>
 cudaError_t launch_ens_step_family(int fam, const ChainDesc* cd, const WorkItem* w, int nw, cudaStream_t st) {
   if (nw <= 0) return cudaSuccess;
@@ -141,10 +156,13 @@ cudaError_t launch_ens_step_family(int fam, const ChainDesc* cd, const WorkItem*
       if constexpr (is_fx<T>()) k_ens_inverse<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
       break;
     case ENS_PLAQ: k_ens_plaq<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
-    case ENS_CLOVER: k_ens_clover<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
+    case ENS_CLOVER:
+      if constexpr (is_fx<T>()) k_ens_clover_half<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
+      k_ens_clover<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_FORCE_WILSON: k_ens_force_wilson<T><<<n, ENS_BLOCK, 0, st>>>(cd, w); break;
     case ENS_FORCE_THETA:
       if constexpr (is_fx<T>()) {
+        k_ens_force_t<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
         k_ens_force_a<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
         k_ens_force_b<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
       } else {

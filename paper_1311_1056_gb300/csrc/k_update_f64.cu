@@ -39,10 +39,10 @@ cudaError_t launch_plaq(int prec, const GeoH& h, const void* U, const void* Ux, 
   return prec == 0 ? StepFx<double>::plaq(h, U, Ux, Ui, Pq, Dq, st) : StepFx<df64>::plaq(h, U, Ux, Ui, Pq, Dq, st);
 }
 cudaError_t launch_clover_rot(int prec, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                              void* F, double sre, double sim, cudaStream_t st) {
+                              void* E, void* F, double sre, double sim, cudaStream_t st) {
   if (prec == 1) return launch_clover_rot_f32(h, U, Dq, F, sre, sim, st);
-  return prec == 0 ? StepFx<double>::clover(h, U, Ux, Ui, Dq, F, sre, sim, st)
-                   : StepFx<df64>::clover(h, U, Ux, Ui, Dq, F, sre, sim, st);
+  return prec == 0 ? StepFx<double>::clover(h, U, Ux, Ui, Dq, E, F, sre, sim, st)
+                   : StepFx<df64>::clover(h, U, Ux, Ui, Dq, E, F, sre, sim, st);
 }
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,

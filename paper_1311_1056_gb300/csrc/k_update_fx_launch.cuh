@@ -14,7 +14,8 @@ template <typename L>
 struct StepFx {
   static cudaError_t links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st);
   static cudaError_t plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq, cudaStream_t st);
-  static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* F, double sre, double sim, cudaStream_t st);
+  static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* E,
+                            void* F, double sre, double sim, cudaStream_t st);
   static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6, cudaStream_t st);
   static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, uint64_t seed, StepDev* sd, bool adaptive, int cexp, cudaStream_t st);
 };
@@ -25,10 +26,11 @@ namespace {
 inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 1) / bs) * planes)); }
 
 // Registers of the plaquette, clover and force kernels: three blocks of 128
-// threads per SM.  Per 32^4 step at caps of 144 / 168 / 208: clover and
-// plaquettes 3.33 / 3.00 / 3.37 ms, force 7.37 / 6.49 / 6.98 ms (two blocks at
-// 208; 144 spills more, 420 bytes a thread at 168).  FP64 arithmetic took 11.95
-// and 26.0 ms.
+// threads per SM.  Per 32^4 step at caps of 144 / 168 / 208, before the clover
+// field and the force were split further: clover and plaquettes 3.33 / 3.00 /
+// 3.37 ms, force 7.37 / 6.49 / 6.98 ms (two blocks at 208; 144 spills more, 420
+// bytes a thread at 168).  Now 2.60 and 6.38 ms; FP64 arithmetic took 11.95 and
+// 26.0 ms.
 const int FX_MAXNREG = 168;
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui) {
@@ -39,12 +41,15 @@ __global__ void __maxnreg__(FX_MAXNREG) k_fx_plaq(Geo g, const typename vec2_of<
                                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq) {
   fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, blockIdx.x);
 }
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_clover_half(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
+                                                         const int4* __restrict__ Dq, int4* E) {
+  fx_clover_half_body(g, Ux, Ui, Dq, E, blockIdx.x);
+}
 template <typename L>
 __global__ void __maxnreg__(FX_MAXNREG) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
-                                                              const int4* __restrict__ Ui,
-                                                              const int4* __restrict__ Dq, int4* F, double sre,
-                                                              double sim) {
-  fx_clover_body<L>(g, U, Ux, Ui, Dq, F, sre, sim, blockIdx.x);
+                                                    const int4* __restrict__ Ui, const int4* __restrict__ Dq,
+                                                    const int4* __restrict__ E, int4* F, double sre, double sim) {
+  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sre, sim, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
@@ -52,6 +57,10 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const
                                                                     const int4* __restrict__ Ui,
                                                                     const int4* __restrict__ Dq, int4* C, double b6) {
   fx_force_wilson_body<L>(g, U, Ux, Ui, Dq, C, b6, blockIdx.x);
+}
+__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_t(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
+                                                     const int4* __restrict__ F, int4* C) {
+  fx_force_t_body(g, Ux, Ui, F, C, blockIdx.x);
 }
 __global__ void __maxnreg__(FX_MAXNREG) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui,
@@ -93,10 +102,11 @@ cudaError_t StepFx<L>::plaq(const GeoH& h, const void* U, const void* Ux, const 
 
 template <typename L>
 cudaError_t StepFx<L>::clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                                  void* F, double sre, double sim, cudaStream_t st) {
+                                  void* E, void* F, double sre, double sim, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = block_of(h, TUNE_CLOVER);
-  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq,
+  k_fx_clover_half<<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)E);
+  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E,
                                                (int4*)F, sre, sim);
   return cudaGetLastError();
 }
@@ -112,6 +122,7 @@ cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const voi
     k_fx_force_wilson<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)C, b6);
     return cudaGetLastError();
   }
+  k_fx_force_t<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)F, (int4*)C);
   k_fx_force_a<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)F, (int4*)Gq,
                                   (int4*)C, b6);
   k_fx_force_b<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Pq, (const int4*)Dq,

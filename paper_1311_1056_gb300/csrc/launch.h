@@ -82,7 +82,7 @@ struct WorkItem {
 enum {
   ENS_INVERSE = 0,      // link inverses, 4 directions
   ENS_PLAQ = 1,         // plaquettes, 6 planes
-  ENS_CLOVER = 2,       // clover field (theta != 0 chains)
+  ENS_CLOVER = 2,       // clover field (theta != 0 chains; FP64: two kernels)
   ENS_FORCE_WILSON = 3, // drift contributions, theta = 0 chains
   ENS_FORCE_THETA = 4,  // drift contributions, theta != 0 chains (FP64: two kernels)
   ENS_UPDATE = 5,       // gather + update, fixed step size
@@ -130,9 +130,11 @@ cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ux
 cudaError_t launch_plaq(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
                         cudaStream_t st);
 cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                              void* F, double scale_re, double scale_im, cudaStream_t st);
-// (theta != 0 runs two kernels, parking partial sums of the transported dual
-// fields in Gq, six planes.)
+                              void* E, void* F, double scale_re, double scale_im, cudaStream_t st);
+// The clover field of the fixed-point forms goes through E, six planes of
+// scratch (the first of C).  Their theta force runs three kernels, parking the
+// transported dual fields and partial sums of them in planes of C (Gq points at
+// some of these).
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
                               double beta, int cexp, cudaStream_t st);
