@@ -161,21 +161,16 @@ cl_status do_steps(cl_lattice* l, double eps, int n) {
       // max |K|, then the step size on the device, then the update from the
       // stored drift
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 2, l->g, l->U, l->C, l->Pq, eps, l->p.seed, l->sd, false, ce, l->st);
+        return launch_update_gather(l->prec, 2, l->g, l->U, l->C, l->Pq, eps, l->k_ref, l->p.seed, l->sd, ce, l->st);
       }));
-      CK(timed(l, CL_PHASE_UPDATE, [&] { return launch_step_eps(l->sd, eps, l->k_ref, l->st); }));
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 3, l->g, l->U, l->Pq, l->Un, eps, l->p.seed, l->sd, true, ce, l->st);
+        return launch_update_gather(l->prec, 3, l->g, l->U, l->Pq, l->Un, eps, l->k_ref, l->p.seed, l->sd, ce, l->st);
       }));
     } else {
       CK(timed(l, CL_PHASE_UPDATE, [&] {
-        return launch_update_gather(l->prec, 0, l->g, l->U, l->C, l->Un, eps, l->p.seed, l->sd, false, ce, l->st);
+        return launch_update_gather(l->prec, 0, l->g, l->U, l->C, l->Un, eps, l->k_ref, l->p.seed, l->sd, ce, l->st);
       }));
     }
-    // one-thread bookkeeping kernel: counted as a launch, not timed (so the update
-    // phase's per-launch time stays that of the update kernel)
-    CK(launch_step_bump(l->sd, eps, adaptive, l->st));
-    l->launches++;
     std::swap(l->U, l->Un);
     l->step++;
   }
@@ -638,7 +633,7 @@ cl_status cl_drift(cl_lattice* l, double* host_aos) {
   const bool th = theta_nonzero(l);
   const int ce = contribution_exponent(l);
   CK(do_force(l, th, clover_scale_re(l), clover_scale_im(l), ce));
-  CK(launch_update_gather(l->prec, 1, l->g, l->U, l->C, l->Un, 0.0, l->p.seed, l->sd, false, ce, l->st));
+  CK(launch_update_gather(l->prec, 1, l->g, l->U, l->C, l->Un, 0.0, 0.0, l->p.seed, l->sd, ce, l->st));
   CK(launch_soa_to_aos(l->prec, l->g, l->Un, l->stage, 4, l->st));
   l->launches += 2;
   CK(cudaMemcpyAsync(host_aos, l->stage, sizeof(double) * 18 * 4 * (size_t)l->g.V,
@@ -856,19 +851,15 @@ cl_status check_batch_member(const cl_batch* b, const cl_lattice* l, double eps,
 }
 
 // ---- fused mode
-// Host plan of a fused step: the work lists of every kernel family and the
-// chain lists of the per-chain kernels, offsets into one device allocation.
+// Host plan of a fused step: the work lists of every kernel family.
 struct FusedPlan {
   std::vector<WorkItem> items;
-  std::vector<int> ints;
   struct List {
     size_t off;
     int n;
   };
   List fam[ENS_NFAM + 3];  // + the gradient of the first sweep (all chains), the first Omega (all), spare
-  List all_chains, adaptive_chains, adaptive_flags;
   int n_iter;
-  bool any_adaptive;
 };
 enum { ENS_FIRST_GRAD = ENS_NFAM, ENS_FIRST_OMEGA = ENS_NFAM + 1 };
 
@@ -911,17 +902,6 @@ FusedPlan plan_fused(const cl_batch* b) {
   add(ENS_COOL_APPLY, four, cb(ENS_COOL_APPLY));
   add(ENS_COOL_GRAD_OMEGA, sp, cb(ENS_COOL_GRAD_OMEGA));
   add(ENS_COOL_APPLY_UN, sp, cb(ENS_COOL_APPLY_UN));
-  P.all_chains.off = P.ints.size();
-  for (int i = 0; i < n; ++i) P.ints.push_back(i);
-  P.all_chains.n = n;
-  P.adaptive_chains.off = P.ints.size();
-  for (int i = 0; i < n; ++i)
-    if (ad(i)) P.ints.push_back(i);
-  P.adaptive_chains.n = (int)(P.ints.size() - P.adaptive_chains.off);
-  P.adaptive_flags.off = P.ints.size();
-  for (int i = 0; i < n; ++i) P.ints.push_back(ad(i) ? 1 : 0);
-  P.adaptive_flags.n = n;
-  P.any_adaptive = P.adaptive_chains.n > 0;
   P.n_iter = 0;
   if (b->with_cooling)
     for (const cl_cool_params& cp : b->cps) P.n_iter = std::max(P.n_iter, cp.forced_sweeps >= 0 ? cp.forced_sweeps : cp.n_max);
@@ -972,7 +952,7 @@ ChainDesc describe(const cl_lattice* l, double eps, const cl_cool_params& cp, bo
 // sweep count of the batch (a chain's own rule marks it done at its count;
 // later launches skip its blocks).  Returns the number of launches.
 cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainDesc* cd, const WorkItem* w,
-                             const int* ints, cudaStream_t st, int64_t* launches) {
+                             cudaStream_t st, int64_t* launches) {
   const int prec = b->lats[0]->prec;
   int64_t nl = 0;
   auto fam = [&](int f, int list, int arg) -> cudaError_t {
@@ -985,15 +965,9 @@ cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainD
   CK(fam(ENS_CLOVER, ENS_CLOVER, 0));
   CK(fam(ENS_FORCE_WILSON, ENS_FORCE_WILSON, 0));
   CK(fam(ENS_FORCE_THETA, ENS_FORCE_THETA, 0));
-  if (P.any_adaptive) {
-    CK(fam(ENS_DRIFTMAX, ENS_DRIFTMAX, 0));
-    CK(launch_ens_step_eps(cd, ints + P.adaptive_chains.off, P.adaptive_chains.n, st));
-    ++nl;
-    CK(fam(ENS_UPDATE_X, ENS_UPDATE_X, 0));
-  }
+  CK(fam(ENS_DRIFTMAX, ENS_DRIFTMAX, 0));
+  CK(fam(ENS_UPDATE_X, ENS_UPDATE_X, 0));
   CK(fam(ENS_UPDATE, ENS_UPDATE, 0));
-  CK(launch_ens_step_bump(cd, ints + P.all_chains.off, ints + P.adaptive_flags.off, P.all_chains.n, st));
-  ++nl;
   if (b->with_cooling) {
     CK(fam(ENS_COOL_GRAD, ENS_FIRST_GRAD, 1));
     for (int k = 0; k < P.n_iter; ++k) {
@@ -1029,16 +1003,13 @@ cl_status capture_batch_fused(cl_batch* b) {
   std::vector<ChainDesc> cd(2 * (size_t)n);
   for (int v = 0; v < 2; ++v)
     for (int i = 0; i < n; ++i) cd[(size_t)v * n + i] = describe(b->lats[i], b->eps[i], b->cps[i], v == 1);
-  const size_t cd_bytes = sizeof(ChainDesc) * cd.size(), w_bytes = sizeof(WorkItem) * P.items.size(),
-               i_bytes = sizeof(int) * P.ints.size();
-  const size_t w_off = (cd_bytes + 255) / 256 * 256, i_off = w_off + (w_bytes + 255) / 256 * 256;
-  CK(cudaMalloc(&b->dmem, i_off + i_bytes + 16));
+  const size_t cd_bytes = sizeof(ChainDesc) * cd.size(), w_bytes = sizeof(WorkItem) * P.items.size();
+  const size_t w_off = (cd_bytes + 255) / 256 * 256;
+  CK(cudaMalloc(&b->dmem, w_off + w_bytes + 16));
   char* base = (char*)b->dmem;
   CK(cudaMemcpy(base, cd.data(), cd_bytes, cudaMemcpyHostToDevice));
   if (w_bytes) CK(cudaMemcpy(base + w_off, P.items.data(), w_bytes, cudaMemcpyHostToDevice));
-  if (i_bytes) CK(cudaMemcpy(base + i_off, P.ints.data(), i_bytes, cudaMemcpyHostToDevice));
   const WorkItem* w = (const WorkItem*)(base + w_off);
-  const int* ints = (const int*)(base + i_off);
   cl_status s = CL_OK;
   int64_t nl = 0;
   for (int v = 0; v < 2 && s == CL_OK; ++v) {
@@ -1046,7 +1017,7 @@ cl_status capture_batch_fused(cl_batch* b) {
     for (int i = 0; i < n; ++i) b->startU[v][i] = v == 0 ? b->lats[i]->U : b->lats[i]->Un;
     cudaError_t e = cudaStreamBeginCapture(b->origin, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return fail(CL_ERR_CUDA, std::string("fused capture: ") + cudaGetErrorString(e));
-    s = enqueue_fused_step(b, P, (const ChainDesc*)base + (size_t)v * n, w, ints, b->origin, &nl);
+    s = enqueue_fused_step(b, P, (const ChainDesc*)base + (size_t)v * n, w, b->origin, &nl);
     cudaGraph_t gr = nullptr;
     e = cudaStreamEndCapture(b->origin, &gr);
     if (s == CL_OK && e != cudaSuccess) s = fail(CL_ERR_CUDA, std::string("fused capture: ") + cudaGetErrorString(e));

@@ -124,25 +124,20 @@ __global__ void __maxnreg__(FORCE_AB_MAXNREG) k_ens_force_ab(const ChainDesc* __
 // after the force); MODE_UPDATE_X reads it back and writes Un at the device
 // step size.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_update(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, 3) k_ens_update(const ChainDesc* __restrict__ cd,
                                                                const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  UpdArgs a;
-  a.cexp = c.cexp;
-  a.beta = 0.0;
-  a.eps = c.eps;
-  a.sqrt_eps = c.sqrt_eps;
-  a.seed = c.seed;
-  a.sd = c.sd;
-  a.adaptive = MODE == MODE_UPDATE_X ? 1 : 0;
+  const UpdArgs a = {c.eps, c.sqrt_eps, c.k_ref, c.seed, c.sd, MODE == MODE_UPDATE_X ? 1 : 0, c.cexp};
   const void* in = MODE == MODE_UPDATE_X ? c.Pq : c.C;
   void* out = MODE == MODE_DRIFTMAX ? c.Pq : c.Un;
+  const uint32_t step = step_begin<MODE>(geo_of(c), a);
   if constexpr (is_fx<T>())
-    fx_update_body<T, MODE>(geo_of(c), (const V2*)c.U, (const int4*)in, out, a, it.vb);
+    fx_update_body<T, MODE>(geo_of(c), (const V2*)c.U, (const int4*)in, out, a, step, it.vb);
   else
-    k_update_gather_body<T, MODE>(geo_of(c), (const V2*)c.U, (const V2*)in, (V2*)out, a, it.vb);
+    k_update_gather_body<T, MODE>(geo_of(c), (const V2*)c.U, (const V2*)in, (V2*)out, a, step, it.vb);
+  step_size<MODE>(geo_of(c), a);
 }
 
 // Launch family fam of the CL step for link type T (FP64 runs the clover

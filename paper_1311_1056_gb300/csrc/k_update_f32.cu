@@ -43,16 +43,9 @@ cudaError_t launch_plaq_force_f32(bool theta, const GeoH& h, const void* U,
 }
 
 cudaError_t launch_update_gather_f32(int mode, const GeoH& h, const void* U, const void* C, void* out,
-                                    double eps, uint64_t seed, StepDev* sd, bool adaptive, cudaStream_t st) {
+                                     double eps, double k_ref, uint64_t seed, StepDev* sd, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  UpdArgs a;
-  a.cexp = 0;
-  a.beta = 0.0;
-  a.eps = eps;
-  a.sqrt_eps = sqrt(eps);
-  a.seed = seed;
-  a.sd = sd;
-  a.adaptive = adaptive ? 1 : 0;
+  const UpdArgs a = update_args(mode, eps, k_ref, seed, sd, 0);
   const int bs = block_of(h, TUNE_UPDATE);
   const dim3 gr = grid(g.V, 4, bs);
   const V2* u = (const V2*)U;

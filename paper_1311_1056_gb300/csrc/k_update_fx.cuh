@@ -478,8 +478,8 @@ __device__ __forceinline__ double drift_fx(const Geo& g, const int4* C, int4* o,
 // below 2^-62).  What does not fit goes through general_update_f64.
 template <typename L>
 __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L>::type* U, const int4* C, const int4* X,
-                                          typename vec2_of<L>::type* out, const UpdArgs& a, int s, const int* x, int MU) {
-  const uint32_t step = a.sd->step;
+                                          typename vec2_of<L>::type* out, const UpdArgs& a, uint32_t step, int s, const int* x,
+                                          int MU) {
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
   const tagged Xt = {const_cast<int4*>(X), ldexp(1.0, a.cexp + 2)};
@@ -535,7 +535,8 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
 // UPDATE_X's C) the drift are fixed-point fields.
 template <typename L, int MODE>
 __device__ __forceinline__ void fx_update_body(Geo g, const typename vec2_of<L>::type* __restrict__ U,
-                                               const int4* __restrict__ C, void* __restrict__ out, UpdArgs a, int vb) {
+                                               const int4* __restrict__ C, void* __restrict__ out, UpdArgs a, uint32_t step,
+                                               int vb) {
   typedef typename vec2_of<L>::type V2;
   const int MU = vb % 4;
   const int s_raw = (vb / 4) * blockDim.x + threadIdx.x;
@@ -550,7 +551,7 @@ __device__ __forceinline__ void fx_update_body(Geo g, const typename vec2_of<L>:
   } else if (MODE == MODE_DRIFTMAX) {
     kmax_update(a.sd, drift_fx(g, C, (int4*)out, a.cexp, s, x, MU, s_raw < g.V));
   } else {
-    update_fx<L>(g, U, MODE == MODE_UPDATE ? C : nullptr, MODE == MODE_UPDATE ? nullptr : C, (V2*)out, a, s, x, MU);
+    update_fx<L>(g, U, MODE == MODE_UPDATE ? C : nullptr, MODE == MODE_UPDATE ? nullptr : C, (V2*)out, a, step, s, x, MU);
   }
 }
 

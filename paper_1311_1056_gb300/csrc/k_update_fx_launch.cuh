@@ -17,7 +17,8 @@ struct StepFx {
   static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* E,
                             void* F, double sre, double sim, cudaStream_t st);
   static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6, cudaStream_t st);
-  static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, uint64_t seed, StepDev* sd, bool adaptive, int cexp, cudaStream_t st);
+  static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, double k_ref,
+                            uint64_t seed, StepDev* sd, int cexp, cudaStream_t st);
 };
 
 namespace {
@@ -77,9 +78,11 @@ __global__ void __maxnreg__(FX_MAXNREG) k_fx_force_b(Geo g, const typename vec2_
   fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, blockIdx.x);
 }
 template <typename L, int MODE>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
+__global__ void __maxnreg__(UPDATE_MAXNREG) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
                                                               const int4* __restrict__ C, void* __restrict__ out, UpdArgs a) {
-  fx_update_body<L, MODE>(g, U, C, out, a, blockIdx.x);
+  const uint32_t step = step_begin<MODE>(g, a);
+  fx_update_body<L, MODE>(g, U, C, out, a, step, blockIdx.x);
+  step_size<MODE>(g, a);
 }
 }  // namespace
 
@@ -131,17 +134,10 @@ cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const voi
 }
 
 template <typename L>
-cudaError_t StepFx<L>::update(int mode, const GeoH& h, const void* U, const void* C, void* out,
-                                    double eps, uint64_t seed, StepDev* sd, bool adaptive, int cexp, cudaStream_t st) {
+cudaError_t StepFx<L>::update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, double k_ref,
+                              uint64_t seed, StepDev* sd, int cexp, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  UpdArgs a;
-  a.cexp = cexp;
-  a.beta = 0.0;
-  a.eps = eps;
-  a.sqrt_eps = sqrt(eps);
-  a.seed = seed;
-  a.sd = sd;
-  a.adaptive = adaptive ? 1 : 0;
+  const UpdArgs a = update_args(mode, eps, k_ref, seed, sd, cexp);
   const int bs = block_of(h, TUNE_UPDATE);
   const dim3 gr = grid(g.V, 4, bs);
   const typename vec2_of<L>::type* u = (const typename vec2_of<L>::type*)U;

@@ -138,18 +138,13 @@ cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
                               double beta, int cexp, cudaStream_t st);
-// mode 0: update from the gathered drift (eps, or the device step size when
-// sd_adaptive); 1: write the drift X_S to out; 2: write X_S to out and fold
-// max |K|^2 into sd->kmax2_bits; 3: update reading X_S from C (a mode-2 output).
+// mode 0: update from the gathered drift, step size eps; 1: write the drift X_S
+// to out; 2: write X_S to out, max |K| and from it the device step size, eps
+// min(1, k_ref / K_max); 3: update reading X_S from C (a mode-2 output), device
+// step size.  Modes 0 and 3 count the step (sd->step, the Philox step word, and
+// sd->t).
 cudaError_t launch_update_gather(int prec, int mode, const GeoH& g, const void* U, const void* C, void* out,
-                                 double eps, uint64_t seed, StepDev* sd, bool sd_adaptive, int cexp,
-                                 cudaStream_t st);
-// step += 1 on the device (the Philox step counter read by the update).
-// After an update: step += 1 and t += the step size taken (eps, or the
-// device step size when adaptive).
-cudaError_t launch_step_bump(StepDev* sd, double eps, bool adaptive, cudaStream_t st);
-// Adaptive step size from the drift pass: eps_n = eps min(1, k_ref / K_max).
-cudaError_t launch_step_eps(StepDev* sd, double eps, double k_ref, cudaStream_t st);
+                                 double eps, double k_ref, uint64_t seed, StepDev* sd, int cexp, cudaStream_t st);
 // Cooling (cool_sweep.cuh).  What a call works on: the links U; the second link
 // buffer Ux, which holds their fixed-point words during a call of the FP64 and
 // DF64 forms (FP32 storage: Ux = U); f (8 FP64 values per site, [a][V]); the
@@ -186,14 +181,8 @@ cudaError_t launch_obs(int prec, const GeoH& g, const void* U, const void* Ux, c
 cudaError_t launch_obs_final(const GeoH& g, const double* partials, double beta, double th_re,
                              double th_im, ObsOut* out, cudaStream_t st);
 // Fused batch: one launch of family fam (ENS_*) over nw work items (device
-// arrays cd, w); FP64 and FP32 storage only.  Per-chain kernels (one thread
-// or one block per chain): the adaptive step size, the step counter, and the
-// cooling rule (first = the call's first sweep).
-// arg: ENS_COOL_GRAD's `first` flag (the call's first gradient runs whatever the rule state); the applies' sweep number.
+// arrays cd, w); FP64 and FP32 storage only.  arg: ENS_COOL_GRAD's `first` flag (the call's first gradient runs whatever the rule state); the applies' sweep number.
 cudaError_t launch_ens(int prec, int fam, const ChainDesc* cd, const WorkItem* w, int nw, int arg, cudaStream_t st);
-cudaError_t launch_ens_step_eps(const ChainDesc* cd, const int* chains, int n, cudaStream_t st);
-cudaError_t launch_ens_step_bump(const ChainDesc* cd, const int* chains, const int* adaptive, int n,
-                                 cudaStream_t st);
 // Integer-pipe float <-> double conversions (cvt.cuh) against the hardware
 // ones on n generated cases; mismatch counts added into bad[0] (float ->
 // double) and bad[1] (double -> float).
