@@ -22,16 +22,22 @@ struct fx_herm {
   cx<fx> o[3];  // 01, 02, 12
 };
 __device__ __forceinline__ fx fx_word(int2 w) { return fx{__int_as_float(w.x), w.y}; }
-__device__ __forceinline__ void fx_load_herm(fx_herm& h, const int2* __restrict__ P, int s, int V, fx_chk& ck) {
+__device__ __forceinline__ void fx_unpack_herm(fx_herm& h, const int2* v, fx_chk& ck) {
   fx w[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) w[k] = fx_word(__ldg(P + (size_t)k * V + s));
+  for (int k = 0; k < 9; ++k) w[k] = fx_word(v[k]);
   if (fx_is_raw(w[0].l)) ck.fail();
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     h.d[k] = w[k];
     h.o[k] = cx<fx>{w[3 + 2 * k], w[4 + 2 * k]};
   }
+}
+__device__ __forceinline__ void fx_load_herm(fx_herm& h, const int2* __restrict__ P, int s, int V, fx_chk& ck) {
+  int2 v[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) v[k] = __ldg(P + (size_t)k * V + s);
+  fx_unpack_herm(h, v, ck);
 }
 __device__ __forceinline__ void fx_store_herm(int2* P, int s, int V, const fx_herm& h) {
 #pragma unroll

@@ -24,7 +24,8 @@ __device__ __forceinline__ Geo geo_of(const ChainDesc& c) {
 }
 
 // Blocks per SM the link-algebra kernels are built for: the FP64 form's as its
-// single-chain kernels (FX_MAXNREG, k_update_fx_launch.cuh).
+// single-chain kernels (FX_BLOCKS_SM, k_update_fx_launch.cuh).
+static_assert(ENS_BLOCK <= FX_BLOCK, "shared-memory slots of a block");
 #define ENS_MIN_BLOCKS(T) (is_fx<T>() ? 3 : 1)
 
 template <typename T>
@@ -40,10 +41,11 @@ template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const ChainDesc* __restrict__ cd,
                                                              const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
+  __shared__ int4 sm[is_fx<T>() ? FX_PIPE : 1];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
-    fx_plaq_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, it.vb);
+    fx_plaq_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, sm, it.vb);
   else
     k_plaq_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Pq, (V2*)c.Dq, it.vb);
 }
@@ -52,27 +54,30 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover_half(const ChainDesc* __restrict__ cd,
                                                                     const WorkItem* __restrict__ w) {
+  __shared__ int4 sm[FX_PIPE];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  fx_clover_half_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C, it.vb);
+  fx_clover_half_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C, sm, it.vb);
 }
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_t(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
+  __shared__ int4 sm[FX_PIPE];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  fx_force_t_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.F, (int4*)c.C, it.vb);
+  fx_force_t_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.F, (int4*)c.C, sm, it.vb);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(const ChainDesc* __restrict__ cd,
                                                                const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
+  __shared__ int4 sm[is_fx<T>() ? FX_PIPE : 1];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
     fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq,
-                      (const int4*)c.C, (int4*)c.F, c.sre, c.sim, it.vb);
+                      (const int4*)c.C, (int4*)c.F, c.sre, c.sim, sm, it.vb);
   else
     k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }

@@ -27,6 +27,43 @@ namespace clgc {
 __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
 
+// Operands of the products on their way from memory: each thread copies the
+// matrices that it will need next into two slots of shared memory (cp.async)
+// while it works on the last one.  Three warps per scheduler do not hide a load
+// of 144 bytes (a quarter of a warp's time), and registers to load ahead are not
+// there.  A slot is a thread's own: element k of slot q at sm[(9 q + k)
+// FX_BLOCK + thread], no barrier.  32^4: plaquettes and clover field 2.60 ->
+// 2.48 ms a step, observables 3.03 -> 2.92 ms.  Stages a and b of the theta
+// force spill registers to the L1 that the slots take (6.34 -> 6.98 ms with
+// them) and load directly.
+const int FX_BLOCK = 128;                  // largest block of the kernels that use it
+const int FX_PIPE = 2 * 9 * FX_BLOCK;      // int4
+struct fx_pipe {
+  int4* sm;
+  int in, out;  // matrices asked for and taken (compile-time constants after unrolling)
+  __device__ __forceinline__ explicit fx_pipe(int4* s) : sm(s + threadIdx.x), in(0), out(0) {}
+  __device__ __forceinline__ void ask(const int4* f, int plane, int site, int V) {
+    const int4* p = f + (size_t)plane * 9 * V + site;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(sm + (in & 1) * 9 * FX_BLOCK);
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + k * FX_BLOCK * 16), "l"(p + (size_t)k * V) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    ++in;
+  }
+  __device__ __forceinline__ void take(mat<fx>& a, fx_chk& ck) {
+    if (in - out > 1)
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const int4* p = sm + (out & 1) * 9 * FX_BLOCK;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a.e[k] = unpack(p[k * FX_BLOCK]);
+    if (fx_is_raw(a.e[0].re.l)) ck.fail();
+    ++out;
+  }
+};
+
 // ------------------------------------------------------ links and inverses
 template <typename L>
 __device__ __forceinline__ void fx_links_body(Geo g, const typename vec2_of<L>::type* __restrict__ U,
@@ -58,26 +95,31 @@ static __device__ __noinline__ void general_plaq(Geo g, const typename vec2_of<L
 }
 template <typename L>
 __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
-                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq, int vb) {
+                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   int x[4];
   site_coords(g, s, x);
   fx_chk ck;
-  mat<fx> P, b;
-  fx_load(P, Ux, mu, s, g.V, ck);
-  fx_load(b, Ux, nu, hop(g, s, x, mu, 1), g.V, ck);
-  fx_mul_left<FX_WIDE>(P, b, ck);
-  fx_load(b, Ui, mu, hop(g, s, x, nu, 1), g.V, ck);
-  fx_mul_left<FX_WIDE>(P, b, ck);
-  fx_load(b, Ui, nu, s, g.V, ck);
-  fx_mul_left<FX_WIDE>(P, b, ck);
-  fx_adj(b, P, ck);
-  store<fx>(Pq, p, s, g.V, P);
+  mat<fx> Pm, b;
+  fx_pipe P(sm);
+  P.ask(Ux, mu, s, g.V);
+  P.ask(Ux, nu, hop(g, s, x, mu, 1), g.V);
+  P.take(Pm, ck);
+  P.ask(Ui, mu, hop(g, s, x, nu, 1), g.V);
+  P.take(b, ck);
+  P.ask(Ui, nu, s, g.V);
+  fx_mul_left<FX_WIDE>(Pm, b, ck);
+  P.take(b, ck);
+  fx_mul_left<FX_WIDE>(Pm, b, ck);
+  P.take(b, ck);
+  fx_mul_left<FX_WIDE>(Pm, b, ck);
+  fx_adj(b, Pm, ck);
+  store<fx>(Pq, p, s, g.V, Pm);
 #pragma unroll
-  for (int k = 0; k < 9; ++k) P.e[k] = cx<fx>{fx_half_diff(P.e[k].re, b.e[k].re), fx_half_diff(P.e[k].im, b.e[k].im)};
-  store<fx>(Dq, p, s, g.V, P);
+  for (int k = 0; k < 9; ++k) Pm.e[k] = cx<fx>{fx_half_diff(Pm.e[k].re, b.e[k].re), fx_half_diff(Pm.e[k].im, b.e[k].im)};
+  store<fx>(Dq, p, s, g.V, Pm);
   if (ck.bad()) general_plaq<L>(g, U, tag(Pq), tag_D(Dq), vb);
 }
 
@@ -93,7 +135,7 @@ static __device__ __noinline__ void general_clover(Geo g, const typename vec2_of
 // six (32^4: plaquettes and clover field 3.00 -> 2.60 ms a step, observables
 // 3.43 -> 3.04 ms; the second pass is partly bound by its 0.9 GB of E).
 __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
-                                                    const int4* __restrict__ Dq, int4* E, int vb) {
+                                                    const int4* __restrict__ Dq, int4* E, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -102,11 +144,16 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
   const int xmm = hop(g, s, x, mu, -1);
   fx_chk ck;
   mat<fx> acc, w, d;
-  fx_load(w, Ui, mu, xmm, g.V, ck);
-  fx_load(d, Dq, p, xmm, g.V, ck);
+  fx_pipe P(sm);
+  P.ask(Ui, mu, xmm, g.V);
+  P.ask(Dq, p, xmm, g.V);
+  P.take(w, ck);
+  P.ask(Ux, mu, xmm, g.V);
+  P.take(d, ck);
+  P.ask(Dq, p, s, g.V);
   fx_mul_left<FX_NARROW, 2>(w, d, ck);
-  fx_load(d, Ux, mu, xmm, g.V, ck);
-  fx_load(acc, Dq, p, s, g.V, ck);
+  P.take(d, ck);
+  P.take(acc, ck);
   fx_mul_acc<FX_WIDE, +1, 2>(acc, w, d, ck);
   if (ck.bad()) acc.e[0].re.l = fx_raw_mark();  // its readers start over from D
   store<fx>(E, p, s, g.V, acc);
@@ -116,7 +163,7 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
 template <typename L>
 __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                const int4* __restrict__ Ui, const int4* __restrict__ Dq,
-                                               const int4* __restrict__ E, int4* F, double sre, double sim, int vb) {
+                                               const int4* __restrict__ E, int4* F, double sre, double sim, int4* sm, int vb) {
   const int p = vb % 6, nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -129,11 +176,16 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
   const int xmn = hop(g, s, x, nu, -1);
   fx_chk ck;
   mat<fx> acc, w, d;
-  fx_load(w, Ui, nu, xmn, g.V, ck);
-  fx_load(d, E, p, xmn, g.V, ck);
+  fx_pipe P(sm);
+  P.ask(Ui, nu, xmn, g.V);
+  P.ask(E, p, xmn, g.V);
+  P.take(w, ck);
+  P.ask(Ux, nu, xmn, g.V);
+  P.take(d, ck);
+  P.ask(E, p, s, g.V);
   fx_mul_left<FX_WIDE>(w, d, ck);
-  fx_load(d, Ux, nu, xmn, g.V, ck);
-  fx_load(acc, E, p, s, g.V, ck);
+  P.take(d, ck);
+  P.take(acc, ck);
   fx_mul_acc<FX_WIDE, +1>(acc, w, d, ck);
   unsigned mag = 0;
   const cx<fx> sc = {fx_of_double(8.0 * sre, mag), fx_of_double(8.0 * sim, mag)};
@@ -192,7 +244,7 @@ __device__ __forceinline__ void fx_force_wilson_body(Geo g, const typename vec2_
 // and (a b) G2 (a b)^{-1} for two: 20 products a plaquette in place of 21.7
 // (theta force of a 32^4 step 6.55 -> 6.38 ms).
 __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
-                                                const int4* __restrict__ F, int4* C, int vb) {
+                                                const int4* __restrict__ F, int4* C, int4* sm, int vb) {
   const int p = vb % 6, nu = plane_nu(p), pc = 5 - p;
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -200,10 +252,14 @@ __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ 
   site_coords(g, s, x);
   fx_chk ck;
   mat<fx> A, B;
-  fx_load(A, Ux, nu, s, g.V, ck);
-  fx_load(B, F, pc, hop(g, s, x, nu, 1), g.V, ck);
+  fx_pipe P(sm);
+  P.ask(Ux, nu, s, g.V);
+  P.ask(F, pc, hop(g, s, x, nu, 1), g.V);
+  P.take(A, ck);
+  P.ask(Ui, nu, s, g.V);
+  P.take(B, ck);
   fx_mul_left<FX_WIDE>(A, B, ck);
-  fx_load(B, Ui, nu, s, g.V, ck);
+  P.take(B, ck);
   fx_mul_left<FX_WIDE>(A, B, ck);
   if (ck.bad()) A.e[0].re.l = fx_raw_mark();  // its readers start over from F
   store<fx>(C, 4 * p + 3, s, g.V, A);
@@ -394,7 +450,7 @@ __device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long
   return !ck.bad();
 }
 // A = 2 eps (X - Tr X / 3) + i sqrt(eps) sqrt(2) g_a lambda_a from the traceless
-// quarter of X 2^-cexp and g / 8.  The noise constant 8 sqrt(2 eps) passes the fixed-point
+// quarter of X 2^-cexp and g / 8 (element j at gs[j TUNE_MAX_BLOCK]).  The noise constant 8 sqrt(2 eps) passes the fixed-point
 // bound at eps = 0.016; from there on A is formed as a quarter.
 __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, const fx* gs, double eps, double sqrt_eps,
                                             int cexp) {
@@ -409,7 +465,7 @@ __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, co
   if (!fx_mag_ok(mag)) return false;
   fx_right R[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) R[j] = fx_rhs(gs[j]);
+  for (int j = 0; j < 8; ++j) R[j] = fx_rhs(gs[j * TUNE_MAX_BLOCK]);
 #pragma unroll
   for (int k = 0; k < 9; ++k)
 #pragma unroll
@@ -422,7 +478,7 @@ __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, co
       if (i == j) {
         if (im) {
           if (i < 2) fx_mac(s, i == 0 ? n : m, R[2]);
-          fx_mac(s, n3, i < 2 ? R[7] : fx_rhs(fx_twice(-gs[7])));
+          fx_mac(s, n3, i < 2 ? R[7] : fx_rhs(fx_twice(-gs[7 * TUNE_MAX_BLOCK])));
         }
       } else {
         const int q = i + j == 1 ? 0 : i + j == 2 ? 3 : 5;
@@ -483,6 +539,18 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
   const tagged Xt = {const_cast<int4*>(X), ldexp(1.0, a.cexp + 2)};
+  // The noise first, one pair at a time into shared memory (a thread's own
+  // words): its code once instead of four times, which the warps fetched (a
+  // sixth of their time; update 0.145 -> 0.136 ms at 16^4, 1.80 -> 1.76 at 32^4).
+  __shared__ fx noise[8 * TUNE_MAX_BLOCK];
+  fx* gs = noise + threadIdx.x;
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {
+    fx g0, g1;
+    normal_pair_fx(g0, g1, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL, (uint32_t)j);
+    gs[2 * j * TUNE_MAX_BLOCK] = g0;
+    gs[(2 * j + 1) * TUNE_MAX_BLOCK] = g1;
+  }
   mat<fx> A;
   bool ok;
   if (C) {
@@ -494,11 +562,7 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
     ok = !ck.bad();
   }
   if (ok) {
-    {
-      fx gs[8];
-      normals_fx<4>(gs, a.seed, step, (uint32_t)s, (uint32_t)MU, STREAM_CL);
-      ok = fx_exponent(A, gs, eps, sqrt_eps, a.cexp);
-    }
+    ok = fx_exponent(A, gs, eps, sqrt_eps, a.cexp);
     ok = ok && fx_expm_traceless(A, fx_norm(A), TAYLOR_TOL_FP64);
     if (ok) {
       fx_chk ck;

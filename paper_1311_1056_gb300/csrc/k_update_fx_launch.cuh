@@ -2,6 +2,7 @@
 // (k_update_fx.cuh) for one link type, instantiated by k_update_f64.cu and
 // k_update_df64.cu.
 #pragma once
+#include <algorithm>
 #include <cmath>
 
 #include "k_update_fx.cuh"
@@ -26,31 +27,34 @@ namespace {
 // cover every plane of a range of sites, so shared neighbours stay in cache.
 inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 1) / bs) * planes)); }
 
-// Registers of the plaquette, clover and force kernels: three blocks of 128
-// threads per SM.  Per 32^4 step at caps of 144 / 168 / 208, before the clover
+// Resident blocks that the plaquette, clover and force kernels are built for
+// (168 registers).  Per 32^4 step at caps of 144 / 168 / 208, before the clover
 // field and the force were split further: clover and plaquettes 3.33 / 3.00 /
 // 3.37 ms, force 7.37 / 6.49 / 6.98 ms (two blocks at 208; 144 spills more, 420
 // bytes a thread at 168).  Now 2.60 and 6.38 ms; FP64 arithmetic took 11.95 and
 // 26.0 ms.
-const int FX_MAXNREG = 168;
+const int FX_BLOCKS_SM = 3;
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui) {
   fx_links_body<L>(g, U, Ux, Ui, blockIdx.x);
 }
 template <typename L>
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_plaq(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_plaq(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq) {
-  fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, sm, blockIdx.x);
 }
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_clover_half(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover_half(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                          const int4* __restrict__ Dq, int4* E) {
-  fx_clover_half_body(g, Ux, Ui, Dq, E, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_clover_half_body(g, Ux, Ui, Dq, E, sm, blockIdx.x);
 }
 template <typename L>
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                     const int4* __restrict__ Ui, const int4* __restrict__ Dq,
                                                     const int4* __restrict__ E, int4* F, double sre, double sim) {
-  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sre, sim, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sre, sim, sm, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
@@ -59,11 +63,12 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const
                                                                     const int4* __restrict__ Dq, int4* C, double b6) {
   fx_force_wilson_body<L>(g, U, Ux, Ui, Dq, C, b6, blockIdx.x);
 }
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_t(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_t(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                      const int4* __restrict__ F, int4* C) {
-  fx_force_t_body(g, Ux, Ui, F, C, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_force_t_body(g, Ux, Ui, F, C, sm, blockIdx.x);
 }
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui,
                                                                const int4* __restrict__ Dq,
                                                                const int4* __restrict__ F, int4* Gq, int4* C,
@@ -71,7 +76,7 @@ __global__ void __maxnreg__(FX_MAXNREG) k_fx_force_a(Geo g, const int4* __restri
   fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, blockIdx.x);
 }
 template <typename L>
-__global__ void __maxnreg__(FX_MAXNREG) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui, const int4* Pq,
                                                                const int4* Dq, const int4* F, const int4* Gq, int4* C,
                                                                double b6) {
@@ -98,7 +103,7 @@ template <typename L>
 cudaError_t StepFx<L>::plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
                             cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  const int bs = block_of(h, TUNE_CLOVER);
+  const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
   k_fx_plaq<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (int4*)Pq, (int4*)Dq);
   return cudaGetLastError();
 }
@@ -107,7 +112,7 @@ template <typename L>
 cudaError_t StepFx<L>::clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
                                   void* E, void* F, double sre, double sim, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  const int bs = block_of(h, TUNE_CLOVER);
+  const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
   k_fx_clover_half<<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)E);
   k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E,
                                                (int4*)F, sre, sim);
@@ -119,7 +124,7 @@ cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const voi
                                   const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
                                   cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  const int bs = block_of(h, TUNE_FORCE);
+  const int bs = std::min(block_of(h, TUNE_FORCE), FX_BLOCK);
   const dim3 gr = grid(g.V, 6, bs);
   if (!theta) {
     k_fx_force_wilson<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)C, b6);

@@ -117,20 +117,22 @@ __device__ __forceinline__ void fx_sincos(uint64_t k, fx& sn, fx& cs) {
   cs = fx_split(fx_sum(b));
 }
 
-// 2 NP normal numbers divided by 8: the pairs of normals_f64.
+// Pair j of the normal numbers of normals_f64, divided by 8.
+__device__ __forceinline__ void normal_pair_fx(fx& g0, fx& g1, uint64_t seed, uint32_t step, uint32_t site, uint32_t slot,
+                                               uint32_t stream, uint32_t j) {
+  const uint4 w = philox_words(seed, step, site, slot, stream, j);
+  const uint64_t k1 = ((uint64_t)(w.x >> 6) << 26) | (w.y >> 6), k2 = ((uint64_t)(w.z >> 6) << 26) | (w.w >> 6);
+  const fx_left r = fx_lhs(fx_radius(k1));
+  fx s, c;
+  fx_sincos(k2, s, c);
+  g0 = fx_times(r, fx_rhs(c));
+  g1 = fx_times(r, fx_rhs(s));
+}
 template <int NP>
 __device__ __forceinline__ void normals_fx(fx* g, uint64_t seed, uint32_t step, uint32_t site, uint32_t slot,
                                            uint32_t stream) {
 #pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    const uint4 w = philox_words(seed, step, site, slot, stream, (uint32_t)j);
-    const uint64_t k1 = ((uint64_t)(w.x >> 6) << 26) | (w.y >> 6), k2 = ((uint64_t)(w.z >> 6) << 26) | (w.w >> 6);
-    const fx_left r = fx_lhs(fx_radius(k1));
-    fx s, c;
-    fx_sincos(k2, s, c);
-    g[2 * j] = fx_times(r, fx_rhs(c));
-    g[2 * j + 1] = fx_times(r, fx_rhs(s));
-  }
+  for (int j = 0; j < NP; ++j) normal_pair_fx(g[2 * j], g[2 * j + 1], seed, step, site, slot, stream, (uint32_t)j);
 }
 
 }  // namespace clgc
