@@ -326,6 +326,41 @@ __device__ __forceinline__ void fx_load(mat<fx>& a, const int4* __restrict__ f, 
   if (fx_is_raw(a.e[0].re.l)) ck.fail();
 }
 
+// Matrices on their way from memory: each thread copies those that it will need
+// next into slots of shared memory (cp.async) while it works on the last one.
+// Three warps per scheduler do not hide a load of 144 bytes (a quarter of a
+// warp's time), and registers to load ahead are not there.  A slot is a
+// thread's own: element k of slot q at sm[(9 q + k) FX_PIPE_THREADS + thread],
+// no barrier.  With two slots `in` and `out` are constants of unrolled code.
+const int FX_PIPE_THREADS = 128;
+template <int SLOTS>
+struct fx_pipe {
+  static const int WORDS = SLOTS * 9 * FX_PIPE_THREADS;  // int4
+  int4* sm;
+  int in, out;  // matrices asked for and taken
+  __device__ __forceinline__ explicit fx_pipe(int4* s) : sm(s + threadIdx.x), in(0), out(0) {}
+  __device__ __forceinline__ void ask(const int4* f, int plane, int site, int V) {
+    const int4* p = f + (size_t)plane * 9 * V + site;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(sm + (in & (SLOTS - 1)) * 9 * FX_PIPE_THREADS);
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + k * FX_PIPE_THREADS * 16), "l"(p + (size_t)k * V) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    ++in;
+  }
+  __device__ __forceinline__ void take(mat<fx>& a, fx_chk& ck) {
+    if (SLOTS > 1 && in - out > 1)
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const int4* p = sm + (out & (SLOTS - 1)) * 9 * FX_PIPE_THREADS;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a.e[k] = unpack(p[k * FX_PIPE_THREADS]);
+    if (fx_is_raw(a.e[0].re.l)) ck.fail();
+    ++out;
+  }
+};
+
 // Plain (coherent) load, for words this kernel also writes; |v| < 1 for a 60-bit integer.
 __device__ __forceinline__ void fx_load_plain(mat<fx>& a, const int4* f, int plane, int site, int V) {
   const int4* p = f + (size_t)plane * 9 * V + site;

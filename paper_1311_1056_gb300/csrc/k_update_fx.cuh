@@ -27,42 +27,12 @@ namespace clgc {
 __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
 
-// Operands of the products on their way from memory: each thread copies the
-// matrices that it will need next into two slots of shared memory (cp.async)
-// while it works on the last one.  Three warps per scheduler do not hide a load
-// of 144 bytes (a quarter of a warp's time), and registers to load ahead are not
-// there.  A slot is a thread's own: element k of slot q at sm[(9 q + k)
-// FX_BLOCK + thread], no barrier.  32^4: plaquettes and clover field 2.60 ->
-// 2.48 ms a step, observables 3.03 -> 2.92 ms.  Stages a and b of the theta
-// force spill registers to the L1 that the slots take (6.34 -> 6.98 ms with
-// them) and load directly.
-const int FX_BLOCK = 128;                  // largest block of the kernels that use it
-const int FX_PIPE = 2 * 9 * FX_BLOCK;      // int4
-struct fx_pipe {
-  int4* sm;
-  int in, out;  // matrices asked for and taken (compile-time constants after unrolling)
-  __device__ __forceinline__ explicit fx_pipe(int4* s) : sm(s + threadIdx.x), in(0), out(0) {}
-  __device__ __forceinline__ void ask(const int4* f, int plane, int site, int V) {
-    const int4* p = f + (size_t)plane * 9 * V + site;
-    const unsigned d = (unsigned)__cvta_generic_to_shared(sm + (in & 1) * 9 * FX_BLOCK);
-#pragma unroll
-    for (int k = 0; k < 9; ++k)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + k * FX_BLOCK * 16), "l"(p + (size_t)k * V) : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    ++in;
-  }
-  __device__ __forceinline__ void take(mat<fx>& a, fx_chk& ck) {
-    if (in - out > 1)
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const int4* p = sm + (out & 1) * 9 * FX_BLOCK;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) a.e[k] = unpack(p[k * FX_BLOCK]);
-    if (fx_is_raw(a.e[0].re.l)) ck.fail();
-    ++out;
-  }
-};
+// The operands of the products come through an fx_pipe of two slots (fixed.cuh):
+// 32^4: plaquettes and clover field 2.60 -> 2.48 ms a step, observables 3.03 ->
+// 2.92 ms.  Stages a and b of the theta force spill registers to the L1 that
+// the slots take (6.34 -> 6.98 ms with them) and load directly.
+const int FX_BLOCK = FX_PIPE_THREADS;  // largest block of the kernels that use it
+const int FX_PIPE = fx_pipe<2>::WORDS;
 
 // ------------------------------------------------------ links and inverses
 template <typename L>
@@ -103,7 +73,7 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
   site_coords(g, s, x);
   fx_chk ck;
   mat<fx> Pm, b;
-  fx_pipe P(sm);
+  fx_pipe<2> P(sm);
   P.ask(Ux, mu, s, g.V);
   P.ask(Ux, nu, hop(g, s, x, mu, 1), g.V);
   P.take(Pm, ck);
@@ -144,7 +114,7 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
   const int xmm = hop(g, s, x, mu, -1);
   fx_chk ck;
   mat<fx> acc, w, d;
-  fx_pipe P(sm);
+  fx_pipe<2> P(sm);
   P.ask(Ui, mu, xmm, g.V);
   P.ask(Dq, p, xmm, g.V);
   P.take(w, ck);
@@ -176,7 +146,7 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
   const int xmn = hop(g, s, x, nu, -1);
   fx_chk ck;
   mat<fx> acc, w, d;
-  fx_pipe P(sm);
+  fx_pipe<2> P(sm);
   P.ask(Ui, nu, xmn, g.V);
   P.ask(E, p, xmn, g.V);
   P.take(w, ck);
@@ -252,7 +222,7 @@ __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ 
   site_coords(g, s, x);
   fx_chk ck;
   mat<fx> A, B;
-  fx_pipe P(sm);
+  fx_pipe<2> P(sm);
   P.ask(Ux, nu, s, g.V);
   P.ask(F, pc, hop(g, s, x, nu, 1), g.V);
   P.take(A, ck);

@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_ens_cool_grad_omega(const ChainD
                                                                    const WorkItem* __restrict__ w) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  sweep_grad_omega_body<L, CS_WIDE_OMEGA>(ens_geo(c), ens_sweep<L>(c), it.vb);
+  sweep_grad_omega_body<L, cs_wide_omega<L>()>(ens_geo(c), ens_sweep<L>(c), it.vb);
 }
 // sweep: which of the call's sweeps this launch is (each chain has its own last one)
 template <typename L, bool RULE>
@@ -796,7 +796,7 @@ cudaError_t launch_cool_grad_omega(int prec, const GeoH& h, const CoolBufs& b, c
     if (cs_narrow(g.V))
       k_cool_grad_omega<L, 1><<<cs_grad_omega_blocks(g.V, 1), CS_THREADS, 0, st>>>(g, a);
     else
-      k_cool_grad_omega<L, CS_WIDE_OMEGA><<<cs_grad_omega_blocks(g.V, CS_WIDE_OMEGA), CS_THREADS, 0, st>>>(g, a);
+      k_cool_grad_omega<L, cs_wide_omega<L>()><<<cs_grad_omega_blocks(g.V, cs_wide_omega<L>()), CS_THREADS, 0, st>>>(g, a);
   });
 }
 cudaError_t launch_cool_apply(int prec, const GeoH& h, const CoolBufs& b, bool rule, bool last, cudaStream_t st) {
@@ -822,7 +822,7 @@ int ens_cool_blocks(int prec, int fam, int V) {
   switch (fam) {
     case ENS_COOL_GRAD: return cs_grad_blocks(V, prec == 0 ? cs_wide_grad<double>() : cs_wide_grad<float>());
     case ENS_COOL_OMEGA: return cs_omega_blocks(V, false);
-    case ENS_COOL_GRAD_OMEGA: return cs_grad_omega_blocks(V, CS_WIDE_OMEGA);
+    case ENS_COOL_GRAD_OMEGA: return cs_grad_omega_blocks(V, prec == 0 ? cs_wide_omega<double>() : cs_wide_omega<float>());
     default: return cs_apply_blocks(V);
   }
 }
