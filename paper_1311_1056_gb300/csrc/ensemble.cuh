@@ -24,7 +24,7 @@ __device__ __forceinline__ Geo geo_of(const ChainDesc& c) {
 }
 
 // Blocks per SM the link-algebra kernels are built for: the FP64 form's as its
-// single-chain kernels (FX_BLOCKS_SM, k_update_fx_launch.cuh).
+// single-chain kernels (k_update_fx_launch.cuh); its force's kernels 2.
 static_assert(ENS_BLOCK <= FX_BLOCK, "shared-memory slots of a block");
 #define ENS_MIN_BLOCKS(T) (is_fx<T>() ? 3 : 1)
 
@@ -83,35 +83,38 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(con
 }
 
 template <typename T>
-__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_wilson(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, is_fx<T>() ? 2 : 1) k_ens_force_wilson(const ChainDesc* __restrict__ cd,
                                                                      const WorkItem* __restrict__ w) {
   typedef typename vec2_of<T>::type V2;
+  __shared__ int4 sm[is_fx<T>() ? FX_PIPE : 1];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
     fx_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C,
-                         ldexp(c.beta / 6.0, -c.cexp), it.vb);
+                         ldexp(c.beta / 6.0, -c.cexp), sm, it.vb);
   else
     k_plaq_force_wilson_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.C,
                               (T)(c.beta / 6.0), it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_a(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_a(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
+  __shared__ int4 sm[FX_PIPE];
   fx_force_a_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (const int4*)c.F, (int4*)c.Gq,
-                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), it.vb);
+                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), sm, it.vb);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_b(const ChainDesc* __restrict__ cd,
+__global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_b(const ChainDesc* __restrict__ cd,
                                                                 const WorkItem* __restrict__ w) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
+  __shared__ int4 sm[FX_PIPE];
   fx_force_b_body<T>(geo_of(c), (const typename vec2_of<T>::type*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
-                  (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), it.vb);
+                  (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), sm, it.vb);
 }
 
 template <typename T>

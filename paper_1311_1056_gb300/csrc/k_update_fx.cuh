@@ -29,8 +29,7 @@ __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cas
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
 // 32^4: plaquettes and clover field 2.60 -> 2.48 ms a step, observables 3.03 ->
-// 2.92 ms.  Stages a and b of the theta force spill registers to the L1 that
-// the slots take (6.34 -> 6.98 ms with them) and load directly.
+// 2.92 ms.
 const int FX_BLOCK = FX_PIPE_THREADS;  // largest block of the kernels that use it
 const int FX_PIPE = fx_pipe<2>::WORDS;
 
@@ -178,7 +177,7 @@ static __device__ __noinline__ void general_force_wilson(Geo g, const typename v
 template <typename L>
 __device__ __forceinline__ void fx_force_wilson_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                      const int4* __restrict__ Ui, const int4* __restrict__ Dq, int4* C,
-                                                     double b6, int vb) {
+                                                     double b6, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -186,22 +185,28 @@ __device__ __forceinline__ void fx_force_wilson_body(Geo g, const typename vec2_
   unsigned mag = 0;
   const fx b = fx_of_double(2.0 * b6, mag);
   mat<fx> M, t, a;
-  fx_load(a, Dq, p, s, g.V, ck);
+  fx_pipe<2> P(sm);
+  P.ask(Dq, p, s, g.V);
+  P.ask(Ui, nu, s, g.V);
+  P.take(a, ck);
+  P.ask(Ux, nu, s, g.V);
   fx_scaled<FX_WIDE>(M, a, b, ck);
   store<fx>(C, 4 * p + 1, s, g.V, M);
   // slot 3: u^{-1} (beta/6 D) u
-  fx_load(t, Ui, nu, s, g.V, ck);
+  P.take(t, ck);
+  P.ask(Ui, mu, s, g.V);
   fx_mul_left<FX_WIDE>(t, M, ck);
-  fx_load(a, Ux, nu, s, g.V, ck);
+  P.take(a, ck);
+  P.ask(Ux, mu, s, g.V);
   fx_mul_left<FX_WIDE>(t, a, ck);
   store<fx>(C, 4 * p + 3, s, g.V, t);
   // slots 0 and 2: -(beta/6) D and the same carried by a
 #pragma unroll
   for (int k = 0; k < 9; ++k) M.e[k] = cx<fx>{-M.e[k].re, -M.e[k].im};
   store<fx>(C, 4 * p + 0, s, g.V, M);
-  fx_load(t, Ui, mu, s, g.V, ck);
+  P.take(t, ck);
   fx_mul_left<FX_WIDE>(t, M, ck);
-  fx_load(a, Ux, mu, s, g.V, ck);
+  P.take(a, ck);
   fx_mul_left<FX_WIDE>(t, a, ck);
   store<fx>(C, 4 * p + 2, s, g.V, t);
   if (ck.bad() || !fx_mag_ok(mag)) general_force_wilson<L>(g, U, tag_D(Dq), tag(C), b6, vb);
@@ -239,10 +244,10 @@ __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ 
 // and the partials of slots 0 and 2 go to Gq and C (planes of this plaquette
 // that only stage b of the same thread's plaquette writes).  Both stages keep
 // at most three matrices in registers at a time, parking and re-reading the
-// rest, so that three blocks of 128 threads fit an SM.
+// rest: with a fourth they would spill.
 __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                 const int4* __restrict__ Dq, const int4* __restrict__ F, int4* Gq,
-                                                int4* C, double b6, int vb) {
+                                                int4* C, double b6, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), pc = 5 - p;
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -254,30 +259,38 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
   const fx nb = fx_of_double(-b6, mag);
   mat<fx> A, B, M;
   // corner c0: half the slot 0 partial, [D, G0] / 2 - (beta/6) D / 2
-  fx_load(A, Dq, p, s, g.V, ck);
-  fx_load(B, F, pc, s, g.V, ck);
+  fx_pipe<2> P(sm);
+  P.ask(Dq, p, s, g.V);
+  P.ask(F, pc, s, g.V);
+  P.take(A, ck);
+  P.ask(Ux, mu, s, g.V);
+  P.take(B, ck);
+  P.ask(F, pc, c1, g.V);
   fx_commutator<FX_NARROW>(M, A, B, nb, ck);
   store<fx>(C, 4 * p + 0, s, g.V, M);
   // corner c1: A = G1^ = a G1 a^{-1}; slot 2 partial = slot 0 partial + [D, G1^]
-  fx_load(A, Ux, mu, s, g.V, ck);
-  fx_load(B, F, pc, c1, g.V, ck);
+  P.take(A, ck);
+  P.ask(Ui, mu, s, g.V);
+  P.take(B, ck);
+  P.ask(Dq, p, s, g.V);
   fx_mul_left<FX_WIDE>(A, B, ck);
-  fx_load(B, Ui, mu, s, g.V, ck);
+  P.take(B, ck);
+  P.ask(F, pc, s, g.V);
   fx_mul_left<FX_NARROW>(A, B, ck);
-  load_rw(M, C, 4 * p + 0, s, g.V);
-  fx_load(B, Dq, p, s, g.V, ck);
+  P.take(B, ck);
+  P.ask(Ux, mu, s, g.V);
   fx_commutator_acc<FX_NARROW>(M, B, A, ck);
   store<fx>(C, 4 * p + 2, s, g.V, M);
-  fx_load(B, F, pc, s, g.V, ck);
-  fx_add(A, B);
-  store<fx>(Gq, GQ_PLANE * p, s, g.V, A);  // G0 + G1^
+  P.take(B, ck);
+  P.ask(C, 4 * p + 3, c1, g.V);
+  M = A;
+  fx_add(M, B);  // G0 + G1^
   // corner c2: G2^ = a T(x+mu) a^{-1}
-  fx_load(A, Ux, mu, s, g.V, ck);
-  fx_load_plain(B, C, 4 * p + 3, c1, g.V);
-  if (fx_is_raw(B.e[0].re.l)) ck.fail();
+  P.take(A, ck);
+  P.ask(Ui, mu, s, g.V);
+  P.take(B, ck);
   fx_mul_left<FX_WIDE>(A, B, ck);
-  fx_load(B, Ui, mu, s, g.V, ck);
-  load_rw(M, Gq, GQ_PLANE * p, s, g.V);
+  P.take(B, ck);
   fx_mul_acc<FX_WIDE, +1>(M, A, B, ck);
   if (ck.bad() || !fx_mag_ok(mag)) M.e[0].re.l = fx_raw_mark();  // stage b starts over
   store<fx>(Gq, GQ_PLANE * p, s, g.V, M);
@@ -292,7 +305,7 @@ static __device__ __noinline__ void general_force(Geo g, const typename vec2_of<
 template <typename L>
 __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                 const int4* __restrict__ Ui, const int4* Pq, const int4* Dq,
-                                                const int4* F, const int4* Gq, int4* C, double b6, int vb) {
+                                                const int4* F, const int4* Gq, int4* C, double b6, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -301,47 +314,60 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   const fx pb = fx_of_double(b6, mag);
   mat<fx> A, B, M;
   // corner c3: A = G3r = T; slot 3 partial = [D, G3r] + (beta/6) D
-  fx_load_plain(A, C, 4 * p + 3, s, g.V);
-  if (fx_is_raw(A.e[0].re.l)) ck.fail();
-  fx_load(B, Dq, p, s, g.V, ck);
+  fx_pipe<2> P(sm);
+  P.ask(C, 4 * p + 3, s, g.V);
+  P.ask(Dq, p, s, g.V);
+  P.take(A, ck);
+  P.ask(Pq, p, s, g.V);
+  P.take(B, ck);
+  P.ask(Dq, p, s, g.V);
   fx_commutator<FX_NARROW>(M, B, A, pb, ck);
   store<fx>(C, 4 * p + 3, s, g.V, M);
   // M = G^ += P G3r P^{-1}, with P^{-1} = P - 2 (D / 2)
-  fx_load(B, Pq, p, s, g.V, ck);
+  P.take(B, ck);
+  P.ask(Pq, p, s, g.V);
   fx_mul_left<FX_WIDE>(B, A, ck);
-  fx_load(A, Dq, p, s, g.V, ck);
-  fx_load(M, Pq, p, s, g.V, ck);
+  P.take(A, ck);
+  P.ask(Gq, GQ_PLANE * p, s, g.V);
+  P.take(M, ck);
+  P.ask(Pq, p, s, g.V);
 #pragma unroll
   for (int k = 0; k < 9; ++k) A.e[k] = cx<fx>{M.e[k].re - fx_twice(A.e[k].re), M.e[k].im - fx_twice(A.e[k].im)};
-  load_rw(M, Gq, GQ_PLANE * p, s, g.V);
-  if (fx_is_raw(M.e[0].re.l)) ck.fail();
+  P.take(M, ck);
+  P.ask(C, 4 * p + 0, s, g.V);
   fx_mul_acc<FX_WIDE, +1>(M, B, A, ck);
   // A = K = P^{-1} G^ + G^ P
   fx_mul_left<FX_WIDE>(A, M, ck);
-  fx_load(B, Pq, p, s, g.V, ck);
+  P.take(B, ck);
+  P.ask(Dq, p, s, g.V);
   fx_mul_acc<FX_NARROW, +1>(A, M, B, ck);
   // slot 0: K + partial; slot 1: -K + (beta/6) D
-  load_rw(M, C, 4 * p + 0, s, g.V);
+  P.take(M, ck);
+  P.ask(Ui, nu, s, g.V);
   fx_twice_add<+1>(M, A);
   store<fx>(C, 4 * p + 0, s, g.V, M);
-  fx_load(M, Dq, p, s, g.V, ck);
+  P.take(M, ck);
+  P.ask(Ux, nu, s, g.V);
   fx_scaled<FX_NARROW>(M, M, pb, ck);
   fx_twice_add<-1>(M, A);
   store<fx>(C, 4 * p + 1, s, g.V, M);
   // slot 3: u^{-1} (-K + partial) u
   load_rw(M, C, 4 * p + 3, s, g.V);
   fx_twice_add<-1>(M, A);
-  fx_load(B, Ui, nu, s, g.V, ck);
+  P.take(B, ck);
+  P.ask(C, 4 * p + 2, s, g.V);
   fx_mul_left<FX_WIDE>(B, M, ck);
-  fx_load(M, Ux, nu, s, g.V, ck);
+  P.take(M, ck);
+  P.ask(Ui, mu, s, g.V);
   fx_mul_left<FX_WIDE>(B, M, ck);
   store<fx>(C, 4 * p + 3, s, g.V, B);
   // slot 2: a^{-1} (K + partial) a
-  load_rw(M, C, 4 * p + 2, s, g.V);
+  P.take(M, ck);
+  P.ask(Ux, mu, s, g.V);
   fx_twice_add<+1>(M, A);
-  fx_load(A, Ui, mu, s, g.V, ck);
+  P.take(A, ck);
   fx_mul_left<FX_WIDE>(A, M, ck);
-  fx_load(M, Ux, mu, s, g.V, ck);
+  P.take(M, ck);
   fx_mul_left<FX_WIDE>(A, M, ck);
   store<fx>(C, 4 * p + 2, s, g.V, A);
   // anything out of range: the whole plaquette again (its slots are its own)

@@ -27,13 +27,14 @@ namespace {
 // cover every plane of a range of sites, so shared neighbours stay in cache.
 inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 1) / bs) * planes)); }
 
-// Resident blocks that the plaquette, clover and force kernels are built for
-// (168 registers).  Per 32^4 step at caps of 144 / 168 / 208, before the clover
-// field and the force were split further: clover and plaquettes 3.33 / 3.00 /
-// 3.37 ms, force 7.37 / 6.49 / 6.98 ms (two blocks at 208; 144 spills more, 420
-// bytes a thread at 168).  Now 2.60 and 6.38 ms; FP64 arithmetic took 11.95 and
-// 26.0 ms.
-const int FX_BLOCKS_SM = 3;
+// Resident blocks of 128 threads that the kernels are built for.  Three (168
+// registers) for the plaquettes and the clover field, whose operands come
+// through the pipe.  Two (255, next to nothing spilled) for the theta force's
+// stages a and b: with the pipe to hide the loads, 5.68 ms per 32^4 step; three blocks
+// spill ~470 bytes a thread and take 6.34 ms without the pipe, 6.98 ms with it
+// (its slots are the spills' L1).  FP64 arithmetic took 26.0 ms, plaquettes and
+// clover field 11.95 (now 2.48).
+const int FX_BLOCKS_SM = 3, FX_BLOCKS_FORCE = 2;
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui) {
   fx_links_body<L>(g, U, Ux, Ui, blockIdx.x);
@@ -57,30 +58,33 @@ __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover(Geo g, con
   fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sre, sim, sm, blockIdx.x);
 }
 template <typename L>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
                                                                     const int4* __restrict__ Ux,
                                                                     const int4* __restrict__ Ui,
                                                                     const int4* __restrict__ Dq, int4* C, double b6) {
-  fx_force_wilson_body<L>(g, U, Ux, Ui, Dq, C, b6, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_force_wilson_body<L>(g, U, Ux, Ui, Dq, C, b6, sm, blockIdx.x);
 }
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_t(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                      const int4* __restrict__ F, int4* C) {
   __shared__ int4 sm[FX_PIPE];
   fx_force_t_body(g, Ux, Ui, F, C, sm, blockIdx.x);
 }
-__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_a(Geo g, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui,
                                                                const int4* __restrict__ Dq,
                                                                const int4* __restrict__ F, int4* Gq, int4* C,
                                                                double b6) {
-  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, sm, blockIdx.x);
 }
 template <typename L>
-__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
+__global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui, const int4* Pq,
                                                                const int4* Dq, const int4* F, const int4* Gq, int4* C,
                                                                double b6) {
-  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, blockIdx.x);
+  __shared__ int4 sm[FX_PIPE];
+  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sm, blockIdx.x);
 }
 template <typename L, int MODE>
 __global__ void __maxnreg__(UPDATE_MAXNREG) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
