@@ -87,7 +87,8 @@ __device__ __forceinline__ void load_herm_mat(mat<double>& m, tagged_herm f, int
 // G_x = sum_mu (U U^+ - U^+_{x-mu} U_{x-mu}) as 60-bit integers: diagonal, and
 // re / im of 01, 02, 12.
 struct fx_gradient {
-  long long d[3], o[6];
+  long long d[3], o[6];  // times 2^-e, below one
+  int e;
 };
 // rows (or conjugated columns) r0, r1, r2 of one link: += sign r_i conj(r_j); n: their squares in float
 __device__ __forceinline__ void fx_outer(fx_acc* D, fx_acc* O, float* n, cx<fx> r0, cx<fx> r1, cx<fx> r2, bool neg) {
@@ -236,17 +237,38 @@ __device__ __forceinline__ void fx_exp_sum(fx_herm& om, const fx_exp_series& S, 
 }
 
 // H = 4 c (G - Tr G / 3), c = -eps alpha_ad (f_a lambda_a = 4 (G - Tr G / 3)).
+// Only the product c G has to fit: c goes in as c 2^t, in [1/2, 1), and G as
+// G 2^-t.  (With c itself as the factor, f >= 1.44 or c >= 0.36 sent a site and
+// with it the links around it through FP64; fields of norm 1.01, where cooled
+// chains live, have some such f at every other site.)
+__device__ __forceinline__ int fx_strength_exponent(double c) {
+  const int e = (__double2hiint(c) >> 20) & 0x7ff;
+  return max(-24, min(24, 1022 - e));
+}
+__device__ __forceinline__ double fx_scaled_double(double x, int t) {  // x 2^t for t within 64 of zero
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0x7ff) return x;
+  if (e < 65) return 0.0;
+  return e > 1980 ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double(hi + t * (1 << 20), __double2loint(x));
+}
+// v 2^-n
+__device__ __forceinline__ fx fx_shifted(long long v, int n, fx_chk& ck) {
+  const long long w = n >= 0 ? v >> n : v << -n;
+  if (n < 0 && (w >> -n) != v) ck.fail();
+  ck.see<FX_WIDE>((int)(w >> 32));
+  return fx_of_bits(w);
+}
 __device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradient& G, double c) {
   fx_chk ck;
   unsigned mag = 0;
-  const fx_left c4 = fx_lhs(fx_of_double(4.0 * c, mag));
+  const int t = fx_strength_exponent(4.0 * c);
+  const fx_left c4 = fx_lhs(fx_of_double(fx_scaled_double(4.0 * c, t), mag));
   const long long third = (G.d[0] + G.d[1] + G.d[2]) / 3;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const long long v = k < 3 ? G.d[k] - third : G.o[k - 3];
-    ck.see<FX_WIDE>((int)(v >> 32));
     fx_acc a = fx_zero();
-    fx_mac(a, c4, fx_rhs(fx_of_bits(v)));
+    fx_mac(a, c4, fx_rhs(fx_shifted(v, t - G.e, ck)));
     const fx w = fx_get<FX_WIDE>(a, ck);
     const int q = (k - 3) >> 1;
     if (k < 3)
@@ -259,21 +281,24 @@ __device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradien
   return !ck.bad() && fx_mag_ok(mag);
 }
 // The same from f: H = c f_a lambda_a.
-__device__ __forceinline__ fx fx_of_real(double x, unsigned& mag) { return fx_of_double(x, mag); }
-__device__ __forceinline__ fx fx_of_real(float x, unsigned& mag) {
+__device__ __forceinline__ fx fx_of_real(double x, int t, unsigned& mag) { return fx_of_double(fx_scaled_double(x, -t), mag); }
+__device__ __forceinline__ fx fx_of_real(float x, int t, unsigned& mag) {
+  x *= __int_as_float((127 - t) << 23);
   if (!(fabsf(x) < 1.4375f)) mag = 0xffffffffu;
   return fx_of_float(x);
 }
 template <typename T>
-__device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const T* f, double c) {
+__device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const T* f, double c0) {
   fx_chk ck;
   unsigned mag = 0;
+  const int t = fx_strength_exponent(c0);
+  const double c = fx_scaled_double(c0, t);
   const fx_left cl = fx_lhs(fx_of_double(c, mag)), cn = fx_lhs(fx_of_double(-c, mag)),
                 c3 = fx_lhs(fx_of_double(c * 0.57735026918962576451, mag)),
                 m3 = fx_lhs(fx_of_double(-2.0 * (c * 0.57735026918962576451), mag));
   fx_right F[8];
 #pragma unroll
-  for (int a = 0; a < 8; ++a) F[a] = fx_rhs(fx_of_real(f[a], mag));
+  for (int a = 0; a < 8; ++a) F[a] = fx_rhs(fx_of_real(f[a], t, mag));
   auto one = [&](const fx_left& x, const fx_right& y) {
     fx_acc s = fx_zero();
     fx_mac(s, x, y);

@@ -367,9 +367,19 @@ __device__ __forceinline__ bool sweep_gradient(fx_gradient& G, const SweepPart<L
   for (int i = 0; i < 3; ++i) G.d[i] = sweep_sum(sm, i);
 #pragma unroll
   for (int i = 0; i < 6; ++i) G.o[i] = sweep_sum(sm, 3 + i);
-  // |G| below 1, as everything formed from it expects
+  // |G| below 1, as everything formed from it expects: an eighth of it if need be
+  bool one = true;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && fx_below_one(G.d[k]) && fx_below_one(G.o[2 * k]) && fx_below_one(G.o[2 * k + 1]);
+  for (int k = 0; k < 3; ++k) one = one && fx_below_one(G.d[k]) && fx_below_one(G.o[2 * k]) && fx_below_one(G.o[2 * k + 1]);
+  G.e = one ? 0 : 3;
+  if (!one) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      G.d[k] >>= 3;
+      G.o[2 * k] >>= 3;
+      G.o[2 * k + 1] >>= 3;
+    }
+  }
   return ok;
 }
 __device__ __forceinline__ void sweep_f(float* fa, const float* q) {
@@ -450,14 +460,14 @@ __device__ __forceinline__ void sweep_grad_site(SweepSums& v, const SweepPart<L,
           o += G.o[k] < 0 ? -G.o[k] : G.o[k];
           const fx w = fx_of_bits(G.o[k]);
           fx_mac(sq, fx_lhs(w), fx_rhs(w));
-          const double d = fx_bits_to_double(G.o[k], 2);
+          const double d = fx_bits_to_double(G.o[k], 2 + G.e);
           fa[k < 2 ? k : k + 1] = (k & 1) ? -d : d;
         }
         const long long d01 = G.d[0] - G.d[1], d2 = G.d[0] + G.d[1] - 2 * G.d[2];
-        fa[2] = fx_bits_to_double(d01, 1);
-        fa[7] = fx_bits_to_double(d2, 1) * 0.57735026918962576451;
+        fa[2] = fx_bits_to_double(d01, 1 + G.e);
+        fa[7] = fx_bits_to_double(d2, 1 + G.e) * 0.57735026918962576451;
         if (with_f) {
-          v.x += fx_bits_to_double(o, 2) + (fabs(fa[2]) + fabs(fa[7]));
+          v.x += fx_bits_to_double(o, 2 + G.e) + (fabs(fa[2]) + fabs(fa[7]));
           // (f_2 / 4)^2 + (f_7 / 4)^2 with f_2 / 4 = d01 / 2, f_7 / 4 = d2 / (2 sqrt 3)
           const fx w2 = fx_of_bits(d01 >> 1);
           unsigned mag = 0;
@@ -467,7 +477,7 @@ __device__ __forceinline__ void sweep_grad_site(SweepSums& v, const SweepPart<L,
           const fx w7 = fx_twice(fx_twice(fx_get<FX_WIDE>(z, ck)));
           fx_mac(sq, fx_lhs(w2), fx_rhs(w2));
           fx_mac(sq, fx_lhs(w7), fx_rhs(w7));
-          v.y += fx_bits_to_double(fx_sum(sq) - (1 << 29), 4);
+          v.y += fx_bits_to_double(fx_sum(sq) - (1 << 29), 4 + 2 * G.e);
         }
         // the unitarity norm; later gradients of D_2 calls need it too
         long long dev = 0;  // of the three diagonals from 4, 2^-58
