@@ -217,7 +217,7 @@ struct sweep_real { typedef typename std::conditional<is_fx<L>(), long long, flo
 template <typename L, int N>
 struct SweepPart {
   typename sweep_real<L>::type q[N][CS_THREADS];
-  int ok[CS_THREADS];
+  float top[CS_THREADS];  // fixed point: largest row or column norm (squared); infinite: not representable
 };
 
 // FP32 storage: the ten numbers of direction mu at site s (sb: the site behind).
@@ -269,6 +269,57 @@ __device__ __forceinline__ void sweep_sums_f32(float* q, bool with_norm, const G
     for (int i = 0; i < 10; ++i)
       if (i < 9 || with_norm) q[i] += p[i];
   }
+}
+
+// Entries beyond the fixed-point bound, up to 2^K times it (chains whose links
+// have skirts keep a few such): the link times 2^-K, from its words or doubles.
+template <int K>
+__device__ __forceinline__ bool fx_load_wild(mat<fx>& u, const int4* Ux, int mu, int s, int V) {
+  fx_load_plain(u, Ux, mu, s, V);
+  unsigned mag = 0;
+  if (fx_is_raw(u.e[0].re.l)) {
+    mat<double> d;
+    load(d, tagged{const_cast<int4*>(Ux), 1.0}, mu, s, V);
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      u.e[k] = cx<fx>{fx_of_double(fx_scaled_double(d.e[k].re, -K), mag), fx_of_double(fx_scaled_double(d.e[k].im, -K), mag)};
+  } else {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_bits(fx_bits(u.e[k].re) >> K), fx_of_bits(fx_bits(u.e[k].im) >> K)};
+  }
+  return fx_mag_ok(mag);
+}
+// A thread's part of the gradient where a link of it is beyond the bound: both
+// links times 1/4, the sums times 16.  (In FP64 the site's eight links are one
+// thread's chain of ~600 instructions: 20 us a sweep for the whole launch.)
+static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* top, const int4* Ux, int mu, int s, int sb, int V) {
+  fx_acc D[3], O[6];
+  float nf[3] = {0.0f, 0.0f, 0.0f}, nb[3] = {0.0f, 0.0f, 0.0f}, m = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) D[i] = fx_zero();
+#pragma unroll
+  for (int i = 0; i < 6; ++i) O[i] = fx_zero();
+  mat<fx> u;
+  if (!fx_load_wild<2>(u, Ux, mu, s, V)) return;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) fx_outer(D, O, nf, u.e[k], u.e[3 + k], u.e[6 + k], false);
+  if (n > 9)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) q[(9 + i) * CS_THREADS] = (fx_sum<true>(D[i]) - (1 << 29)) << 4;
+  if (!fx_load_wild<2>(u, Ux, mu, sb, V)) return;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const cx<fx> a = u.e[3 * k], b = u.e[3 * k + 1], c = u.e[3 * k + 2];
+    fx_outer(D, O, nb, cx<fx>{a.re, -a.im}, cx<fx>{b.re, -b.im}, cx<fx>{c.re, -c.im}, true);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    q[i * CS_THREADS] = (fx_sum<true>(D[i]) - (1 << 29)) << 4;
+    m = fmaxf(m, fmaxf(nf[i], nb[i]));
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) q[(3 + i) * CS_THREADS] = (fx_sum<true>(O[i]) - (1 << 29)) << 4;
+  *top = m * 0x1p-56f;
 }
 
 // First half: this thread's direction (warp) and site.  FIRST: the links are
@@ -337,15 +388,16 @@ __device__ __forceinline__ void sweep_part(SweepPart<L, N>& sm, const Geo& g, co
       const cx<fx> p = u.e[3 * k], q = u.e[3 * k + 1], r = u.e[3 * k + 2];
       fx_outer(D, O, nb, cx<fx>{p.re, -p.im}, cx<fx>{q.re, -q.im}, cx<fx>{r.re, -r.im}, true);
     }
-    // sums over the four directions must stay below 8: rows and columns below 1.9 each
+    float top = 0.0f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       sm.q[i][t] = fx_sum<true>(D[i]) - (1 << 29);
-      ok = ok && nf[i] < 1.9f * 0x1p60f && nb[i] < 1.9f * 0x1p60f;
+      top = fmaxf(top, fmaxf(nf[i], nb[i]));
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i) sm.q[3 + i][t] = fx_sum<true>(O[i]) - (1 << 29);
-    sm.ok[t] = ok && !ck.bad();
+    sm.top[t] = ok && !ck.bad() ? top * 0x1p-60f : __int_as_float(0x7f800000);
+    if (!FIRST && ck.bad()) sweep_part_wild(&sm.q[0][t], N, &sm.top[t], Ux, mu, s, sb, g.V);
   } else {
     float q[N];
     sweep_part_f32(q, N > 9, (const V2*)a.U, mu, s, sb, g.V);
@@ -362,7 +414,8 @@ __device__ __forceinline__ typename sweep_real<L>::type sweep_sum(const SweepPar
 template <typename L, int N>
 __device__ __forceinline__ bool sweep_gradient(fx_gradient& G, const SweepPart<L, N>& sm) {
   const int l = threadIdx.x & 31;
-  bool ok = sm.ok[l] && sm.ok[32 + l] && sm.ok[64 + l] && sm.ok[96 + l];
+  // the sums over the four directions must stay below 8
+  const bool ok = ((sm.top[l] + sm.top[32 + l]) + sm.top[64 + l]) + sm.top[96 + l] < 7.6f;
 #pragma unroll
   for (int i = 0; i < 3; ++i) G.d[i] = sweep_sum(sm, i);
 #pragma unroll
@@ -752,6 +805,26 @@ static __device__ __noinline__ double general_cool_apply(const Geo g, int4* Ux, 
 // Norms are summed as integers, exactly, within a record: a link's Tr U U^+ - 3
 // (below 1.9) in units of 2^(sh - 60), so that R groups of 128 links fit; links
 // beyond that (wild) in FP64.
+// The apply is linear in the link: one beyond the bound goes through it times
+// 1/8, and back into fixed point where it fits.  Returns Tr U U^+.
+static __device__ __noinline__ double far_cool_apply(const Geo g, int4* Ux, int2* Om, int2* Omi, int mu, int s, int sp) {
+  fx_chk ck;
+  fx_herm o, oi;
+  mat<fx> u;
+  fx_load_herm(o, Om, s, g.V, ck);
+  fx_load_herm(oi, Omi, sp, g.V, ck);
+  if (!fx_load_wild<3>(u, Ux, mu, s, g.V)) ck.fail();
+  fx_apply_ops ops;
+  fx_lhs(ops, o);
+  long long dev = 0;
+  fx_apply_link<false>(u, ops, oi, ck, dev);
+  if (ck.bad()) return general_cool_apply(g, Ux, Om, Omi, mu, s, sp);
+  mat<double> d;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) d.e[k] = cx<double>{fx_to_double(u.e[k].re, 3), fx_to_double(u.e[k].im, 3)};
+  store(tagged{Ux, 1.0}, mu, s, g.V, d);
+  return norm2(d);
+}
 // A thread's next link and its two Omegas on their way into shared memory while
 // it works on the current ones (lattices where a block takes several groups:
 // apply of a 32^4 step of ten sweeps 4.03 -> 3.36 ms).
@@ -778,7 +851,6 @@ struct sweep_pipe {
       u.e[k] = unpack(sm[k * CS_THREADS]);
       h[k] = sm[(9 + k) * CS_THREADS];
     }
-    if (fx_is_raw(u.e[0].re.l)) ck.fail();
     int2 w[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) w[k] = make_int2(h[k].x, h[k].y);
@@ -843,8 +915,8 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
         fx_load_herm(o, (const int2*)a.Om, s, g.V, ck);
         fx_load_herm(oi, (const int2*)a.Omi, sp, g.V, ck);
         fx_load_plain(u, Ux, mu, s, g.V);
-        if (fx_is_raw(u.e[0].re.l)) ck.fail();
       }
+      if (fx_is_raw(u.e[0].re.l)) ck.fail();
       fx_apply_ops ops;
       fx_lhs(ops, o);
       long long dev = 0;
@@ -854,7 +926,7 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
         if (!last || !RULE) store<fx>(Ux, mu, s, g.V, u);  // D_2 calls end with a gradient
         acc += dev >> sh;
       } else {
-        wild += general_cool_apply(g, Ux, (int2*)a.Om, (int2*)a.Omi, mu, s, sp) - 3.0;
+        wild += far_cool_apply(g, Ux, (int2*)a.Om, (int2*)a.Omi, mu, s, sp) - 3.0;
         nwild = 1;
         if (last) unload_link(U, Ux, mu, s, g.V);
       }
@@ -880,31 +952,43 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
   if constexpr (RULE) {
     if (stopped) return;
     __shared__ long long sums[CS_THREADS / 32];
-    __shared__ double wilds[CS_THREADS];
+    __shared__ double wilds[CS_THREADS / 32];
+    const auto warp_sum = [](double w) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
+      return w;
+    };
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = acc;
-    wilds[threadIdx.x] = wild;
+    const bool any_warp = __any_sync(0xffffffffu, nwild != 0);
+    const double w = any_warp ? warp_sum(wild) : 0.0;
+    if ((threadIdx.x & 31) == 0) {
+      sums[threadIdx.x >> 5] = acc;
+      wilds[threadIdx.x >> 5] = w;
+    }
     const int any = __syncthreads_or(nwild);
     SweepNorm* n = sweep_norm(a, g.V);
     if (threadIdx.x == 0) {
       const long long t = sums[0] + sums[1] + sums[2] + sums[3];
       atomicAdd(&n->hi, (unsigned long long)(t >> 20));
       atomicAdd(&n->lo, (unsigned long long)(t & 0xfffff));
-      double w = 0.0;
-      if (any) {
-        for (int j = 0; j < CS_THREADS; ++j) w += wilds[j];
-        atomicAdd(&n->wild, 1u);
-      }
-      __stcg(a.rec + 2 * vb, make_double2(w, 0.0));
+      if (any) atomicAdd(&n->wild, 1u);
+      __stcg(a.rec + 2 * vb, make_double2(any ? (wilds[0] + wilds[1]) + (wilds[2] + wilds[3]) : 0.0, 0.0));
     }
     const int nb = cs_apply_blocks(g.V);
-    if (!sweep_last(a, nb) || threadIdx.x != 0) return;
+    if (!sweep_last(a, nb)) return;
+    double far = 0.0;  // links beyond the bound, by the whole block
+    if (__ldcg(&n->wild) != 0u) {
+      for (int b = threadIdx.x; b < nb; b += CS_THREADS) far += __ldcg(a.rec + 2 * b).x;
+      far = warp_sum(far);
+      if ((threadIdx.x & 31) == 0) wilds[threadIdx.x >> 5] = far;
+      __syncthreads();
+      far = (wilds[0] + wilds[1]) + (wilds[2] + wilds[3]);
+    }
+    if (threadIdx.x != 0) return;
     const CoolState old = *a.cs;
     const long long hi = (long long)__ldcg(&n->hi), lo = (long long)__ldcg(&n->lo);
-    double dev = fx_bits_to_double(hi, sh + 20) + fx_bits_to_double(lo, sh);
-    if (__ldcg(&n->wild) != 0u)
-      for (int b = 0; b < nb; ++b) dev += __ldcg(a.rec + 2 * b).x;
+    const double dev = fx_bits_to_double(hi, sh + 20) + fx_bits_to_double(lo, sh) + far;
     cool_rule(1.0 + dev * ((1.0 / 3.0) * a.ca.inv_links), 0.0, 0.0, false, a.ca, old, a.cs, 0);
     *n = SweepNorm{0ull, 0ull, 0u, 0u};
     *a.ticket = 0u;

@@ -382,6 +382,7 @@ __device__ __forceinline__ double fx_raw_first(int2 v) { return __hiloint2double
 struct tagged {
   int4* p;
   double sc;
+  unsigned lim = 0x3FF70000u;  // words below this (high word of a double; 1.4375)
 };
 __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int site, int V) {
   const int4* p = f.p + (size_t)plane * 9 * V + site;
@@ -400,14 +401,25 @@ __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int si
     a.e[k].im *= f.sc;
   }
 }
+// In fixed point where it fits, so that one number out of range does not send
+// its readers the same way.
 __device__ __forceinline__ void store(tagged f, int plane, int site, int V, const mat<double>& a) {
   int4* p = f.p + (size_t)plane * 9 * V + site;
   const double isc = 1.0 / f.sc;
+  unsigned mag = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    mag = max(mag, max((unsigned)__double2hiint(a.e[k].re * isc) & 0x7fffffffu, (unsigned)__double2hiint(a.e[k].im * isc) & 0x7fffffffu));
+  const bool fits = mag < f.lim;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const double re = a.e[k].re * isc, im = a.e[k].im * isc;
-    const int2 w = k == 0 ? fx_raw_first(re) : make_int2(__double2loint(re), __double2hiint(re));
-    p[(size_t)k * V] = make_int4(w.x, w.y, __double2loint(im), __double2hiint(im));
+    if (fits) {
+      p[(size_t)k * V] = pack(cx<fx>{fx_of_double(re, mag), fx_of_double(im, mag)});
+    } else {
+      const int2 w = k == 0 ? fx_raw_first(re) : make_int2(__double2loint(re), __double2hiint(re));
+      p[(size_t)k * V] = make_int4(w.x, w.y, __double2loint(im), __double2hiint(im));
+    }
   }
 }
 

@@ -10,13 +10,14 @@
 // the pair 02|13), C is 2^-e times the contribution.
 //
 // A thread whose inputs or results leave the fixed-point range calls the
-// general path, the FP64 bodies of k_update.cuh on the same fields, for its
-// plaquette; that code is out of line and costs the others nothing.
+// general path, FP64 on the same fields (the whole warp for one plaquette,
+// general_warp.cuh, or the bodies of k_update.cuh), for its plaquette; that code is out of line and costs the others nothing.
 //
 // Scales that keep every number within the fixed-point bound: D is stored
 // halved (|D| < 2.9), the clover sum is formed as an eighth of F.
 #pragma once
 #include "fixed.cuh"
+#include "general_warp.cuh"
 #include "k_update.cuh"
 #include "link_fx.cuh"
 #include "noise_fx.cuh"
@@ -25,6 +26,7 @@ namespace clgc {
 
 // Fields of the general path.
 __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
+__device__ __forceinline__ tagged tag_F(int4* f) { return tagged{f, 1.0, 0x3FD70000u}; }  // 0.359375 (FX_NARROW)
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
@@ -89,7 +91,8 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
 #pragma unroll
   for (int k = 0; k < 9; ++k) Pm.e[k] = cx<fx>{fx_half_diff(Pm.e[k].re, b.e[k].re), fx_half_diff(Pm.e[k].im, b.e[k].im)};
   store<fx>(Dq, p, s, g.V, Pm);
-  if (ck.bad()) general_plaq<L>(g, U, tag(Pq), tag_D(Dq), vb);
+  general_path(ck.bad(), s, g.V, [&](unsigned m, int t) { warp_plaq<L>(m, g, U, tag(Pq), tag_D(Dq), p, t); },
+               [&] { general_plaq<L>(g, U, tagged{Pq, 1.0, 0u}, tag_D(Dq), vb); });
 }
 
 // ------------------------------------------------------------ clover field
@@ -166,7 +169,9 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
     acc.e[k] = cx<fx>{fx_get<FX_NARROW>(re, ck), fx_get<FX_NARROW>(im, ck)};
   }
   store<fx>(F, p, s, g.V, acc);
-  if (ck.bad() || !fx_mag_ok(mag)) general_clover<L>(g, U, tag_D(Dq), tag(F), sre, sim, vb);
+  general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
+               [&](unsigned m, int t) { warp_clover<L>(m, g, U, tag_D(Dq), tag_F(F), sre, sim, p, t); },
+               [&] { general_clover<L>(g, U, tag_D(Dq), tag_F(F), sre, sim, vb); });
 }
 
 // ------------------------------------------------------- plaquette drift
@@ -209,7 +214,9 @@ __device__ __forceinline__ void fx_force_wilson_body(Geo g, const typename vec2_
   P.take(a, ck);
   fx_mul_left<FX_WIDE>(t, a, ck);
   store<fx>(C, 4 * p + 2, s, g.V, t);
-  if (ck.bad() || !fx_mag_ok(mag)) general_force_wilson<L>(g, U, tag_D(Dq), tag(C), b6, vb);
+  general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
+               [&](unsigned m, int t) { warp_force_wilson<L>(m, g, U, tag_D(Dq), tag(C), b6, p, t); },
+               [&] { general_force_wilson<L>(g, U, tag_D(Dq), tag(C), b6, vb); });
 }
 
 // The dual field of plaquette p's corner c3 carried to its base point,
@@ -371,7 +378,9 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   fx_mul_left<FX_WIDE>(A, M, ck);
   store<fx>(C, 4 * p + 2, s, g.V, A);
   // anything out of range: the whole plaquette again (its slots are its own)
-  if (ck.bad() || !fx_mag_ok(mag)) general_force<L>(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb);
+  general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
+               [&](unsigned m, int t) { warp_force<L>(m, g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, p, t); },
+               [&] { general_force<L>(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb); });
 }
 
 // --------------------------------------------------------------- gather
@@ -513,15 +522,51 @@ __device__ __forceinline__ double drift_fx(const Geo& g, const int4* C, int4* o,
       fx_mac(n, fx_lhs(Q.e[k].im), fx_rhs(Q.e[k].im));
       nf = fmaf((float)Q.e[k].re.h, (float)Q.e[k].re.h, fmaf((float)Q.e[k].im.h, (float)Q.e[k].im.h, nf));
     }
-    if (nf < 7.5f * 0x1p60f) {
-      if (write) store<fx>(o, MU, s, g.V, Q);
-      return fx_bits_to_double(fx_sum(n) - (1 << 29), 2 * cexp + 5);
-    }
+    if (write) store<fx>(o, MU, s, g.V, Q);
+    write = false;  // the words an update from C would use: the same step bit for bit
+    if (nf < 7.5f * 0x1p60f) return fx_bits_to_double(fx_sum(n) - (1 << 29), 2 * cexp + 5);
   }
   mat<double> Xd;
   gather_f64(Xd, g, s, x, MU, C, cexp);
-  if (write) store(tagged{o, ldexp(1.0, cexp + 2)}, MU, s, g.V, Xd);
+  if (write) store(tagged{o, ldexp(1.0, cexp + 2), 0u}, MU, s, g.V, Xd);  // doubles: words are the traceless quarter
   return general_k2(Xd);
+}
+
+// The general update's X from the contributions, as drift_fx would have stored it.
+static __device__ __noinline__ void general_operand(mat<double>& X, const Geo g, int s, const int* x, int MU, const int4* C,
+                                                    int cexp) {
+  long long v[18];
+  mat<fx> Q;
+  if (fx_gather(v, g, s, x, MU, C) && fx_traceless_quarter(Q, v)) {
+    const double sc = ldexp(1.0, cexp + 2);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X.e[k] = cx<double>{fx_to_double(Q.e[k].re) * sc, fx_to_double(Q.e[k].im) * sc};
+  } else {
+    gather_f64(X, g, s, x, MU, C, cexp);
+  }
+}
+
+// An eighth of a link beyond the fixed-point range (exp(A) U is linear in it),
+// and the end of its update.
+template <typename L>
+static __device__ __noinline__ bool fx_link_eighth(mat<fx>& u, const typename vec2_of<L>::type* U, int mu, int s, int V) {
+  mat<double> d;
+  load_link_d<L>(d, U, mu, s, V);
+  unsigned mag = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    u.e[k] = cx<fx>{fx_of_double(0.125 * d.e[k].re, mag), fx_of_double(0.125 * d.e[k].im, mag)};
+  return fx_mag_ok(mag);
+}
+template <class V2>
+static __device__ __noinline__ void update_far(V2* out, const mat<fx>& W, int mu, int s, int V) {
+  mat<double> d;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) d.e[k] = cx<double>{fx_to_double(W.e[k].re, 3), fx_to_double(W.e[k].im, 3)};
+  const cx<double> z = det_inv_cuberoot(det(d));
+#pragma unroll
+  for (int k = 0; k < 9; ++k) d.e[k] = cmul(d.e[k], z);
+  store_link(out, mu, s, V, d);
 }
 
 // The whole update in fixed point: exp(A) U with U the fixed-point word that
@@ -564,8 +609,14 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
       fx_chk ck;
       mat<fx> u;
       fx_load_plain(u, reinterpret_cast<const int4*>(out), MU, s, g.V);
-      if (fx_is_raw(u.e[0].re.l)) ck.fail();
+      const bool far = fx_is_raw(u.e[0].re.l);
+      if (far && !fx_link_eighth<L>(u, U, MU, s, g.V)) ck.fail();
       fx_mul_left<FX_WIDE>(A, u, ck);
+      if (far && !ck.bad()) {
+        const mat<fx> W = A;  // a local of its own: its address goes out of line
+        update_far(out, W, MU, s, g.V);
+        return;
+      }
       const cx<fx> e = fx_det_minus_one(A, ck);
       if (!ck.bad() && e.re.h == 0 && e.im.h == 0) {
         const float er = e.re.l * (-1.0f / 3.0f), ei = e.im.l * (-1.0f / 3.0f);  // units of 2^-60
@@ -583,7 +634,7 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
   }
   mat<double> Xg, u, r;
   if (C)
-    gather_f64(Xg, g, s, x, MU, C, a.cexp);
+    general_operand(Xg, g, s, x, MU, C, a.cexp);
   else
     load(Xg, Xt, MU, s, g.V);
   load_link_d<L>(u, U, MU, s, g.V);
