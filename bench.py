@@ -48,9 +48,10 @@ CPU_SAMPLE_L = (8, 8, 8, 8)
 # Box-Muller noise are not counted).  Building blocks: 3x3 complex product
 # 198, product-accumulate 216, adjugate 126, Hermitian-times-general 162.
 # ncu's executed-instruction counters agree within 1 % on these sources
-# (profiles/ncu_fp64_counts_24x4.md).  "pipe" is the unit the kernel loads:
-# the FP64 pipe in the FP64 form; in the FP32-storage form only the
-# exponentials, the re-projection and the cooling Omega stay on it.
+# (profiles/ncu_fp64_counts_24x4.md, taken when this arithmetic was FP64).
+# "pipe" is what the kernel loads: the FP64 and DF64 forms, and the FP32-storage
+# form's exponentials, re-projection and cooling Omega, run in fixed point on the
+# integer and FP32 pipes ("fixed"); the rest of the FP32-storage form is FP32.
 MUL, MULACC, ADJ, HERM = 198, 216, 126, 162
 
 
@@ -65,13 +66,15 @@ FP32_STORAGE_FP64_FLOPS = {"update": 4 * 663, "cool_omega": 163, "cool_grad_omeg
 def flop_model(prec, theta_on=True, n_taylor=15):
     expm = MUL + 6 + 72 + 36 + 16 * n_taylor + 9 * (6 + 8) + 6  # Cayley-Hamilton + Horner
     det_root = 64 + 19                                           # det + three-term cube-root series
-    if theta_on:
-        force = 6 * (12 * MUL + ADJ + 9 * MULACC + 162)          # per-plaquette drift, 6 planes
+    if theta_on and prec == "fp64":
+        force = 6 * (11 * MUL + 9 * MULACC + 162)                # per-plaquette drift, 6 planes, corner transport shared
+    elif theta_on:
+        force = 6 * (12 * MUL + ADJ + 9 * MULACC + 162)
     else:
         force = 6 * (4 * MUL + 36)
     m = {
         "force": force,
-        "clover": 4 * ADJ + 6 * (3 * MUL + ADJ + 18) + (6 * (3 * (MUL + MULACC) + 54) if theta_on else 0),
+        "clover": 4 * ADJ + 6 * (3 * MUL + ADJ + 18) + (6 * ((2 if prec == "fp64" else 3) * (MUL + MULACC) + 54) if theta_on else 0),
         "cool_grad": 914,
         "cool_omega": 209,
         "cool_apply": 4 * 2 * HERM,
@@ -79,18 +82,13 @@ def flop_model(prec, theta_on=True, n_taylor=15):
     }
     if prec == "fp64":
         m["update"] = 4 * (12 * 18 + 32 + 38 + expm + MUL + det_root + 54)
-        pipe = {k: "fp64" for k in m}
+        pipe = {k: "fixed" for k in m}
     else:
         pipe = {k: "fp32" for k in m}
         for k, v in FP32_STORAGE_FP64_FLOPS.items():  # FP64 part only
             m[k] = v
-            pipe[k] = "fp64"
+            pipe[k] = "fixed"
     return m, pipe
-
-
-def fp64_peak_tflops(sm_max_mhz):
-    # 152 SMs x 2 FP64 FMA per SM per clock (4 flops) x clock: 1.259 TFLOP/s at 2070 MHz.
-    return 152 * 4 * sm_max_mhz * 1e6 / 1e12
 
 
 def measured_peaks():
@@ -104,10 +102,10 @@ def measured_peaks():
 
 # The sources of the kernels the bench launches (their launch shapes included);
 # the host runtime, the server and the chain kernel do not change them.
-KERNEL_SOURCES = ("bm_tables.cuh", "df64.cuh", "expm.cuh", "k_update.cuh", "k_update_df64.cu", "k_update_f32.cu",
-                  "k_update_f64.cu",
-                  "kernels.cu", "launch.h",
-                  "lattice.cuh", "philox.cuh", "su3.cuh")
+KERNEL_SOURCES = ("bm_tables.cuh", "cool_fx.cuh", "cool_sweep.cuh", "df64.cuh", "expm.cuh", "expm_fx.cuh", "fixed.cuh",
+                  "general_warp.cuh", "k_update.cuh", "k_update_df64.cu", "k_update_f32.cu", "k_update_f64.cu",
+                  "k_update_fx.cuh", "k_update_fx_launch.cuh", "kernels.cu", "launch.h", "lattice.cuh", "link_fx.cuh",
+                  "noise_fx.cuh", "noise_fx_tables.cuh", "philox.cuh", "su3.cuh")
 
 
 def kernel_source_hash():
@@ -152,6 +150,14 @@ TRAFFIC_FAMILIES = {
              "update": ("k_update_gather<df64, 0>",), "cool_apply": ("k_cool_apply_df",),
              "cool_grad": ("k_cool_grad_df",), "cool_omega": ("k_cool_omega<df64>",)},
 }
+
+
+# The same under the kernels' present names (the ones above are those of older launch lists).
+TRAFFIC_FAMILIES_FX = {
+    form: {"force": ("k_fx_force_t", "k_fx_force_a", "k_fx_force_b<%s>" % t), "update": ("k_fx_update<%s, 0>" % t,),
+           "cool_apply": ("k_cool_apply<%s, 1>" % t,), "cool_grad_omega": ("k_cool_grad_omega<%s, 3>" % t,)}
+    for form, t in (("fp64", "double"), ("df64", "df64"))}
+TRAFFIC_FAMILIES_FX["fp32"] = {"cool_apply": ("k_cool_apply<float, 1>",), "cool_grad_omega": ("k_cool_grad_omega<float, 4>",)}
 
 
 def ingest_ncu(path, out_json=None, capture_sites=None):
@@ -203,7 +209,7 @@ def ingest_ncu(path, out_json=None, capture_sites=None):
     out = {"source_hash": h}
     if capture_sites:
         out["capture_sites"] = capture_sites
-    for form, fams in TRAFFIC_FAMILIES.items():
+    for form, fams in list(TRAFFIC_FAMILIES.items()) + list(TRAFFIC_FAMILIES_FX.items()):
         for fam, kernels in fams.items():
             if all(k in agg for k in kernels):
                 b = sum((agg[k]["rd"] + agg[k]["wr"]) / agg[k]["n"] for k in kernels)
@@ -382,18 +388,11 @@ def e2e_measure(cl, torch, lat, V, one_step, steps):
                                  "step_and_get_links": round(t_get / steps * 1e3, 3)}}
 
 
-# FP32 instructions per site that the DF64 kernels execute, from ncu's
-# executed-instruction counters on one launch at 24^4
-# (smsp__sass_thread_inst_executed_op_{ffma,fadd,fmul}_pred_on.sum divided by
-# the 331,776 sites; profiles/ncu_df64_fp32_ops_24x4.md).  These kernels load
-# the FP32 pipe, so their roofline is that pipe: flops (FFMA = 2) against the
-# FP32 peak, and FP32-pipe instructions against the pipe's issue rate (the
-# error-free transformations are mostly FADDs, one flop per issue slot).
-DF64_FP32_OPS_PER_SITE = {
-    "force": {"ffma": 43740, "fadd": 126684, "fmul": 14580},
-    "cool_grad": {"ffma": 1323, "fadd": 4211, "fmul": 513},
-    "cool_apply": {"ffma": 2160, "fadd": 5472, "fmul": 720},
-}
+def fixed_peak_tflops(sm_max_mhz):
+    # A real multiply-accumulate in fixed point takes 6 dispatch cycles of a scheduler for a warp (IMAD.WIDE and
+    # the 64-bit add and the packed FFMA2, two cycles each): 152 SMs x 4 schedulers x 32 lanes / 6 x 2 flops x
+    # clock, 13.4 TFLOP/s at 2070 MHz (the FP64 pipe: 1.26).
+    return 152 * 4 * 32 / 6 * 2 * sm_max_mhz * 1e6 / 1e12
 
 
 def fp32_peak_tflops(sm_max_mhz):
@@ -410,31 +409,11 @@ def roofline_of(prec_name, V, phases, sm_max_mhz, theta_on=True):
     dom = max(single, key=lambda k: single[k][0])
     ms_tot, n = phases[dom]
     per = ms_tot / max(n, 1)
-    if prec_name == "df64":
-        # double-float arithmetic runs on the FP32 pipe: its executed FP32
-        # operations (ncu counts) against the FP32 peak
-        ops = DF64_FP32_OPS_PER_SITE.get(dom)
-        peak = fp32_peak_tflops(sm_max_mhz)
-        src = ("executed FP32 operations of the double-float kernels (ncu, 24^4, FFMA = 2 flops) against "
-               "152 SMs x 128 FP32 FMA/clk x %d MHz (FP32 is not in MEASURED_PEAKS.json)" % sm_max_mhz)
-        if not ops:
-            return {"kernel": dom, "bound": "alu", "pipe": "fp32", "achieved": None, "peak": round(peak, 4),
-                    "unit": "TFLOP/s", "frac": None, "traffic": dram_traffic(dom, prec_name, V),
-                    "avg_launch_ms": round(per, 4), "launches": n, "peak_source": src}
-        flops = (2 * ops["ffma"] + ops["fadd"] + ops["fmul"]) * V
-        inst = (ops["ffma"] + ops["fadd"] + ops["fmul"]) * V
-        ach = flops / (per * 1e-3) / 1e12
-        inst_rate = inst / (per * 1e-3) / 1e12
-        inst_peak = peak / 2
-        return {"kernel": dom, "bound": "alu", "pipe": "fp32", "achieved": round(ach, 4),
-                "peak": round(peak, 4), "unit": "TFLOP/s", "frac": round(ach / peak, 4),
-                "fp32_pipe_inst_per_s": round(inst_rate * 1e12, 1), "fp32_pipe_inst_frac": round(inst_rate / inst_peak, 4),
-                "traffic": dram_traffic(dom, prec_name, V), "flops_per_launch": flops,
-                "avg_launch_ms": round(per, 4), "launches": n, "peak_source": src}
     flops = fm[dom] * V
-    if pipe[dom] == "fp64":
-        peak = fp64_peak_tflops(sm_max_mhz)
-        src = "152 SMs x 2 FP64 FMA/clk x %d MHz (FP64 is not in MEASURED_PEAKS.json)" % sm_max_mhz
+    if pipe[dom] == "fixed":
+        peak = fixed_peak_tflops(sm_max_mhz)
+        src = ("152 SMs x 4 schedulers x 32 lanes, 6 dispatch cycles a fixed-point multiply-accumulate, x %d MHz "
+               "(not in MEASURED_PEAKS.json)" % sm_max_mhz)
     else:
         peak = fp32_peak_tflops(sm_max_mhz)
         src = "152 SMs x 128 FP32 FMA/clk x %d MHz" % sm_max_mhz
@@ -476,7 +455,7 @@ def native(args):
                    "beta": WORKLOAD["beta"], "theta": WORKLOAD["theta"], "eps": WORKLOAD["eps"],
                    "cooling": "alpha_ad = alpha / D_1 (normalised unitarity norm), alpha 1, "
                               "10 sweeps per step (fixed count)",
-                   "precision": "fp64 links and arithmetic",
+                   "precision": "fp64 links; products, noise and exponentials in 60-bit fixed point, errors below fp64's",
                    "l2": "no flush: the link fields (604 MB fp64 / 302 MB fp32) exceed the 129 MB L2",
                    "parallelism": "replicas x%d (independent chains)" % ws},
         "gpu_launches": launches,
@@ -511,8 +490,7 @@ def native(args):
         msd = rank_max(msd, "cuda")
         result.setdefault("forms", {})["df64"] = {
             "value": job_value(Vd, msd, ws), "ms_per_step": msd, "gpu_launches": ld,
-            "dtype": "df64 links (hi + lo floats); link algebra, noise, exponentials and re-projection "
-                     "in double-float on the FP32 pipe; f64 final sums of the reductions",
+            "dtype": "df64 links (hi + lo floats); fixed-point link algebra as in the FP64 form",
             "phases_ms_per_step": {k: round(v[0] / args.steps, 4) for k, v in phd.items()},
             "roofline": roofline_of("df64", Vd, phd, sm_max),
             "observables_after": {k: obsd[k] for k in ("plaq_re", "un", "q_re", "q_im")},
