@@ -327,7 +327,7 @@ static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* 
 // PIPE: the links come through a pipe, the forward one asked for by
 // the call for the group before (next; the first group's by the caller), so that each
 // link's load runs under the outer products of the one before (gradient + Omega
-// of a 32^4 step of ten sweeps 2.53 -> 2.30 ms).
+// of a 32^4 step of ten sweeps 2.53 -> 2.37 ms).
 __device__ __forceinline__ void sweep_ask(fx_pipe<1>& P, const Geo& g, const SweepArgs& a, int group) {
   const int mu = threadIdx.x >> 5, s = group * CS_SITES + (threadIdx.x & 31);
   if (s < g.V) P.ask((const int4*)a.Ux, mu, s, g.V);
@@ -827,7 +827,7 @@ static __device__ __noinline__ double far_cool_apply(const Geo g, int4* Ux, int2
 }
 // A thread's next link and its two Omegas on their way into shared memory while
 // it works on the current ones (lattices where a block takes several groups:
-// apply of a 32^4 step of ten sweeps 4.03 -> 3.36 ms).
+// apply of a 32^4 step of ten sweeps 4.03 -> 3.74 ms).
 // Item k of a thread at sm[k CS_THREADS + thread]; a thread's own, no barrier.
 struct sweep_pipe {
   int4* sm;

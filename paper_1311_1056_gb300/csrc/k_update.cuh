@@ -1,5 +1,5 @@
 // k_update.cuh -- the CL step: plaquettes, clover field, per-plaquette drift
-// contributions, and the per-link gather + noise + FP64 exponential update
+// contributions, and the per-link gather + noise + exponential update
 // with det re-projection.
 //
 // Action (Sec. 5, eq. "eq:st"): S = S_W - i theta sum_x q_L(x) with the
@@ -30,7 +30,7 @@
 // Update (the CL step of the method, Sec. 2 and its refs):
 //   K_a = -D_a S,  A = i lambda_a (eps K_a + sqrt(eps) eta_a)
 //     = 2 eps (X_S - Tr X_S / 3) + i sqrt(eps) eta_a lambda_a,  <eta_a eta_b> = 2 delta_ab,
-//   U' = exp(A) U  (exp in FP64),  U' <- U' det(U')^{-1/3}  (FP64 factor).
+//   U' = exp(A) U,  U' <- U' det(U')^{-1/3}  (both to FP64 precision).
 #pragma once
 #include <type_traits>
 
@@ -343,8 +343,8 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
   store(C, 4 * p + 3, s, g.V, M);
 }
 
-// The FP64 and DF64 forms run the stages as two kernels, the partial G^ parked
-// in Gq.  Gq is not a buffer of its own: the partial of plaquette (p, s) sits
+// The FP64 and DF64 forms run the stages as two of three kernels
+// (k_update_fx.cuh), the partial G^ parked in Gq.  Gq is not a buffer of its own: the partial of plaquette (p, s) sits
 // in plane 4p + 1 of C (Gq points at plane 1 of C, so Gq plane GQ_PLANE * p is
 // C plane 4p + 1), the slot-1 contribution of that same plaquette, which only
 // stage b writes, and only after the same thread has read the partial back.
