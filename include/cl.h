@@ -88,7 +88,9 @@ typedef struct {
   double alpha;      /* alpha_gf (alpha of alpha_ad = alpha / D) */
   cl_adapt mode;     /* choice of D */
   int n_min, n_max;  /* sweep-count bounds of the adaptive stop rule */
-  double tol_rel;    /* stop when UN_prev - UN < tol_rel (UN_prev - 1) */
+  double tol_rel;    /* stop when UN_prev - UN < tol_rel (UN_prev - 1); a chain
+                        that meets this within rounding may take a sweep more
+                        or less in another form or another build */
   double d_floor;    /* stop when UN - 1 < d_floor */
   double d_guard;    /* no sweep when D < d_guard (gradient at rounding level) */
   int forced_sweeps; /* >= 0: exactly this many sweeps (reproducible counts) */

@@ -10,11 +10,13 @@
 // lattices below ~50,000 sites, a warp or two per scheduler, run at the length
 // of that chain: gradient + Omega and apply 13 us each at 10x8x12x9, now ~8.
 // Where the second half would leave most of the block idle and the lattice
-// fills the GPU anyway, a block takes several groups before it (CS_WIDE); a
-// site's numbers are the same either way.
+// fills the GPU anyway, a block takes several groups before it (the wide shape); a
+// site's numbers are the same either way.  FP32 storage, whose sums keep one
+// order (sweep_add_f32), splits a site by the entries of G instead of by direction,
+// and in the wide shape not at all.
 //
 // The rule (Sec. 4) needs sums over the lattice.  Every group (of large
-// lattices: every few groups, cs_per_record) leaves one record; the block that
+// lattices: every few groups, cs_rounds) leaves one record; the block that
 // finds, by a counter, that it is the last one sums the records in a fixed order
 // and applies the rule.  No block waits.  (A launch of its own for the rule cost
 // ~6 us a sweep.)  The records do not depend on how the groups are dealt to
@@ -30,21 +32,30 @@ namespace clgc {
 
 const int CS_SITES = 32, CS_THREADS = 128, CS_NARROW_SITES = 24576;
 __host__ __device__ inline int cs_groups(int V) { return (V + CS_SITES - 1) / CS_SITES; }
-// Groups per record: at most ~2,048 records, which one block sums in ~3 us.
-__host__ __device__ inline int cs_per_record(int V) { return (cs_groups(V) + 2047) / 2048; }
 // Groups that a block of the wide shape takes at once.
 template <typename L>
 __host__ __device__ constexpr int cs_wide_grad() { return is_fx<L>() ? 2 : 4; }
 template <typename L>
 __host__ __device__ constexpr int cs_wide_omega() { return is_fx<L>() ? 3 : 4; }  // 3: what shared memory holds with the pipe
+// Rounds of a block: the links of fixed-point forms keep at most ~2,048 records
+// (which one block sums in ~3 us), one per warp; FP32 storage, whose kernels are
+// short, at most 2,048 blocks of four groups a round (with the records' number
+// for its blocks', 512 at 32^4: first gradient 0.134 against 0.091 ms).
+template <typename L>
+__host__ __device__ inline int cs_rounds(int V) {
+  const int n = is_fx<L>() ? 2048 : 8192;
+  return (cs_groups(V) + n - 1) / n;
+}
 // Blocks: gradient (width w: 1 or cs_wide_grad), gradient + Omega (width 1 or
-// cs_wide_omega), apply.
+// cs_wide_omega), apply (FP32 storage: width 1 or 4).
+template <typename L>
 __host__ __device__ inline int cs_grad_blocks(int V, int w) {
-  const int n = w * cs_per_record(V);
+  const int n = w * cs_rounds<L>(V);
   return (cs_groups(V) + n - 1) / n;
 }
 __host__ __device__ inline int cs_grad_omega_blocks(int V, int w) { return (cs_groups(V) + w - 1) / w; }
-__host__ __device__ inline int cs_apply_blocks(int V) { return cs_grad_blocks(V, 1); }
+template <typename L>
+__host__ __device__ inline int cs_apply_blocks(int V, int w) { return cs_grad_blocks<L>(V, is_fx<L>() ? 1 : w); }
 // Whether a lattice on its own runs the narrow shape.
 inline bool cs_narrow(int V) { return V <= CS_NARROW_SITES; }
 
@@ -83,6 +94,9 @@ __device__ __forceinline__ void unload_link(V2* U, const int4* Ux, int mu, int s
 // (or its RMS).  Sweep count: at least n_min, at most n_max; stop once the
 // norm decreases by less than tol_rel of its distance from 1 or that distance
 // is below d_floor; no sweep when D < d_guard; forced_sweeps >= 0 fixes the count.
+// Both sides of the tol_rel test are differences of nearly equal norms, and chains
+// do meet it within rounding: a count is reproducible for one build and form, and
+// by one sweep sensitive to any change in the rounding of the links or of the sums.
 // un: the norm; tot0, tot1: sum |f_ax|, sum f_ax^2; old: the state before.
 // One thread runs this at the end of a kernel: the state comes in one read, and
 // FP64 divisions (~0.5 us each) are left out where the divisor is known before.
@@ -147,7 +161,8 @@ __device__ __forceinline__ void sweep_record(const SweepArgs& a, int r, double x
 // rule takes and zeroes them.
 struct SweepNorm {
   unsigned long long hi, lo;  // sum over blocks of acc >> 20 and of its low 20 bits
-  unsigned wild, pad;         // blocks with links out of range
+  double far;                 // FP32 storage: sites beyond the integers' range
+  unsigned wild, pad;         // fixed point: blocks with links out of range
 };
 __device__ __forceinline__ SweepNorm* sweep_norm(const SweepArgs& a, int V) {
   return reinterpret_cast<SweepNorm*>(a.rec + 2 * (cs_groups(V) + 4));
@@ -203,71 +218,98 @@ __device__ __forceinline__ void sweep_rule(const Geo& g, const SweepArgs& a, boo
 #pragma unroll
   for (int q = 0; q < 3; ++q) tot[q] = (part[0][q] + part[1][q]) + (part[2][q] + part[3][q]);
   cool_rule(tot[2] * a.ca.inv_links, tot[0], tot[1], nonfinite, a.ca, old, a.cs, first);
-  if (first) *sweep_norm(a, g.V) = SweepNorm{0ull, 0ull, 0u, 0u};
+  if (first) *sweep_norm(a, g.V) = SweepNorm{0ull, 0ull, 0.0, 0u, 0u};
   *a.ticket = 0u;
 }
 
 // --------------------------------------------------------------- gradient
-// Partial sums of one direction, in shared memory between the two halves of
-// the gradient: fixed point 60-bit integers, FP32 storage floats.
+// The gradient between its two halves, in shared memory.  Fixed point: partial
+// sums of one direction, 60-bit integers.  FP32 storage: a site's sums, floats.
 template <typename L>
 struct sweep_real { typedef typename std::conditional<is_fx<L>(), long long, float>::type type; };
 // N: 9 numbers, g00, g11, g22, then re / im of g01, g02, g12; 12 with the norm
-// (fixed point: the three diagonals of its forward links; float: their sum).
+// (the three diagonals of the forward links).
 template <typename L, int N>
 struct SweepPart {
-  typename sweep_real<L>::type q[N][CS_THREADS];
-  float top[CS_THREADS];  // fixed point: largest row or column norm (squared); infinite: not representable
+  static const int WIDTH = is_fx<L>() ? CS_THREADS : CS_SITES;
+  typename sweep_real<L>::type q[N][WIDTH];
+  float top[is_fx<L>() ? CS_THREADS : 1];  // largest row or column norm (squared); infinite: not representable
 };
 
-// FP32 storage: the ten numbers of direction mu at site s (sb: the site behind).
-__device__ __forceinline__ void sweep_part_f32(float* q, bool with_norm, const float2* __restrict__ U, int mu, int s, int sb,
-                                               int V) {
+// FP32 storage.  The rule compares differences of norms, themselves sums of
+// rounded floats, with a threshold that chains often meet within rounding, so
+// a site's numbers are summed in one order in every shape: the forward links
+// mu = 0 .. 3, then the backward ones.  (Summed direction by direction the same
+// chains stopped a sweep earlier or later now and then.)
+// One column k of a link's rows (or conjugated columns) a, b, c: d += |c|^2, o += a conj(b).
+__device__ __forceinline__ void sweep_add_f32(float& d, cx<float>& o, cx<float> a, cx<float> b, cx<float> c) {
+  d = fmaf(c.re, c.re, fmaf(c.im, c.im, d));
+  o = cfma(a, cx<float>{b.re, -b.im}, o);
+}
+__device__ __forceinline__ void sweep_sub_f32(float& d, cx<float>& o, cx<float> a, cx<float> b, cx<float> c) {
+  d = fmaf(-c.re, c.re, fmaf(-c.im, c.im, d));
+  o = cfms(cx<float>{a.re, -a.im}, b, o);
+}
+// Rows of pair p: g01 with g00, g12 with g11, g02 with g22.
+__host__ __device__ constexpr int pair_a(int p) { return p == 1 ? 1 : 0; }
+__host__ __device__ constexpr int pair_b(int p) { return p == 0 ? 1 : 2; }
+__host__ __device__ constexpr int pair_off(int p) { return p == 0 ? 3 : p == 1 ? 7 : 5; }  // its slot among the nine numbers
+// Pair P of a site, for the narrow shape, a warp a pair (9 chains of 48 dependent
+// multiply-adds, a third of them a warp's).  fwd: the diagonal after the forward links.
+template <int P>
+__device__ __forceinline__ void sweep_pair_f32(float& d, float& fwd, cx<float>& o, const Geo& g, const float2* __restrict__ U, int s) {
+  constexpr int A = pair_a(P), B = pair_b(P);
+  int x[4];
+  site_coords(g, s, x);
+  d = 0.0f;
+  o = cx<float>{0.0f, 0.0f};
+#pragma unroll
+  for (int dir = 0; dir < 8; ++dir) {
+    const int mu = dir & 3;
+    const float2* p = U + (size_t)mu * 9 * g.V + (dir < 4 ? s : hop(g, s, x, mu, -1));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const cx<float> a = unpack(__ldg(p + (size_t)(dir < 4 ? 3 * A + k : 3 * k + A) * g.V));
+      const cx<float> b = unpack(__ldg(p + (size_t)(dir < 4 ? 3 * B + k : 3 * k + B) * g.V));
+      if (dir < 4)
+        sweep_add_f32(d, o, a, b, P == 2 ? b : a);
+      else
+        sweep_sub_f32(d, o, a, b, P == 2 ? b : a);
+    }
+    if (dir == 3) fwd = d;
+  }
+}
+// The wide shape's site: all of it by one thread; q[9] the norm.
+__device__ __forceinline__ void sweep_sums_f32(float* q, const Geo& g, const float2* __restrict__ U, int s) {
+  int x[4];
+  site_coords(g, s, x);
   float d[3] = {0.0f, 0.0f, 0.0f};
   cx<float> o[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
   mat<float> u;
-  load(u, U, mu, s, V);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {  // + U U^+
-    const cx<float> r0 = u.e[k], r1 = u.e[3 + k], r2 = u.e[6 + k];
-    d[0] = fmaf(r0.re, r0.re, fmaf(r0.im, r0.im, d[0]));
-    d[1] = fmaf(r1.re, r1.re, fmaf(r1.im, r1.im, d[1]));
-    d[2] = fmaf(r2.re, r2.re, fmaf(r2.im, r2.im, d[2]));
-    o[0] = cfma(r0, cx<float>{r1.re, -r1.im}, o[0]);
-    o[1] = cfma(r0, cx<float>{r2.re, -r2.im}, o[1]);
-    o[2] = cfma(r1, cx<float>{r2.re, -r2.im}, o[2]);
+  for (int mu = 0; mu < 4; ++mu) {
+    load(u, U, mu, s, g.V);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        sweep_add_f32(d[p], o[p], u.e[3 * pair_a(p) + k], u.e[3 * pair_b(p) + k], u.e[3 * p + k]);
   }
-  if (with_norm) q[9] = d[0] + d[1] + d[2];
-  load(u, U, mu, sb, V);
+  q[9] = d[0] + d[1] + d[2];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {  // - U^+ U
-    const cx<float> c0 = u.e[3 * k], c1 = u.e[3 * k + 1], c2 = u.e[3 * k + 2];
-    d[0] = fmaf(-c0.re, c0.re, fmaf(-c0.im, c0.im, d[0]));
-    d[1] = fmaf(-c1.re, c1.re, fmaf(-c1.im, c1.im, d[1]));
-    d[2] = fmaf(-c2.re, c2.re, fmaf(-c2.im, c2.im, d[2]));
-    o[0] = cfms(cx<float>{c0.re, -c0.im}, c1, o[0]);
-    o[1] = cfms(cx<float>{c0.re, -c0.im}, c2, o[1]);
-    o[2] = cfms(cx<float>{c1.re, -c1.im}, c2, o[2]);
+  for (int mu = 0; mu < 4; ++mu) {
+    load(u, U, mu, hop(g, s, x, mu, -1), g.V);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        sweep_sub_f32(d[p], o[p], u.e[3 * k + pair_a(p)], u.e[3 * k + pair_b(p)], u.e[3 * k + p]);
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    q[i] = d[i];
-    q[3 + 2 * i] = o[i].re;
-    q[4 + 2 * i] = o[i].im;
-  }
-}
-// The wide shape's site: the same numbers in the same order, no exchange.
-__device__ __forceinline__ void sweep_sums_f32(float* q, bool with_norm, const Geo& g, const float2* __restrict__ U, int s) {
-  int x[4];
-  site_coords(g, s, x);
-  sweep_part_f32(q, with_norm, U, 0, s, hop(g, s, x, 0, -1), g.V);
-#pragma unroll
-  for (int mu = 1; mu < 4; ++mu) {
-    float p[10];
-    sweep_part_f32(p, with_norm, U, mu, s, hop(g, s, x, mu, -1), g.V);
-#pragma unroll
-    for (int i = 0; i < 10; ++i)
-      if (i < 9 || with_norm) q[i] += p[i];
+  for (int p = 0; p < 3; ++p) {
+    q[p] = d[p];
+    q[pair_off(p)] = o[p].re;
+    q[pair_off(p) + 1] = o[p].im;
   }
 }
 
@@ -322,8 +364,9 @@ static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* 
   *top = m * 0x1p-56f;
 }
 
-// First half: this thread's direction (warp) and site.  FIRST: the links are
-// read from U and (fixed point) their words written to Ux.
+// First half: this thread's direction (fixed point) or pair (FP32 storage), a warp
+// each, and site.  FIRST: the links are read from U and (fixed point) their words
+// written to Ux.
 // PIPE: the links come through a pipe, the forward one asked for by
 // the call for the group before (next; the first group's by the caller), so that each
 // link's load runs under the outer products of the one before (gradient + Omega
@@ -338,10 +381,10 @@ __device__ __forceinline__ void sweep_part(SweepPart<L, N>& sm, const Geo& g, co
   typedef typename vec2_of<L>::type V2;
   const int mu = threadIdx.x >> 5, s = group * CS_SITES + (threadIdx.x & 31), t = threadIdx.x;
   if (s >= g.V) return;
-  int x[4];
-  site_coords(g, s, x);
-  const int sb = hop(g, s, x, mu, -1);
   if constexpr (is_fx<L>()) {
+    int x[4];
+    site_coords(g, s, x);
+    const int sb = hop(g, s, x, mu, -1);
     const V2* U = (const V2*)a.U;
     int4* Ux = (int4*)a.Ux;
     fx_acc D[3], O[6];
@@ -398,11 +441,17 @@ __device__ __forceinline__ void sweep_part(SweepPart<L, N>& sm, const Geo& g, co
     for (int i = 0; i < 6; ++i) sm.q[3 + i][t] = fx_sum<true>(O[i]) - (1 << 29);
     sm.top[t] = ok && !ck.bad() ? top * 0x1p-60f : __int_as_float(0x7f800000);
     if (!FIRST && ck.bad()) sweep_part_wild(&sm.q[0][t], N, &sm.top[t], Ux, mu, s, sb, g.V);
-  } else {
-    float q[N];
-    sweep_part_f32(q, N > 9, (const V2*)a.U, mu, s, sb, g.V);
-#pragma unroll
-    for (int i = 0; i < (N > 9 ? 10 : 9); ++i) sm.q[i][t] = q[i];
+  } else if (mu < 3) {
+    float d, fwd;
+    cx<float> o;
+    if (mu == 0) sweep_pair_f32<0>(d, fwd, o, g, (const V2*)a.U, s);
+    if (mu == 1) sweep_pair_f32<1>(d, fwd, o, g, (const V2*)a.U, s);
+    if (mu == 2) sweep_pair_f32<2>(d, fwd, o, g, (const V2*)a.U, s);
+    const int l = t & 31;
+    sm.q[mu][l] = d;
+    sm.q[pair_off(mu)][l] = o.re;
+    sm.q[pair_off(mu) + 1][l] = o.im;
+    if constexpr (N > 9) sm.q[9 + mu][l] = fwd;
   }
 }
 // Second half (after a barrier), one thread per site: the sums over directions.
@@ -573,7 +622,8 @@ __device__ __forceinline__ void sweep_grad_site(SweepSums& v, const SweepPart<L,
   }
 }
 // W: groups at once.  Record W vb + w of a block is that of its warp w: the
-// groups W (R vb + j) + w, j < R = cs_per_record.
+// groups W (R vb + j) + w, j < R = cs_rounds.  FP32 storage beyond 2,048 groups:
+// record vb, the block's.
 template <typename L, bool FIRST, int W>
 __device__ __forceinline__ void sweep_grad_body(const Geo& g, const SweepArgs& a, int vb, bool rule) {
   if (!FIRST && a.cs->done) return;
@@ -582,7 +632,7 @@ __device__ __forceinline__ void sweep_grad_body(const Geo& g, const SweepArgs& a
   __shared__ SweepPart<L, 12> sm[ALONE ? 1 : W];
   SweepSums v;
   const bool with_f = a.ca.mode >= 2;
-  const int ng = cs_groups(g.V), R = cs_per_record(g.V), w = threadIdx.x >> 5;
+  const int ng = cs_groups(g.V), R = cs_rounds<L>(g.V), w = threadIdx.x >> 5;
   constexpr bool PIPE = is_fx<L>() && !FIRST && W > 1;
   __shared__ int4 slot[PIPE ? fx_pipe<1>::WORDS : 1];
   fx_pipe<1> P(slot);
@@ -592,20 +642,24 @@ __device__ __forceinline__ void sweep_grad_body(const Geo& g, const SweepArgs& a
     const int s = (g0 + w) * CS_SITES + ((int)threadIdx.x & 31);
     float q[10];
     if constexpr (ALONE) {
-      if (s < g.V) sweep_sums_f32(q, true, g, (const float2*)a.U, s);
+      if (s < g.V) sweep_sums_f32(q, g, (const float2*)a.U, s);
     } else {
       if (j > 0) __syncthreads();
 #pragma unroll 1
       for (int p = 0; p < W; ++p) sweep_part<L, FIRST, PIPE, 12>(sm[p], g, a, g0 + p, P, p + 1 < W || j + 1 < R ? g0 + p + 1 : -1);
       __syncthreads();
       if constexpr (!is_fx<L>())
-        if (w < W && s < g.V)
+        if (w < W && s < g.V) {
+          const int l = threadIdx.x & 31;
 #pragma unroll
-          for (int i = 0; i < 10; ++i) q[i] = sweep_sum(sm[w], i);
+          for (int i = 0; i < 9; ++i) q[i] = sm[w].q[i][l];
+          q[9] = (sm[w].q[9][l] + sm[w].q[10][l]) + sm[w].q[11][l];
+        }
     }
     if (w < W && s < g.V) sweep_grad_site<L, FIRST>(v, sm[ALONE ? 0 : w], q, g, a, s, with_f);
   }
   if (!rule) return;
+  const bool one = !is_fx<L>() && ng > 2048;  // one record for the block
   if (w < W) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -615,15 +669,31 @@ __device__ __forceinline__ void sweep_grad_body(const Geo& g, const SweepArgs& a
       }
       v.z += __shfl_down_sync(0xffffffffu, v.z, o);
     }
-    const bool bad = __any_sync(0xffffffffu, v.w != 0.0);
-    if ((threadIdx.x & 31) == 0 && (R > 1 || W * vb + w < ng)) sweep_record(a, W * vb + w, v.x, v.y, v.z, bad ? 1.0 : 0.0);
+    v.w = __any_sync(0xffffffffu, v.w != 0.0) ? 1.0 : 0.0;
+    if (!one && (threadIdx.x & 31) == 0 && (R > 1 || W * vb + w < ng)) sweep_record(a, W * vb + w, v.x, v.y, v.z, v.w);
+  }
+  if constexpr (ALONE) {
+    if (one) {
+      __shared__ SweepSums part[W];
+      if ((threadIdx.x & 31) == 0) part[w] = v;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        for (int q = 1; q < W; ++q) {
+          v.x += part[q].x;
+          v.y += part[q].y;
+          v.z += part[q].z;
+          v.w += part[q].w;
+        }
+        sweep_record(a, vb, v.x, v.y, v.z, v.w);
+      }
+    }
   }
   if (W > 1) {
     __threadfence();
     __syncthreads();
   }
-  const int nb = cs_grad_blocks(g.V, W);
-  sweep_rule(g, a, with_f, nb, R > 1 ? W * nb : ng, FIRST ? 1 : 0);
+  const int nb = cs_grad_blocks<L>(g.V, W);
+  sweep_rule(g, a, with_f, nb, one ? nb : R > 1 ? W * nb : ng, FIRST ? 1 : 0);
 }
 
 
@@ -735,7 +805,7 @@ __host__ __device__ inline int cs_omega_blocks(int V, bool split) {
 // Single-pass sweep of the D_0 / D_1 rules: their strength needs only the
 // unitarity norm, which the previous sweep's apply summed, so the gradient
 // goes straight into Omega.
-// W = 1: two warps take the signs; W = 4: a thread per site forms both.
+// W = 1: two warps take the signs; W > 1: a thread per site forms both.
 template <typename L, int W>
 __device__ __forceinline__ void sweep_grad_omega_body(const Geo& g, const SweepArgs& a, int vb) {
   if (a.cs->done) return;
@@ -762,12 +832,12 @@ __device__ __forceinline__ void sweep_grad_omega_body(const Geo& g, const SweepA
     fx_gradient G;
     ok = sweep_gradient(G, sm) && fx_herm_of_gradient(H, G, c);
   } else {
-    float r[9];
+    float r[10];
     if constexpr (ALONE) {
-      sweep_sums_f32(r, false, g, (const float2*)a.U, s);
+      sweep_sums_f32(r, g, (const float2*)a.U, s);
     } else {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) r[i] = sweep_sum(sm, i);
+      for (int i = 0; i < 9; ++i) r[i] = sm.q[i][threadIdx.x & 31];
     }
     sweep_f(ff, r);
     ok = fx_herm_of_f(H, ff, c);
@@ -863,18 +933,18 @@ struct sweep_pipe {
 template <typename L, bool RULE>
 __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& a, int vb, bool last) {
   typedef typename vec2_of<L>::type V2;
-  const int mu = threadIdx.x >> 5, R = cs_per_record(g.V);
+  const int mu = threadIdx.x >> 5, R = cs_rounds<L>(g.V);
   V2* U = (V2*)const_cast<void*>(a.U);
   const bool stopped = a.cs && a.cs->done;
-  if (stopped && !(is_fx<L>() && last && a.cs->sweeps > 0)) return;
+  if (stopped && !(last && a.cs->sweeps > 0)) return;
   const int sh = 6 + (R > 1 ? 32 - __clz(R - 1) : 0);
   long long acc = 0;
   double wild = 0.0;
   int nwild = 0;
-  __shared__ int4 sm[is_fx<L>() ? 18 * CS_THREADS : 1];
+  __shared__ int4 sm[18 * CS_THREADS];
   const sweep_pipe P = {sm + threadIdx.x};
-  int sp0 = 0;  // fixed point: the next site's neighbour, asked for already
-  if (is_fx<L>() && R > 1 && !stopped) {
+  int sp0 = 0;  // the next site's neighbour, asked for already
+  if (R > 1 && !stopped) {
     const int s = R * vb * CS_SITES + ((int)threadIdx.x & 31);
     if (s < g.V) {
       int x[4];
@@ -886,67 +956,44 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
   for (int j = 0; j < R; ++j) {
     const int s = (R * vb + j) * CS_SITES + ((int)threadIdx.x & 31);
     if (s >= g.V) break;
-    if constexpr (is_fx<L>()) {
-      if (stopped) {
-        unload_link(U, (const int4*)a.Ux, mu, s, g.V);
-        continue;
-      }
+    if (stopped) {
+      unload_link(U, (const int4*)a.Ux, mu, s, g.V);
+      continue;
     }
     int x[4];
     int sp = sp0;
-    if (!is_fx<L>() || R == 1) {
-      site_coords(g, s, x);
-      sp = hop(g, s, x, mu, 1);
-    }
-    if constexpr (is_fx<L>()) {
-      int4* Ux = (int4*)a.Ux;
-      fx_chk ck;
-      fx_herm o, oi;
-      mat<fx> u;
-      if (R > 1) {
-        P.take(u, o, oi, ck);
-        const int s1 = s + CS_SITES;
-        if (j + 1 < R && s1 < g.V) {
-          site_coords(g, s1, x);
-          sp0 = hop(g, s1, x, mu, 1);
-          P.ask(a, mu, s1, sp0, g.V);
-        }
-      } else {
-        fx_load_herm(o, (const int2*)a.Om, s, g.V, ck);
-        fx_load_herm(oi, (const int2*)a.Omi, sp, g.V, ck);
-        fx_load_plain(u, Ux, mu, s, g.V);
-      }
-      if (fx_is_raw(u.e[0].re.l)) ck.fail();
-      fx_apply_ops ops;
-      fx_lhs(ops, o);
-      long long dev = 0;
-      fx_apply_link<RULE>(u, ops, oi, ck, dev);
-      if (!ck.bad()) {
-        if (last) fx_store_link(U, mu, s, g.V, u);
-        if (!last || !RULE) store<fx>(Ux, mu, s, g.V, u);  // D_2 calls end with a gradient
-        acc += dev >> sh;
-      } else {
-        wild += far_cool_apply(g, Ux, (int2*)a.Om, (int2*)a.Omi, mu, s, sp) - 3.0;
-        nwild = 1;
-        if (last) unload_link(U, Ux, mu, s, g.V);
+    int4* Ux = (int4*)a.Ux;
+    fx_chk ck;
+    fx_herm o, oi;
+    mat<fx> u;
+    if (R > 1) {
+      P.take(u, o, oi, ck);
+      const int s1 = s + CS_SITES;
+      if (j + 1 < R && s1 < g.V) {
+        site_coords(g, s1, x);
+        sp0 = hop(g, s1, x, mu, 1);
+        P.ask(a, mu, s1, sp0, g.V);
       }
     } else {
-      mat<L> o, oi, u, w;
-      load_herm_mat(o, (const L*)a.Om, s, g.V);
-      load_herm_mat(oi, (const L*)a.Omi, sp, g.V);
-      load(u, U, mu, s, g.V);
-      mul_herm_left(w, o, u);
-      mul_herm_right(u, w, oi);
-      store(U, mu, s, g.V, u);
-      if (RULE) {
-        const float n = norm2(u);
-        if (n < 4.9f) {
-          acc += (fx_bits(fx_of_float(0.25f * n)) - (3ll << 58)) >> (sh - 2);
-        } else {
-          wild += cvt<double>(n) - 3.0;
-          nwild = 1;
-        }
-      }
+      site_coords(g, s, x);
+      sp = hop(g, s, x, mu, 1);
+      fx_load_herm(o, (const int2*)a.Om, s, g.V, ck);
+      fx_load_herm(oi, (const int2*)a.Omi, sp, g.V, ck);
+      fx_load_plain(u, Ux, mu, s, g.V);
+    }
+    if (fx_is_raw(u.e[0].re.l)) ck.fail();
+    fx_apply_ops ops;
+    fx_lhs(ops, o);
+    long long dev = 0;
+    fx_apply_link<RULE>(u, ops, oi, ck, dev);
+    if (!ck.bad()) {
+      if (last) fx_store_link(U, mu, s, g.V, u);
+      if (!last || !RULE) store<fx>(Ux, mu, s, g.V, u);  // D_2 calls end with a gradient
+      acc += dev >> sh;
+    } else {
+      wild += far_cool_apply(g, Ux, (int2*)a.Om, (int2*)a.Omi, mu, s, sp) - 3.0;
+      nwild = 1;
+      if (last) unload_link(U, Ux, mu, s, g.V);
     }
   }
   if constexpr (RULE) {
@@ -975,7 +1022,7 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
       if (any) atomicAdd(&n->wild, 1u);
       __stcg(a.rec + 2 * vb, make_double2(any ? (wilds[0] + wilds[1]) + (wilds[2] + wilds[3]) : 0.0, 0.0));
     }
-    const int nb = cs_apply_blocks(g.V);
+    const int nb = cs_apply_blocks<L>(g.V, 1);
     if (!sweep_last(a, nb)) return;
     double far = 0.0;  // links beyond the bound, by the whole block
     if (__ldcg(&n->wild) != 0u) {
@@ -990,9 +1037,103 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
     const long long hi = (long long)__ldcg(&n->hi), lo = (long long)__ldcg(&n->lo);
     const double dev = fx_bits_to_double(hi, sh + 20) + fx_bits_to_double(lo, sh) + far;
     cool_rule(1.0 + dev * ((1.0 / 3.0) * a.ca.inv_links), 0.0, 0.0, false, a.ca, old, a.cs, 0);
-    *n = SweepNorm{0ull, 0ull, 0u, 0u};
+    *n = SweepNorm{0ull, 0ull, 0.0, 0u, 0u};
     *a.ticket = 0u;
   }
+}
+
+// FP32 storage: the apply of one link; returns Tr U U^+.
+__device__ __forceinline__ float sweep_apply_f32(float2* U, const mat<float>& o, const float* Omi, const Geo& g, int mu, int s,
+                                                 const int* x) {
+  mat<float> oi, u, w;
+  load_herm_mat(oi, Omi, hop(g, s, x, mu, 1), g.V);
+  load(u, U, mu, s, g.V);
+  mul_herm_left(w, o, u);
+  mul_herm_right(u, w, oi);
+  store(U, mu, s, g.V, u);
+  return norm2(u);
+}
+// W = 1: a group, a warp per direction; W = 4: a thread per site, which loads
+// Omega_x once, cs_rounds rounds of 128 sites (32^4, ten sweeps: 1.20 ms against
+// 1.25; 16^4: 0.153 against 0.173).  RULE as above; a site's norm is the float sum over mu = 0 .. 3
+// (the order matters, see sweep_add_f32), the lattice's an exact one: integers
+// in units of 2^-36, which hold every float above 2^-12; sites of norm beyond
+// 1,024 (or not finite) in FP64.
+template <bool RULE, int W>
+__device__ __forceinline__ void sweep_apply_f32_body(const Geo& g, const SweepArgs& a, int vb) {
+  if (a.cs && a.cs->done) return;
+  float2* U = (float2*)const_cast<void*>(a.U);
+  const float *Om = (const float*)a.Om, *Omi = (const float*)a.Omi;
+  long long acc = 0;
+  double far = 0.0;
+  int nfar = 0;
+  const auto site = [&](float un) {
+    if (un < 1024.0f) {
+      acc += __float2ll_rn(un * 0x1p36f) - (12ll << 36);
+    } else {
+      far += cvt<double>(un) - 12.0;
+      nfar = 1;
+    }
+  };
+  mat<float> o;
+  int x[4];
+  if (W > 1) {
+    const int R = cs_rounds<float>(g.V);
+    for (int j = 0; j < R; ++j) {
+      const int s = (R * vb + j) * CS_THREADS + (int)threadIdx.x;
+      if (s >= g.V) break;
+      site_coords(g, s, x);
+      load_herm_mat(o, Om, s, g.V);
+      float un = 0.0f;
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) un += sweep_apply_f32(U, o, Omi, g, mu, s, x);
+      if (RULE) site(un);
+    }
+  } else {
+    __shared__ float n[4][CS_SITES];
+    const int mu = threadIdx.x >> 5, l = threadIdx.x & 31, s = vb * CS_SITES + l;
+    if (s < g.V) {
+      site_coords(g, s, x);
+      load_herm_mat(o, Om, s, g.V);
+      n[mu][l] = sweep_apply_f32(U, o, Omi, g, mu, s, x);
+    }
+    if (RULE) {
+      __syncthreads();
+      if (mu == 0 && s < g.V) site(((n[0][l] + n[1][l]) + n[2][l]) + n[3][l]);
+    }
+  }
+  if constexpr (RULE) {
+    __shared__ long long sums[CS_THREADS / 32];
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, k);
+    if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = acc;
+    SweepNorm* n = sweep_norm(a, g.V);
+    if (nfar) atomicAdd(&n->far, far);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const long long t = sums[0] + sums[1] + sums[2] + sums[3];
+      atomicAdd(&n->hi, (unsigned long long)(t >> 20));
+      atomicAdd(&n->lo, (unsigned long long)(t & 0xfffff));
+    }
+    if (!sweep_last(a, cs_apply_blocks<float>(g.V, W))) return;
+    if (threadIdx.x != 0) return;
+    const CoolState old = *a.cs;
+    const long long hi = (long long)__ldcg(&n->hi), lo = (long long)__ldcg(&n->lo);
+    const double dev = fx_bits_to_double(hi, 44) + fx_bits_to_double(lo, 24) + __ldcg(&n->far);
+    cool_rule(1.0 + dev * ((1.0 / 3.0) * a.ca.inv_links), 0.0, 0.0, false, a.ca, old, a.cs, 0);
+    *n = SweepNorm{0ull, 0ull, 0.0, 0u, 0u};
+    *a.ticket = 0u;
+  }
+}
+
+// The apply of either field; wide: FP32 storage at W = 4.
+template <typename L, bool RULE, bool WIDE>
+__device__ __forceinline__ void sweep_apply(const Geo& g, const SweepArgs& a, int vb, bool last) {
+  if constexpr (is_fx<L>())
+    sweep_apply_body<L, RULE>(g, a, vb, last);
+  else
+    sweep_apply_f32_body<RULE, WIDE ? 4 : 1>(g, a, vb);
 }
 
 }  // namespace clgc

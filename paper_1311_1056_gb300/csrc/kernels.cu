@@ -268,9 +268,9 @@ template <typename L, int W>
 __global__ void __launch_bounds__(CS_THREADS) k_cool_grad_omega(Geo g, SweepArgs a) {
   sweep_grad_omega_body<L, W>(g, a, blockIdx.x);
 }
-template <typename L, bool RULE>
+template <typename L, bool RULE, bool WIDE>
 __global__ void __launch_bounds__(CS_THREADS, CS_APPLY_BLOCKS(L)) k_cool_apply(Geo g, SweepArgs a, int last) {
-  sweep_apply_body<L, RULE>(g, a, blockIdx.x, last != 0);
+  sweep_apply<L, RULE, WIDE>(g, a, blockIdx.x, last != 0);
 }
 // The links' fixed-point words, for an apply without a gradient before it.
 template <typename L>
@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(CS_THREADS, CS_APPLY_BLOCKS(L)) k_ens_cool_app
                                                                   const WorkItem* __restrict__ w, int sweep) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  sweep_apply_body<L, RULE>(ens_geo(c), ens_sweep<L>(c), it.vb, sweep == cs_sweeps(c.ca) - 1);
+  sweep_apply<L, RULE, true>(ens_geo(c), ens_sweep<L>(c), it.vb, sweep == cs_sweeps(c.ca) - 1);
 }
 
 template <typename L>
@@ -762,7 +762,7 @@ cudaError_t launch_cool_grad(int prec, const GeoH& h, const CoolBufs& b, bool fi
   return by_prec(prec, [&](auto t) {
     using L = decltype(t);
     constexpr int W = cs_wide_grad<L>();
-    const int n = cs_grad_blocks(g.V, cs_narrow(g.V) ? 1 : W);
+    const int n = cs_grad_blocks<L>(g.V, cs_narrow(g.V) ? 1 : W);
     if (cs_narrow(g.V)) {
       if (first)
         k_cool_grad<L, true, 1><<<n, CS_THREADS, 0, st>>>(g, a, r);
@@ -802,13 +802,22 @@ cudaError_t launch_cool_grad_omega(int prec, const GeoH& h, const CoolBufs& b, c
 cudaError_t launch_cool_apply(int prec, const GeoH& h, const CoolBufs& b, bool rule, bool last, cudaStream_t st) {
   Geo g = to_geo(h);
   const SweepArgs a = sweep_args(b);
-  const int n = cs_apply_blocks(g.V);
+  const int k = last ? 1 : 0;
   return by_prec(prec, [&](auto t) {
     using L = decltype(t);
-    if (rule)
-      k_cool_apply<L, true><<<n, CS_THREADS, 0, st>>>(g, a, last ? 1 : 0);
-    else
-      k_cool_apply<L, false><<<n, CS_THREADS, 0, st>>>(g, a, last ? 1 : 0);
+    const bool wide = is_fx<L>() || !cs_narrow(g.V);  // fixed point: one shape
+    const int n = cs_apply_blocks<L>(g.V, wide ? 4 : 1);
+    if (wide) {
+      if (rule)
+        k_cool_apply<L, true, true><<<n, CS_THREADS, 0, st>>>(g, a, k);
+      else
+        k_cool_apply<L, false, true><<<n, CS_THREADS, 0, st>>>(g, a, k);
+    } else if constexpr (!is_fx<L>()) {
+      if (rule)
+        k_cool_apply<L, true, false><<<n, CS_THREADS, 0, st>>>(g, a, k);
+      else
+        k_cool_apply<L, false, false><<<n, CS_THREADS, 0, st>>>(g, a, k);
+    }
   });
 }
 cudaError_t launch_cool_load(int prec, const GeoH& h, const void* U, void* Ux, cudaStream_t st) {
@@ -820,10 +829,11 @@ cudaError_t launch_cool_load(int prec, const GeoH& h, const void* U, void* Ux, c
 }
 int ens_cool_blocks(int prec, int fam, int V) {
   switch (fam) {
-    case ENS_COOL_GRAD: return cs_grad_blocks(V, prec == 0 ? cs_wide_grad<double>() : cs_wide_grad<float>());
+    case ENS_COOL_GRAD:
+      return prec == 0 ? cs_grad_blocks<double>(V, cs_wide_grad<double>()) : cs_grad_blocks<float>(V, cs_wide_grad<float>());
     case ENS_COOL_OMEGA: return cs_omega_blocks(V, false);
     case ENS_COOL_GRAD_OMEGA: return cs_grad_omega_blocks(V, prec == 0 ? cs_wide_omega<double>() : cs_wide_omega<float>());
-    default: return cs_apply_blocks(V);
+    default: return prec == 0 ? cs_apply_blocks<double>(V, 4) : cs_apply_blocks<float>(V, 4);
   }
 }
 
