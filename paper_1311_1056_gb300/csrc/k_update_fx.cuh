@@ -444,10 +444,11 @@ __device__ __forceinline__ void gather_f64(mat<double>& X, const Geo& g, int s, 
 // (X - Tr X / 3) / 4 of the 60-bit integers X; false out of range.
 __device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long* X) {
   fx_chk ck;
-  const long long tr = (X[0] + X[8] + X[16]) / 3, ti = (X[1] + X[9] + X[17]) / 3;
+  // of the quarters: three diagonals of up to 8 leave 64 bits
+  const long long tr = ((X[0] >> 2) + (X[8] >> 2) + (X[16] >> 2)) / 3, ti = ((X[1] >> 2) + (X[9] >> 2) + (X[17] >> 2)) / 3;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    const long long re = (X[2 * k] - (k % 4 == 0 ? tr : 0)) >> 2, im = (X[2 * k + 1] - (k % 4 == 0 ? ti : 0)) >> 2;
+    const long long re = (X[2 * k] >> 2) - (k % 4 == 0 ? tr : 0), im = (X[2 * k + 1] >> 2) - (k % 4 == 0 ? ti : 0);
     ck.see<FX_WIDE>((int)(re >> 32));
     ck.see<FX_WIDE>((int)(im >> 32));
     Q.e[k] = cx<fx>{fx_of_bits(re), fx_of_bits(im)};
