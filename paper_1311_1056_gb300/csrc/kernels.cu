@@ -325,7 +325,8 @@ static __device__ __noinline__ double general_obs_link(const typename vec2_of<T>
   *det2 = fmax(*det2, h * h);
   return norm2(u);
 }
-// Tr of a stored matrix times 1/4 as a 60-bit integer (FP32 storage: of its float trace).
+// Tr of a stored matrix times 1/4 as a 60-bit integer (FP32 storage: of its float
+// trace).  Six of them are added: each below 5.3 / 4 (fixed point: 3 1.4375 / 4).
 __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const float2* f, int p, int s, int V) {
   float tr = 0.0f, ti = 0.0f;
 #pragma unroll
@@ -334,7 +335,7 @@ __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const fl
     tr += w.x;
     ti += w.y;
   }
-  if (!(fabsf(tr) < 7.0f && fabsf(ti) < 7.0f)) return false;
+  if (!(fabsf(tr) < 5.3f && fabsf(ti) < 5.3f)) return false;
   re = fx_bits(fx_of_float(0.25f * tr));
   im = fx_bits(fx_of_float(0.25f * ti));
   return true;

@@ -36,3 +36,29 @@ def test_drift_of_large_trace(cl, prec, a):
     assert abs(k_gpu - k) <= 1e-12 * X
     assert abs(e_gpu - e) <= 1e-12 * eps
     assert err <= 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("p", [1.0, 2.4, 2.6, 2.9, 3.3])
+def test_fp32_storage_observables_of_large_traces(cl, p):
+    """The six plaquettes at one site are h = diag(p, p, p^-2): real traces of 3 to 6.7, whose sum passes 32 at
+    p = 2.65 (at its neighbours, where h^-1 stands, earlier).  Entries of P and P^-1 reach p^2 = 11 and carry ~10 roundings of 6e-8 each: 1e-5 per trace, on 6 of
+    the 6 V plaquettes and the ~30 that share a link with them."""
+    L, beta = (3, 4, 3, 5), 6.0
+    V = I.volume(L)
+    x = I.coords(L)
+    U = np.zeros((V, 4, 3, 3), np.complex64)
+    U[:] = np.eye(3)
+    base = np.array([1, 2, 0, 3])
+    for mu in range(4):
+        for nu in range(mu + 1, 4):
+            y = base.copy()
+            y[mu] = (y[mu] + 1) % L[mu]
+            s = int(np.flatnonzero((x == y).all(1))[0])
+            U[s, nu] = np.diag([p, p, p ** -2])
+    U = U.astype(np.complex128)
+    ref = O.observables(L, U, beta, 0.0)
+    with cl.Lattice(L, beta=beta, prec=cl.CL_FP32_STORAGE) as lat:
+        lat.set_links(U)
+        obs = lat.observables()
+    assert abs(obs["plaq_re"] - ref["plaq_re"]) <= 36 * 1e-5 / (18.0 * V)
+    assert abs(obs["sw_re"] - ref["sw_re"]) <= beta / 6.0 * 36 * 2e-5
