@@ -181,7 +181,10 @@ __device__ __forceinline__ bool fx_exp_setup(fx_exp_series& S, const fx_herm& H,
     Q.o[2] = cx<fx>{fx_get<FX_WIDE>(re, ck), fx_get<FX_WIDE>(im, ck)};
   }
   // c1 = Tr H^2 / 2, c0 = det H = Tr H^3 / 3 = (sum_i Q_ii d_i + 2 Re sum Q_ij conj(o_ij)) / 3
-  const fx c1 = fx_of_bits((fx_bits(Q.d[0]) + fx_bits(Q.d[1]) + fx_bits(Q.d[2])) >> 1);
+  // Tr H^2 / 2 in 64 bits: as a number it would wrap at 2 and pass for a small one
+  const long long h2 = (fx_bits(Q.d[0]) + fx_bits(Q.d[1]) + fx_bits(Q.d[2])) >> 1;
+  if (ck.bad() || h2 > (1ll << 56)) return false;  // |H|_F above 0.354
+  const fx c1 = fx_of_bits(h2);
   fx_acc t = fx_zero(), t2 = fx_zero();
 #pragma unroll
   for (int i = 0; i < 3; ++i) {

@@ -62,3 +62,27 @@ def test_fp32_storage_observables_of_large_traces(cl, p):
         obs = lat.observables()
     assert abs(obs["plaq_re"] - ref["plaq_re"]) <= 36 * 1e-5 / (18.0 * V)
     assert abs(obs["sw_re"] - ref["sw_re"]) <= beta / 6.0 * 36 * 2e-5
+
+
+@pytest.mark.parametrize("prec,tol", [("CL_FP64", 1e-12), ("CL_DF64", 1e-12), ("CL_FP32_STORAGE", 1e-5)])
+@pytest.mark.parametrize("h", [0.05, 0.12, 0.5, 0.8, 0.82, 0.84, 0.846, 0.86])
+def test_cooling_exponents_whose_square_passes_two(cl, prec, tol, h):
+    """One link B with B^2 = a + b J (J all ones): at its two ends H has a zero diagonal and +-h off it, so that the
+    diagonal of H^2, 2 h^2, is in range up to h = 0.8478 while half its trace, 3 h^2, passes 2 at h = 0.8165.
+    The result is three matrices of size up to e^(2 h); 1e-12 (1e-5) of it is hundreds of its roundings."""
+    L, eps = (3, 4, 3, 5), 1.92  # a strength just below a power of two, so that f = H / eps is in range as well
+    b = h / (4 * eps)
+    a = min(r.real for r in np.roots([1.0, 3 * b, 0.0, -1.0]) if abs(r.imag) < 1e-12 and r.real > 0)
+    w, v = np.linalg.eigh(a * np.eye(3) + b * np.ones((3, 3)))
+    U = np.zeros((I.volume(L), 4, 3, 3), complex)
+    U[:] = np.eye(3)
+    U[37, 2] = (v * np.sqrt(w)) @ v.T
+    kw = dict(eps=eps, alpha=1.0, forced_sweeps=1)
+    if prec == "CL_FP32_STORAGE":
+        U = U.astype(np.complex64).astype(complex)
+    ref, _ = O.cool(L, U, O.cool_params(mode=O.D0, **kw))
+    with cl.Lattice(L, prec=getattr(cl, prec)) as lat:
+        lat.set_links(U)
+        lat.cool(cl.make_cool(mode=cl.CL_D0, **kw))
+        got = lat.links()
+    assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
