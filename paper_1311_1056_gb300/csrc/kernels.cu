@@ -295,7 +295,8 @@ __global__ void __launch_bounds__(CS_THREADS) k_cool_load(Geo g, const typename 
 // are widened to FP64 once (GB300's FP64 rate again: 430 us at 16^4 with the
 // plaquettes, determinants and traces formed in FP64).
 
-// One link's Tr U U^+ - 3 (60-bit integer) and |det U - 1|^2; false out of range.
+// One link's Tr U U^+ - 3 (60-bit integer, within 1.95 of zero: four are added)
+// and |det U - 1|^2; false out of range.
 __device__ __forceinline__ bool obs_link(const mat<fx>& u, long long& dev, double& det2) {
   fx_chk ck;
   fx_acc n = fx_zero();
@@ -307,7 +308,7 @@ __device__ __forceinline__ bool obs_link(const mat<fx>& u, long long& dev, doubl
     nf = fmaf((float)u.e[k].re.h, (float)u.e[k].re.h, fmaf((float)u.e[k].im.h, (float)u.e[k].im.h, nf));
   }
   const cx<fx> e = fx_det_minus_one(u, ck);
-  if (ck.bad() || !(nf < 4.9f * 0x1p60f)) return false;
+  if (ck.bad() || !(nf > 1.05f * 0x1p60f && nf < 4.9f * 0x1p60f)) return false;
   dev += fx_sum(n) - ((3ll << 60) + (1 << 29));
   const double re = fx_to_double(e.re), im = fx_to_double(e.im);
   det2 = fmax(det2, fma(re, re, im * im));

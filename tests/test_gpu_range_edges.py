@@ -86,3 +86,19 @@ def test_cooling_exponents_whose_square_passes_two(cl, prec, tol, h):
         lat.cool(cl.make_cool(mode=cl.CL_D0, **kw))
         got = lat.links()
     assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("prec,tol", [("CL_FP64", 1e-14), ("CL_DF64", 1e-13), ("CL_FP32_STORAGE", 1e-6)])
+@pytest.mark.parametrize("a", [0.0, 0.1, 0.5, 0.58, 0.6])
+def test_norm_of_small_links(cl, prec, tol, a):
+    """Links a U, off determinant one as a caller's may be: (1/3) Tr U U^+ = a^2.  A sum of V positive numbers."""
+    L = (3, 4, 3, 5)
+    U = a * I.su3_lattice(L, 4)
+    if prec == "CL_FP32_STORAGE":
+        U = U.astype(np.complex64).astype(complex)
+    un = np.sum(np.abs(U) ** 2) / (12.0 * I.volume(L))
+    with cl.Lattice(L, prec=getattr(cl, prec)) as lat:
+        lat.set_links(U)
+        obs = lat.observables()
+    assert abs(obs["un"] - un) <= tol * max(un, 1.0)
+    assert abs(obs["max_det_dev"] - np.abs(np.linalg.det(U) - 1.0).max()) <= max(tol, 1e-13)
