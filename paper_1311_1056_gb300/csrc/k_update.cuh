@@ -32,6 +32,7 @@
 //     = 2 eps (X_S - Tr X_S / 3) + i sqrt(eps) eta_a lambda_a,  <eta_a eta_b> = 2 delta_ab,
 //   U' = exp(A) U,  U' <- U' det(U')^{-1/3}  (both to FP64 precision).
 #pragma once
+#include <cstddef>
 #include <type_traits>
 
 #include "expm_fx.cuh"
@@ -475,23 +476,28 @@ __device__ __forceinline__ void kmax_update(StepDev* sd, double kk) {
 // 1.68, FP32 storage 1.10 -> 0.90.
 const int UPDATE_MAXNREG = 168;
 // The step's bookkeeping without kernels of its own (of one thread, 3 us each).
-__device__ __forceinline__ bool last_of_blocks(StepDev* sd, const Geo& g) {
-  const bool last = atomicAdd(&sd->pad, 1u) + 1u == 4u * ((unsigned)(g.V + blockDim.x - 1) / blockDim.x);
-  if (last) sd->pad = 0u;
-  return last;
-}
+__device__ __forceinline__ unsigned update_blocks(const Geo& g) { return 4u * ((unsigned)(g.V + blockDim.x - 1) / blockDim.x); }
 // An update kernel's step number.  The last block to have read it counts the
-// step: step += 1, t += the step size taken.  (Counted when the blocks finish
-// instead, the barrier at the end of each costs the update 8 %.)
+// step: step += 1, t += the step size taken.  A block reads the step by the same
+// 64-bit atomic that counts it (step and pad are one word), so the last one's
+// write comes after every read without a fence.  (Counted when the blocks finish
+// instead, the barrier at the end of each costs the update 8 %; read and counted
+// apart, with the release that this needs, also 8 %.)
 template <int MODE>
 __device__ __forceinline__ uint32_t step_begin(const Geo& g, const UpdArgs& a) {
   if (MODE == MODE_DRIFT || MODE == MODE_DRIFTMAX) return 0u;
-  const uint32_t step = *(volatile const uint32_t*)&a.sd->step;
-  __syncthreads();
-  if (threadIdx.x == 0 && last_of_blocks(a.sd, g)) {
-    a.sd->step = step + 1u;
-    a.sd->t += a.adaptive ? a.sd->eps_n : a.eps;
+  static_assert(offsetof(StepDev, step) == 0 && offsetof(StepDev, pad) == 4, "one 64-bit word");
+  __shared__ uint32_t step;
+  if (threadIdx.x == 0) {
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(&a.sd->step);
+    const unsigned long long old = atomicAdd(w, 1ull << 32);
+    step = (uint32_t)old;
+    if ((unsigned)(old >> 32) + 1u == update_blocks(g)) {
+      *w = (unsigned long long)((uint32_t)old + 1u);
+      a.sd->t += a.adaptive ? a.sd->eps_n : a.eps;
+    }
   }
+  __syncthreads();
   return step;
 }
 // After the drift pass, by its last block: the adaptive step size eps min(1,
@@ -503,7 +509,9 @@ __device__ __forceinline__ void step_size(const Geo& g, const UpdArgs& a) {
   if (threadIdx.x != 0) return;
   __threadfence();
   StepDev* sd = a.sd;
-  if (!last_of_blocks(sd, g)) return;
+  if (atomicAdd(&sd->pad, 1u) + 1u != update_blocks(g)) return;
+  __threadfence();
+  sd->pad = 0u;
   const double kmax = sqrt(__longlong_as_double((long long)atomicExch(&sd->kmax2_bits, 0ull)));
   const double e = kmax > a.k_ref ? a.eps * (a.k_ref / kmax) : a.eps;
   sd->eps_n = e;
