@@ -467,7 +467,7 @@ __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, co
   const double kd = ldexp(quarter ? 2.0 * eps : 8.0 * eps, cexp);  // times X / 4
   const fx kf = fx_of_double(ks, mag);
   const fx_left d = fx_lhs(fx_of_double(kd, mag)), n = fx_lhs(kf), m = fx_lhs_neg(kf),
-                n3 = fx_lhs(fx_times(n, fx_rhs(fx_constant(NFX_RSQRT3_H, NFX_RSQRT3_L))));
+                n3 = fx_lhs(fx_times(n, fx_rhs(fx_constant(NFX_RSQRT3_H, NFX_RSQRT3_L)))), m3 = {-n3.h, fx_neg(n3.p)};
   if (!fx_mag_ok(mag)) return false;
   fx_right R[8];
 #pragma unroll
@@ -484,7 +484,8 @@ __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, co
       if (i == j) {
         if (im) {
           if (i < 2) fx_mac(s, i == 0 ? n : m, R[2]);
-          fx_mac(s, n3, i < 2 ? R[7] : fx_rhs(fx_twice(-gs[7 * TUNE_MAX_BLOCK])));
+          fx_mac(s, i < 2 ? n3 : m3, R[7]);
+          if (i == 2) fx_mac(s, m3, R[7]);  // (2 g7 / 8 passes the range at g7 = 8; |g| goes up to 8.6)
         }
       } else {
         const int q = i + j == 1 ? 0 : i + j == 2 ? 3 : 5;
