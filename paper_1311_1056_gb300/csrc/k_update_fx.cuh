@@ -457,12 +457,15 @@ __device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long
 }
 // A = 2 eps (X - Tr X / 3) + i sqrt(eps) sqrt(2) g_a lambda_a from the traceless
 // quarter of X 2^-cexp and g / 8 (element j at gs[j TUNE_MAX_BLOCK]).  The noise constant 8 sqrt(2 eps) passes the fixed-point
-// bound at eps = 0.016; from there on A is formed as a quarter.
+// bound at eps = 0.016, the drift's 8 eps 2^cexp at eps = 0.0112 for beta = 12 .. 24 (cexp = 4),
+// half that for the next octave of beta: from the lower one on A is formed as a
+// quarter.  (Out of range, every link takes the FP64 path: 16^4 step at beta = 24,
+// eps = 0.01, 1.06 ms against 0.72.)
 __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, const fx* gs, double eps, double sqrt_eps,
                                             int cexp) {
   fx_chk ck;
   unsigned mag = 0;
-  const bool quarter = !(sqrt_eps < 0.12);
+  const bool quarter = !(sqrt_eps < 0.12 && ldexp(8.0 * eps, cexp) < 1.4375);
   const double ks = sqrt_eps * (quarter ? 2.0 * 1.41421356237309504880 : 8.0 * 1.41421356237309504880);
   const double kd = ldexp(quarter ? 2.0 * eps : 8.0 * eps, cexp);  // times X / 4
   const fx kf = fx_of_double(ks, mag);

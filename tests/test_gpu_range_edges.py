@@ -102,3 +102,19 @@ def test_norm_of_small_links(cl, prec, tol, a):
         obs = lat.observables()
     assert abs(obs["un"] - un) <= tol * max(un, 1.0)
     assert abs(obs["max_det_dev"] - np.abs(np.linalg.det(U) - 1.0).max()) <= max(tol, 1e-13)
+
+
+@pytest.mark.parametrize("beta,theta", [(6.0, 1.0), (11.9, 0.0), (12.0, 0.0), (12.5, 2.0), (23.9, 0.0), (24.5, 0.0), (100.0, 1.0)])
+@pytest.mark.parametrize("eps", [0.0027, 0.0056, 0.0057, 0.0112, 0.0113, 0.012, 0.0145, 0.05])
+def test_update_on_both_sides_of_the_drift_constant(cl, beta, theta, eps):
+    """The drift's constant 8 eps 2^cexp on both sides of the fixed-point bound, with the noise's inside and outside.
+    The update is three products of matrices of size max |U| exp(|A|): 1e-12 of the result."""
+    L = (4, 3, 2, 5)
+    U = I.su3_lattice(L, 12)
+    ref = O.cl_step(L, U, beta, theta, eps, 99, 4)
+    with cl.Lattice(L, beta=beta, theta=theta, seed=99) as lat:
+        lat.set_links(U)
+        cl.cl_set_step(lat.h, 4)
+        lat.step(eps)
+        got = lat.links()
+    assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
