@@ -138,13 +138,12 @@ cudaError_t do_force(cl_lattice* l, bool th, double sre, double sim, int ce) {
     e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); });
   if (e == cudaSuccess && th)
     e = timed(l, CL_PHASE_CLOVER, [&] {
-      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, ldexp(sre, -ce), ldexp(sim, -ce),
-                               l->st);
+      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, sre, sim, l->st);
     }, clover_kernels(l));
   if (e == cudaSuccess)
     e = timed(l, CL_PHASE_FORCE, [&] {
       return launch_plaq_force(l->prec, th, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->F, l->Gq, l->C, l->p.beta,
-                               ce, l->st);
+                               sre, sim, ce, l->st);
     }, (th && l->prec != 1) ? 3 : 1);  // FP64 and DF64 split the theta force in three kernels
   return e;
 }
@@ -241,7 +240,7 @@ cl_status do_obs(cl_lattice* l, ObsOut* dst, double* q_site) {
     CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
-    return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, obs_clover_scale(l->prec), 0.0, l->st);
+    return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, 1.0, 0.0, l->st);
   }, clover_kernels(l)));
   CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->Un, l->Pq, l->Dq, l->F, l->partials, q_site, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
@@ -379,7 +378,8 @@ cl_status cl_init_lattice(const cl_params* params, void* cuda_stream, cl_lattice
     l->Omi = c + sizeof(double) * 8 * Vs + real_size(l) * 9 * Vs;
     l->crec = (double*)(c + align256(sizeof(double) * 8 * Vs + 2 * real_size(l) * 9 * Vs));
   }
-  cudaError_t e = init_state(l);
+  cudaError_t e = prepare_step_kernels(l->prec);
+  if (e == cudaSuccess) e = init_state(l);
   if (e != cudaSuccess) {
     cl_free(l);
     return fail(CL_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e));

@@ -248,12 +248,6 @@ __device__ __forceinline__ int fx_strength_exponent(double c) {
   const int e = (__double2hiint(c) >> 20) & 0x7ff;
   return max(-24, min(24, 1022 - e));
 }
-__device__ __forceinline__ double fx_scaled_double(double x, int t) {  // x 2^t for t within 64 of zero
-  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-  if (e == 0x7ff) return x;
-  if (e < 65) return 0.0;
-  return e > 1980 ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double(hi + t * (1 << 20), __double2loint(x));
-}
 // v 2^-n
 __device__ __forceinline__ fx fx_shifted(long long v, int n, fx_chk& ck) {
   const long long w = n >= 0 ? v >> n : v << -n;

@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(con
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
     fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq,
-                      (const int4*)c.C, (int4*)c.F, c.sre, c.sim, sm, it.vb);
+                      (const int4*)c.C, (int4*)c.F, sm, it.vb);
   else
     k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }
@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_a(const ChainDesc* _
                                                                 const WorkItem* __restrict__ w) {
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  __shared__ int4 sm[FX_PIPE];
+  extern __shared__ int4 sm_park[];
   fx_force_a_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (const int4*)c.F, (int4*)c.Gq,
-                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), sm, it.vb);
+                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), c.sre, c.sim, sm_park, it.vb);
 }
 
 template <typename T>
@@ -114,7 +114,8 @@ __global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_b(const ChainDesc* _
   const ChainDesc& c = cd[it.chain];
   __shared__ int4 sm[FX_PIPE];
   fx_force_b_body<T>(geo_of(c), (const typename vec2_of<T>::type*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
-                  (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), sm, it.vb);
+                  (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), c.sre,
+                  c.sim, sm, it.vb);
 }
 
 template <typename T>
@@ -148,6 +149,11 @@ __global__ void __launch_bounds__(ENS_BLOCK, 3) k_ens_update(const ChainDesc* __
   step_size<MODE>(geo_of(c), a);
 }
 
+template <typename T>
+cudaError_t prepare_ens_step() {
+  return cudaFuncSetAttribute(k_ens_force_a<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_PARK_BYTES);
+}
+
 // Launch family fam of the CL step for link type T (FP64 runs the clover
 // field and the theta force as two and three kernels).
 template <typename T>
@@ -166,7 +172,7 @@ cudaError_t launch_ens_step_family(int fam, const ChainDesc* cd, const WorkItem*
     case ENS_FORCE_THETA:
       if constexpr (is_fx<T>()) {
         k_ens_force_t<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
-        k_ens_force_a<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
+        k_ens_force_a<T><<<n, ENS_BLOCK, FX_PARK_BYTES, st>>>(cd, w);
         k_ens_force_b<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);
       } else {
         k_ens_force_ab<T><<<n, ENS_BLOCK, 0, st>>>(cd, w);

@@ -49,27 +49,38 @@ __device__ __forceinline__ fx_pair fx_fma2(fx_pair a, fx_pair b, fx_pair c) {
 __device__ __forceinline__ fx_pair fx_neg(fx_pair a) { return a ^ 0x8000000080000000ull; }
 
 // Range check: the largest of the results' high words, offset to be unsigned.
-// WIDE: |x| < 1.4375; NARROW: |x| < 0.359375, for results that are added to
-// others before their next use.
-enum { FX_WIDE = 0, FX_NARROW = 1 };
+// WIDE: |x| < 1.4375; NARROW: |x| < 0.359375, for results that are multiplied by
+// four; MID: |x| < 1, for results that are added to others (a sum below 2.5625
+// cannot wrap into the bound of WIDE).
+enum { FX_WIDE = 0, FX_NARROW = 1, FX_MID = 2 };
 struct fx_chk {
-  unsigned m0, m1;
-  __device__ __forceinline__ fx_chk() : m0(0), m1(0) {}
+  unsigned m0, m1, m2;
+  __device__ __forceinline__ fx_chk() : m0(0), m1(0), m2(0) {}
   template <int B>
   __device__ __forceinline__ void see(int hi) {  // hi: units of 2^-28
     if (B == FX_WIDE)
       m0 = max(m0, (unsigned)hi + 0x17000000u);
-    else
+    else if (B == FX_NARROW)
       m1 = max(m1, (unsigned)hi + 0x05C00000u);
+    else
+      m2 = max(m2, (unsigned)hi + 0x10000000u);
   }
   __device__ __forceinline__ void fail() { m0 = 0xffffffffu; }
-  __device__ __forceinline__ bool bad() const { return m0 >= 0x2E000000u || m1 >= 0x0B800000u; }
+  __device__ __forceinline__ bool bad() const { return m0 >= 0x2E000000u || m1 >= 0x0B800000u || m2 >= 0x20000000u; }
 };
 
 __device__ __forceinline__ fx operator-(fx a) { return fx{-a.l, -a.h}; }
 __device__ __forceinline__ fx operator+(fx a, fx b) { return fx{a.l + b.l, a.h + b.h}; }
 __device__ __forceinline__ fx operator-(fx a, fx b) { return fx{a.l - b.l, a.h - b.h}; }
 __device__ __forceinline__ fx fx_twice(fx a) { return fx{2.0f * a.l, 2 * a.h}; }
+// a + SIGN b with the low limb brought back below 2^29 (the carry by rounding the
+// limbs' sum to a multiple of 2^30), so that nothing is lost in it.
+template <int SIGN>
+__device__ __forceinline__ fx fx_sum_of(fx a, fx b) {
+  const float bl = SIGN > 0 ? b.l : -b.l;
+  const float r = (a.l + bl) + 0x1.8p53f, c = r - 0x1.8p53f;
+  return fx{fmaf(-0.5f, c, a.l) + fmaf(-0.5f, c, bl), a.h + SIGN * b.h + (__float_as_int(r) - __float_as_int(0x1.8p53f))};
+}
 
 // The 60-bit integer of a number, and back.
 __device__ __forceinline__ long long fx_bits(fx a) { return mad_wide(a.h, 1 << 30, (long long)__float2int_rn(a.l)); }
@@ -261,20 +272,22 @@ __device__ __forceinline__ void fx_adj(mat<fx>& r, mat<fx>& a, fx_chk& ck) {
   }
 }
 
-__device__ __forceinline__ void fx_add(mat<fx>& c, const mat<fx>& a) {
-#pragma unroll
-  for (int k = 0; k < 9; ++k) c.e[k] = cx<fx>{c.e[k].re + a.e[k].re, c.e[k].im + a.e[k].im};
-}
-// c <- 2 c + SIGN a
+// c <- c + SIGN a, |a| < 1
 template <int SIGN>
-__device__ __forceinline__ void fx_twice_add(mat<fx>& c, const mat<fx>& a) {
+__device__ __forceinline__ void fx_add_to(mat<fx>& c, const mat<fx>& a, fx_chk& ck) {
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    const cx<fx> t = {fx_twice(c.e[k].re), fx_twice(c.e[k].im)};
-    c.e[k] = SIGN > 0 ? cx<fx>{t.re + a.e[k].re, t.im + a.e[k].im} : cx<fx>{t.re - a.e[k].re, t.im - a.e[k].im};
+    c.e[k] = cx<fx>{fx_sum_of<SIGN>(c.e[k].re, a.e[k].re), fx_sum_of<SIGN>(c.e[k].im, a.e[k].im)};
+    ck.see<FX_WIDE>(c.e[k].re.h >> 2);
+    ck.see<FX_WIDE>(c.e[k].im.h >> 2);
   }
 }
-
+// c <- (c + a) / 4
+__device__ __forceinline__ void fx_quarter_sum(mat<fx>& c, const mat<fx>& a) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    c.e[k] = cx<fx>{fx_of_bits((fx_bits(c.e[k].re) + fx_bits(a.e[k].re)) >> 2), fx_of_bits((fx_bits(c.e[k].im) + fx_bits(a.e[k].im)) >> 2)};
+}
 // ---------------------------------------------------------- conversions
 // Double to fixed point, rounded to nearest (ties away).  Only |x| < 2 has an
 // image; `mag` collects the magnitudes' high words for the caller's check.
@@ -294,6 +307,55 @@ __device__ __forceinline__ long long fx_bits_of_double(double x, unsigned& mag) 
 __device__ __forceinline__ fx fx_of_double(double x, unsigned& mag) { return fx_of_bits(fx_bits_of_double(x, mag)); }
 // Whether the largest magnitude seen is below FX_BOUND (false for NaN and Inf).
 __device__ __forceinline__ bool fx_mag_ok(unsigned mag) { return mag < 0x3FF70000u; }  // 1.4375
+
+__device__ __forceinline__ double fx_scaled_double(double x, int t) {  // x 2^t for t within 64 of zero
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0x7ff) return x;
+  if (e < 65) return 0.0;
+  return e > 1980 ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double(hi + t * (1 << 20), __double2loint(x));
+}
+// A complex constant below one, times 2^t so that its larger part is in [1/2, 1):
+// a small one keeps its 53 bits (down to 2^-32; what it multiplies is then below
+// the numbers' resolution).
+struct fx_cscale {
+  fx_cleft m;
+  int t;
+  bool imag;  // real part zero
+  // (re + i im) 2^up
+  __device__ __forceinline__ fx_cscale(double re, double im, int up, unsigned& mag) {
+    const int e = max((__double2hiint(re) >> 20) & 0x7ff, (__double2hiint(im) >> 20) & 0x7ff);
+    t = max(0, min(31, 1022 - up - e));
+    imag = re == 0.0;
+    m = fx_lhs(cx<fx>{fx_of_double(fx_scaled_double(re, up + t), mag), fx_of_double(fx_scaled_double(im, up + t), mag)});
+  }
+};
+// a <- s a
+template <int B>
+__device__ __forceinline__ void fx_cscaled(mat<fx>& a, const fx_cscale& s, fx_chk& ck) {
+  const long long up = (1ll << 29) - (1ll << (29 - min(s.t, 29)));
+  const auto get = [&](const fx_acc& x, bool see) {
+    const long long r = fx_sum(x);  // offset by 2^29
+    const int hi = (int)(r >> 32), w = hi >> s.t;
+    if (see) ck.see<B>(w);
+    return fx_split((long long)(((unsigned long long)(unsigned)w << 32) | __funnelshift_r((unsigned)r, (unsigned)hi, s.t)) + up);
+  };
+  if (s.imag) {  // theta real
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      fx_acc re = fx_zero(), im = fx_zero();
+      fx_mac(re, s.m.nim, fx_rhs(a.e[k].im));
+      fx_mac(im, s.m.im, fx_rhs(a.e[k].re));
+      a.e[k] = cx<fx>{get(re, false), get(im, false)};  // no larger than a
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      fx_acc re = fx_zero(), im = fx_zero();
+      fx_cmac(re, im, s.m, fx_rhs(a.e[k]));
+      a.e[k] = cx<fx>{get(re, true), get(im, true)};
+    }
+  }
+}
 
 // v 2^(e - 60) as a double, rounded to nearest even.
 __device__ __forceinline__ double fx_bits_to_double(long long v, int e = 0) {
@@ -361,6 +423,21 @@ struct fx_pipe {
   }
 };
 
+// One matrix of a thread set aside in shared memory, laid out as a slot.
+struct fx_park {
+  static const int WORDS = 9 * FX_PIPE_THREADS;  // int4
+  int4* sm;
+  __device__ __forceinline__ explicit fx_park(int4* s) : sm(s + threadIdx.x) {}
+  __device__ __forceinline__ void put(const mat<fx>& a) const {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) sm[k * FX_PIPE_THREADS] = pack(a.e[k]);
+  }
+  __device__ __forceinline__ void get(mat<fx>& a) const {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) a.e[k] = unpack(sm[k * FX_PIPE_THREADS]);
+  }
+};
+
 // Plain (coherent) load, for words this kernel also writes; |v| < 1 for a 60-bit integer.
 __device__ __forceinline__ void fx_load_plain(mat<fx>& a, const int4* f, int plane, int site, int V) {
   const int4* p = f + (size_t)plane * 9 * V + site;
@@ -400,6 +477,16 @@ __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int si
     a.e[k].re *= f.sc;
     a.e[k].im *= f.sc;
   }
+}
+// The same times a complex factor (the clover field in the force).
+struct tagged_c {
+  tagged f;
+  cx<double> sc;
+};
+__device__ __forceinline__ void load(mat<double>& a, tagged_c f, int plane, int site, int V) {
+  load(a, f.f, plane, site, V);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a.e[k] = cmul(a.e[k], f.sc);
 }
 // In fixed point where it fits, so that one number out of range does not send
 // its readers the same way.

@@ -59,6 +59,7 @@ struct warp_ops {
     }
     return wmat{cx<double>{r.re * f.sc, r.im * f.sc}};
   }
+  __device__ __forceinline__ wmat load(tagged_c f, int plane, int s, int V) const { return wmat{cmul(load(f.f, plane, s, V).v, f.sc)}; }
   // In fixed point where it fits, as store(tagged).
   __device__ __forceinline__ void store(tagged f, int plane, int s, int V, const wmat& a) const {
     const double isc = 1.0 / f.sc, re = a.v.re * isc, im = a.v.im * isc;
@@ -93,7 +94,7 @@ static __device__ __noinline__ void warp_plaq(unsigned mask, Geo g, const typena
 }
 template <typename L>
 static __device__ __noinline__ void warp_clover(unsigned mask, Geo g, const typename vec2_of<L>::type* U, tagged Dq, tagged F,
-                                                double sre, double sim, int p, int s) {
+                                                double scale, int p, int s) {
   const warp_ops W(mask);
   const int mu = plane_mu(p), nu = plane_nu(p);
   int x[4];
@@ -106,7 +107,7 @@ static __device__ __noinline__ void warp_clover(unsigned mask, Geo g, const type
   const wmat d = W.load(Dq, p, xmn, g.V) + W.carry(W.adj(u), W.load(Dq, p, xmm_mn, g.V), u);
   u = W.link<L>(U, nu, xmn, g.V);
   acc = acc + W.carry(W.adj(u), d, u);
-  W.store(F, p, s, g.V, wmat{cmul(acc.v, cx<double>{sre, sim})});
+  W.store(F, p, s, g.V, scale * acc);
 }
 template <typename L>
 static __device__ __noinline__ void warp_force_wilson(unsigned mask, Geo g, const typename vec2_of<L>::type* U, tagged Dq,
@@ -121,7 +122,7 @@ static __device__ __noinline__ void warp_force_wilson(unsigned mask, Geo g, cons
 }
 template <typename L>
 static __device__ __noinline__ void warp_force(unsigned mask, Geo g, const typename vec2_of<L>::type* U, tagged Pq, tagged Dq,
-                                               tagged F, tagged C, double b6, int p, int s) {
+                                               tagged_c F, tagged C, double b6, int p, int s) {
   const warp_ops W(mask);
   const int mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
   int x[4];

@@ -245,7 +245,7 @@ __device__ __forceinline__ void force_stage_a(mat<T>& Gh, const Geo& g, int s, c
                                               FC C, T beta6) {
   const int mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
   // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
-  const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
+  const unsigned long long m = !std::is_same<FF, tagged_c>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c1 = hop(g, s, x, mu, 1);
   mat<T> D, M, t, q;
   load(D, Dq, p, s, g.V);
@@ -286,7 +286,7 @@ __device__ __forceinline__ void force_stage_b(mat<T>& Gh, const Geo& g, int s, c
                                               FC C, T beta6) {
   const int mu = plane_mu(p), nu = plane_nu(p), pc = 5 - p;
   // the fixed-point clover field is stored with its sign (k_update_fx.cuh)
-  const unsigned long long m = !std::is_same<FF, tagged>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
+  const unsigned long long m = !std::is_same<FF, tagged_c>::value && (p == 1 || p == 4) ? 0x8000000000000000ull : 0ull;
   const int c3 = hop(g, s, x, nu, 1);
   mat<T> D, M, t, q;
   // corner c3: G3r = u G3 u^{-1}; slot 3 partial = [D, G3r] + (beta/6) D

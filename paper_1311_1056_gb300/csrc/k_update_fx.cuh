@@ -4,17 +4,24 @@
 //
 // Fields between the kernels (int4 words, SoA as the links): Ux, the links in
 // fixed point, in the buffer that the update writes at the step's end; Ui
-// their inverses; P, D, F, C.  F and C carry the factor 2^-e that keeps the
-// drift contributions below one (drift_exponent, launch.h): F is -i theta
-// kappa 2^-e times the clover field, negated for planes 1 and 4 (the sign of
-// the pair 02|13), C is 2^-e times the contribution.
+// their inverses; P, D, F, C.  F is an eighth of the clover field, negated for
+// planes 1 and 4 (the sign of the pair 02|13); its factor -i theta kappa (s below)
+// comes in where the force is formed, times 2^-e, the factor that keeps the
+// contributions C within bounds (drift_exponent, launch.h).
+//
+// A fixed-point number's error is the same whatever its size, ~1e-17, so fields are
+// kept as large as the bounds allow.  (With F held times s 2^-e and C four times
+// smaller, errors against 80-bit arithmetic on links scattered by 0.27: drift at
+// theta = 1 1.3e-15 of its size, charge density 1.6e-15; now 1.7e-16 and 5.1e-16; FP64
+// arithmetic 2.7e-16 and 4.5e-16.)
 //
 // A thread whose inputs or results leave the fixed-point range calls the
 // general path, FP64 on the same fields (the whole warp for one plaquette,
 // general_warp.cuh, or the bodies of k_update.cuh), for its plaquette; that code is out of line and costs the others nothing.
 //
 // Scales that keep every number within the fixed-point bound: D is stored
-// halved (|D| < 2.9), the clover sum is formed as an eighth of F.
+// halved (|D| < 2.9), the sums of leaves are averages, the sum of the dual fields
+// over a plaquette's corners is a quarter.
 #pragma once
 #include "fixed.cuh"
 #include "general_warp.cuh"
@@ -26,14 +33,15 @@ namespace clgc {
 
 // Fields of the general path.
 __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
-__device__ __forceinline__ tagged tag_F(int4* f) { return tagged{f, 1.0, 0x3FD70000u}; }  // 0.359375 (FX_NARROW)
+// the clover field times s
+__device__ __forceinline__ tagged_c tag_F(const int4* f, double sre, double sim) { return tagged_c{tagged{const_cast<int4*>(f), 8.0}, cx<double>{sre, sim}}; }
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
 // 32^4: plaquettes and clover field 2.60 -> 2.48 ms a step, observables 3.03 ->
 // 2.92 ms.
 const int FX_BLOCK = FX_PIPE_THREADS;  // largest block of the kernels that use it
-const int FX_PIPE = fx_pipe<2>::WORDS;
+const int FX_PIPE = fx_pipe<2>::WORDS, FX_PARK_BYTES = (FX_PIPE + fx_park::WORDS) * (int)sizeof(int4);
 
 // ------------------------------------------------------ links and inverses
 template <typename L>
@@ -97,11 +105,10 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
 
 // ------------------------------------------------------------ clover field
 template <typename L>
-static __device__ __noinline__ void general_clover(Geo g, const typename vec2_of<L>::type* U, tagged Dq, tagged F, double sre, double sim,
-                                                   int vb) {
-  k_clover_rot_body<double>(g, link_field<L>{U}, Dq, F, sre, sim, vb);
+static __device__ __noinline__ void general_clover(Geo g, const typename vec2_of<L>::type* U, tagged Dq, tagged F, double scale, int vb) {
+  k_clover_rot_body<double>(g, link_field<L>{U}, Dq, F, scale, 0.0, vb);
 }
-// Half of the leaves: E(x) = [D(x) + U_mu(x-mu)^{-1} D(x-mu) U_mu(x-mu)] / 8,
+// Half of the leaves: E(x) = [D(x) + U_mu(x-mu)^{-1} D(x-mu) U_mu(x-mu)] / 4,
 // the leaves L1 and L2 of x.  L3 and L4 of x are the same of x - nu carried
 // along U_nu(x-nu), so two passes of two products each do what one pass does in
 // six (32^4: plaquettes and clover field 3.00 -> 2.60 ms a step, observables
@@ -123,26 +130,22 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
   P.ask(Ux, mu, xmm, g.V);
   P.take(d, ck);
   P.ask(Dq, p, s, g.V);
-  fx_mul_left<FX_NARROW, 2>(w, d, ck);
+  fx_mul_left<FX_WIDE, 1>(w, d, ck);
   P.take(d, ck);
   P.take(acc, ck);
-  fx_mul_acc<FX_WIDE, +1, 2>(acc, w, d, ck);
+  fx_mul_acc<FX_WIDE, +1, 1>(acc, w, d, ck);
   if (ck.bad()) acc.e[0].re.l = fx_raw_mark();  // its readers start over from D
   store<fx>(E, p, s, g.V, acc);
 }
-// F = E(x) + U_nu(x-nu)^{-1} E(x-nu) U_nu(x-nu), scaled.
-// sre, sim: the scale of plane p's F, |sre|, |sim| <= 1/32
+// F = +- [E(x) + U_nu(x-nu)^{-1} E(x-nu) U_nu(x-nu)] / 2.
 template <typename L>
 __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                const int4* __restrict__ Ui, const int4* __restrict__ Dq,
-                                               const int4* __restrict__ E, int4* F, double sre, double sim, int4* sm, int vb) {
+                                               const int4* __restrict__ E, int4* F, int4* sm, int vb) {
   const int p = vb % 6, nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
-  if (p == 1 || p == 4) {
-    sre = -sre;
-    sim = -sim;
-  }
+  const bool neg = p == 1 || p == 4;
   int x[4];
   site_coords(g, s, x);
   const int xmn = hop(g, s, x, nu, -1);
@@ -155,23 +158,18 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
   P.ask(Ux, nu, xmn, g.V);
   P.take(d, ck);
   P.ask(E, p, s, g.V);
-  fx_mul_left<FX_WIDE>(w, d, ck);
+  fx_mul_left<FX_WIDE, 1>(w, d, ck);
   P.take(d, ck);
   P.take(acc, ck);
-  fx_mul_acc<FX_WIDE, +1>(acc, w, d, ck);
-  unsigned mag = 0;
-  const cx<fx> sc = {fx_of_double(8.0 * sre, mag), fx_of_double(8.0 * sim, mag)};
-  const fx_cleft x8 = fx_lhs(sc);
+  fx_mul_acc<FX_WIDE, +1, 1>(acc, w, d, ck);
+  if (neg) {
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    fx_acc re = fx_zero(), im = fx_zero();
-    fx_cmac(re, im, x8, fx_rhs(acc.e[k]));
-    acc.e[k] = cx<fx>{fx_get<FX_NARROW>(re, ck), fx_get<FX_NARROW>(im, ck)};
+    for (int k = 0; k < 9; ++k) acc.e[k] = cx<fx>{-acc.e[k].re, -acc.e[k].im};
   }
   store<fx>(F, p, s, g.V, acc);
-  general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
-               [&](unsigned m, int t) { warp_clover<L>(m, g, U, tag_D(Dq), tag_F(F), sre, sim, p, t); },
-               [&] { general_clover<L>(g, U, tag_D(Dq), tag_F(F), sre, sim, vb); });
+  general_path(ck.bad(), s, g.V,
+               [&](unsigned m, int t) { warp_clover<L>(m, g, U, tag_D(Dq), tag(F), neg ? -0.125 : 0.125, p, t); },
+               [&] { general_clover<L>(g, U, tag_D(Dq), tag(F), neg ? -0.125 : 0.125, vb); });
 }
 
 // ------------------------------------------------------- plaquette drift
@@ -247,14 +245,15 @@ __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ 
   store<fx>(C, 4 * p + 3, s, g.V, A);
 }
 
-// Stage a of the theta force: corners c0 .. c2.  The sum of the dual fields
-// and the partials of slots 0 and 2 go to Gq and C (planes of this plaquette
+// Stage a of the theta force: corners c0 .. c2.  A quarter of the dual fields'
+// sum and the partials of slots 0 and 2 go to Gq and C (planes of this plaquette
 // that only stage b of the same thread's plaquette writes).  Both stages keep
 // at most three matrices in registers at a time, parking and re-reading the
-// rest: with a fourth they would spill.
+// rest: with a fourth they would spill.  s: the scale -i theta kappa 2^-e, |s| <=
+// 1/32; it multiplies D (and P), so the fields' errors are scaled down with it.
 __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                 const int4* __restrict__ Dq, const int4* __restrict__ F, int4* Gq,
-                                                int4* C, double b6, int4* sm, int vb) {
+                                                int4* C, double b6, double sre, double sim, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), pc = 5 - p;
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -263,19 +262,12 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
   const int c1 = hop(g, s, x, mu, 1);
   fx_chk ck;
   unsigned mag = 0;
-  const fx nb = fx_of_double(-b6, mag);
   mat<fx> A, B, M;
-  // corner c0: half the slot 0 partial, [D, G0] / 2 - (beta/6) D / 2
   fx_pipe<2> P(sm);
-  P.ask(Dq, p, s, g.V);
-  P.ask(F, pc, s, g.V);
-  P.take(A, ck);
+  const fx_park K(sm + FX_PIPE);
+  // corner c1: G1^ = a G1 a^{-1}
   P.ask(Ux, mu, s, g.V);
-  P.take(B, ck);
   P.ask(F, pc, c1, g.V);
-  fx_commutator<FX_NARROW>(M, A, B, nb, ck);
-  store<fx>(C, 4 * p + 0, s, g.V, M);
-  // corner c1: A = G1^ = a G1 a^{-1}; slot 2 partial = slot 0 partial + [D, G1^]
   P.take(A, ck);
   P.ask(Ui, mu, s, g.V);
   P.take(B, ck);
@@ -283,20 +275,28 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
   fx_mul_left<FX_WIDE>(A, B, ck);
   P.take(B, ck);
   P.ask(F, pc, s, g.V);
-  fx_mul_left<FX_NARROW>(A, B, ck);
+  fx_mul_left<FX_WIDE>(A, B, ck);
+  K.put(A);
+  // slot 0 partial -(beta/6) D + [s D, G0], slot 2 partial the same + [s D, G1^]
+  P.take(A, ck);
+  P.ask(F, pc, s, g.V);
+  fx_scaled<FX_WIDE>(M, A, fx_of_double(-2.0 * b6, mag), ck);
+  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 4, mag), ck);  // 8 s D = 16 s (D / 2)
   P.take(B, ck);
   P.ask(Ux, mu, s, g.V);
-  fx_commutator_acc<FX_NARROW>(M, B, A, ck);
+  fx_commutator_acc<FX_WIDE>(M, A, B, ck);
+  store<fx>(C, 4 * p + 0, s, g.V, M);
+  K.get(B);
+  fx_commutator_acc<FX_WIDE>(M, A, B, ck);
   store<fx>(C, 4 * p + 2, s, g.V, M);
-  P.take(B, ck);
+  P.take(M, ck);
   P.ask(C, 4 * p + 3, c1, g.V);
-  M = A;
-  fx_add(M, B);  // G0 + G1^
+  fx_quarter_sum(M, B);  // (G0 + G1^) / 4
   // corner c2: G2^ = a T(x+mu) a^{-1}
   P.take(A, ck);
   P.ask(Ui, mu, s, g.V);
   P.take(B, ck);
-  fx_mul_left<FX_WIDE>(A, B, ck);
+  fx_mul_left<FX_WIDE, 2>(A, B, ck);
   P.take(B, ck);
   fx_mul_acc<FX_WIDE, +1>(M, A, B, ck);
   if (ck.bad() || !fx_mag_ok(mag)) M.e[0].re.l = fx_raw_mark();  // stage b starts over
@@ -304,7 +304,7 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
 }
 
 template <typename L>
-static __device__ __noinline__ void general_force(Geo g, const typename vec2_of<L>::type* U, tagged Pq, tagged Dq, tagged F, tagged C,
+static __device__ __noinline__ void general_force(Geo g, const typename vec2_of<L>::type* U, tagged Pq, tagged Dq, tagged_c F, tagged C,
                                                   double b6, int vb) {
   k_plaq_force_ab_body<double>(g, link_field<L>{U}, Pq, Dq, F, C, b6, vb);
 }
@@ -312,28 +312,31 @@ static __device__ __noinline__ void general_force(Geo g, const typename vec2_of<
 template <typename L>
 __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                 const int4* __restrict__ Ui, const int4* Pq, const int4* Dq,
-                                                const int4* F, const int4* Gq, int4* C, double b6, int4* sm, int vb) {
+                                                const int4* F, const int4* Gq, int4* C, double b6, double sre, double sim,
+                                                int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   fx_chk ck;
   unsigned mag = 0;
-  const fx pb = fx_of_double(b6, mag);
+  const fx pb = fx_of_double(2.0 * b6, mag);
   mat<fx> A, B, M;
-  // corner c3: A = G3r = T; slot 3 partial = [D, G3r] + (beta/6) D
+  // corner c3: A = G3r = T; slot 3 partial = [s D, G3r] + (beta/6) D
   fx_pipe<2> P(sm);
+  P.ask(Dq, p, s, g.V);
   P.ask(C, 4 * p + 3, s, g.V);
-  P.ask(Dq, p, s, g.V);
+  P.take(B, ck);
+  P.ask(Pq, p, s, g.V);
+  fx_scaled<FX_WIDE>(M, B, pb, ck);
+  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 4, mag), ck);  // 8 s D
   P.take(A, ck);
-  P.ask(Pq, p, s, g.V);
-  P.take(B, ck);
   P.ask(Dq, p, s, g.V);
-  fx_commutator<FX_NARROW>(M, B, A, pb, ck);
+  fx_commutator_acc<FX_WIDE>(M, B, A, ck);
   store<fx>(C, 4 * p + 3, s, g.V, M);
-  // M = G^ += P G3r P^{-1}, with P^{-1} = P - 2 (D / 2)
+  // M = G^ / 4 += P G3r P^{-1} / 4, with P^{-1} = P - 2 (D / 2)
   P.take(B, ck);
   P.ask(Pq, p, s, g.V);
-  fx_mul_left<FX_WIDE>(B, A, ck);
+  fx_mul_left<FX_WIDE, 2>(B, A, ck);
   P.take(A, ck);
   P.ask(Gq, GQ_PLANE * p, s, g.V);
   P.take(M, ck);
@@ -343,24 +346,26 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   P.take(M, ck);
   P.ask(C, 4 * p + 0, s, g.V);
   fx_mul_acc<FX_WIDE, +1>(M, B, A, ck);
-  // A = K = P^{-1} G^ + G^ P
-  fx_mul_left<FX_WIDE>(A, M, ck);
+  // K = 32 s (P^{-1} G^ / 4 + G^ / 4 P), s taken with P^{-1} and P
   P.take(B, ck);
   P.ask(Dq, p, s, g.V);
-  fx_mul_acc<FX_NARROW, +1>(A, M, B, ck);
-  // slot 0: K + partial; slot 1: -K + (beta/6) D
+  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 5, mag), ck);
+  fx_mul_left<FX_WIDE>(A, M, ck);
+  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 5, mag), ck);
+  fx_mul_acc<FX_MID, +1>(A, M, B, ck);
+  // slot 0: partial + K; slot 1: (beta/6) D - K
   P.take(M, ck);
   P.ask(Ui, nu, s, g.V);
-  fx_twice_add<+1>(M, A);
+  fx_add_to<+1>(M, A, ck);
   store<fx>(C, 4 * p + 0, s, g.V, M);
   P.take(M, ck);
   P.ask(Ux, nu, s, g.V);
-  fx_scaled<FX_NARROW>(M, M, pb, ck);
-  fx_twice_add<-1>(M, A);
+  fx_scaled<FX_WIDE>(M, M, pb, ck);
+  fx_add_to<-1>(M, A, ck);
   store<fx>(C, 4 * p + 1, s, g.V, M);
-  // slot 3: u^{-1} (-K + partial) u
+  // slot 3: u^{-1} (partial - K) u
   load_rw(M, C, 4 * p + 3, s, g.V);
-  fx_twice_add<-1>(M, A);
+  fx_add_to<-1>(M, A, ck);
   P.take(B, ck);
   P.ask(C, 4 * p + 2, s, g.V);
   fx_mul_left<FX_WIDE>(B, M, ck);
@@ -368,10 +373,10 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   P.ask(Ui, mu, s, g.V);
   fx_mul_left<FX_WIDE>(B, M, ck);
   store<fx>(C, 4 * p + 3, s, g.V, B);
-  // slot 2: a^{-1} (K + partial) a
+  // slot 2: a^{-1} (partial + K) a
   P.take(M, ck);
   P.ask(Ux, mu, s, g.V);
-  fx_twice_add<+1>(M, A);
+  fx_add_to<+1>(M, A, ck);
   P.take(A, ck);
   fx_mul_left<FX_WIDE>(A, M, ck);
   P.take(M, ck);
@@ -379,8 +384,8 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   store<fx>(C, 4 * p + 2, s, g.V, A);
   // anything out of range: the whole plaquette again (its slots are its own)
   general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
-               [&](unsigned m, int t) { warp_force<L>(m, g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, p, t); },
-               [&] { general_force<L>(g, U, tag(Pq), tag_D(Dq), tag(F), tag(C), b6, vb); });
+               [&](unsigned m, int t) { warp_force<L>(m, g, U, tag(Pq), tag_D(Dq), tag_F(F, sre, sim), tag(C), b6, p, t); },
+               [&] { general_force<L>(g, U, tag(Pq), tag_D(Dq), tag_F(F, sre, sim), tag(C), b6, vb); });
 }
 
 // --------------------------------------------------------------- gather
@@ -457,10 +462,10 @@ __device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long
 }
 // A = 2 eps (X - Tr X / 3) + i sqrt(eps) sqrt(2) g_a lambda_a from the traceless
 // quarter of X 2^-cexp and g / 8 (element j at gs[j TUNE_MAX_BLOCK]).  The noise constant 8 sqrt(2 eps) passes the fixed-point
-// bound at eps = 0.016, the drift's 8 eps 2^cexp at eps = 0.0112 for beta = 12 .. 24 (cexp = 4),
-// half that for the next octave of beta: from the lower one on A is formed as a
-// quarter.  (Out of range, every link takes the FP64 path: 16^4 step at beta = 24,
-// eps = 0.01, 1.06 ms against 0.72.)
+// bound at eps = 0.016, the drift's 8 eps 2^cexp at eps = 0.0112 for beta = 24 .. 48
+// (cexp = 4), half that for the next octave of beta: from the lower one on A is
+// formed as a quarter.  (Out of range every link takes the FP64 path: 16^4 step 1.06
+// ms against 0.72.)
 __device__ __forceinline__ bool fx_exponent(mat<fx>& A /* in: the quarter */, const fx* gs, double eps, double sqrt_eps,
                                             int cexp) {
   fx_chk ck;

@@ -13,11 +13,13 @@ namespace clgc {
 // The step's launches for links of type L (k_update_fx_launch.cuh).
 template <typename L>
 struct StepFx {
+  static cudaError_t prepare();  // once per device: shared memory of the theta force
   static cudaError_t links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st);
   static cudaError_t plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq, cudaStream_t st);
   static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* E,
-                            void* F, double sre, double sim, cudaStream_t st);
-  static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6, cudaStream_t st);
+                            void* F, cudaStream_t st);
+  static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
+                           double sre, double sim, cudaStream_t st);
   static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, double k_ref,
                             uint64_t seed, StepDev* sd, int cexp, cudaStream_t st);
 };
@@ -53,9 +55,9 @@ __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover_half(Geo g
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                     const int4* __restrict__ Ui, const int4* __restrict__ Dq,
-                                                    const int4* __restrict__ E, int4* F, double sre, double sim) {
+                                                    const int4* __restrict__ E, int4* F) {
   __shared__ int4 sm[FX_PIPE];
-  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sre, sim, sm, blockIdx.x);
+  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sm, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
@@ -74,17 +76,17 @@ __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_a(Geo g,
                                                                const int4* __restrict__ Ui,
                                                                const int4* __restrict__ Dq,
                                                                const int4* __restrict__ F, int4* Gq, int4* C,
-                                                               double b6) {
-  __shared__ int4 sm[FX_PIPE];
-  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, sm, blockIdx.x);
+                                                               double b6, double sre, double sim) {
+  extern __shared__ int4 sm_park[];
+  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, sre, sim, sm_park, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui, const int4* Pq,
                                                                const int4* Dq, const int4* F, const int4* Gq, int4* C,
-                                                               double b6) {
+                                                               double b6, double sre, double sim) {
   __shared__ int4 sm[FX_PIPE];
-  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sm, blockIdx.x);
+  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, sm, blockIdx.x);
 }
 template <typename L, int MODE>
 __global__ void __maxnreg__(UPDATE_MAXNREG) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
@@ -94,6 +96,11 @@ __global__ void __maxnreg__(UPDATE_MAXNREG) k_fx_update(Geo g, const typename ve
   step_size<MODE>(g, a);
 }
 }  // namespace
+
+template <typename L>
+cudaError_t StepFx<L>::prepare() {
+  return cudaFuncSetAttribute(k_fx_force_a, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_PARK_BYTES);
+}
 
 template <typename L>
 cudaError_t StepFx<L>::links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st) {
@@ -114,19 +121,18 @@ cudaError_t StepFx<L>::plaq(const GeoH& h, const void* U, const void* Ux, const 
 
 template <typename L>
 cudaError_t StepFx<L>::clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                                  void* E, void* F, double sre, double sim, cudaStream_t st) {
+                                  void* E, void* F, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
   k_fx_clover_half<<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)E);
-  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E,
-                                               (int4*)F, sre, sim);
+  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E, (int4*)F);
   return cudaGetLastError();
 }
 
 template <typename L>
 cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui,
                                   const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
-                                  cudaStream_t st) {
+                                  double sre, double sim, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_FORCE), FX_BLOCK);
   const dim3 gr = grid(g.V, 6, bs);
@@ -135,10 +141,10 @@ cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const voi
     return cudaGetLastError();
   }
   k_fx_force_t<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)F, (int4*)C);
-  k_fx_force_a<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)F, (int4*)Gq,
-                                  (int4*)C, b6);
+  k_fx_force_a<<<gr, bs, FX_PARK_BYTES, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)F, (int4*)Gq,
+                                  (int4*)C, b6, sre, sim);
   k_fx_force_b<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Pq, (const int4*)Dq,
-                                  (const int4*)F, (const int4*)Gq, (int4*)C, b6);
+                                  (const int4*)F, (const int4*)Gq, (int4*)C, b6, sre, sim);
   return cudaGetLastError();
 }
 

@@ -443,11 +443,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
     v[1] += ti * (1.0 / 3.0);
     v[2] += 2.0 * tr - (fx_bits_to_double(dr, FX ? 3 : 2) + wp[2]);
     v[3] += 2.0 * ti - (fx_bits_to_double(di, FX ? 3 : 2) + wp[3]);
-    // topological charge density; F carries obs_clover_scale
+    // topological charge density (fixed point: F is an eighth of the clover field)
     cx<double> q = {0.0, 0.0};
     if constexpr (FX) {
       fx_acc re = fx_zero(), im = fx_zero();
       fx_chk ck;
+      float nf = 0.0f;  // sum of |F|^2, twice a bound of the traces' sum
 #pragma unroll 1
       for (int p = 0; p < 3; ++p) {  // the planes 1 and 4 are both stored negated
         mat<fx> F1, F2;
@@ -456,10 +457,14 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-          for (int k = 0; k < 3; ++k)
-            fx_cmac(re, im, p == 1 ? fx_lhs_neg(F1.e[3 * i + k]) : fx_lhs(F1.e[3 * i + k]), fx_rhs(F2.e[3 * k + i]));
+          for (int k = 0; k < 3; ++k) {
+            const cx<fx> x = F1.e[3 * i + k], y = F2.e[3 * k + i];
+            fx_cmac(re, im, p == 1 ? fx_lhs_neg(x) : fx_lhs(x), fx_rhs(y));
+            nf = fmaf((float)x.re.h, (float)x.re.h, fmaf((float)x.im.h, (float)x.im.h, nf));
+            nf = fmaf((float)y.re.h, (float)y.re.h, fmaf((float)y.im.h, (float)y.im.h, nf));
+          }
       }
-      if (!ck.bad()) {  // |F| < 0.36: 54 products stay below 7
+      if (!ck.bad() && nf < 15.0f * 0x1p60f) {
         q.re = fx_bits_to_double(fx_sum<true>(re) - (1 << 29));
         q.im = fx_bits_to_double(fx_sum<true>(im) - (1 << 29));
       } else {
@@ -470,8 +475,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
           q.im += p == 1 ? -t[1] : t[1];
         }
       }
-      q.re *= 1024.0 * KAPPA_Q;
-      q.im *= 1024.0 * KAPPA_Q;
+      q.re *= 64.0 * KAPPA_Q;
+      q.im *= 64.0 * KAPPA_Q;
     } else {
 #pragma unroll
       for (int p = 0; p < 3; ++p) {

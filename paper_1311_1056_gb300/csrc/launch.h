@@ -113,14 +113,14 @@ cudaError_t launch_soa_to_aos(int prec, const GeoH& g, const void* U, double* ao
                               cudaStream_t st);
 // The FP64 and DF64 forms run the step's link algebra in 64-bit fixed point
 // (k_update_fx.cuh): Ux receives the links in fixed point (the update's target
-// buffer, free until then), the clover scale and the contributions C carry the
-// factor 2^-cexp, cexp = drift_exponent(beta, scale_re, scale_im).  FP32
-// storage ignores Ux and Ui and takes cexp = 0.
+// buffer, free until then), the contributions C carry the factor 2^-cexp, cexp =
+// drift_exponent(beta, scale_re, scale_im).  FP32 storage ignores Ux and Ui and
+// takes cexp = 0.
 int drift_exponent(double beta, double sre, double sim);
-// Scale of the clover field that launch_obs expects (fixed point: entries below one).
-inline double obs_clover_scale(int prec) { return prec != 1 ? 0.03125 : 1.0; }
+cudaError_t prepare_step_kernels(int prec);  // before a device's first step of that form
 // The CL step (k_update.cuh): link inverses Ui; plaquettes P and D = P - P^{-1}
-// (six planes); the clover field F^ = scale * F_{mu nu}(x) built from the D's;
+// (six planes); the clover field F^ = scale * F_{mu nu}(x) built from the D's (fixed
+// point: F_{mu nu} / 8 whatever the scale, which the force then applies);
 // the per-plaquette drift contributions C (24 planes: 4 links x 6 planes);
 // then per link the gather of its six contributions followed by the update
 // (mode 0) or by storing the drift matrix X_S (mode 1).
@@ -137,7 +137,7 @@ cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void
 // some of these).
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
-                              double beta, int cexp, cudaStream_t st);
+                              double beta, double scale_re, double scale_im, int cexp, cudaStream_t st);
 // mode 0: update from the gathered drift, step size eps; 1: write the drift X_S
 // to out; 2: write X_S to out, max |K| and from it the device step size, eps
 // min(1, k_ref / K_max); 3: update reading X_S from C (a mode-2 output), device
@@ -174,7 +174,7 @@ cudaError_t launch_cool_apply(int prec, const GeoH& g, const CoolBufs& b, bool r
 // Ux from U (FP64, DF64), for an apply without a gradient before it.
 cudaError_t launch_cool_load(int prec, const GeoH& g, const void* U, void* Ux, cudaStream_t st);
 // Observables: per-site pass over the links, the plaquette pass's fields and
-// the clover field F (scale obs_clover_scale), then the final fixed-order
+// the clover field F (FP32 storage: of scale one), then the final fixed-order
 // reduction into *out.
 cudaError_t launch_obs(int prec, const GeoH& g, const void* U, const void* Ux, const void* Pq, const void* Dq,
                        const void* F, double* partials, double* q_site, cudaStream_t st);

@@ -104,7 +104,8 @@ def test_norm_of_small_links(cl, prec, tol, a):
     assert abs(obs["max_det_dev"] - np.abs(np.linalg.det(U) - 1.0).max()) <= max(tol, 1e-13)
 
 
-@pytest.mark.parametrize("beta,theta", [(6.0, 1.0), (11.9, 0.0), (12.0, 0.0), (12.5, 2.0), (23.9, 0.0), (24.5, 0.0), (100.0, 1.0)])
+@pytest.mark.parametrize("beta,theta", [(6.0, 1.0), (11.9, 0.0), (12.0, 0.0), (12.5, 2.0), (23.9, 0.0), (24.5, 0.0), (48.5, 0.0),
+                                        (100.0, 1.0)])
 @pytest.mark.parametrize("eps", [0.0027, 0.0056, 0.0057, 0.0112, 0.0113, 0.012, 0.0145, 0.05])
 def test_update_on_both_sides_of_the_drift_constant(cl, beta, theta, eps):
     """The drift's constant 8 eps 2^cexp on both sides of the fixed-point bound, with the noise's inside and outside.
