@@ -88,7 +88,7 @@ __device__ __forceinline__ void load_herm_mat(mat<double>& m, tagged_herm f, int
 // re / im of 01, 02, 12.
 struct fx_gradient {
   long long d[3], o[6];  // times 2^-e, below one
-  int e;
+  int e, wild;           // wild: e, where it comes from links beyond the bound
 };
 // rows (or conjugated columns) r0, r1, r2 of one link: += sign r_i conj(r_j); n: their squares in float
 __device__ __forceinline__ void fx_outer(fx_acc* D, fx_acc* O, float* n, cx<fx> r0, cx<fx> r1, cx<fx> r2, bool neg) {

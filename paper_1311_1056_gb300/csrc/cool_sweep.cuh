@@ -233,7 +233,9 @@ template <typename L, int N>
 struct SweepPart {
   static const int WIDTH = is_fx<L>() ? CS_THREADS : CS_SITES;
   typename sweep_real<L>::type q[N][WIDTH];
-  float top[is_fx<L>() ? CS_THREADS : 1];  // largest row or column norm (squared); infinite: not representable
+  // fixed point: largest row or column norm (squared); negative: of a direction whose
+  // sums are in sixteenths; infinite: not representable
+  float top[is_fx<L>() ? CS_THREADS : 1];
 };
 
 // FP32 storage.  The rule compares differences of norms, themselves sums of
@@ -331,10 +333,26 @@ __device__ __forceinline__ bool fx_load_wild(mat<fx>& u, const int4* Ux, int mu,
   }
   return fx_mag_ok(mag);
 }
-// A thread's part of the gradient where a link of it is beyond the bound: both
-// links times 1/4, the sums times 16.  (In FP64 the site's eight links are one
-// thread's chain of ~600 instructions: 20 us a sweep for the whole launch.)
-static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* top, const int4* Ux, int mu, int s, int sb, int V) {
+// A thread's part of the gradient where a link of it is beyond the bound or a sum
+// beyond 8: both links times 1/4, the sums in sixteenths.  (In FP64 the site's eight
+// links are one thread's chain of ~600 instructions: 20 us a sweep for the whole
+// launch, and at a unitarity norm of 1.2 all sites': 24^4, five sweeps, 10.0 ms
+// against 4.4.)
+template <typename L, bool FIRST>
+static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* top, const void* U, const int4* Ux, int mu, int s, int sb,
+                                                    int V) {
+  const auto get = [&](mat<fx>& u, int site) {
+    if constexpr (FIRST) {  // the neighbour's words may not be there yet
+      mat<double> d;
+      load_link_d<L>(d, (const typename vec2_of<L>::type*)U, mu, site, V);
+      unsigned mag = 0;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_double(fx_scaled_double(d.e[k].re, -2), mag), fx_of_double(fx_scaled_double(d.e[k].im, -2), mag)};
+      return fx_mag_ok(mag);
+    } else {
+      return fx_load_wild<2>(u, Ux, mu, site, V);
+    }
+  };
   fx_acc D[3], O[6];
   float nf[3] = {0.0f, 0.0f, 0.0f}, nb[3] = {0.0f, 0.0f, 0.0f}, m = 0.0f;
 #pragma unroll
@@ -342,13 +360,14 @@ static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* 
 #pragma unroll
   for (int i = 0; i < 6; ++i) O[i] = fx_zero();
   mat<fx> u;
-  if (!fx_load_wild<2>(u, Ux, mu, s, V)) return;
+  *top = __int_as_float(0x7f800000);
+  if (!get(u, s)) return;
 #pragma unroll
   for (int k = 0; k < 3; ++k) fx_outer(D, O, nf, u.e[k], u.e[3 + k], u.e[6 + k], false);
   if (n > 9)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) q[(9 + i) * CS_THREADS] = (fx_sum<true>(D[i]) - (1 << 29)) << 4;
-  if (!fx_load_wild<2>(u, Ux, mu, sb, V)) return;
+    for (int i = 0; i < 3; ++i) q[(9 + i) * CS_THREADS] = fx_sum<true>(D[i]) - (1 << 29);
+  if (!get(u, sb)) return;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const cx<fx> a = u.e[3 * k], b = u.e[3 * k + 1], c = u.e[3 * k + 2];
@@ -356,12 +375,12 @@ static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* 
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    q[i * CS_THREADS] = (fx_sum<true>(D[i]) - (1 << 29)) << 4;
+    q[i * CS_THREADS] = fx_sum<true>(D[i]) - (1 << 29);
     m = fmaxf(m, fmaxf(nf[i], nb[i]));
   }
 #pragma unroll
-  for (int i = 0; i < 6; ++i) q[(3 + i) * CS_THREADS] = (fx_sum<true>(O[i]) - (1 << 29)) << 4;
-  *top = m * 0x1p-56f;
+  for (int i = 0; i < 6; ++i) q[(3 + i) * CS_THREADS] = fx_sum<true>(O[i]) - (1 << 29);
+  if (m < 7.6f * 0x1p60f) *top = -16.0f * 0x1p-60f * m;
 }
 
 // First half: this thread's direction (fixed point) or pair (FP32 storage), a warp
@@ -439,8 +458,9 @@ __device__ __forceinline__ void sweep_part(SweepPart<L, N>& sm, const Geo& g, co
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i) sm.q[3 + i][t] = fx_sum<true>(O[i]) - (1 << 29);
-    sm.top[t] = ok && !ck.bad() ? top * 0x1p-60f : __int_as_float(0x7f800000);
-    if (!FIRST && ck.bad()) sweep_part_wild(&sm.q[0][t], N, &sm.top[t], Ux, mu, s, sb, g.V);
+    top *= 0x1p-60f;
+    sm.top[t] = ok && !ck.bad() && top < 7.6f ? top : __int_as_float(0x7f800000);
+    if (!ok || ck.bad() || !(top < 7.6f)) sweep_part_wild<L, FIRST>(&sm.q[0][t], N, &sm.top[t], a.U, Ux, mu, s, sb, g.V);
   } else if (mu < 3) {
     float d, fwd;
     cx<float> o;
@@ -460,11 +480,30 @@ __device__ __forceinline__ typename sweep_real<L>::type sweep_sum(const SweepPar
   const int l = threadIdx.x & 31;
   return ((sm.q[q][l] + sm.q[q][32 + l]) + sm.q[q][64 + l]) + sm.q[q][96 + l];
 }
+// The sum of number q times 2^-n, for sites with directions in sixteenths.
+template <typename L, int N>
+static __device__ __noinline__ long long sweep_sum_wild(const SweepPart<L, N>& sm, int q, int n) {
+  long long v = 0;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const int l = (threadIdx.x & 31) + 32 * mu, k = sm.top[l] < 0.0f ? n - 4 : n;
+    v += k >= 0 ? sm.q[q][l] >> k : sm.q[q][l] << -k;
+  }
+  return v;
+}
+// The sum of the norms' diagonals, Tr U U^+ over the four forward links, likewise.
+template <typename L, int N>
+static __device__ __noinline__ double sweep_norm_wild(const SweepPart<L, N>& sm, int n) {
+  double un = 0.0;
+  for (int i = 0; i < 3; ++i) un += fx_bits_to_double(sweep_sum_wild(sm, 9 + i, n), n);
+  return un;
+}
 template <typename L, int N>
 __device__ __forceinline__ bool sweep_gradient(fx_gradient& G, const SweepPart<L, N>& sm) {
   const int l = threadIdx.x & 31;
   // the sums over the four directions must stay below 8
-  const bool ok = ((sm.top[l] + sm.top[32 + l]) + sm.top[64 + l]) + sm.top[96 + l] < 7.6f;
+  const float t0 = sm.top[l], t1 = sm.top[32 + l], t2 = sm.top[64 + l], t3 = sm.top[96 + l];
+  const bool tame = fminf(fminf(t0, t1), fminf(t2, t3)) >= 0.0f && ((t0 + t1) + t2) + t3 < 7.6f;
 #pragma unroll
   for (int i = 0; i < 3; ++i) G.d[i] = sweep_sum(sm, i);
 #pragma unroll
@@ -474,6 +513,7 @@ __device__ __forceinline__ bool sweep_gradient(fx_gradient& G, const SweepPart<L
 #pragma unroll
   for (int k = 0; k < 3; ++k) one = one && fx_below_one(G.d[k]) && fx_below_one(G.o[2 * k]) && fx_below_one(G.o[2 * k + 1]);
   G.e = one ? 0 : 3;
+  G.wild = 0;
   if (!one) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -482,7 +522,17 @@ __device__ __forceinline__ bool sweep_gradient(fx_gradient& G, const SweepPart<L
       G.o[2 * k + 1] >>= 3;
     }
   }
-  return ok;
+  if (!tame) {
+    const float top = ((fabsf(t0) + fabsf(t1)) + fabsf(t2)) + fabsf(t3);
+    if (!(top < 1024.0f)) return false;
+    const int n = max(1, ((__float_as_int(top) >> 23) & 0xff) - 126);  // top 2^-n in [1/2, 1)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) G.d[i] = sweep_sum_wild(sm, i, n);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) G.o[i] = sweep_sum_wild(sm, 3 + i, n);
+    G.e = G.wild = n;
+  }
+  return true;
 }
 __device__ __forceinline__ void sweep_f(float* fa, const float* q) {
   fa[0] = 4.0f * q[3];
@@ -585,7 +635,7 @@ __device__ __forceinline__ void sweep_grad_site(SweepSums& v, const SweepPart<L,
         long long dev = 0;  // of the three diagonals from 4, 2^-58
 #pragma unroll
         for (int i = 0; i < 3; ++i) dev += (sweep_sum(sm, 9 + i) - (4ll << 60)) >> 2;
-        un = 12.0 + fx_bits_to_double(dev, 2);
+        un = G.wild ? sweep_norm_wild(sm, G.wild) : 12.0 + fx_bits_to_double(dev, 2);
       } else {
         double fg[8];
         un = general_cool_grad<L, FIRST>(g, a.U, a.Ux, s, fg);
@@ -887,13 +937,25 @@ static __device__ __noinline__ double far_cool_apply(const Geo g, int4* Ux, int2
   fx_apply_ops ops;
   fx_lhs(ops, o);
   long long dev = 0;
-  fx_apply_link<false>(u, ops, oi, ck, dev);
+  fx_apply_link<true>(u, ops, oi, ck, dev);
   if (ck.bad()) return general_cool_apply(g, Ux, Om, Omi, mu, s, sp);
-  mat<double> d;
+  int top = 0;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) d.e[k] = cx<double>{fx_to_double(u.e[k].re, 3), fx_to_double(u.e[k].im, 3)};
-  store(tagged{Ux, 1.0}, mu, s, g.V, d);
-  return norm2(d);
+  for (int k = 0; k < 9; ++k) top = max(top, max(abs(u.e[k].re.h), abs(u.e[k].im.h)));
+  const bool fits = top < (int)(1.4375 / 8 * (1 << 30)) - 1;
+  int4* p = Ux + (size_t)mu * 9 * g.V + s;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const long long re = fx_bits(u.e[k].re), im = fx_bits(u.e[k].im);
+    if (fits) {
+      p[(size_t)k * g.V] = pack(cx<fx>{fx_of_bits(re << 3), fx_of_bits(im << 3)});
+    } else {
+      const double x = fx_bits_to_double(re, 3), y = fx_bits_to_double(im, 3);
+      const int2 w = k == 0 ? fx_raw_first(x) : make_int2(__double2loint(x), __double2hiint(x));
+      p[(size_t)k * g.V] = make_int4(w.x, w.y, __double2loint(y), __double2hiint(y));
+    }
+  }
+  return 192.0 + fx_bits_to_double(dev, 6);  // dev: Tr (U / 8) (U / 8)^+ - 3
 }
 // A thread's next link and its two Omegas on their way into shared memory while
 // it works on the current ones (lattices where a block takes several groups:
@@ -981,11 +1043,14 @@ __device__ __forceinline__ void sweep_apply_body(const Geo& g, const SweepArgs& 
       fx_load_herm(oi, (const int2*)a.Omi, sp, g.V, ck);
       fx_load_plain(u, Ux, mu, s, g.V);
     }
-    if (fx_is_raw(u.e[0].re.l)) ck.fail();
-    fx_apply_ops ops;
-    fx_lhs(ops, o);
     long long dev = 0;
-    fx_apply_link<RULE>(u, ops, oi, ck, dev);
+    if (fx_is_raw(u.e[0].re.l)) {
+      ck.fail();
+    } else {
+      fx_apply_ops ops;
+      fx_lhs(ops, o);
+      fx_apply_link<RULE>(u, ops, oi, ck, dev);
+    }
     if (!ck.bad()) {
       if (last) fx_store_link(U, mu, s, g.V, u);
       if (!last || !RULE) store<fx>(Ux, mu, s, g.V, u);  // D_2 calls end with a gradient

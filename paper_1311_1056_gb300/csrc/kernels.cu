@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(256) k_soa_to_aos(Geo g, const typename vec2_o
 // --------------------------------------------------------------- cooling
 // The kernels of cool_sweep.cuh, one launch per lattice.
 template <typename L, bool FIRST, int W>
-__global__ void __launch_bounds__(CS_THREADS) k_cool_grad(Geo g, SweepArgs a, int rule) {
+__global__ void __launch_bounds__(CS_THREADS, is_fx<L>() ? 4 : 0) k_cool_grad(Geo g, SweepArgs a, int rule) {
   sweep_grad_body<L, FIRST, W>(g, a, blockIdx.x, rule != 0);
 }
 template <typename L, bool SPLIT>
