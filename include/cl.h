@@ -176,16 +176,18 @@ cl_status cl_trajectory(cl_lattice* lat, double eps, int n_steps, const cl_cool_
  * update), CL_TUNE_OMEGA (cooling transformation), CL_TUNE_APPLY (cooling
  * apply).  The reductions keep a fixed shape so that their summation order,
  * and hence every result, is the same under any tuning.  The cooling kernels
- * choose their own shape by lattice size: the last two families are accepted,
- * timed and stored, and change no launch.
+ * choose their own shape by lattice size: the last two families are accepted and
+ * stored, and change no launch.  The FP64 and DF64 forms' first two families launch
+ * at most 128 threads a block.
  * cl_set_blocks: blocks[CL_NTUNE], each 0 (default, 128) or a multiple of 32
  *   in [32, 256]; takes effect for later launches (graphs already captured
  *   keep the shape they were captured with).
  * cl_get_blocks: the block sizes in effect.
  * cl_autotune: times one CL step + 2 cooling sweeps (eps, cp with the sweep
  *   count forced to 2) reps times for every candidate block size in
- *   {32, 64, 128, 256}, sets the fastest per family and writes it to
- *   blocks_out (may be NULL).  ms_out (may be NULL) receives the mean
+ *   {32, 64, 128, 256}, sets the fastest per family (of sizes that launch the
+ *   same, the one that is launched, with the smallest of their times) and writes
+ *   it to blocks_out (may be NULL).  ms_out (may be NULL) receives the mean
  *   per-step milliseconds, [4 candidates][CL_NTUNE].  The lattice is left as
  *   it was (links, step counter, cooling state; snapshot in a temporary
  *   device buffer of one link field).  With use_cache != 0 and ms_out NULL a

@@ -1290,6 +1290,14 @@ TuneKey tune_key(const cl_lattice* l) {
   return k;
 }
 
+// What a family launches when block size b is asked for: the fixed-point link
+// algebra takes at most 128 threads (its shared-memory slots), the cooling kernels
+// have one shape.
+int launched_block(const cl_lattice* l, int fam, int b) {
+  if (fam == TUNE_OMEGA || fam == TUNE_APPLY) return TUNE_DEFAULT_BLOCK;
+  return l->prec != 1 && fam != TUNE_UPDATE ? std::min(b, 128) : b;
+}
+
 bool valid_block(int b) { return b == 0 || (b >= 32 && b <= TUNE_MAX_BLOCK && b % 32 == 0); }
 
 }  // namespace
@@ -1399,9 +1407,20 @@ cl_status cl_autotune(cl_lattice* l, double eps, const cl_cool_params* cp, int r
   }
   std::array<int, NTUNE> best;
   for (int f = 0; f < NTUNE; ++f) {
-    int bc = 0;
-    for (int c = 1; c < N_TUNE_CANDIDATES; ++c)
-      if (table[c][f] < table[bc][f]) bc = c;
+    // sizes of the same launch have one time, the smallest measured, and the first
+    // of them that is what is launched is taken
+    const auto launched = [&](int c) { return launched_block(l, f, TUNE_CANDIDATES[c]); };
+    double ms[N_TUNE_CANDIDATES];
+    for (int c = 0; c < N_TUNE_CANDIDATES; ++c) {
+      ms[c] = table[c][f];
+      for (int d = 0; d < N_TUNE_CANDIDATES; ++d)
+        if (launched(d) == launched(c)) ms[c] = std::min(ms[c], table[d][f]);
+    }
+    int bc = -1;
+    for (int c = 0; c < N_TUNE_CANDIDATES; ++c) {
+      table[c][f] = ms[c];
+      if (TUNE_CANDIDATES[c] == launched(c) && (bc < 0 || ms[c] < ms[bc])) bc = c;
+    }
     best[f] = TUNE_CANDIDATES[bc];
     l->g.blk[f] = best[f];
   }

@@ -105,7 +105,7 @@ cudaError_t StepFx<L>::prepare() {
 template <typename L>
 cudaError_t StepFx<L>::links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
-  const int bs = block_of(h, TUNE_CLOVER);
+  const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
   k_fx_links<L><<<grid(g.V, 4, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (int4*)Ux, (int4*)Ui);
   return cudaGetLastError();
 }
