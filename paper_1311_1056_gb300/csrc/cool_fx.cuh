@@ -259,7 +259,7 @@ __device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradien
   fx_chk ck;
   unsigned mag = 0;
   const int t = fx_strength_exponent(4.0 * c);
-  const fx_left c4 = fx_lhs(fx_of_double(fx_scaled_double(4.0 * c, t), mag));
+  const fx_left c4 = fx_lhs(fx_of_double(fx_pow2(4.0 * c, t), mag));
   const long long third = (G.d[0] + G.d[1] + G.d[2]) / 3;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -278,7 +278,7 @@ __device__ __forceinline__ bool fx_herm_of_gradient(fx_herm& H, const fx_gradien
   return !ck.bad() && fx_mag_ok(mag);
 }
 // The same from f: H = c f_a lambda_a.
-__device__ __forceinline__ fx fx_of_real(double x, int t, unsigned& mag) { return fx_of_double(fx_scaled_double(x, -t), mag); }
+__device__ __forceinline__ fx fx_of_real(double x, int t, unsigned& mag) { return fx_of_double(fx_pow2(x, -t), mag); }
 __device__ __forceinline__ fx fx_of_real(float x, int t, unsigned& mag) {
   x *= __int_as_float((127 - t) << 23);
   if (!(fabsf(x) < 1.4375f)) mag = 0xffffffffu;
@@ -289,7 +289,7 @@ __device__ __forceinline__ bool fx_herm_of_f(fx_herm& H, const T* f, double c0) 
   fx_chk ck;
   unsigned mag = 0;
   const int t = fx_strength_exponent(c0);
-  const double c = fx_scaled_double(c0, t);
+  const double c = fx_pow2(c0, t);
   const fx_left cl = fx_lhs(fx_of_double(c, mag)), cn = fx_lhs(fx_of_double(-c, mag)),
                 c3 = fx_lhs(fx_of_double(c * 0.57735026918962576451, mag)),
                 m3 = fx_lhs(fx_of_double(-2.0 * (c * 0.57735026918962576451), mag));

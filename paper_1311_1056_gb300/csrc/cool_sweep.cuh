@@ -83,7 +83,7 @@ __device__ __forceinline__ void unload_link(V2* U, const int4* Ux, int mu, int s
     fx_store_link(U, mu, s, V, u);
   } else {
     mat<double> d;
-    load(d, tagged{const_cast<int4*>(Ux), 1.0}, mu, s, V);
+    load(d, tagged{const_cast<int4*>(Ux), 0}, mu, s, V);
     store_link(U, mu, s, V, d);
   }
 }
@@ -323,10 +323,10 @@ __device__ __forceinline__ bool fx_load_wild(mat<fx>& u, const int4* Ux, int mu,
   unsigned mag = 0;
   if (fx_is_raw(u.e[0].re.l)) {
     mat<double> d;
-    load(d, tagged{const_cast<int4*>(Ux), 1.0}, mu, s, V);
+    load(d, tagged{const_cast<int4*>(Ux), 0}, mu, s, V);
 #pragma unroll
     for (int k = 0; k < 9; ++k)
-      u.e[k] = cx<fx>{fx_of_double(fx_scaled_double(d.e[k].re, -K), mag), fx_of_double(fx_scaled_double(d.e[k].im, -K), mag)};
+      u.e[k] = cx<fx>{fx_of_double(fx_pow2(d.e[k].re, -K), mag), fx_of_double(fx_pow2(d.e[k].im, -K), mag)};
   } else {
 #pragma unroll
     for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_bits(fx_bits(u.e[k].re) >> K), fx_of_bits(fx_bits(u.e[k].im) >> K)};
@@ -347,7 +347,7 @@ static __device__ __noinline__ void sweep_part_wild(long long* q, int n, float* 
       load_link_d<L>(d, (const typename vec2_of<L>::type*)U, mu, site, V);
       unsigned mag = 0;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_double(fx_scaled_double(d.e[k].re, -2), mag), fx_of_double(fx_scaled_double(d.e[k].im, -2), mag)};
+      for (int k = 0; k < 9; ++k) u.e[k] = cx<fx>{fx_of_double(fx_pow2(d.e[k].re, -2), mag), fx_of_double(fx_pow2(d.e[k].im, -2), mag)};
       return fx_mag_ok(mag);
     } else {
       return fx_load_wild<2>(u, Ux, mu, site, V);
@@ -422,7 +422,7 @@ __device__ __forceinline__ void sweep_part(SweepPart<L, N>& sm, const Geo& g, co
       } else {
         mat<double> d;
         load_link_d<L>(d, U, mu, s, g.V);
-        store(tagged{Ux, 1.0}, mu, s, g.V, d);
+        store(tagged{Ux, 0}, mu, s, g.V, d);
       }
     } else if constexpr (PIPE) {
       P.take(u, ck);
@@ -590,7 +590,7 @@ __device__ __forceinline__ double cool_grad_site(const Geo& g, FU U, int s, doub
 template <typename L, bool FIRST>
 static __device__ __noinline__ double general_cool_grad(const Geo g, const void* U, void* Ux, int s, double* fa) {
   if constexpr (FIRST) return cool_grad_site(g, link_field<L>{(const typename vec2_of<L>::type*)U}, s, fa);
-  return cool_grad_site(g, tagged{(int4*)Ux, 1.0}, s, fa);
+  return cool_grad_site(g, tagged{(int4*)Ux, 0}, s, fa);
 }
 
 // The gradient f into [a][V] (FP64), and the rule.  FIRST: the call's first
@@ -911,10 +911,10 @@ static __device__ __noinline__ double general_cool_apply(const Geo g, int4* Ux, 
   mat<double> o, oi, u, t;
   load_herm_mat(o, tagged_herm{Om}, s, g.V);
   load_herm_mat(oi, tagged_herm{Omi}, sp, g.V);
-  load(u, tagged{Ux, 1.0}, mu, s, g.V);
+  load(u, tagged{Ux, 0}, mu, s, g.V);
   mul_herm_left(t, o, u);
   mul_herm_right(u, t, oi);
-  store(tagged{Ux, 1.0}, mu, s, g.V, u);
+  store(tagged{Ux, 0}, mu, s, g.V, u);
   return norm2(u);
 }
 // U_{x,mu} <- Omega_x U_{x,mu} Omega_{x+mu}^{-1}, all links at once (in place:

@@ -308,11 +308,12 @@ __device__ __forceinline__ fx fx_of_double(double x, unsigned& mag) { return fx_
 // Whether the largest magnitude seen is below FX_BOUND (false for NaN and Inf).
 __device__ __forceinline__ bool fx_mag_ok(unsigned mag) { return mag < 0x3FF70000u; }  // 1.4375
 
-__device__ __forceinline__ double fx_scaled_double(double x, int t) {  // x 2^t for t within 64 of zero
+// x 2^n on the integer pipe; zero below the smallest normal number.
+__device__ __forceinline__ double fx_pow2(double x, int n) {
   const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
   if (e == 0x7ff) return x;
-  if (e < 65) return 0.0;
-  return e > 1980 ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double(hi + t * (1 << 20), __double2loint(x));
+  if (e == 0 || e + n <= 0) return 0.0;
+  return e + n >= 0x7ff ? __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0) : __hiloint2double(hi + n * (1 << 20), __double2loint(x));
 }
 // A complex constant below one, times 2^t so that its larger part is in [1/2, 1):
 // a small one keeps its 53 bits (down to 2^-32; what it multiplies is then below
@@ -326,7 +327,7 @@ struct fx_cscale {
     const int e = max((__double2hiint(re) >> 20) & 0x7ff, (__double2hiint(im) >> 20) & 0x7ff);
     t = max(0, min(31, 1022 - up - e));
     imag = re == 0.0;
-    m = fx_lhs(cx<fx>{fx_of_double(fx_scaled_double(re, up + t), mag), fx_of_double(fx_scaled_double(im, up + t), mag)});
+    m = fx_lhs(cx<fx>{fx_of_double(fx_pow2(re, up + t), mag), fx_of_double(fx_pow2(im, up + t), mag)});
   }
 };
 // a <- s a
@@ -455,11 +456,13 @@ __device__ __forceinline__ int2 fx_raw_first(double x) {
 }
 __device__ __forceinline__ double fx_raw_first(int2 v) { return __hiloint2double(v.x, v.y) * 0x1p-400; }
 
-// The general path's view of such a field; its numbers are the field's times sc.
+// The general path's view of such a field; its numbers are the field's times 2^ex.
+// (As a factor in FP64 that power cost as much as a sixth of a product for every
+// matrix read or written.)
 struct tagged {
   int4* p;
-  double sc;
-  unsigned lim = 0x3FF70000u;  // words below this (high word of a double; 1.4375)
+  int ex;
+  unsigned lim = 0x3FF70000u;  // stored as words below this (high word of a double; 1.4375)
 };
 __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int site, int V) {
   const int4* p = f.p + (size_t)plane * 9 * V + site;
@@ -468,14 +471,12 @@ __device__ __forceinline__ void load(mat<double>& a, tagged f, int plane, int si
   for (int k = 0; k < 9; ++k) {
     const int4 v = p[(size_t)k * V];
     if (raw) {
-      a.e[k] = cx<double>{__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
-      if (k == 0) a.e[0].re = fx_raw_first(make_int2(v.x, v.y));
+      const double re = k == 0 ? fx_raw_first(make_int2(v.x, v.y)) : __hiloint2double(v.y, v.x), im = __hiloint2double(v.w, v.z);
+      a.e[k] = f.ex ? cx<double>{fx_pow2(re, f.ex), fx_pow2(im, f.ex)} : cx<double>{re, im};
     } else {
       const cx<fx> w = unpack(v);
-      a.e[k] = cx<double>{fx_to_double(w.re), fx_to_double(w.im)};
+      a.e[k] = cx<double>{fx_to_double(w.re, f.ex), fx_to_double(w.im, f.ex)};
     }
-    a.e[k].re *= f.sc;
-    a.e[k].im *= f.sc;
   }
 }
 // The same times a complex factor (the clover field in the force).
@@ -492,15 +493,14 @@ __device__ __forceinline__ void load(mat<double>& a, tagged_c f, int plane, int 
 // its readers the same way.
 __device__ __forceinline__ void store(tagged f, int plane, int site, int V, const mat<double>& a) {
   int4* p = f.p + (size_t)plane * 9 * V + site;
-  const double isc = 1.0 / f.sc;
   unsigned mag = 0;
 #pragma unroll
   for (int k = 0; k < 9; ++k)
-    mag = max(mag, max((unsigned)__double2hiint(a.e[k].re * isc) & 0x7fffffffu, (unsigned)__double2hiint(a.e[k].im * isc) & 0x7fffffffu));
-  const bool fits = mag < f.lim;
+    mag = max(mag, max((unsigned)__double2hiint(a.e[k].re) & 0x7fffffffu, (unsigned)__double2hiint(a.e[k].im) & 0x7fffffffu));
+  const bool fits = (int)(mag >> 20) < 0x7ff && (int)mag - f.ex * (1 << 20) < (int)f.lim;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    const double re = a.e[k].re * isc, im = a.e[k].im * isc;
+    const double re = f.ex ? fx_pow2(a.e[k].re, -f.ex) : a.e[k].re, im = f.ex ? fx_pow2(a.e[k].im, -f.ex) : a.e[k].im;
     if (fits) {
       p[(size_t)k * V] = pack(cx<fx>{fx_of_double(re, mag), fx_of_double(im, mag)});
     } else {

@@ -49,20 +49,18 @@ struct warp_ops {
   __device__ __forceinline__ wmat load(tagged f, int plane, int s, int V) const {
     const int4* p = f.p + (size_t)plane * 9 * V + s;
     const int4 v = p[(size_t)k * V];
-    cx<double> r;
     if (fx_is_raw(__int_as_float(p[0].x))) {
-      r = cx<double>{__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
+      cx<double> r = {__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
       if (k == 0) r.re = fx_raw_first(make_int2(v.x, v.y));
-    } else {
-      const cx<fx> w = unpack(v);
-      r = cx<double>{fx_to_double(w.re), fx_to_double(w.im)};
+      return wmat{cx<double>{fx_pow2(r.re, f.ex), fx_pow2(r.im, f.ex)}};
     }
-    return wmat{cx<double>{r.re * f.sc, r.im * f.sc}};
+    const cx<fx> w = unpack(v);
+    return wmat{cx<double>{fx_to_double(w.re, f.ex), fx_to_double(w.im, f.ex)}};
   }
   __device__ __forceinline__ wmat load(tagged_c f, int plane, int s, int V) const { return wmat{cmul(load(f.f, plane, s, V).v, f.sc)}; }
   // In fixed point where it fits, as store(tagged).
   __device__ __forceinline__ void store(tagged f, int plane, int s, int V, const wmat& a) const {
-    const double isc = 1.0 / f.sc, re = a.v.re * isc, im = a.v.im * isc;
+    const double re = fx_pow2(a.v.re, -f.ex), im = fx_pow2(a.v.im, -f.ex);
     unsigned mag = 0;
     const cx<fx> w = {fx_of_double(re, mag), fx_of_double(im, mag)};
     const bool fits = __all_sync(mask, mag < f.lim);

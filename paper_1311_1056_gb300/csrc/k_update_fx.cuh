@@ -32,10 +32,10 @@
 namespace clgc {
 
 // Fields of the general path.
-__device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 1.0}; }
+__device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 0}; }
 // the clover field times s
-__device__ __forceinline__ tagged_c tag_F(const int4* f, double sre, double sim) { return tagged_c{tagged{const_cast<int4*>(f), 8.0}, cx<double>{sre, sim}}; }
-__device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 2.0}; }
+__device__ __forceinline__ tagged_c tag_F(const int4* f, double sre, double sim) { return tagged_c{tagged{const_cast<int4*>(f), 3}, cx<double>{sre, sim}}; }
+__device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 1}; }
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
 // 32^4: plaquettes and clover field 2.60 -> 2.48 ms a step, observables 3.03 ->
@@ -100,7 +100,7 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
   for (int k = 0; k < 9; ++k) Pm.e[k] = cx<fx>{fx_half_diff(Pm.e[k].re, b.e[k].re), fx_half_diff(Pm.e[k].im, b.e[k].im)};
   store<fx>(Dq, p, s, g.V, Pm);
   general_path(ck.bad(), s, g.V, [&](unsigned m, int t) { warp_plaq<L>(m, g, U, tag(Pq), tag_D(Dq), p, t); },
-               [&] { general_plaq<L>(g, U, tagged{Pq, 1.0, 0u}, tag_D(Dq), vb); });
+               [&] { general_plaq<L>(g, U, tagged{Pq, 0, 0u}, tag_D(Dq), vb); });
 }
 
 // ------------------------------------------------------------ clover field
@@ -538,7 +538,7 @@ __device__ __forceinline__ double drift_fx(const Geo& g, const int4* C, int4* o,
   }
   mat<double> Xd;
   gather_f64(Xd, g, s, x, MU, C, cexp);
-  if (write) store(tagged{o, ldexp(1.0, cexp + 2), 0u}, MU, s, g.V, Xd);  // doubles: words are the traceless quarter
+  if (write) store(tagged{o, cexp + 2, 0u}, MU, s, g.V, Xd);  // doubles: words are the traceless quarter
   return general_k2(Xd);
 }
 
@@ -589,7 +589,7 @@ __device__ __forceinline__ void update_fx(const Geo& g, const typename vec2_of<L
                                           int MU) {
   const double eps = a.adaptive ? a.sd->eps_n : a.eps;
   const double sqrt_eps = a.adaptive ? a.sd->sqrt_eps_n : a.sqrt_eps;
-  const tagged Xt = {const_cast<int4*>(X), ldexp(1.0, a.cexp + 2)};
+  const tagged Xt = {const_cast<int4*>(X), a.cexp + 2};
   // The noise first, one pair at a time into shared memory (a thread's own
   // words): its code once instead of four times, which the warps fetched (a
   // sixth of their time; update 0.145 -> 0.136 ms at 16^4, 1.80 -> 1.76 at 32^4).

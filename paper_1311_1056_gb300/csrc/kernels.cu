@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_cool_load(Geo g, const typename 
   } else {
     mat<double> d;
     load_link_d<L>(d, U, mu, s, g.V);
-    store(tagged{Ux, 1.0}, mu, s, g.V, d);
+    store(tagged{Ux, 0}, mu, s, g.V, d);
   }
 }
 
@@ -353,14 +353,14 @@ __device__ __forceinline__ bool obs_trace(long long& re, long long& im, const in
   }
   return ok;
 }
-static __device__ __noinline__ void general_obs_trace(const int4* f, int p, int s, int V, double sc, double* out) {
+static __device__ __noinline__ void general_obs_trace(const int4* f, int p, int s, int V, int ex, double* out) {
   mat<double> m;
-  load(m, tagged{const_cast<int4*>(f), sc}, p, s, V);
+  load(m, tagged{const_cast<int4*>(f), ex}, p, s, V);
   const cx<double> t = trace(m);
   out[0] = t.re;
   out[1] = t.im;
 }
-static __device__ __noinline__ void general_obs_trace(const float2* f, int p, int s, int V, double, double* out) {
+static __device__ __noinline__ void general_obs_trace(const float2* f, int p, int s, int V, int, double* out) {
   mat<float> m;
   load(m, f, p, s, V);
   const cx<float> t = trace(m);
@@ -370,8 +370,8 @@ static __device__ __noinline__ void general_obs_trace(const float2* f, int p, in
 // Tr F_p F_{5-p} in FP64.
 static __device__ __noinline__ void general_obs_ff(const int4* F, int p, int s, int V, double* out) {
   mat<double> F1, F2;
-  load(F1, tagged{const_cast<int4*>(F), 1.0}, p, s, V);
-  load(F2, tagged{const_cast<int4*>(F), 1.0}, 5 - p, s, V);
+  load(F1, tagged{const_cast<int4*>(F), 0}, p, s, V);
+  load(F2, tagged{const_cast<int4*>(F), 0}, 5 - p, s, V);
   const cx<double> t = trace_mul(F1, F2);
   out[0] = t.re;
   out[1] = t.im;
@@ -430,10 +430,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
         di += d;
       } else {
         double t[2];
-        general_obs_trace(Pq, p, s, g.V, 1.0, t);
+        general_obs_trace(Pq, p, s, g.V, 0, t);
         wp[0] += t[0];
         wp[1] += t[1];
-        general_obs_trace(Dq, p, s, g.V, 2.0, t);
+        general_obs_trace(Dq, p, s, g.V, 1, t);
         wp[2] += t[0];
         wp[3] += t[1];
       }
