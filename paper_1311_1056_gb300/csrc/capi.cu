@@ -133,17 +133,17 @@ int clover_kernels(const cl_lattice* l) { return l->prec != 1 ? 2 : 1; }
 cudaError_t do_force(cl_lattice* l, bool th, double sre, double sim, int ce) {
   cudaError_t e = cudaSuccess;
   if (needs_inverse_pass(l))
-    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); });
+    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->sd, l->st); });
   if (e == cudaSuccess)
-    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); });
+    e = timed(l, CL_PHASE_CLOVER, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->sd, l->st); });
   if (e == cudaSuccess && th)
     e = timed(l, CL_PHASE_CLOVER, [&] {
-      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, sre, sim, l->st);
+      return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, sre, sim, l->sd, l->st);
     }, clover_kernels(l));
   if (e == cudaSuccess)
     e = timed(l, CL_PHASE_FORCE, [&] {
       return launch_plaq_force(l->prec, th, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->F, l->Gq, l->C, l->p.beta,
-                               sre, sim, ce, l->st);
+                               sre, sim, ce, l->sd, l->st);
     }, (th && l->prec != 1) ? 3 : 1);  // FP64 and DF64 split the theta force in three kernels
   return e;
 }
@@ -237,12 +237,12 @@ cl_status do_cool(cl_lattice* l, const cl_cool_params* cp) {
 
 cl_status do_obs(cl_lattice* l, ObsOut* dst, double* q_site) {
   if (needs_inverse_pass(l))
-    CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->st); }));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->st); }));
+    CK(timed(l, CL_PHASE_OBS, [&] { return launch_link_inverse(l->prec, l->g, l->U, l->Un, l->Ui, l->sd, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] { return launch_plaq(l->prec, l->g, l->U, l->Un, l->Ui, l->Pq, l->Dq, l->sd, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
-    return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, 1.0, 0.0, l->st);
+    return launch_clover_rot(l->prec, l->g, l->U, l->Un, l->Ui, l->Dq, l->C, l->F, 1.0, 0.0, l->sd, l->st);
   }, clover_kernels(l)));
-  CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->Un, l->Pq, l->Dq, l->F, l->partials, q_site, l->st); }));
+  CK(timed(l, CL_PHASE_OBS, [&] { return launch_obs(l->prec, l->g, l->U, l->Un, l->Pq, l->Dq, l->F, l->partials, q_site, l->sd, l->st); }));
   CK(timed(l, CL_PHASE_OBS, [&] {
     return launch_obs_final(l->g, l->partials, l->p.beta, l->p.theta_re, l->p.theta_im, dst, l->st);
   }));
@@ -288,7 +288,7 @@ cudaError_t init_state(cl_lattice* l) {
   const cl_params* params = &l->p;
   l->step = 0;
   cudaError_t e = cudaMemsetAsync(l->cs, 0, sizeof(CoolState), l->st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(l->sd, 0, sizeof(StepDev), l->st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(l->sd, 0, STEP_DEV_BYTES, l->st);
   if (e == cudaSuccess)
     e = params->start == CL_START_HOT ? launch_hot(l->prec, l->g, l->U, params->seed, l->st)
                                       : launch_cold(l->prec, l->g, l->U, l->st);
@@ -353,7 +353,7 @@ cl_status cl_init_lattice(const cl_params* params, void* cuda_stream, cl_lattice
   alloc((void**)&l->partials, sizeof(double) * NQ_OBS * (size_t)reduce_blocks(l->g.V));
   alloc((void**)&l->cs, sizeof(CoolState));
   alloc((void**)&l->obs, sizeof(ObsOut));
-  alloc((void**)&l->sd, sizeof(StepDev));
+  alloc((void**)&l->sd, STEP_DEV_BYTES);
   if (s != CL_OK) {
     cl_free(l);
     return s;

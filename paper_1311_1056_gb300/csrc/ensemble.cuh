@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_ens_inverse(const ChainDesc*
   typedef typename vec2_of<T>::type V2;
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  fx_links_body<T>(geo_of(c), (const V2*)c.U, (int4*)c.Un, (int4*)c.Ui, it.vb);
+  fx_links_body<T>(geo_of(c), (const V2*)c.U, (int4*)c.Un, (int4*)c.Ui, field_top(c.sd), it.vb);
 }
 
 template <typename T>
@@ -45,7 +45,8 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_plaq(const
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
-    fx_plaq_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, sm, it.vb);
+    fx_plaq_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (int4*)c.Pq, (int4*)c.Dq, field_top(c.sd),
+                    sm, it.vb);
   else
     k_plaq_body<T>(geo_of(c), (const V2*)c.U, (V2*)c.Pq, (V2*)c.Dq, it.vb);
 }
@@ -57,7 +58,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover_hal
   __shared__ int4 sm[FX_PIPE];
   const WorkItem it = w[blockIdx.x];
   const ChainDesc& c = cd[it.chain];
-  fx_clover_half_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C, sm, it.vb);
+  fx_clover_half_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (int4*)c.C, field_top(c.sd), sm, it.vb);
 }
 template <typename T>
 __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_force_t(const ChainDesc* __restrict__ cd,
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, ENS_MIN_BLOCKS(T)) k_ens_clover(con
   const ChainDesc& c = cd[it.chain];
   if constexpr (is_fx<T>())
     fx_clover_body<T>(geo_of(c), (const V2*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq,
-                      (const int4*)c.C, (int4*)c.F, sm, it.vb);
+                      (const int4*)c.C, (int4*)c.F, field_top(c.sd), sm, it.vb);
   else
     k_clover_rot_body<T>(geo_of(c), (const V2*)c.U, (const V2*)c.Dq, (V2*)c.F, c.sre, c.sim, it.vb);
 }
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_a(const ChainDesc* _
   const ChainDesc& c = cd[it.chain];
   extern __shared__ int4 sm_park[];
   fx_force_a_body(geo_of(c), (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Dq, (const int4*)c.F, (int4*)c.Gq,
-                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), c.sre, c.sim, sm_park, it.vb);
+                  (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), c.sre, c.sim, field_top(c.sd), sm_park, it.vb);
 }
 
 template <typename T>
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(ENS_BLOCK, 2) k_ens_force_b(const ChainDesc* _
   __shared__ int4 sm[FX_PIPE];
   fx_force_b_body<T>(geo_of(c), (const typename vec2_of<T>::type*)c.U, (const int4*)c.Un, (const int4*)c.Ui, (const int4*)c.Pq,
                   (const int4*)c.Dq, (const int4*)c.F, (const int4*)c.Gq, (int4*)c.C, ldexp(c.beta / 6.0, -c.cexp), c.sre,
-                  c.sim, sm, it.vb);
+                  c.sim, field_top(c.sd), sm, it.vb);
 }
 
 template <typename T>

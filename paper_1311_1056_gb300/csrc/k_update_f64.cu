@@ -37,29 +37,30 @@ cudaError_t prepare_step_kernels(int prec) {
   return e == cudaSuccess ? prepare_ens_step<double>() : e;
 }
 
-cudaError_t launch_link_inverse(int prec, const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st) {
+cudaError_t launch_link_inverse(int prec, const GeoH& h, const void* U, void* Ux, void* Ui, StepDev* sd, cudaStream_t st) {
   if (prec == 1) return cudaSuccess;
-  return prec == 0 ? StepFx<double>::links(h, U, Ux, Ui, st) : StepFx<df64>::links(h, U, Ux, Ui, st);
+  return prec == 0 ? StepFx<double>::links(h, U, Ux, Ui, sd, st) : StepFx<df64>::links(h, U, Ux, Ui, sd, st);
 }
 cudaError_t launch_plaq(int prec, const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
-                        cudaStream_t st) {
+                        StepDev* sd, cudaStream_t st) {
   if (prec == 1) return launch_plaq_f32(h, U, Pq, Dq, st);
-  return prec == 0 ? StepFx<double>::plaq(h, U, Ux, Ui, Pq, Dq, st) : StepFx<df64>::plaq(h, U, Ux, Ui, Pq, Dq, st);
+  return prec == 0 ? StepFx<double>::plaq(h, U, Ux, Ui, Pq, Dq, sd, st) : StepFx<df64>::plaq(h, U, Ux, Ui, Pq, Dq, sd, st);
 }
 cudaError_t launch_clover_rot(int prec, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                              void* E, void* F, double sre, double sim, cudaStream_t st) {
+                              void* E, void* F, double sre, double sim, StepDev* sd, cudaStream_t st) {
   if (prec == 1) return launch_clover_rot_f32(h, U, Dq, F, sre, sim, st);
-  return prec == 0 ? StepFx<double>::clover(h, U, Ux, Ui, Dq, E, F, st) : StepFx<df64>::clover(h, U, Ux, Ui, Dq, E, F, st);
+  return prec == 0 ? StepFx<double>::clover(h, U, Ux, Ui, Dq, E, F, sd, st)
+                   : StepFx<df64>::clover(h, U, Ux, Ui, Dq, E, F, sd, st);
 }
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
-                              double beta, double sre, double sim, int cexp, cudaStream_t st) {
+                              double beta, double sre, double sim, int cexp, StepDev* sd, cudaStream_t st) {
   if (prec == 1) return launch_plaq_force_f32(theta, h, U, Pq, Dq, F, C, beta, st);
   const double b6 = ldexp(beta / 6.0, -cexp);
   sre = ldexp(sre, -cexp);
   sim = ldexp(sim, -cexp);
-  return prec == 0 ? StepFx<double>::force(theta, h, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, st)
-                   : StepFx<df64>::force(theta, h, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, st);
+  return prec == 0 ? StepFx<double>::force(theta, h, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, sd, st)
+                   : StepFx<df64>::force(theta, h, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, sd, st);
 }
 cudaError_t launch_update_gather(int prec, int mode, const GeoH& h, const void* U, const void* C,
                                  void* out, double eps, double k_ref, uint64_t seed, StepDev* sd,

@@ -5,7 +5,8 @@
 // Fields between the kernels (int4 words, SoA as the links): Ux, the links in
 // fixed point, in the buffer that the update writes at the step's end; Ui
 // their inverses; P, D, F, C.  F is an eighth of the clover field, negated for
-// planes 1 and 4 (the sign of the pair 02|13); its factor -i theta kappa (s below)
+// planes 1 and 4 (the sign of the pair 02|13), times 2^k that keeps the lattice's
+// largest D / 2 just below the bound (fx_field_shift); its factor -i theta kappa (s below)
 // comes in where the force is formed, times 2^-e, the factor that keeps the
 // contributions C within bounds (drift_exponent, launch.h).
 //
@@ -33,8 +34,10 @@ namespace clgc {
 
 // Fields of the general path.
 __device__ __forceinline__ tagged tag(const int4* f) { return tagged{const_cast<int4*>(f), 0}; }
-// the clover field times s
-__device__ __forceinline__ tagged_c tag_F(const int4* f, double sre, double sim) { return tagged_c{tagged{const_cast<int4*>(f), 3}, cx<double>{sre, sim}}; }
+// the clover field (kept times 2^k / 8) times s
+__device__ __forceinline__ tagged_c tag_F(const int4* f, int k, double sre, double sim) {
+  return tagged_c{tagged{const_cast<int4*>(f), 3 - k}, cx<double>{sre, sim}};
+}
 __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cast<int4*>(f), 1}; }
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
@@ -46,7 +49,8 @@ const int FX_PIPE = fx_pipe<2>::WORDS, FX_PARK_BYTES = (FX_PIPE + fx_park::WORDS
 // ------------------------------------------------------ links and inverses
 template <typename L>
 __device__ __forceinline__ void fx_links_body(Geo g, const typename vec2_of<L>::type* __restrict__ U,
-                                              int4* __restrict__ Ux, int4* __restrict__ Ui, int vb) {
+                                              int4* __restrict__ Ux, int4* __restrict__ Ui, unsigned* top, int vb) {
+  if (vb == 0 && threadIdx.x == 0) *top = 0u;  // for the plaquette pass
   const int mu = vb % 4;
   const int s = (vb / 4) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -74,7 +78,8 @@ static __device__ __noinline__ void general_plaq(Geo g, const typename vec2_of<L
 }
 template <typename L>
 __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
-                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq, int4* sm, int vb) {
+                                             const int4* __restrict__ Ui, int4* Pq, int4* Dq, unsigned* top, int4* sm,
+                                             int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -99,6 +104,17 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
 #pragma unroll
   for (int k = 0; k < 9; ++k) Pm.e[k] = cx<fx>{fx_half_diff(Pm.e[k].re, b.e[k].re), fx_half_diff(Pm.e[k].im, b.e[k].im)};
   store<fx>(Dq, p, s, g.V, Pm);
+  {
+    int hi = ck.bad() ? 1 << 30 : 0, lo = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      hi = max(hi, max(Pm.e[k].re.h, Pm.e[k].im.h));
+      lo = min(lo, min(Pm.e[k].re.h, Pm.e[k].im.h));
+    }
+    const int n = g.V - (s - (int)(threadIdx.x & 31));  // the warp's sites
+    const unsigned m = __reduce_max_sync(n >= 32 ? 0xffffffffu : (1u << n) - 1u, (unsigned)max(hi, -lo));
+    if ((threadIdx.x & 31) == 0 && m > *(volatile unsigned*)top) atomicMax(top, m);
+  }
   general_path(ck.bad(), s, g.V, [&](unsigned m, int t) { warp_plaq<L>(m, g, U, tag(Pq), tag_D(Dq), p, t); },
                [&] { general_plaq<L>(g, U, tagged{Pq, 0, 0u}, tag_D(Dq), vb); });
 }
@@ -114,7 +130,7 @@ static __device__ __noinline__ void general_clover(Geo g, const typename vec2_of
 // six (32^4: plaquettes and clover field 3.00 -> 2.60 ms a step, observables
 // 3.43 -> 3.04 ms; the second pass is partly bound by its 0.9 GB of E).
 __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
-                                                    const int4* __restrict__ Dq, int4* E, int4* sm, int vb) {
+                                                    const int4* __restrict__ Dq, int4* E, const unsigned* top, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -126,13 +142,16 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
   fx_pipe<2> P(sm);
   P.ask(Ui, mu, xmm, g.V);
   P.ask(Dq, p, xmm, g.V);
+  const int shift = fx_field_shift(top);
   P.take(w, ck);
   P.ask(Ux, mu, xmm, g.V);
   P.take(d, ck);
   P.ask(Dq, p, s, g.V);
+  if (shift) fx_shift_up(d, shift);
   fx_mul_left<FX_WIDE, 1>(w, d, ck);
   P.take(d, ck);
   P.take(acc, ck);
+  if (shift) fx_shift_up(acc, shift);
   fx_mul_acc<FX_WIDE, +1, 1>(acc, w, d, ck);
   if (ck.bad()) acc.e[0].re.l = fx_raw_mark();  // its readers start over from D
   store<fx>(E, p, s, g.V, acc);
@@ -141,7 +160,7 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
 template <typename L>
 __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                const int4* __restrict__ Ui, const int4* __restrict__ Dq,
-                                               const int4* __restrict__ E, int4* F, int4* sm, int vb) {
+                                               const int4* __restrict__ E, int4* F, const unsigned* top, int4* sm, int vb) {
   const int p = vb % 6, nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -167,9 +186,9 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
     for (int k = 0; k < 9; ++k) acc.e[k] = cx<fx>{-acc.e[k].re, -acc.e[k].im};
   }
   store<fx>(F, p, s, g.V, acc);
-  general_path(ck.bad(), s, g.V,
-               [&](unsigned m, int t) { warp_clover<L>(m, g, U, tag_D(Dq), tag(F), neg ? -0.125 : 0.125, p, t); },
-               [&] { general_clover<L>(g, U, tag_D(Dq), tag(F), neg ? -0.125 : 0.125, vb); });
+  const auto scale = [&] { return ldexp(neg ? -0.125 : 0.125, fx_field_shift(top)); };
+  general_path(ck.bad(), s, g.V, [&](unsigned m, int t) { warp_clover<L>(m, g, U, tag_D(Dq), tag(F), scale(), p, t); },
+               [&] { general_clover<L>(g, U, tag_D(Dq), tag(F), scale(), vb); });
 }
 
 // ------------------------------------------------------- plaquette drift
@@ -253,7 +272,7 @@ __device__ __forceinline__ void fx_force_t_body(Geo g, const int4* __restrict__ 
 // 1/32; it multiplies D (and P), so the fields' errors are scaled down with it.
 __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
                                                 const int4* __restrict__ Dq, const int4* __restrict__ F, int4* Gq,
-                                                int4* C, double b6, double sre, double sim, int4* sm, int vb) {
+                                                int4* C, double b6, double sre, double sim, const unsigned* top, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), pc = 5 - p;
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -281,7 +300,7 @@ __device__ __forceinline__ void fx_force_a_body(Geo g, const int4* __restrict__ 
   P.take(A, ck);
   P.ask(F, pc, s, g.V);
   fx_scaled<FX_WIDE>(M, A, fx_of_double(-2.0 * b6, mag), ck);
-  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 4, mag), ck);  // 8 s D = 16 s (D / 2)
+  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 4 - fx_field_shift(top), mag), ck);  // 8 s D = 16 s (D / 2)
   P.take(B, ck);
   P.ask(Ux, mu, s, g.V);
   fx_commutator_acc<FX_WIDE>(M, A, B, ck);
@@ -313,13 +332,14 @@ template <typename L>
 __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                 const int4* __restrict__ Ui, const int4* Pq, const int4* Dq,
                                                 const int4* F, const int4* Gq, int4* C, double b6, double sre, double sim,
-                                                int4* sm, int vb) {
+                                                const unsigned* top, int4* sm, int vb) {
   const int p = vb % 6, mu = plane_mu(p), nu = plane_nu(p);
   const int s = (vb / 6) * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   fx_chk ck;
   unsigned mag = 0;
   const fx pb = fx_of_double(2.0 * b6, mag);
+  const int shift = fx_field_shift(top);
   mat<fx> A, B, M;
   // corner c3: A = G3r = T; slot 3 partial = [s D, G3r] + (beta/6) D
   fx_pipe<2> P(sm);
@@ -328,7 +348,7 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   P.take(B, ck);
   P.ask(Pq, p, s, g.V);
   fx_scaled<FX_WIDE>(M, B, pb, ck);
-  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 4, mag), ck);  // 8 s D
+  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 4 - shift, mag), ck);  // 8 s D
   P.take(A, ck);
   P.ask(Dq, p, s, g.V);
   fx_commutator_acc<FX_WIDE>(M, B, A, ck);
@@ -349,9 +369,9 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   // K = 32 s (P^{-1} G^ / 4 + G^ / 4 P), s taken with P^{-1} and P
   P.take(B, ck);
   P.ask(Dq, p, s, g.V);
-  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 5, mag), ck);
+  fx_cscaled<FX_WIDE>(A, fx_cscale(sre, sim, 5 - shift, mag), ck);
   fx_mul_left<FX_WIDE>(A, M, ck);
-  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 5, mag), ck);
+  fx_cscaled<FX_WIDE>(B, fx_cscale(sre, sim, 5 - shift, mag), ck);
   fx_mul_acc<FX_MID, +1>(A, M, B, ck);
   // slot 0: partial + K; slot 1: (beta/6) D - K
   P.take(M, ck);
@@ -384,8 +404,8 @@ __device__ __forceinline__ void fx_force_b_body(Geo g, const typename vec2_of<L>
   store<fx>(C, 4 * p + 2, s, g.V, A);
   // anything out of range: the whole plaquette again (its slots are its own)
   general_path(ck.bad() || !fx_mag_ok(mag), s, g.V,
-               [&](unsigned m, int t) { warp_force<L>(m, g, U, tag(Pq), tag_D(Dq), tag_F(F, sre, sim), tag(C), b6, p, t); },
-               [&] { general_force<L>(g, U, tag(Pq), tag_D(Dq), tag_F(F, sre, sim), tag(C), b6, vb); });
+               [&](unsigned m, int t) { warp_force<L>(m, g, U, tag(Pq), tag_D(Dq), tag_F(F, shift, sre, sim), tag(C), b6, p, t); },
+               [&] { general_force<L>(g, U, tag(Pq), tag_D(Dq), tag_F(F, shift, sre, sim), tag(C), b6, vb); });
 }
 
 // --------------------------------------------------------------- gather

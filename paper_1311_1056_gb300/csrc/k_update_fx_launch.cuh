@@ -14,12 +14,13 @@ namespace clgc {
 template <typename L>
 struct StepFx {
   static cudaError_t prepare();  // once per device: shared memory of the theta force
-  static cudaError_t links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st);
-  static cudaError_t plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq, cudaStream_t st);
+  static cudaError_t links(const GeoH& h, const void* U, void* Ux, void* Ui, StepDev* sd, cudaStream_t st);
+  static cudaError_t plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq, StepDev* sd,
+                          cudaStream_t st);
   static cudaError_t clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq, void* E,
-                            void* F, cudaStream_t st);
+                            void* F, StepDev* sd, cudaStream_t st);
   static cudaError_t force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
-                           double sre, double sim, cudaStream_t st);
+                           double sre, double sim, StepDev* sd, cudaStream_t st);
   static cudaError_t update(int mode, const GeoH& h, const void* U, const void* C, void* out, double eps, double k_ref,
                             uint64_t seed, StepDev* sd, int cexp, cudaStream_t st);
 };
@@ -38,26 +39,27 @@ inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 
 // clover field 11.95 (now 2.48).
 const int FX_BLOCKS_SM = 3, FX_BLOCKS_FORCE = 2;
 template <typename L>
-__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui) {
-  fx_links_body<L>(g, U, Ux, Ui, blockIdx.x);
+__global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui,
+                                                             unsigned* top) {
+  fx_links_body<L>(g, U, Ux, Ui, top, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_plaq(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
-                                                            const int4* __restrict__ Ui, int4* Pq, int4* Dq) {
+                                                            const int4* __restrict__ Ui, int4* Pq, int4* Dq, unsigned* top) {
   __shared__ int4 sm[FX_PIPE];
-  fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, sm, blockIdx.x);
+  fx_plaq_body<L>(g, U, Ux, Ui, Pq, Dq, top, sm, blockIdx.x);
 }
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover_half(Geo g, const int4* __restrict__ Ux, const int4* __restrict__ Ui,
-                                                         const int4* __restrict__ Dq, int4* E) {
+                                                         const int4* __restrict__ Dq, int4* E, const unsigned* top) {
   __shared__ int4 sm[FX_PIPE];
-  fx_clover_half_body(g, Ux, Ui, Dq, E, sm, blockIdx.x);
+  fx_clover_half_body(g, Ux, Ui, Dq, E, top, sm, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_SM) k_fx_clover(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                     const int4* __restrict__ Ui, const int4* __restrict__ Dq,
-                                                    const int4* __restrict__ E, int4* F) {
+                                                    const int4* __restrict__ E, int4* F, const unsigned* top) {
   __shared__ int4 sm[FX_PIPE];
-  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, sm, blockIdx.x);
+  fx_clover_body<L>(g, U, Ux, Ui, Dq, E, F, top, sm, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_wilson(Geo g, const typename vec2_of<L>::type* U,
@@ -76,17 +78,17 @@ __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_a(Geo g,
                                                                const int4* __restrict__ Ui,
                                                                const int4* __restrict__ Dq,
                                                                const int4* __restrict__ F, int4* Gq, int4* C,
-                                                               double b6, double sre, double sim) {
+                                                               double b6, double sre, double sim, const unsigned* top) {
   extern __shared__ int4 sm_park[];
-  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, sre, sim, sm_park, blockIdx.x);
+  fx_force_a_body(g, Ux, Ui, Dq, F, Gq, C, b6, sre, sim, top, sm_park, blockIdx.x);
 }
 template <typename L>
 __global__ void __launch_bounds__(FX_BLOCK, FX_BLOCKS_FORCE) k_fx_force_b(Geo g, const typename vec2_of<L>::type* U, const int4* __restrict__ Ux,
                                                                const int4* __restrict__ Ui, const int4* Pq,
                                                                const int4* Dq, const int4* F, const int4* Gq, int4* C,
-                                                               double b6, double sre, double sim) {
+                                                               double b6, double sre, double sim, const unsigned* top) {
   __shared__ int4 sm[FX_PIPE];
-  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, sm, blockIdx.x);
+  fx_force_b_body<L>(g, U, Ux, Ui, Pq, Dq, F, Gq, C, b6, sre, sim, top, sm, blockIdx.x);
 }
 template <typename L, int MODE>
 __global__ void __maxnreg__(UPDATE_MAXNREG) k_fx_update(Geo g, const typename vec2_of<L>::type* __restrict__ U,
@@ -103,36 +105,36 @@ cudaError_t StepFx<L>::prepare() {
 }
 
 template <typename L>
-cudaError_t StepFx<L>::links(const GeoH& h, const void* U, void* Ux, void* Ui, cudaStream_t st) {
+cudaError_t StepFx<L>::links(const GeoH& h, const void* U, void* Ux, void* Ui, StepDev* sd, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
-  k_fx_links<L><<<grid(g.V, 4, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (int4*)Ux, (int4*)Ui);
+  k_fx_links<L><<<grid(g.V, 4, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (int4*)Ux, (int4*)Ui, field_top(sd));
   return cudaGetLastError();
 }
 
 template <typename L>
 cudaError_t StepFx<L>::plaq(const GeoH& h, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
-                            cudaStream_t st) {
+                            StepDev* sd, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
-  k_fx_plaq<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (int4*)Pq, (int4*)Dq);
+  k_fx_plaq<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (int4*)Pq, (int4*)Dq, field_top(sd));
   return cudaGetLastError();
 }
 
 template <typename L>
 cudaError_t StepFx<L>::clover(const GeoH& h, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                                  void* E, void* F, cudaStream_t st) {
+                                  void* E, void* F, StepDev* sd, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_CLOVER), FX_BLOCK);
-  k_fx_clover_half<<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)E);
-  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E, (int4*)F);
+  k_fx_clover_half<<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (int4*)E, field_top(sd));
+  k_fx_clover<L><<<grid(g.V, 6, bs), bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)E, (int4*)F, field_top(sd));
   return cudaGetLastError();
 }
 
 template <typename L>
 cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const void* Ux, const void* Ui,
                                   const void* Pq, const void* Dq, const void* F, void* Gq, void* C, double b6,
-                                  double sre, double sim, cudaStream_t st) {
+                                  double sre, double sim, StepDev* sd, cudaStream_t st) {
   Geo g = make_geo(h.L, h.V);
   const int bs = std::min(block_of(h, TUNE_FORCE), FX_BLOCK);
   const dim3 gr = grid(g.V, 6, bs);
@@ -142,9 +144,9 @@ cudaError_t StepFx<L>::force(bool theta, const GeoH& h, const void* U, const voi
   }
   k_fx_force_t<<<gr, bs, 0, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)F, (int4*)C);
   k_fx_force_a<<<gr, bs, FX_PARK_BYTES, st>>>(g, (const int4*)Ux, (const int4*)Ui, (const int4*)Dq, (const int4*)F, (int4*)Gq,
-                                  (int4*)C, b6, sre, sim);
+                                  (int4*)C, b6, sre, sim, field_top(sd));
   k_fx_force_b<L><<<gr, bs, 0, st>>>(g, (const typename vec2_of<L>::type*)U, (const int4*)Ux, (const int4*)Ui, (const int4*)Pq, (const int4*)Dq,
-                                  (const int4*)F, (const int4*)Gq, (int4*)C, b6, sre, sim);
+                                  (const int4*)F, (const int4*)Gq, (int4*)C, b6, sre, sim, field_top(sd));
   return cudaGetLastError();
 }
 

@@ -368,10 +368,10 @@ static __device__ __noinline__ void general_obs_trace(const float2* f, int p, in
   out[1] = (double)t.im;
 }
 // Tr F_p F_{5-p} in FP64.
-static __device__ __noinline__ void general_obs_ff(const int4* F, int p, int s, int V, double* out) {
+static __device__ __noinline__ void general_obs_ff(const int4* F, int p, int s, int V, int ex, double* out) {
   mat<double> F1, F2;
-  load(F1, tagged{const_cast<int4*>(F), 0}, p, s, V);
-  load(F2, tagged{const_cast<int4*>(F), 0}, 5 - p, s, V);
+  load(F1, tagged{const_cast<int4*>(F), ex}, p, s, V);
+  load(F2, tagged{const_cast<int4*>(F), ex}, 5 - p, s, V);
   const cx<double> t = trace_mul(F1, F2);
   out[0] = t.re;
   out[1] = t.im;
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
                                                     const typename obs_word<T>::type* __restrict__ Pq,
                                                     const typename obs_word<T>::type* __restrict__ Dq,
                                                     const typename obs_word<T>::type* __restrict__ F,
-                                                    double* partials, double* q_site) {
+                                                    double* partials, double* q_site, const unsigned* top) {
   constexpr bool FX = is_fx<T>();
   double v[NQ_OBS];
 #pragma unroll
@@ -448,6 +448,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
     if constexpr (FX) {
       fx_acc re = fx_zero(), im = fx_zero();
       fx_chk ck;
+      const int shift = fx_field_shift(top);
       float nf = 0.0f;  // sum of |F|^2, twice a bound of the traces' sum
 #pragma unroll 1
       for (int p = 0; p < 3; ++p) {  // the planes 1 and 4 are both stored negated
@@ -465,12 +466,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_obs(Geo g, const typename vec2_
           }
       }
       if (!ck.bad() && nf < 15.0f * 0x1p60f) {
-        q.re = fx_bits_to_double(fx_sum<true>(re) - (1 << 29));
-        q.im = fx_bits_to_double(fx_sum<true>(im) - (1 << 29));
+        q.re = fx_bits_to_double(fx_sum<true>(re) - (1 << 29), -2 * shift);
+        q.im = fx_bits_to_double(fx_sum<true>(im) - (1 << 29), -2 * shift);
       } else {
         for (int p = 0; p < 3; ++p) {
           double t[2];
-          general_obs_ff(F, p, s, g.V, t);
+          general_obs_ff(F, p, s, g.V, -shift, t);
           q.re += p == 1 ? -t[0] : t[0];
           q.im += p == 1 ? -t[1] : t[1];
         }
@@ -845,13 +846,13 @@ int ens_cool_blocks(int prec, int fam, int V) {
 }
 
 cudaError_t launch_obs(int prec, const GeoH& h, const void* U, const void* Ux, const void* Pq, const void* Dq,
-                       const void* F, double* partials, double* q_site, cudaStream_t st) {
+                       const void* F, double* partials, double* q_site, StepDev* sd, cudaStream_t st) {
   Geo g = to_geo(h);
   return by_prec(prec, [&](auto t) {
     using T = decltype(t);
     typedef typename obs_word<T>::type W;
     k_obs<T><<<reduce_blocks(g.V), RED_THREADS, 0, st>>>(g, (const typename vec2_of<T>::type*)U, (const int4*)Ux,
-                                                        (const W*)Pq, (const W*)Dq, (const W*)F, partials, q_site);
+                                                        (const W*)Pq, (const W*)Dq, (const W*)F, partials, q_site, field_top(sd));
   });
 }
 

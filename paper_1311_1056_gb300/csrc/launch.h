@@ -32,6 +32,12 @@ struct StepDev {
   unsigned long long kmax2_bits; // running max of |K|^2 (non-negative doubles order as integers)
 };
 
+// Behind it in the same allocation: the largest entry of the plaquette pass's D / 2
+// (the high limb's magnitude), from which the FP64 and DF64 forms take the power of
+// two that their clover field is kept at.
+__host__ __device__ inline unsigned* field_top(StepDev* sd) { return reinterpret_cast<unsigned*>(sd + 1); }
+const size_t STEP_DEV_BYTES = sizeof(StepDev) + sizeof(unsigned);
+
 // Packed results of the cooling rule, resident on the device.
 struct CoolState {
   double alpha_ad;       // alpha / D of the sweep about to run
@@ -120,24 +126,25 @@ int drift_exponent(double beta, double sre, double sim);
 cudaError_t prepare_step_kernels(int prec);  // before a device's first step of that form
 // The CL step (k_update.cuh): link inverses Ui; plaquettes P and D = P - P^{-1}
 // (six planes); the clover field F^ = scale * F_{mu nu}(x) built from the D's (fixed
-// point: F_{mu nu} / 8 whatever the scale, which the force then applies);
+// point: F_{mu nu} / 8 times the power of two of field_top, whatever the scale, which
+// the force then applies);
 // the per-plaquette drift contributions C (24 planes: 4 links x 6 planes);
 // then per link the gather of its six contributions followed by the update
 // (mode 0) or by storing the drift matrix X_S (mode 1).
 cudaError_t launch_noise_sample(int prec, int site0, int n, uint64_t seed, uint32_t step, int mu, double* out,
                                 cudaStream_t st);
-cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ux, void* Ui, cudaStream_t st);
+cudaError_t launch_link_inverse(int prec, const GeoH& g, const void* U, void* Ux, void* Ui, StepDev* sd, cudaStream_t st);
 cudaError_t launch_plaq(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, void* Pq, void* Dq,
-                        cudaStream_t st);
+                        StepDev* sd, cudaStream_t st);
 cudaError_t launch_clover_rot(int prec, const GeoH& g, const void* U, const void* Ux, const void* Ui, const void* Dq,
-                              void* E, void* F, double scale_re, double scale_im, cudaStream_t st);
+                              void* E, void* F, double scale_re, double scale_im, StepDev* sd, cudaStream_t st);
 // The clover field of the fixed-point forms goes through E, six planes of
 // scratch (the first of C).  Their theta force runs three kernels, parking the
 // transported dual fields and partial sums of them in planes of C (Gq points at
 // some of these).
 cudaError_t launch_plaq_force(int prec, bool theta, const GeoH& g, const void* U, const void* Ux, const void* Ui,
                               const void* Pq, const void* Dq, const void* F, void* Gq, void* C,
-                              double beta, double scale_re, double scale_im, int cexp, cudaStream_t st);
+                              double beta, double scale_re, double scale_im, int cexp, StepDev* sd, cudaStream_t st);
 // mode 0: update from the gathered drift, step size eps; 1: write the drift X_S
 // to out; 2: write X_S to out, max |K| and from it the device step size, eps
 // min(1, k_ref / K_max); 3: update reading X_S from C (a mode-2 output), device
@@ -177,7 +184,7 @@ cudaError_t launch_cool_load(int prec, const GeoH& g, const void* U, void* Ux, c
 // the clover field F (FP32 storage: of scale one), then the final fixed-order
 // reduction into *out.
 cudaError_t launch_obs(int prec, const GeoH& g, const void* U, const void* Ux, const void* Pq, const void* Dq,
-                       const void* F, double* partials, double* q_site, cudaStream_t st);
+                       const void* F, double* partials, double* q_site, StepDev* sd, cudaStream_t st);
 cudaError_t launch_obs_final(const GeoH& g, const double* partials, double beta, double th_re,
                              double th_im, ObsOut* out, cudaStream_t st);
 // Fused batch: one launch of family fam (ENS_*) over nw work items (device

@@ -2,7 +2,8 @@
 
 Fixed point has one absolute error for numbers of any size, so a field kept too small for its range loses bits that
 FP64 would keep.  The bounds are 1.5 times the rms error that an FP64 evaluation of the same formulas shows on these
-links (of the result's rms: drift 2.7e-16 at spread 0.27 and 2.5e-16 at 0.1, charge density 4.5e-16 and 6.0e-16)."""
+links (of the result's rms: drift 2.7e-16 at spread 0.27 and 2.5e-16 at 0.1, charge density 4.5e-16 and 6.0e-16; of
+smooth links 1.45e-15 and 3.8e-15 at 0.01, 1.8e-14 and 4.8e-14 at 0.001)."""
 import numpy as np
 import pytest
 
@@ -87,8 +88,8 @@ def drift(U, P, D, F, beta, theta):
     return X
 
 
-def links(spread, seed):
-    """SU(3) links exp(i spread h) with a non-unitary part of 0.012, det = 1."""
+def links(spread, seed, rough=0.012):
+    """SU(3) links exp(i spread h) with a non-unitary part of size rough, det = 1."""
     r = np.random.default_rng(seed)
 
     def gauss():
@@ -103,7 +104,7 @@ def links(spread, seed):
 
     h = gauss()
     h = expm(0.25j * spread * (h + h.conj().swapaxes(-1, -2)))
-    U = mm(expm(0.012 * gauss()), h, h, h, h)
+    U = mm(expm(rough * gauss()), h, h, h, h)
     return U * (np.linalg.det(U) ** (-1 / 3))[..., None, None]
 
 
@@ -121,3 +122,14 @@ def test_drift_and_charge_density_keep_double_precision(cl, spread, drift_bound,
             lat.set_links(U)
             assert rms(lat.drift() - drift(U.astype(LD), P, D, F, beta, theta), drift(U.astype(LD), P, D, F, beta, theta)) <= drift_bound
             assert rms(lat.qdensity() - q, q) <= density_bound
+
+
+@pytest.mark.parametrize("spread,rough,drift_bound,density_bound", [(0.01, 1e-4, 2.2e-15, 5.7e-15), (0.001, 1e-5, 2.7e-14, 7.2e-14)])
+def test_smooth_links_keep_double_precision(cl, spread, rough, drift_bound, density_bound):
+    U = links(spread, 1, rough)
+    P, D, F = fields(U.astype(LD))
+    X, q = drift(U.astype(LD), P, D, F, 6.0, 1.0), density(F)
+    with cl.Lattice(L, beta=6.0, theta=1.0) as lat:
+        lat.set_links(U)
+        assert rms(lat.drift() - X, X) <= drift_bound
+        assert rms(lat.qdensity() - q, q) <= density_bound
