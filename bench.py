@@ -67,14 +67,15 @@ def flop_model(prec, theta_on=True, n_taylor=15):
     expm = MUL + 6 + 72 + 36 + 16 * n_taylor + 9 * (6 + 8) + 6  # Cayley-Hamilton + Horner
     det_root = 64 + 19                                           # det + three-term cube-root series
     if theta_on and prec == "fp64":
-        force = 6 * (11 * MUL + 9 * MULACC + 162)                # per-plaquette drift, 6 planes, corner transport shared
+        # per-plaquette drift, 6 planes, corner transport shared, theta's scale on D, P and P^-1
+        force = 6 * (11 * MUL + 9 * MULACC + 162 + 3 * 54)
     elif theta_on:
         force = 6 * (12 * MUL + ADJ + 9 * MULACC + 162)
     else:
         force = 6 * (4 * MUL + 36)
     m = {
         "force": force,
-        "clover": 4 * ADJ + 6 * (3 * MUL + ADJ + 18) + (6 * ((2 if prec == "fp64" else 3) * (MUL + MULACC) + 54) if theta_on else 0),
+        "clover": 4 * ADJ + 6 * (3 * MUL + ADJ + 18) + (6 * (2 * (MUL + MULACC) if prec == "fp64" else 3 * (MUL + MULACC) + 54) if theta_on else 0),
         "cool_grad": 914,
         "cool_omega": 209,
         "cool_apply": 4 * 2 * HERM,
@@ -136,8 +137,9 @@ def dram_traffic(kernel, prec, V=None, path=None):
         return None
 
 
-# Kernels of each roofline family, per form (a family's bytes per launch sum
-# over its kernels: the split force runs a then b once per step).
+# Kernels of each roofline family, per form, under the names of launch lists taken
+# before the fixed-point kernels (a family's bytes per launch sum over its kernels:
+# the split force ran a then b once per step).
 TRAFFIC_FAMILIES = {
     "fp64": {"force": ("k_plaq_force_a<double>", "k_plaq_force_b<double>"),
              "update": ("k_update_gather<double, 0>",), "cool_apply": ("k_cool_apply_tiles<double>",),
@@ -152,12 +154,16 @@ TRAFFIC_FAMILIES = {
 }
 
 
-# The same under the kernels' present names (the ones above are those of older launch lists).
+# The same under the kernels' present names (one launch per lattice, the wide shape).
 TRAFFIC_FAMILIES_FX = {
     form: {"force": ("k_fx_force_t", "k_fx_force_a", "k_fx_force_b<%s>" % t), "update": ("k_fx_update<%s, 0>" % t,),
-           "cool_apply": ("k_cool_apply<%s, 1>" % t,), "cool_grad_omega": ("k_cool_grad_omega<%s, 3>" % t,)}
+           "cool_apply": ("k_cool_apply<%s, 1, 1>" % t,), "cool_grad_omega": ("k_cool_grad_omega<%s, 3>" % t,),
+           "cool_grad": ("k_cool_grad<%s, 1, 2>" % t,), "cool_omega": ("k_cool_omega<%s, 0>" % t,)}
     for form, t in (("fp64", "double"), ("df64", "df64"))}
-TRAFFIC_FAMILIES_FX["fp32"] = {"cool_apply": ("k_cool_apply<float, 1>",), "cool_grad_omega": ("k_cool_grad_omega<float, 4>",)}
+TRAFFIC_FAMILIES_FX["fp32"] = {
+    "force": ("k_plaq_force_ab<float>",), "update": ("k_update_gather<float, 0>",),
+    "cool_apply": ("k_cool_apply<float, 1, 1>",), "cool_grad_omega": ("k_cool_grad_omega<float, 4>",),
+    "cool_grad": ("k_cool_grad<float, 1, 4>",), "cool_omega": ("k_cool_omega<float, 0>",)}
 
 
 def ingest_ncu(path, out_json=None, capture_sites=None):

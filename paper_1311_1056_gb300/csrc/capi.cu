@@ -365,11 +365,11 @@ cl_status cl_init_lattice(const cl_params* params, void* cuda_stream, cl_lattice
   //    slot that stage b writes only after reading the partial back;
   //  * the cooling fields f (8 FP64 per site, [a][V]) and the packed
   //    Hermitian Omega, Omega^{-1} (9 reals per site each), then, on a
-  //    256-byte boundary, the single-pass apply's tile records (16 bytes per
-  //    tile, at most V / 128 + L3 tiles); used only by the cooling sweeps and
-  //    the start's gauge transformation, never while C holds drift
-  //    contributions.  They need at most 64 + 144 + 17 bytes per site plus
-  //    256, and C has 24 * 9 * 8 bytes per site or more.
+  //    256-byte boundary, the cooling kernels' records (32 bytes per 32 sites
+  //    and 160 bytes); used only by the cooling sweeps and the start's gauge
+  //    transformation, never while C holds drift contributions.  They need at
+  //    most 64 + 144 + 2 bytes per site plus 512, and C has 24 * 9 * 8 bytes
+  //    per site or more.
   {
     char* c = (char*)l->C;
     l->Gq = c + l->esz * 9 * Vs;
@@ -929,7 +929,6 @@ ChainDesc describe(const cl_lattice* l, double eps, const cl_cool_params& cp, bo
   c.f = l->f;
   c.Om = l->Om;
   c.Omi = l->Omi;
-  c.partials = l->partials;
   c.arec = l->crec;
   c.cs = l->cs;
   c.sd = l->sd;

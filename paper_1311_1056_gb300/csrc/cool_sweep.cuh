@@ -66,7 +66,7 @@ struct SweepArgs {
   void* Ux;
   double* f;
   void *Om, *Omi;
-  double2* rec;       // one record of four doubles per block
+  double2* rec;       // records of four doubles (sweep_grad_body)
   unsigned* ticket;   // blocks done, zero between launches
   CoolState* cs;
   CoolArgs ca;
@@ -605,7 +605,8 @@ __device__ __forceinline__ void sweep_grad_site(SweepSums& v, const SweepPart<L,
       double un;
       if (sweep_gradient(G, sm)) {
         long long o = 0;
-        fx_acc sq = fx_zero();  // sum (f / 4)^2
+        fx_acc sq = fx_zero();  // sum (f / 4)^2: six below 1, and the diagonal's two, which are
+                                // (sum d^2 - (sum d)^2 / 3) / 2 < 4 / 3 together: below 8
         fx_chk ck;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {

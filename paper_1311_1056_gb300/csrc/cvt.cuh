@@ -1,12 +1,9 @@
 // cvt.cuh -- float <-> double conversions on the integer pipe.
 //
 // On this GPU a conversion between float and double issues on the FP64 pipe
-// at that pipe's rate (two per SM per clock, the rate of a DFMA).  In the
-// FP32-storage form the FP64 pipe carries the exponentials, the det
-// re-projection and the reductions, and the conversions into and out of
-// them (the exponent into FP64, the exponential and the det factor back to
-// float, the product back to FP64 for its det) took about a fifth of that
-// pipe's issue slots.
+// at that pipe's rate (two per SM per clock, the rate of a DFMA).  The
+// FP32-storage form's sums of gradients, norms and observables widen a few
+// floats per site; done so, they keep off that pipe.
 //
 // IEEE-754 binary32 and binary64 differ only in field widths (8/23 vs 11/52
 // exponent/mantissa bits) and exponent bias (127 vs 1023).  So a normal

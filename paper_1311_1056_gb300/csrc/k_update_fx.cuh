@@ -480,6 +480,8 @@ __device__ __forceinline__ bool fx_traceless_quarter(mat<fx>& Q, const long long
   }
   return !ck.bad();
 }
+// (The constant 8 eps 2^cexp is held to 2^-57 like every number: at small eps that is
+// fewer bits of it than a double has, but times |Q| < 1.44 still below what A resolves.)
 // A = 2 eps (X - Tr X / 3) + i sqrt(eps) sqrt(2) g_a lambda_a from the traceless
 // quarter of X 2^-cexp and g / 8 (element j at gs[j TUNE_MAX_BLOCK]).  The noise constant 8 sqrt(2 eps) passes the fixed-point
 // bound at eps = 0.016, the drift's 8 eps 2^cexp at eps = 0.0112 for beta = 24 .. 48

@@ -59,7 +59,7 @@ struct ObsOut {
   double nonfinite;
 };
 
-enum { NQ_OBS = 9, NQ_COOL = 4, RED_THREADS = 128, RED_MAX_BLOCKS = 1216 };
+enum { NQ_OBS = 9, RED_THREADS = 128, RED_MAX_BLOCKS = 1216 };
 
 // One chain of a fused batch (the ensemble kernels below): its geometry (the
 // fields of lattice.cuh's Geo), device buffers and per-chain parameters.  U
@@ -68,7 +68,6 @@ enum { NQ_OBS = 9, NQ_COOL = 4, RED_THREADS = 128, RED_MAX_BLOCKS = 1216 };
 struct ChainDesc {
   int L[4], stride[4], V;
   void *U, *Un, *Ui, *Pq, *Dq, *F, *C, *Gq, *f, *Om, *Omi;
-  double* partials;
   double* arec;             // the cooling kernels' block records
   CoolState* cs;
   StepDev* sd;
