@@ -960,7 +960,7 @@ static __device__ __noinline__ double far_cool_apply(const Geo g, int4* Ux, int2
 }
 // A thread's next link and its two Omegas on their way into shared memory while
 // it works on the current ones (lattices where a block takes several groups:
-// apply of a 32^4 step of ten sweeps 4.03 -> 3.74 ms).
+// apply of a 32^4 step of ten sweeps 4.03 -> 3.74 ms; now 3.63).
 // Item k of a thread at sm[k CS_THREADS + thread]; a thread's own, no barrier.
 struct sweep_pipe {
   int4* sm;

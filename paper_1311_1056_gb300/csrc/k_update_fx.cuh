@@ -13,7 +13,7 @@
 // A fixed-point number's error is the same whatever its size, ~1e-17, so fields are
 // kept as large as the bounds allow.  (With F held times s 2^-e and C four times
 // smaller, errors against 80-bit arithmetic on links scattered by 0.27: drift at
-// theta = 1 1.3e-15 of its size, charge density 1.6e-15; now 1.7e-16 and 5.1e-16; FP64
+// theta = 1 1.3e-15 of its size, charge density 1.6e-15; now 1.5e-16 and 4.4e-16; FP64
 // arithmetic 2.7e-16 and 4.5e-16.)
 //
 // A thread whose inputs or results leave the fixed-point range calls the
@@ -42,7 +42,7 @@ __device__ __forceinline__ tagged tag_D(const int4* f) { return tagged{const_cas
 
 // The operands of the products come through an fx_pipe of two slots (fixed.cuh):
 // 32^4: plaquettes and clover field 2.60 -> 2.48 ms a step, observables 3.03 ->
-// 2.92 ms.
+// 2.92 ms (2.59 and 3.03 since their sums are the fine ones).
 const int FX_BLOCK = FX_PIPE_THREADS;  // largest block of the kernels that use it
 const int FX_PIPE = fx_pipe<2>::WORDS, FX_PARK_BYTES = (FX_PIPE + fx_park::WORDS) * (int)sizeof(int4);
 
@@ -57,7 +57,7 @@ __device__ __forceinline__ void fx_links_body(Geo g, const typename vec2_of<L>::
   mat<fx> x, xi;
   const bool in = fx_load_link<L>(x, U, mu, s, g.V);
   fx_chk ck;
-  fx_adj(xi, x, ck);
+  fx_adj<fx_acc_fine>(xi, x, ck);
   if (!in || ck.bad()) {  // readers of either turn to U itself
     x.e[0].re.l = fx_raw_mark();
     xi.e[0].re.l = fx_raw_mark();
@@ -94,12 +94,12 @@ __device__ __forceinline__ void fx_plaq_body(Geo g, const typename vec2_of<L>::t
   P.ask(Ui, mu, hop(g, s, x, nu, 1), g.V);
   P.take(b, ck);
   P.ask(Ui, nu, s, g.V);
-  fx_mul_left<FX_WIDE>(Pm, b, ck);
+  fx_mul_left<FX_WIDE, 0, fx_acc_fine>(Pm, b, ck);
   P.take(b, ck);
-  fx_mul_left<FX_WIDE>(Pm, b, ck);
+  fx_mul_left<FX_WIDE, 0, fx_acc_fine>(Pm, b, ck);
   P.take(b, ck);
-  fx_mul_left<FX_WIDE>(Pm, b, ck);
-  fx_adj(b, Pm, ck);
+  fx_mul_left<FX_WIDE, 0, fx_acc_fine>(Pm, b, ck);
+  fx_adj<fx_acc_fine>(b, Pm, ck);
   store<fx>(Pq, p, s, g.V, Pm);
 #pragma unroll
   for (int k = 0; k < 9; ++k) Pm.e[k] = cx<fx>{fx_half_diff(Pm.e[k].re, b.e[k].re), fx_half_diff(Pm.e[k].im, b.e[k].im)};
@@ -148,11 +148,11 @@ __device__ __forceinline__ void fx_clover_half_body(Geo g, const int4* __restric
   P.take(d, ck);
   P.ask(Dq, p, s, g.V);
   if (shift) fx_shift_up(d, shift);
-  fx_mul_left<FX_WIDE, 1>(w, d, ck);
+  fx_mul_left<FX_WIDE, 1, fx_acc_fine>(w, d, ck);
   P.take(d, ck);
   P.take(acc, ck);
   if (shift) fx_shift_up(acc, shift);
-  fx_mul_acc<FX_WIDE, +1, 1>(acc, w, d, ck);
+  fx_mul_acc<FX_WIDE, +1, 1, fx_acc_fine>(acc, w, d, ck);
   if (ck.bad()) acc.e[0].re.l = fx_raw_mark();  // its readers start over from D
   store<fx>(E, p, s, g.V, acc);
 }
@@ -177,10 +177,10 @@ __device__ __forceinline__ void fx_clover_body(Geo g, const typename vec2_of<L>:
   P.ask(Ux, nu, xmn, g.V);
   P.take(d, ck);
   P.ask(E, p, s, g.V);
-  fx_mul_left<FX_WIDE, 1>(w, d, ck);
+  fx_mul_left<FX_WIDE, 1, fx_acc_fine>(w, d, ck);
   P.take(d, ck);
   P.take(acc, ck);
-  fx_mul_acc<FX_WIDE, +1, 1>(acc, w, d, ck);
+  fx_mul_acc<FX_WIDE, +1, 1, fx_acc_fine>(acc, w, d, ck);
   if (neg) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc.e[k] = cx<fx>{-acc.e[k].re, -acc.e[k].im};

@@ -33,10 +33,11 @@ inline dim3 grid(int V, int planes, int bs) { return dim3((unsigned)(((V + bs - 
 // Resident blocks of 128 threads that the kernels are built for.  Three (168
 // registers) for the plaquettes and the clover field, whose operands come
 // through the pipe.  Two (255, next to nothing spilled) for the theta force's
-// stages a and b: with the pipe to hide the loads, 5.68 ms per 32^4 step; three blocks
-// spill ~470 bytes a thread and take 6.34 ms without the pipe, 6.98 ms with it
+// stages a and b: 5.68 ms per 32^4 step when this was chosen (with the transport pass; now,
+// with the theta scale applied here, 6.17); three blocks
+// spill ~470 bytes a thread and took 6.34 ms without the pipe, 6.98 ms with it
 // (its slots are the spills' L1).  FP64 arithmetic took 26.0 ms, plaquettes and
-// clover field 11.95 (now 2.48).
+// clover field 11.95 (now 2.59).
 const int FX_BLOCKS_SM = 3, FX_BLOCKS_FORCE = 2;
 template <typename L>
 __global__ void __launch_bounds__(TUNE_MAX_BLOCK) k_fx_links(Geo g, const typename vec2_of<L>::type* __restrict__ U, int4* Ux, int4* Ui,
