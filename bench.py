@@ -461,7 +461,7 @@ def native(args):
                    "beta": WORKLOAD["beta"], "theta": WORKLOAD["theta"], "eps": WORKLOAD["eps"],
                    "cooling": "alpha_ad = alpha / D_1 (normalised unitarity norm), alpha 1, "
                               "10 sweeps per step (fixed count)",
-                   "precision": "fp64 links; products, noise and exponentials in 60-bit fixed point, errors below fp64's",
+                   "precision": "fp64 links; products, noise and exponentials in 60-bit fixed point, rounding errors of fp64's size or below",
                    "l2": "no flush: the link fields (604 MB fp64 / 302 MB fp32) exceed the 129 MB L2",
                    "parallelism": "replicas x%d (independent chains)" % ws},
         "gpu_launches": launches,

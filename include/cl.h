@@ -30,8 +30,12 @@
  *    A lattice is not thread-safe: one host thread per lattice at a time.
  *  - Precision (cl_precision): CL_FP64 keeps links in FP64; its matrix
  *    products, noise and exponentials run in 60-bit fixed point with FP32
- *    low-order terms (errors at or below FP64's for links near SU(3); wherever
- *    a number leaves the fixed-point range, in FP64), the rest in FP64.
+ *    low-order terms, wherever a number leaves the fixed-point range in FP64,
+ *    the rest in FP64.  Rounding errors are at or below those of FP64
+ *    arithmetic, but for a site's charge density (up to 1.2 times, by the
+ *    size of the field) and the theta drift alone at beta = 0 (up to 2.6
+ *    times).  A CL step of links far from SU(3) (unitarity norm above ~1.1)
+ *    takes up to 7 times as long as one near it, in CL_DF64 up to 8.
  *    CL_FP32_STORAGE stores and multiplies links in FP32; the matrix
  *    exponentials of the Langevin and cooling updates and the det U = 1
  *    re-projection keep FP64's precision, every global reduction is FP64.

@@ -947,7 +947,7 @@ ChainDesc describe(const cl_lattice* l, double eps, const cl_cool_params& cp, bo
 // One fused step of every chain, enqueued on st from descriptor table cd.
 // Each chain runs exactly the kernels and the order of its own step: the CL
 // step (force by theta, update by step-size mode), then its cooling sweeps,
-// single-pass for D_0 / D_1 and four kernels otherwise, up to the largest
+// single-pass for D_0 / D_1 and three kernels otherwise, up to the largest
 // sweep count of the batch (a chain's own rule marks it done at its count;
 // later launches skip its blocks).  Returns the number of launches.
 cl_status enqueue_fused_step(const cl_batch* b, const FusedPlan& P, const ChainDesc* cd, const WorkItem* w,
